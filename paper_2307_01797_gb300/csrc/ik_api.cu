@@ -957,9 +957,17 @@ int itokmc_init(const itokmc_config* cfg, itokmc_handle** out)
         L.h = P.h[0] * (double)(n / m);
         L.phi = dalloc_n<double>(h, cells, &rc);
         L.rhs = dalloc_n<double>(h, cells, &rc);
-        L.res = nullptr;
         L.phi32 = dalloc_n<float>(h, cells, &rc);
         L.rhs32 = dalloc_n<float>(h, cells, &rc);
+        const bool f64 = h->field_prec == ITOKMC_FP64;
+        L.alt = m > 32 ? dalloc(h, cells * (f64 ? sizeof(double) : sizeof(float)), &rc) : nullptr;
+        L.phi_fix = reinterpret_cast<long long*>(L.phi);
+        L.rhs_fix = reinterpret_cast<long long*>(L.rhs);
+        if (l == 0 && f64) {
+            L.phi_fix = dalloc_n<long long>(h, cells, &rc);
+            L.rhs_fix = dalloc_n<long long>(h, cells, &rc);
+            d.fix = dalloc_n<ik::FixScale>(h, 1, &rc);
+        }
     }
     d.nlev = l;
     const size_t nb = (size_t)R * n * n * n / 256 + 16;
@@ -967,7 +975,7 @@ int itokmc_init(const itokmc_config* cfg, itokmc_handle** out)
     d.norm_out = dalloc_n<double>(h, 2 * R, &rc);
     if (!rc && cudaMallocHost(reinterpret_cast<void**>(&h->rb), sizeof(*h->rb)) != cudaSuccess)
         rc = fail(h, ITOKMC_ERR_OOM, "pinned host buffer");
-    if (!rc && cudaMallocHost(reinterpret_cast<void**>(&d.norm_host), 2 * R * sizeof(double)) != cudaSuccess)
+    if (!rc && cudaMallocHost(reinterpret_cast<void**>(&d.norm_host), (2 * R + ik::FIX_DOUBLES) * sizeof(double)) != cudaSuccess)
         rc = fail(h, ITOKMC_ERR_OOM, "pinned host buffer");
     for (int e = 0; e < 8 && !rc; ++e)
         if (cudaEventCreate(&h->ev[e]) != cudaSuccess) rc = fail(h, ITOKMC_ERR_CUDA, "event create");
@@ -1238,10 +1246,10 @@ int itokmc_autotune(itokmc_handle* h, itokmc_tuning* out)
                 best_cyc = cyc;
             }
         }
-    // restore the potential and the field of the initial state
+    // restore the potential of the initial state (the trials form no field)
     IK_CHECK(h, cudaMemcpyAsync(phi0, d.stage, cells * sizeof(double), cudaMemcpyDeviceToDevice, h->s));
     d.phi_F = F0;
-    ik::launch_efield(h->P, d, h->s);
+    d.fix_result = false;                // the trials' potential is dropped
     IK_CHECK(h, cudaStreamSynchronize(h->s));
     if (best < 0) return fail(h, ITOKMC_ERR_NOCONV, "autotune: no smoother pair converged");
     h->cfg.mg_nu1 = t.nu_tried[best][0];

@@ -9,15 +9,20 @@
 // restriction, trilinear cell-centred prolongation, and a one-block
 // red-black solve at the bottom (the paper uses BiCGSTAB there).
 //
-// Two forms: FP64 V-cycles on the FP64 system, or FP32 V-cycles on the
-// correction equation inside FP64 residual iterative refinement
-// (phi += V32(b - A phi) until the FP64 residual meets the tolerance).
+// Two forms: V-cycles on the system in 64-bit fixed point (the FP64 form; with
+// FP64 V-cycles where the integers' range does not serve), or FP32 V-cycles
+// on the correction equation inside residual iterative refinement
+// (phi += V32(b - A phi) until the residual meets the tolerance).
 // Realizations are stacked (slowest index) and solved together; each has
 // its own convergence test.  Norms are reduced in a fixed order.
 #include <algorithm>
 #include <cmath>
 #include <cstdio>
+#include <cstring>
 #include <mutex>
+#include <type_traits>
+
+#include <cooperative_groups.h>
 
 #include "../../include/itokmc.h"
 #include "ik_common.cuh"
@@ -26,6 +31,8 @@
 namespace ik {
 
 namespace {
+
+namespace cg = cooperative_groups;
 
 struct Geo {      // one level, all realizations
     int n, log2n, R;
@@ -74,19 +81,85 @@ __device__ __forceinline__ T diag_val(int d)
     }
 }
 
-// 1/diag for the diagonal counts 1..8 (a multiply instead of a divide).
+// 1/diag for the diagonal counts 4..9 (a multiply instead of a divide).
 template <class T>
 __device__ __forceinline__ T inv_diag(int d)
 {
-    switch (d) {
-    case 4: return (T)(1.0 / 4.0);
-    case 5: return (T)(1.0 / 5.0);
-    case 6: return (T)(1.0 / 6.0);
-    case 7: return (T)(1.0 / 7.0);
-    case 8: return (T)(1.0 / 8.0);
-    case 9: return (T)(1.0 / 9.0);
-    default: return (T)1 / (T)d;
+    if (d == 6) return (T)(1.0 / 6.0);
+    return d == 5 ? (T)(1.0 / 5.0) : d == 7 ? (T)(1.0 / 7.0) : d == 4 ? (T)(1.0 / 4.0) : d == 8 ? (T)(1.0 / 8.0) : (T)(1.0 / 9.0);
+}
+
+// The arithmetic of the multigrid on values of type T.  float and double round
+// each operation in the order written.  long long is the fixed-point form of
+// the FP64 solve (see field_solve): sums are exact, the relaxed value and the
+// interpolated correction are rounded to the nearest unit.  GB300 has 2 FP64
+// lanes per SM and clock and 64 or more integer ones, so a relaxed cell costs
+// about 30 integer instructions in the place of 7 FP64 ones that occupy the
+// pipe for as long as 220.
+template <class T>
+struct MG {
+    static __device__ __forceinline__ T relax(T sum, T rhs, int diag) { return (sum - rhs) * inv_diag<T>(diag); }
+    static __device__ __forceinline__ T resid(T sum, T rhs, T phi, int diag) { return fma(diag_val<T>(diag), phi, rhs - sum); }
+    static __device__ __forceinline__ T half(T acc) { return acc * (T)0.5; }
+    static __device__ __forceinline__ T axpy3(T a, T b) { return fma((T)3, a, b); }
+    static __device__ __forceinline__ T div64(T a) { return a * (T)(1.0 / 64.0); }
+};
+template <>
+struct MG<long long> {
+    // t / d to within a unit for |t| < 2^62: the product with floor(2^63 / d) =
+    // mh 2^32 + ml (ml signed), without the product of the low halves
+    static __device__ __forceinline__ long long mul(long long t, int mh, int ml)
+    {
+        const int th = (int)(t >> 32);
+        const unsigned tl = (unsigned)t;
+        const long long mid = (long long)th * ml + (long long)((unsigned long long)tl * (unsigned)mh);
+        return (((long long)th * mh) << 1) + (mid >> 31);
     }
+    static __device__ __forceinline__ void magic(int diag, int& mh, int& ml)
+    {
+        mh = diag == 6 ? 0x15555555 : diag == 5 ? 0x1999999a : diag == 7 ? 0x12492492
+           : diag == 4 ? 0x20000000 : diag == 8 ? 0x10000000 : 0x0e38e38e;
+        ml = diag == 6 ? 0x55555555 : diag == 5 ? -0x66666667 : diag == 7 ? 0x49249249 : diag == 9 ? 0x38e38e38 : 0;
+    }
+    static __device__ __forceinline__ long long relax(long long sum, long long rhs, int diag)
+    {
+        int mh, ml;
+        magic(diag, mh, ml);
+        return mul(sum - rhs + 3, mh, ml);
+    }
+    static __device__ __forceinline__ long long resid(long long sum, long long rhs, long long phi, int diag)
+    {
+        return rhs - sum + (long long)diag * phi;
+    }
+    static __device__ __forceinline__ long long half(long long acc) { return (acc + 1) >> 1; }
+    static __device__ __forceinline__ long long axpy3(long long a, long long b) { return a + (a << 1) + b; }
+    static __device__ __forceinline__ long long div64(long long a) { return (a + 32) >> 6; }
+};
+
+// A cell's divisor prepared for several relaxations.
+template <class T>
+struct Inv {
+    T v;
+    __device__ __forceinline__ Inv() {}
+    __device__ __forceinline__ explicit Inv(int d) : v(inv_diag<T>(d)) {}
+    __device__ __forceinline__ T relax(T sum, T rhs) const { return (sum - rhs) * v; }
+};
+template <>
+struct Inv<long long> {
+    int mh, ml;
+    __device__ __forceinline__ Inv() {}
+    __device__ __forceinline__ explicit Inv(int d) { MG<long long>::magic(d, mh, ml); }
+    __device__ __forceinline__ long long relax(long long sum, long long rhs) const
+    {
+        return MG<long long>::mul(sum - rhs + 3, mh, ml);
+    }
+};
+
+// Diagonal count of cell (i, j, k): 6, one less per Neumann side face, one
+// more per electrode face.
+__device__ __forceinline__ int diag_count(int i, int j, int k, int n)
+{
+    return 6 - (i == 0) - (i == n - 1) - (j == 0) - (j == n - 1) + (k == 0) + (k == n - 1);
 }
 
 template <class T>
@@ -104,7 +177,7 @@ __global__ void k_smooth(T* __restrict__ phi, const T* __restrict__ rhs, Geo G, 
         const uint64_t idx = ((r * n + k) * n + j) * n + i;
         int diag;
         const T s = nbr_sum(phi, idx, n, i, j, k, diag);
-        phi[idx] = (s - rhs[idx]) * inv_diag<T>(diag);
+        phi[idx] = MG<T>::relax(s, rhs[idx], diag);
     }
 }
 
@@ -112,8 +185,8 @@ __global__ void k_smooth(T* __restrict__ phi, const T* __restrict__ rhs, Geo G, 
 // into the coarse right-hand side.  Every level stores h^2 b (the multigrid
 // systems are scaled by h^2), so the coarse value h_c^2 mean(r) is half the
 // sum of the children's h_f^2 r = h_f^2 b - (neighbour sum - diag phi).
-template <class T, class TC>
-__global__ void k_resid_restrict(const T* __restrict__ phi, const T* __restrict__ rhs, TC* __restrict__ rhs_c,
+template <class T>
+__global__ void k_resid_restrict(const T* __restrict__ phi, const T* __restrict__ rhs, T* __restrict__ rhs_c,
                                  Geo Gc, int nf)
 {
     for (uint64_t t = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; t < Gc.cells; t += (uint64_t)gridDim.x * blockDim.x) {
@@ -126,9 +199,9 @@ __global__ void k_resid_restrict(const T* __restrict__ phi, const T* __restrict_
             const uint64_t idx = (((uint64_t)r * nf + k) * nf + j) * nf + i;
             int diag;
             const T s = nbr_sum(phi, idx, nf, i, j, k, diag);
-            acc += fma(diag_val<T>(diag), phi[idx], rhs[idx] - s);
+            acc += MG<T>::resid(s, rhs[idx], phi[idx], diag);
         }
-        rhs_c[t] = (TC)(acc * (T)0.5);
+        rhs_c[t] = MG<T>::half(acc);
     }
 }
 
@@ -136,7 +209,7 @@ __global__ void k_resid_restrict(const T* __restrict__ phi, const T* __restrict_
 // weights 3/4, 1/4 per axis written as (3 a + b) / 4 with fused multiply-
 // adds (ghosts: Neumann e, Dirichlet -e, i.e. (3 a - a) / 4 in z).
 template <class T>
-__device__ __forceinline__ T prolong_at(const T* __restrict__ ec, int nc, int i, int j, int k)
+__device__ __forceinline__ T prolong_at(const T* __restrict__ ec, int nc, int i, int j, int k, int z0 = 0)
 {
     const int I = i >> 1, J = j >> 1, K = k >> 1;
     int I2 = I + ((i & 1) ? 1 : -1), J2 = J + ((j & 1) ? 1 : -1), K2 = K + ((k & 1) ? 1 : -1);
@@ -144,19 +217,19 @@ __device__ __forceinline__ T prolong_at(const T* __restrict__ ec, int nc, int i,
     if (I2 < 0 || I2 >= nc) I2 = I;
     if (J2 < 0 || J2 >= nc) J2 = J;
     if (K2 < 0 || K2 >= nc) { K2 = K; sz = (T)-1; }
-    const int iz[2] = { K, K2 }, iy[2] = { J, J2 };
+    const int iz[2] = { K - z0, K2 - z0 }, iy[2] = { J, J2 };
     T m[2];
 #pragma unroll
     for (int c = 0; c < 2; ++c) {
         T q[2];
 #pragma unroll
         for (int b = 0; b < 2; ++b) {
-            const T* row = ec + ((uint64_t)iz[c] * nc + iy[b]) * nc;
-            q[b] = fma((T)3, row[I], row[I2]);
+            const T* row = ec + ((int64_t)iz[c] * nc + iy[b]) * nc;
+            q[b] = MG<T>::axpy3(row[I], row[I2]);
         }
-        m[c] = fma((T)3, q[0], q[1]);
+        m[c] = MG<T>::axpy3(q[0], q[1]);
     }
-    return fma((T)3, m[0], sz * m[1]) * (T)(1.0 / 64.0);
+    return MG<T>::div64(MG<T>::axpy3(m[0], sz < (T)0 ? -m[1] : m[1]));
 }
 
 template <class T>
@@ -168,32 +241,6 @@ __global__ void k_prolong(T* __restrict__ phi_f, const T* __restrict__ e_c, Geo 
         decode(t, Gf.log2n, r, k, j, i);
         phi_f[t] += prolong_at(e_c + (uint64_t)r * nc * nc * nc, nc, i, j, k);
     }
-}
-
-// Bottom solve: one block per realization, red-black sweeps in shared memory.
-template <class T>
-__global__ void k_bottom(T* __restrict__ phi, const T* __restrict__ rhs, int n, int sweeps)
-{
-    extern __shared__ unsigned char smem_raw[];
-    T* s = reinterpret_cast<T*>(smem_raw);
-    T* b = s + n * n * n;
-    const int cells = n * n * n;
-    const uint64_t base = (uint64_t)blockIdx.x * cells;
-    for (int c = threadIdx.x; c < cells; c += blockDim.x) { s[c] = phi[base + c]; b[c] = rhs[base + c]; }
-    __syncthreads();
-    for (int it = 0; it < sweeps; ++it) {
-        for (int color = 0; color < 2; ++color) {
-            for (int c = threadIdx.x; c < cells; c += blockDim.x) {
-                const int i = c % n, j = (c / n) % n, k = c / (n * n);
-                if (((i + j + k) & 1) != color) continue;
-                int diag;
-                const T sum = nbr_sum(s, (uint64_t)c, n, i, j, k, diag);
-                s[c] = (sum - b[c]) * inv_diag<T>(diag);
-            }
-            __syncthreads();
-        }
-    }
-    for (int c = threadIdx.x; c < cells; c += blockDim.x) phi[base + c] = s[c];
 }
 
 // FP64 residual, its squared norm per block (fixed order), and optionally
@@ -357,6 +404,203 @@ __global__ void k_efield_fixed(const long long* __restrict__ Phi, E64* __restric
     }
 }
 
+// ---- the FP64 form's fixed-point cycles
+// The FP64 solve runs its V-cycles on 64-bit integers: Phi = phi 2^F and B =
+// h^2 b 2^F, |Phi| below 2^57 (2^-57 of the bound on |phi|, FP64 keeps 2^-53
+// of the value), with the relaxations, residuals and transfers of MG<long
+// long>.  The potential is FP64 before and after (the start guess, the
+// checkpoint, itokmc_read_densities).  FIX_LIM marks an iterate that left its
+// range: the solve then goes on with FP64 cycles.
+constexpr long long FIX_LIM = 1ll << 59;
+
+// x 2^F rounded to the nearest integer, |x| 2^F < 2^62, by integer steps.
+__device__ __forceinline__ long long to_fixed(double x, int F)
+{
+    const long long b = __double_as_longlong(x);
+    const int e = (int)((b >> 52) & 0x7ff);
+    if (e == 0) return 0;                                       // zero (or subnormal)
+    const long long m = (b & 0xfffffffffffffll) | (1ll << 52);
+    const int sh = e - 1075 + F;
+    const long long v = sh >= 0 ? m << sh : (sh < -54 ? 0ll : (m + (1ll << (-sh - 1))) >> -sh);
+    return b < 0 ? -v : v;
+}
+
+// The start guess (extrapolated in time when asked) and the largest |guess|
+// and |h^2 b| (the electrode's share of the top layer's b taken out), as the
+// bits of the non-negative doubles.
+__global__ void __launch_bounds__(256) k_fix_start(double* __restrict__ phi, double* __restrict__ prev, int extrapolate,
+                                                   int have, const double* __restrict__ rhs, Geo G, double bc,
+                                                   FixScale* __restrict__ fs)
+{
+    unsigned long long mp = 0, mb = 0;
+    for (uint64_t t = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; t < G.cells; t += (uint64_t)gridDim.x * blockDim.x) {
+        double v = phi[t];
+        if (extrapolate) {
+            const double old = v;
+            if (have) {
+                v = (v + v) - prev[t];
+                phi[t] = v;
+            }
+            prev[t] = old;
+        }
+        double b = rhs[t];
+        if (((t >> (2 * G.log2n)) & (uint64_t)(G.n - 1)) == (uint64_t)(G.n - 1)) b += bc;
+        const unsigned long long vb = (unsigned long long)__double_as_longlong(v) & 0x7fffffffffffffffull,
+                                 bb = (unsigned long long)__double_as_longlong(b) & 0x7fffffffffffffffull;
+        mp = vb > mp ? vb : mp;
+        mb = bb > mb ? bb : mb;
+    }
+#pragma unroll
+    for (int d = 16; d > 0; d >>= 1) {
+        const unsigned long long a = __shfl_xor_sync(0xffffffffu, mp, d), c = __shfl_xor_sync(0xffffffffu, mb, d);
+        mp = a > mp ? a : mp;
+        mb = c > mb ? c : mb;
+    }
+    __shared__ unsigned long long sp[8], sb[8];
+    if ((threadIdx.x & 31) == 0) { sp[threadIdx.x >> 5] = mp; sb[threadIdx.x >> 5] = mb; }
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        for (int w = 1; w < 8; ++w) {
+            mp = sp[w] > mp ? sp[w] : mp;
+            mb = sb[w] > mb ? sb[w] : mb;
+        }
+        atomicMax(&fs->max_phi, mp);
+        atomicMax(&fs->max_b, mb);
+    }
+}
+
+// The scale.  Mc bounds |phi| of the solution: electrode potential plus the
+// 1D Dirichlet bound max|h^2 b| n^2 / 8, doubled.  A guess extrapolated from
+// the last steps is near the solution: four times its modulus bounds it (Mc
+// is loose by orders of magnitude for a localised charge).  use64: the guess
+// is not finite or far above the solution.
+__global__ void k_fix_scale(FixScale* fs, double phi_top, int n, int near, int sh)
+{
+    if (sh) {                                                   // a rescaling of a running solve
+        fs->F += sh;
+    } else {
+        const double mp = __longlong_as_double((long long)fs->max_phi), mb = __longlong_as_double((long long)fs->max_b);
+        const double Mc = 2.0 * (fabs(phi_top) + mb * (double)n * (double)n / 8.0);
+        double M = near && mp * 16384.0 >= Mc ? fmin(Mc, fmax(4.0 * mp, 2.0 * (mb + fabs(phi_top)))) : fmax(Mc, 2.0 * mp);
+        M = fmax(M, 0x1p-400);
+        fs->use64 = !(mp <= 16.0 * Mc) || !(Mc < 0x1p400);
+        if (!(M < 0x1p400)) M = 1.0;
+        fs->F = 57 - (ilogb(M) + 1);
+    }
+    fs->max_fix = 0;
+    fs->down = scalbn(1.0, -fs->F);
+    fs->top = to_fixed(phi_top, fs->F);
+}
+
+// Phi and B from phi and the right-hand side (sh = 0), or Phi shifted up by
+// sh bits and B formed again at the new scale.
+__global__ void k_fix_load(const double* __restrict__ phi, const double* __restrict__ rhs, long long* __restrict__ Phi,
+                           long long* __restrict__ B, uint64_t cells, const FixScale* __restrict__ fs, int sh)
+{
+    const int F = fs->F;
+    if (fs->use64) return;
+    for (uint64_t t = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; t < cells; t += (uint64_t)gridDim.x * blockDim.x) {
+        Phi[t] = sh ? Phi[t] << sh : to_fixed(phi[t], F);
+        B[t] = to_fixed(rhs[t], F);
+    }
+}
+
+// The potential back in FP64.
+__global__ void k_fix_store(const long long* __restrict__ Phi, double* __restrict__ phi, uint64_t cells,
+                            const FixScale* __restrict__ fs)
+{
+    const double sc = fs->down;
+    for (uint64_t t = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; t < cells; t += (uint64_t)gridDim.x * blockDim.x)
+        phi[t] = (double)Phi[t] * sc;
+}
+
+// Squared norms of the exact integer residual and of B (units of 2^30 steps:
+// FP32 holds their squares), summed as in k_resid_fixed, and the largest
+// |Phi|.  The norms serve the convergence test alone.
+__global__ void __launch_bounds__(NORM_TPB) k_resid_norm_fix(const long long* __restrict__ Phi,
+                                                             const long long* __restrict__ B, Geo G,
+                                                             double* __restrict__ part, int with_b, int items,
+                                                             FixScale* __restrict__ fs)
+{
+    __shared__ double red[NORM_TPB / 32][2];
+    __shared__ unsigned long long redm[NORM_TPB / 32];
+    const uint64_t base = ((uint64_t)blockIdx.x * NORM_TPB) * items;
+    float acc = 0.f, bacc = 0.f;
+    unsigned long long mx = 0;
+    for (int q = 0; q < items; ++q) {
+        const uint64_t t = base + (uint64_t)q * NORM_TPB + threadIdx.x;
+        if (t >= G.cells) break;
+        int r, k, j, i;
+        decode(t, G.log2n, r, k, j, i);
+        int diag;
+        const long long s = nbr_sum(Phi, t, G.n, i, j, k, diag);
+        const long long pc = Phi[t], b = B[t];
+        const unsigned long long ap = (unsigned long long)(pc < 0 ? -pc : pc);
+        mx = ap > mx ? ap : mx;
+        const float res = __ll2float_rn(MG<long long>::resid(s, b, pc, diag)) * 0x1p-30f;
+        acc = __fmaf_rn(res, res, acc);
+        if (with_b) {
+            const float bf = __ll2float_rn(b) * 0x1p-30f;
+            bacc = __fmaf_rn(bf, bf, bacc);
+        }
+    }
+    double a = fs->use64 || mx >= (unsigned long long)FIX_LIM ? (double)INFINITY : (double)acc, bb = (double)bacc;
+#pragma unroll
+    for (int d = 16; d > 0; d >>= 1) {
+        a += __shfl_xor_sync(0xffffffffu, a, d);
+        bb += __shfl_xor_sync(0xffffffffu, bb, d);
+        const unsigned long long o = __shfl_xor_sync(0xffffffffu, mx, d);
+        mx = o > mx ? o : mx;
+    }
+    if ((threadIdx.x & 31) == 0) { red[threadIdx.x >> 5][0] = a; red[threadIdx.x >> 5][1] = bb; redm[threadIdx.x >> 5] = mx; }
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        double x = 0.0, y = 0.0;
+        for (int w = 0; w < NORM_TPB / 32; ++w) {
+            x += red[w][0];
+            y += red[w][1];
+            mx = redm[w] > mx ? redm[w] : mx;
+        }
+        part[2 * (uint64_t)blockIdx.x] = x;
+        part[2 * (uint64_t)blockIdx.x + 1] = y;
+        atomicMax(&fs->max_fix, mx);
+    }
+}
+
+// E = -grad(phi) from the fixed-point potential (exact integer differences
+// times 2^-F / 2h) into E, and the potential itself in FP64.
+__global__ void k_efield_fix(const long long* __restrict__ Phi, E64* __restrict__ E, float4* __restrict__ E32,
+                             double* __restrict__ phi, Geo G, double inv2h, const FixScale* __restrict__ fs)
+{
+    if (fs->use64) return;                        // nothing was solved here (replayed steps: the host solves again)
+    const double down = fs->down, sc = down * inv2h;
+    const float inv2hf = (float)inv2h;
+    const long long top2 = 2 * fs->top;
+    for (uint64_t t = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; t < G.cells; t += (uint64_t)gridDim.x * blockDim.x) {
+        int r, k, j, i;
+        decode(t, G.log2n, r, k, j, i);
+        const int n = G.n;
+        const uint64_t sy = (uint64_t)n, sz = (uint64_t)n * n;
+        const long long c = Phi[t];
+        const long long xm = i > 0 ? Phi[t - 1] : c, xp = i < n - 1 ? Phi[t + 1] : c;
+        const long long ym = j > 0 ? Phi[t - sy] : c, yp = j < n - 1 ? Phi[t + sy] : c;
+        const long long zm = k > 0 ? Phi[t - sz] : -c, zp = k < n - 1 ? Phi[t + sz] : top2 - c;
+        phi[t] = (double)c * down;
+        if (E) {
+            const double ex = (double)(xm - xp) * sc, ey = (double)(ym - yp) * sc, ez = (double)(zm - zp) * sc;
+            const double m = sqrt((ex * ex + ey * ey) + ez * ez);
+            reinterpret_cast<double2*>(E + t)[0] = make_double2(ex, ey);
+            reinterpret_cast<double2*>(E + t)[1] = make_double2(ez, m);
+            if (E32) E32[t] = make_float4((float)ex, (float)ey, (float)ez, (float)m);
+        } else {
+            // as k_efield: differences in FP64, scaling and |E| in FP32
+            const float ex = (float)((double)(xm - xp) * down) * inv2hf, ey = (float)((double)(ym - yp) * down) * inv2hf,
+                        ez = (float)((double)(zm - zp) * down) * inv2hf;
+            E32[t] = make_float4(ex, ey, ez, sqrtf(ex * ex + ey * ey + ez * ez));
+        }
+    }
+}
+
 // B = round(b h^2 2^F) with b formed exactly as the FP64 right-hand side.
 __global__ void k_rhs_fixed(const int64_t* __restrict__ rho, long long* __restrict__ B, Geo G, double qscale,
                             double bc_top, double bfix)
@@ -377,13 +621,12 @@ __global__ void k_shift_fixed(long long* __restrict__ Phi, int sh, uint64_t cell
         Phi[t] = (Phi[t] + half) >> sh;
 }
 
-// phi <- 2 phi - prev, prev <- the old phi (with no previous potential yet:
-// prev <- phi only).
-template <class T>
-__global__ void k_extrapolate(T* __restrict__ phi, T* __restrict__ prev, uint64_t cells, bool have)
+// Phi <- 2 Phi - prev, prev <- the old Phi (with no previous potential yet:
+// prev <- Phi only).
+__global__ void k_extrapolate(long long* __restrict__ phi, long long* __restrict__ prev, uint64_t cells, bool have)
 {
     for (uint64_t t = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; t < cells; t += (uint64_t)gridDim.x * blockDim.x) {
-        const T v = phi[t];
+        const long long v = phi[t];
         if (have) phi[t] = (v + v) - prev[t];
         prev[t] = v;
     }
@@ -393,13 +636,6 @@ __global__ void k_phi_to_double(const long long* __restrict__ Phi, double* __res
 {
     for (uint64_t t = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; t < cells; t += (uint64_t)gridDim.x * blockDim.x)
         out[t] = (double)Phi[t] * sc;
-}
-
-template <class T>
-__global__ void k_zero(T* __restrict__ a, uint64_t cells)
-{
-    for (uint64_t t = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; t < cells; t += (uint64_t)gridDim.x * blockDim.x)
-        a[t] = (T)0;
 }
 
 // E = -grad(phi) by centred differences with the boundary ghosts, and |E|.
@@ -450,91 +686,469 @@ Geo geo(const Dev& d, int l, int R)
 }
 
 // ---------------------------------------------------------------------------
-// The coarse end of the V-cycle (levels of at most 16^3 cells) in one launch:
-// one block per realization runs pre-smoothing, residual restriction, the
-// bottom sweeps, prolongation and post-smoothing level by level, with block
-// barriers between the phases (the arrays are tiny and stay in cache).
-constexpr int COARSE_N = 16;
+// The coarse end of the V-cycle (levels of at most 32^3 cells) in one launch:
+// a cluster of 8 blocks per realization.  The 32^3 and 16^3 levels are split
+// into slabs of n/8 planes.  A thread owns an x pair of cells in every plane
+// of its block's slab and keeps their values, right-hand sides and divisors
+// in registers; the values also lie in shared memory, one array per colour
+// with a rim of zeros, for the neighbours in x and y.  A half-sweep stores the
+// slab's two outer planes into the neighbour blocks' halo planes (distributed
+// shared memory) and ends with a cluster barrier.  The 8^3 level runs in the
+// cluster's first block, the 4^3 bottom (48 red-black sweep pairs) in one warp
+// with the cells in registers.  What bounds it is a chain of latencies (21
+// cluster barriers, 96 warp half-sweeps), not bandwidth: 39 us in fixed point,
+// 31 us in FP32 from 32^3 down; one block per realization from 16^3 down took
+// 159 us in FP64 and 96 us in FP32, after 10 launches for the 32^3 level.
+constexpr int COARSE_N = 32, COARSE_CL = 8, COARSE_TPB = 512, BOTTOM_SWEEPS = 48;
 
-struct CoarseLevels {
-    int nlev;            // levels in the fused range, finest first
-    int n[MAX_LEVELS];
-    void* phi[MAX_LEVELS];
-    void* rhs[MAX_LEVELS];
+template <class T>
+struct CoarseTop {       // the level the kernel starts at (n <= COARSE_N)
+    T* phi;
+    const T* rhs;
+    int n;
+};
+
+// One half-sweep of the 4^3 level by one warp: a lane holds the colour-0 and
+// the colour-1 cell of the x pair (2 ih, 2 ih + 1) of its row, five shuffles
+// bring the neighbours of the relaxed one (other: the lane's cell of the other
+// colour; xl the lane of the x neighbour outside the pair).
+template <class T>
+__device__ __forceinline__ T bottom_update(T other, T rhs, const Inv<T>& inv, int xl, unsigned ok, unsigned lane)
+{
+    const unsigned full = 0xffffffffu;
+    const T xo = __shfl_sync(full, other, xl);
+    const T ym = __shfl_sync(full, other, lane - 2), yp = __shfl_sync(full, other, lane + 2);
+    const T zm = __shfl_sync(full, other, lane - 8), zp = __shfl_sync(full, other, lane + 8);
+    T s = other + ((ok & 1u) ? xo : (T)0);
+    s += (ok & 2u) ? ym : (T)0;
+    s += (ok & 4u) ? yp : (T)0;
+    s += (ok & 8u) ? zm : (T)0;
+    s += (ok & 16u) ? zp : (T)0;
+    return inv.relax(s, rhs);
+}
+
+template <class T>
+__device__ void bottom_solve(T* phi, const T* rhs, unsigned lane)
+{
+    const int ih = lane & 1, j = (lane >> 1) & 3, k = lane >> 3;
+    const int p0 = (j + k) & 1, p1 = p0 ^ 1;
+    const int c0 = (k * 4 + j) * 4 + 2 * ih + p0, c1 = (k * 4 + j) * 4 + 2 * ih + p1;
+    const int x0 = (int)lane + (p0 ? 1 : -1), x1 = (int)lane + (p1 ? 1 : -1);
+    const unsigned yz = (j > 0 ? 2u : 0u) | (j < 3 ? 4u : 0u) | (k > 0 ? 8u : 0u) | (k < 3 ? 16u : 0u);
+    const unsigned ok0 = yz | (p0 ? (ih < 1) : (ih > 0)), ok1 = yz | (p1 ? (ih < 1) : (ih > 0));
+    const Inv<T> i0(diag_count(2 * ih + p0, j, k, 4)), i1(diag_count(2 * ih + p1, j, k, 4));
+    T a = phi[c0], b = phi[c1];
+    const T ra = rhs[c0], rb = rhs[c1];
+#pragma unroll 1
+    for (int it = 0; it < BOTTOM_SWEEPS; ++it) {
+        a = bottom_update(b, ra, i0, x0, ok0, lane);
+        b = bottom_update(a, rb, i1, x1, ok1, lane);
+    }
+    phi[c0] = a;
+    phi[c1] = b;
+}
+
+// The planes of one level in one block: PL own planes and a halo plane below
+// and above, each as two colour arrays with a rim of zeros.
+template <int N, int PLANES>
+struct SlabShape {
+    static constexpr int PL = PLANES, W = N / 2 + 2, PLANE = (N + 2) * W, COLOR = (PL + 2) * PLANE, SIZE = 2 * COLOR;
+    static constexpr int PAIRS = N * N / 2;                     // threads that own a pair column
 };
 
 template <class T>
-__device__ void blk_smooth(T* phi, const T* rhs, int n, int color)
-{
-    const int half = n * n * n / 2;
-    for (int t = threadIdx.x; t < half; t += blockDim.x) {
-        const int ih = t % (n / 2), j = (t / (n / 2)) % n, k = t / (n * n / 2);
-        const int i = 2 * ih + ((j + k + color) & 1);
-        const uint64_t idx = ((uint64_t)k * n + j) * n + i;
-        int diag;
-        const T sum = nbr_sum(phi, idx, n, i, j, k, diag);
-        phi[idx] = (sum - rhs[idx]) * inv_diag<T>(diag);
+struct CoarseSmem {
+    T p32[SlabShape<32, 4>::SIZE], p16[SlabShape<16, 2>::SIZE], p8[SlabShape<8, 8>::SIZE];
+    T res[4 * 1024];               // residuals of a level's slab, then corrections of the level below, in cell order
+    T r16[2 * 256], r8[512], e8[512];
+    T p4[64], r4[64];
+};
+
+// A thread's pair column of a level: PER planes of the PLANES in the block.
+template <class T, int N, int PLANES, int PER>
+struct Slab {
+    using S = SlabShape<N, PLANES>;
+    static constexpr int PL = PER;
+    T v[PL][2], r[PL][2];          // value and right-hand side per plane and colour
+    Inv<T> inv[PL][2];
+    T *own, *below, *above;        // the level's array here and in the neighbour blocks (nullptr: none)
+    int at, ih, j, k0;             // the pair's place in a plane's rim array; the slab's first plane
+    bool act;
+
+    __device__ __forceinline__ void init(T* base, T* lower, T* upper, int first)
+    {
+        const int z = threadIdx.x / S::PAIRS * PER;     // the column's first plane in the slab
+        own = base; below = lower; above = upper; k0 = first + z;
+        act = z < PLANES;
+        ih = threadIdx.x % (N / 2);
+        j = threadIdx.x / (N / 2) % N;
+        at = z * S::PLANE + (j + 1) * S::W + ih + 1;
+#pragma unroll
+        for (int q = 0; q < PL; ++q)
+#pragma unroll
+            for (int c = 0; c < 2; ++c) {
+                inv[q][c] = Inv<T>(diag_count(2 * ih + ((j + k0 + q + c) & 1), j, k0 + q, N));
+                v[q][c] = r[q][c] = (T)0;
+            }
     }
-    __syncthreads();
+    // x parity of the colour-c cell of own plane q
+    __device__ __forceinline__ int par(int q, int c) const { return (j + k0 + q + c) & 1; }
+    // its place in cell order, from the column's first plane
+    __device__ __forceinline__ int cell(int q, int p) const { return (q * N + j) * N + 2 * ih + p; }
+    __device__ __forceinline__ T sum(int q, int c) const
+    {
+        const int o = c ^ 1;
+        const T* b = own + o * S::COLOR + (q + 1) * S::PLANE + at;
+        T s = v[q][o] + b[par(q, c) ? 1 : -1];
+        s += b[-S::W];
+        s += b[S::W];
+        s += q > 0 ? v[q - 1][o] : b[-S::PLANE];
+        s += q < PL - 1 ? v[q + 1][o] : b[S::PLANE];
+        return s;
+    }
+    __device__ __forceinline__ void put(int q, int c, T w)
+    {
+        v[q][c] = w;
+        own[c * S::COLOR + (q + 1) * S::PLANE + at] = w;
+        if (q == 0 && below) below[c * S::COLOR + (PL + 1) * S::PLANE + at] = w;
+        if (q == PL - 1 && above) above[c * S::COLOR + at] = w;
+    }
+    __device__ __forceinline__ void relax(int c)
+    {
+        if (!act) return;
+        T w[PL];
+#pragma unroll
+        for (int q = 0; q < PL; ++q) w[q] = inv[q][c].relax(sum(q, c), r[q][c]);
+#pragma unroll
+        for (int q = 0; q < PL; ++q) put(q, c, w[q]);
+    }
+    // right-hand side from cell order
+    __device__ __forceinline__ void set_rhs(const T* rhs)
+    {
+        if (!act) return;
+#pragma unroll
+        for (int q = 0; q < PL; ++q)
+#pragma unroll
+            for (int c = 0; c < 2; ++c) r[q][c] = rhs[cell(q, par(q, c))];
+    }
+    __device__ __forceinline__ void residuals(T* res) const
+    {
+        if (!act) return;
+#pragma unroll
+        for (int q = 0; q < PL; ++q)
+#pragma unroll
+            for (int c = 0; c < 2; ++c)
+                res[cell(q, par(q, c))] =
+                    MG<T>::resid(sum(q, c), r[q][c], v[q][c], diag_count(2 * ih + par(q, c), j, k0 + q, N));
+    }
+    // values in cell order, with the halo planes first and last
+    __device__ __forceinline__ void values(T* out) const
+    {
+        if (!act) return;
+#pragma unroll
+        for (int q = -1; q <= PL; ++q)
+#pragma unroll
+            for (int c = 0; c < 2; ++c)
+                out[cell(q + 1, par(q, c))] = own[c * S::COLOR + (q + 1) * S::PLANE + at];
+    }
+    // plus the correction of the level below (cell order, planes from z0 on)
+    __device__ __forceinline__ void correct(const T* ec, int z0)
+    {
+        if (!act) return;
+#pragma unroll
+        for (int q = 0; q < PL; ++q)
+#pragma unroll
+            for (int c = 0; c < 2; ++c)
+                put(q, c, v[q][c] + prolong_at(ec, N / 2, 2 * ih + par(q, c), j, k0 + q, z0));
+    }
+};
+
+// Half the sums of eight residuals (cell order, planes 2 K and 2 K + 1 of an
+// N x N slab) into planes of the level below.
+template <class T, int N>
+__device__ __forceinline__ void restrict_planes(const T* res, T* rc, int planes)
+{
+    constexpr int NC = N / 2;
+    for (int t = threadIdx.x; t < planes * NC * NC; t += COARSE_TPB) {
+        const int I = t % NC, J = (t / NC) % NC, K = t / (NC * NC);
+        T acc = (T)0;
+#pragma unroll
+        for (int c = 0; c < 8; ++c) acc += res[((2 * K + (c >> 2)) * N + 2 * J + ((c >> 1) & 1)) * N + 2 * I + (c & 1)];
+        rc[t] = MG<T>::half(acc);
+    }
 }
 
+// zero: the starting level's potential is taken as zero (not read).
 template <class T>
-__device__ void blk_resid_restrict(const T* phi, const T* rhs, T* rhs_c, int nf)
+__global__ void __cluster_dims__(COARSE_CL, 1, 1) __launch_bounds__(COARSE_TPB)
+    k_vcycle_coarse(CoarseTop<T> top, int zero, int nu1, int nu2)
 {
-    const int nc = nf / 2;
-    for (int t = threadIdx.x; t < nc * nc * nc; t += blockDim.x) {
-        const int I = t % nc, J = (t / nc) % nc, K = t / (nc * nc);
-        T acc = 0;
-        for (int c = 0; c < 8; ++c) {
-            const int i = 2 * I + (c & 1), j = 2 * J + ((c >> 1) & 1), k = 2 * K + (c >> 2);
-            const uint64_t idx = ((uint64_t)k * nf + j) * nf + i;
-            int diag;
-            const T sum = nbr_sum(phi, idx, nf, i, j, k, diag);
-            acc += fma(diag_val<T>(diag), phi[idx], rhs[idx] - sum);
-        }
-        rhs_c[t] = acc * (T)0.5;
-    }
-    __syncthreads();
-}
-
-template <class T>
-__device__ void blk_prolong(T* phi_f, const T* e_c, int nf)
-{
-    const int nc = nf / 2;
-    for (int t = threadIdx.x; t < nf * nf * nf; t += blockDim.x) {
-        const int i = t % nf, j = (t / nf) % nf, k = t / (nf * nf);
-        phi_f[t] += prolong_at(e_c, nc, i, j, k);
-    }
-    __syncthreads();
-}
-
-template <class T>
-__global__ void __launch_bounds__(1024) k_vcycle_coarse(CoarseLevels C, int nu1, int nu2, int bottom_sweeps)
-{
-    const int r = blockIdx.x;
-    auto PHI = [&](int l) { return reinterpret_cast<T*>(C.phi[l]) + (uint64_t)r * C.n[l] * C.n[l] * C.n[l]; };
-    auto RHS = [&](int l) { return reinterpret_cast<T*>(C.rhs[l]) + (uint64_t)r * C.n[l] * C.n[l] * C.n[l]; };
-    const int L = C.nlev - 1;
-    for (int l = 0; l < L; ++l) {
+    extern __shared__ __align__(16) unsigned char csm[];
+    CoarseSmem<T>& S = *reinterpret_cast<CoarseSmem<T>*>(csm);
+    cg::cluster_group cl = cg::this_cluster();
+    const int rank = (int)cl.block_rank(), n = top.n;
+    const uint64_t base = (uint64_t)(blockIdx.x / COARSE_CL) * n * n * n;
+    T* gp = top.phi + base;
+    const T* gr = top.rhs + base;
+    // zeros everywhere (rims, domain halos, the corrections' start)
+    for (int t = threadIdx.x; t < SlabShape<32, 4>::SIZE; t += COARSE_TPB) S.p32[t] = (T)0;
+    for (int t = threadIdx.x; t < SlabShape<16, 2>::SIZE; t += COARSE_TPB) S.p16[t] = (T)0;
+    for (int t = threadIdx.x; t < SlabShape<8, 8>::SIZE; t += COARSE_TPB) S.p8[t] = (T)0;
+    Slab<T, 32, 4, 4> a;
+    Slab<T, 16, 2, 2> b;
+    Slab<T, 8, 8, 1> c;
+    auto lower = [&](T* p) { return rank > 0 ? cl.map_shared_rank(p, rank - 1) : nullptr; };
+    auto upper = [&](T* p) { return rank < COARSE_CL - 1 ? cl.map_shared_rank(p, rank + 1) : nullptr; };
+    a.init(S.p32, lower(S.p32), upper(S.p32), rank * 4);
+    b.init(S.p16, lower(S.p16), upper(S.p16), rank * 2);
+    c.init(S.p8, nullptr, nullptr, 0);
+    // the starting level's right-hand side and potential
+    auto load = [&](auto& L, int N) {
+        const int64_t o = (int64_t)L.k0 * N * N;
+        L.set_rhs(gr + o);
+        if (zero || !L.act) return;
+#pragma unroll
+        for (int q = 0; q < L.PL; ++q)
+#pragma unroll
+            for (int x = 0; x < 2; ++x) L.put(q, x, gp[o + L.cell(q, L.par(q, x))]);
+    };
+    cl.sync();                                        // zeros in place before a neighbour's store
+    if (n == 32) load(a, 32);
+    if (n == 16) load(b, 16);
+    if (n == 8 && rank == 0) load(c, 8);
+    cl.sync();
+    if (n >= 32) {
         for (int it = 0; it < nu1; ++it) {
-            blk_smooth<T>(PHI(l), RHS(l), C.n[l], 0);
-            blk_smooth<T>(PHI(l), RHS(l), C.n[l], 1);
+            a.relax(0); cl.sync();
+            a.relax(1); cl.sync();
         }
-        blk_resid_restrict<T>(PHI(l), RHS(l), RHS(l + 1), C.n[l]);
-        T* pc = PHI(l + 1);
-        for (int t = threadIdx.x; t < C.n[l + 1] * C.n[l + 1] * C.n[l + 1]; t += blockDim.x) pc[t] = (T)0;
+        a.residuals(S.res);
         __syncthreads();
+        restrict_planes<T, 32>(S.res, S.r16, 2);
+        __syncthreads();
+        b.set_rhs(S.r16);
     }
-    for (int it = 0; it < bottom_sweeps; ++it) {
-        blk_smooth<T>(PHI(L), RHS(L), C.n[L], 0);
-        blk_smooth<T>(PHI(L), RHS(L), C.n[L], 1);
-    }
-    for (int l = L - 1; l >= 0; --l) {
-        blk_prolong<T>(PHI(l), PHI(l + 1), C.n[l]);
-        for (int it = 0; it < nu2; ++it) {
-            blk_smooth<T>(PHI(l), RHS(l), C.n[l], 1);
-            blk_smooth<T>(PHI(l), RHS(l), C.n[l], 0);
+    if (n >= 16) {
+        for (int it = 0; it < nu1; ++it) {
+            b.relax(0); cl.sync();
+            b.relax(1); cl.sync();
         }
+        b.residuals(S.res);
+        __syncthreads();
+        restrict_planes<T, 16>(S.res, cl.map_shared_rank(S.r8, 0) + rank * 64, 1);
+        cl.sync();
+    }
+    if (rank == 0) {
+        if (n >= 16) c.set_rhs(S.r8 + c.k0 * 64);
+        for (int it = 0; it < nu1; ++it) {
+            c.relax(0); __syncthreads();
+            c.relax(1); __syncthreads();
+        }
+        c.residuals(S.res + c.k0 * 64);
+        __syncthreads();
+        restrict_planes<T, 8>(S.res, S.r4, 4);
+        if (threadIdx.x < 64) S.p4[threadIdx.x] = (T)0;
+        __syncthreads();
+        if (threadIdx.x < 32) bottom_solve(S.p4, S.r4, threadIdx.x);
+        __syncthreads();
+        c.correct(S.p4, 0);
+        __syncthreads();
+        for (int it = 0; it < nu2; ++it) {
+            c.relax(1); __syncthreads();
+            c.relax(0); __syncthreads();
+        }
+        if (c.act)
+#pragma unroll
+            for (int x = 0; x < 2; ++x) (n == 8 ? gp : S.e8)[c.k0 * 64 + c.cell(0, c.par(0, x))] = c.v[0][x];
+    }
+    if (n >= 16) {
+        cl.sync();
+        const T* e0 = cl.map_shared_rank(S.e8, 0);
+        for (int t = threadIdx.x; t < 512; t += COARSE_TPB) S.res[t] = e0[t];
+        __syncthreads();
+        b.correct(S.res, 0);
+        cl.sync();
+        for (int it = 0; it < nu2; ++it) {
+            b.relax(1); cl.sync();
+            b.relax(0); cl.sync();
+        }
+    }
+    auto store = [&](auto& L, int N) {
+        if (!L.act) return;
+#pragma unroll
+        for (int q = 0; q < L.PL; ++q)
+#pragma unroll
+            for (int x = 0; x < 2; ++x) gp[(int64_t)L.k0 * N * N + L.cell(q, L.par(q, x))] = L.v[q][x];
+    };
+    if (n >= 32) {
+        b.values(S.res);
+        __syncthreads();
+        a.correct(S.res, rank * 2 - 1);
+        cl.sync();
+        for (int it = 0; it < nu2; ++it) {
+            a.relax(1); cl.sync();
+            a.relax(0); cl.sync();
+        }
+        store(a, 32);
+    } else if (n == 16) {
+        store(b, 16);
+    }
+    cl.sync();                     // no block's shared memory goes while another may still write to it
+}
+
+// ---------------------------------------------------------------------------
+// Two red-black sweeps (four half-sweeps) of a level of at least 64^3 cells in
+// one pass over memory.  A block owns a TX x TY column of a z chunk and
+// marches up in z: while plane t (with a halo of four cells on each side)
+// enters, half-sweep K runs on plane t - K, so that each plane is read once,
+// relaxed four times and written once.  A thread keeps its x pairs of cells
+// of the last planes in registers, one value of each colour (A: the colour of
+// the first half-sweep, B: the other): a cell's z neighbours and one x
+// neighbour are its own, of the other colour whatever the plane.  The other x
+// neighbour and the two y neighbours come from a ring of planes in shared
+// memory, one half plane per colour (no bank conflicts).  They were last
+// written a step before (half-sweep K of step t reads what half-sweep K - 1
+// left on the same plane in step t - 1), so one barrier per step orders
+// everything.  In step t the cell that half-sweep K relaxes has x parity
+// (y + t + c0 + 1) mod 2 for every K.  The next plane's values are loaded
+// into registers a step ahead; the right-hand side never leaves them.  Pairs
+// at the rim of the halo relax with what lies beside them; what is wrong
+// there moves one cell inwards per half-sweep and ends before the tile.  Out
+// of place (dst must not be src): neighbouring blocks read the halo's old
+// values.  src == nullptr: a zero initial guess.  Every cell gets the
+// operations of four plain half-sweeps in their order, so the result is the
+// same to the last bit.  Two sweeps of 256^3 cells: 202 us in fixed point (66%
+// issue utilisation: bound by its integer instructions, 1.9 TB/s of DRAM)
+// against 508 us for four FP64 half-sweeps (FP64 pipe 82% busy).
+template <class T>
+struct SweepTile {
+    static constexpr int TX = sizeof(T) == 4 ? 64 : 32, TY = 32, H = 4;
+    static constexpr int EX = TX + 2 * H, EY = TY + 2 * H, PX = EX / 2;
+    static constexpr int NT = sizeof(T) == 4 ? 720 : 800, PP = sizeof(T) == 4 ? 2 : 1, RING = 5;
+    static constexpr int GUARD = PX + 1;           // elements before and after the ring that rim pairs read
+    static constexpr size_t SMEM = sizeof(T) * (RING * EX * EY + 2 * GUARD);
+    static_assert(PX * EY == PP * NT, "whole pairs per thread");
+};
+
+template <class T>
+struct __align__(2 * sizeof(T)) Pair { T v[2]; };
+
+template <class T>
+__global__ void __launch_bounds__(SweepTile<T>::NT, 1)
+    k_sweep4(const T* __restrict__ src, const T* __restrict__ rhs, T* __restrict__ dst, int n, int c0, int zc)
+{
+    using Q = SweepTile<T>;
+    constexpr int H = Q::H, PP = Q::PP, PX = Q::PX, EY = Q::EY, PLH = PX * EY;   // PLH: the cells of one colour
+    extern __shared__ __align__(16) unsigned char ssm[];
+    T* ring = reinterpret_cast<T*>(ssm) + Q::GUARD;
+    const int tiles_x = n / Q::TX;
+    const int x0 = (int)(blockIdx.x % tiles_x) * Q::TX - H, y0 = (int)(blockIdx.x / tiles_x) * Q::TY - H;
+    const int z0 = (int)blockIdx.y * zc, z1 = z0 + zc;
+    const int64_t nn = (int64_t)n * n;
+    bool in[PP], tile[PP];                         // inside the domain; inside the block's own column
+    int d0[PP], d1[PP];                            // in-plane diagonal counts of the even and the odd cell
+    unsigned odd[PP];                              // y + c0
+    Inv<T> i0[PP], i1[PP];
+    int64_t off[PP];
+#pragma unroll
+    for (int m = 0; m < PP; ++m) {
+        const int q = threadIdx.x + m * Q::NT;
+        const int ey = q / PX, px = q - ey * PX, gi = x0 + 2 * px, gj = y0 + ey;
+        in[m] = gi >= 0 && gi < n && gj >= 0 && gj < n;       // pairs lie wholly inside or outside
+        tile[m] = px >= H / 2 && px < PX - H / 2 && ey >= H && ey < EY - H;
+        const int dy = 6 - (gj == 0) - (gj == n - 1);
+        d0[m] = dy - (gi == 0);
+        d1[m] = dy - (gi + 2 == n);
+        i0[m] = Inv<T>(d0[m]);
+        i1[m] = Inv<T>(d1[m]);
+        odd[m] = (unsigned)(gj + c0);
+        off[m] = (int64_t)blockIdx.z * nn * n + (int64_t)gj * n + gi;
+    }
+    // in step t: v[K] and r[K - 1] are plane t - K's values and right-hand
+    // side, colour A in .v[0], colour B in .v[1]
+    Pair<T> v[H + 2][PP], r[H][PP], nv[PP], nr[PP];
+    auto fetch = [&](const T* __restrict__ a, int p, Pair<T>* to) {
+#pragma unroll
+        for (int m = 0; m < PP; ++m) {
+            to[m].v[0] = to[m].v[1] = (T)0;
+            if (in[m] && p >= 0 && p < n) to[m] = *reinterpret_cast<const Pair<T>*>(a + off[m] + (int64_t)p * nn);
+        }
+    };
+#pragma unroll
+    for (int m = 0; m < PP; ++m) {
+        nv[m].v[0] = nv[m].v[1] = (T)0;
+#pragma unroll
+        for (int K = 0; K < H + 2; ++K) v[K][m] = nv[m];
+#pragma unroll
+        for (int K = 0; K < H; ++K) r[K][m] = nv[m];
+    }
+    if (src) fetch(src, z0 - H, nv);
+    int s = 0;                                     // ring slot of plane t
+    // one step; EDGE: some plane of it is outside the march's range or at a
+    // domain face (else no plane needs a look)
+    auto step = [&](auto edge, int t) {
+        constexpr bool EDGE = decltype(edge)::value;
+        bool par[PP];
+        Inv<T> ic[PP];
+#pragma unroll
+        for (int m = 0; m < PP; ++m) {
+            par[m] = (odd[m] + (unsigned)t + 1u) & 1u;
+            ic[m] = par[m] ? i1[m] : i0[m];
+            T* c = ring + s * (2 * PLH) + threadIdx.x + m * Q::NT;
+            if (src) {
+                v[0][m].v[0] = par[m] ? nv[m].v[0] : nv[m].v[1];
+                v[0][m].v[1] = par[m] ? nv[m].v[1] : nv[m].v[0];
+            }
+            c[0] = v[0][m].v[0];
+            c[PLH] = v[0][m].v[1];
+        }
+        if (src) fetch(src, t + 1, nv);
+        fetch(rhs, t, nr);
+#pragma unroll
+        for (int K = 1; K <= H; ++K) {
+            const int p = t - K;
+            if (EDGE && (p < 0 || p >= n || p < z0 - (H - K) || p >= z1 + (H - K))) continue;
+            const int c = (K & 1) ? 0 : 1, o = c ^ 1;         // relaxed colour and the other
+            const int dz = EDGE ? (p == 0) + (p == n - 1) : 0;
+            T* plane = ring + (s >= K ? s - K : s + Q::RING - K) * (2 * PLH) + threadIdx.x;
+#pragma unroll
+            for (int m = 0; m < PP; ++m) {
+                if (!in[m]) continue;                         // cells outside the domain stay zero
+                const T* oth = plane + o * PLH + m * Q::NT;
+                T sum = v[K][m].v[o] + oth[par[m] ? 1 : -1];
+                sum += oth[-PX];
+                sum += oth[PX];
+                sum += v[K + 1][m].v[o];
+                sum += v[K - 1][m].v[o];
+                T w;
+                if (EDGE && dz) w = Inv<T>((par[m] ? d1[m] : d0[m]) + dz).relax(sum, r[K - 1][m].v[c]);
+                else w = ic[m].relax(sum, r[K - 1][m].v[c]);
+                v[K][m].v[c] = w;
+                if (K < H) plane[c * PLH + m * Q::NT] = w;
+                if (K == H && tile[m]) {
+                    Pair<T> q;
+                    q.v[0] = par[m] ? v[H][m].v[0] : w;
+                    q.v[1] = par[m] ? w : v[H][m].v[0];
+                    *reinterpret_cast<Pair<T>*>(dst + off[m] + (int64_t)p * nn) = q;
+                }
+            }
+        }
+        __syncthreads();
+#pragma unroll
+        for (int m = 0; m < PP; ++m) {
+#pragma unroll
+            for (int K = H + 1; K > 0; --K) v[K][m] = v[K - 1][m];
+#pragma unroll
+            for (int K = H - 1; K > 0; --K) r[K][m] = r[K - 1][m];
+            r[0][m].v[0] = par[m] ? nr[m].v[0] : nr[m].v[1];
+            r[0][m].v[1] = par[m] ? nr[m].v[1] : nr[m].v[0];
+        }
+        s = s + 1 == Q::RING ? 0 : s + 1;
+    };
+#pragma unroll 1
+    for (int t = z0 - H; t < z1 + H; ++t) {
+        if (t - H >= z0 && t <= z1 && t - H > 0 && t < n) step(std::false_type{}, t);
+        else step(std::true_type{}, t);
     }
 }
 
@@ -544,62 +1158,94 @@ template <>
 double* lphi<double>(MGLevel& L) { return L.phi; }
 template <>
 float* lphi<float>(MGLevel& L) { return L.phi32; }
+template <>
+long long* lphi<long long>(MGLevel& L) { return L.phi_fix; }
 template <class T>
 T* lrhs(MGLevel& L);
 template <>
 double* lrhs<double>(MGLevel& L) { return L.rhs; }
 template <>
 float* lrhs<float>(MGLevel& L) { return L.rhs32; }
+template <>
+long long* lrhs<long long>(MGLevel& L) { return L.rhs_fix; }
 
+// Shared memory beyond 48 KB needs an opt-in per kernel and device.
+template <class F>
+void allow_smem(F* kernel, size_t bytes)
+{
+    static std::mutex mtx;
+    static bool done[64] = {};
+    int dev = 0;
+    cudaGetDevice(&dev);
+    std::lock_guard<std::mutex> lk(mtx);
+    if (dev >= 0 && dev < 64 && done[dev]) return;
+    cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+    if (dev >= 0 && dev < 64) done[dev] = true;
+}
+
+// Two sweeps of level l from src (nullptr: zeros) into dst.  The z chunk is
+// the one with the least modelled time: waves of resident blocks (one per SM)
+// times the planes each block marches over, the chunk and its halo of 2 x 4.
 template <class T>
-void vcycle(Dev& d, int l, int R, int nu1, int nu2, cudaStream_t s)
+void launch_sweep4(const T* src, const T* rhs, T* dst, const Geo& G, int c0, cudaStream_t s)
+{
+    using Q = SweepTile<T>;
+    allow_smem(k_sweep4<T>, Q::SMEM);
+    const uint64_t tiles = (uint64_t)(G.n / Q::TX) * (G.n / Q::TY);
+    int zc = G.n;
+    uint64_t best = ~0ull;
+    for (int c = G.n; c >= 4; c >>= 1) {
+        const uint64_t blocks = tiles * G.R * (G.n / c), cost = ((blocks + 151) / 152) * (c + 2 * Q::H);
+        if (cost < best) { best = cost; zc = c; }
+    }
+    ++g_launches;
+    k_sweep4<T><<<dim3((unsigned)tiles, G.n / zc, G.R), Q::NT, Q::SMEM, s>>>(src, rhs, dst, G.n, c0, zc);
+}
+
+// One V-cycle from level l; zero: the level's potential counts as zero (it is
+// not read).  Levels of 64^3 and more take two sweeps per pass, between the
+// level's two arrays; an odd sweep runs as two plain half-sweeps in place.
+template <class T>
+void vcycle(Dev& d, int l, int R, int nu1, int nu2, cudaStream_t s, bool zero)
 {
     MGLevel& L = d.lev[l];
     const Geo G = geo(d, l, R);
-    T* phi = lphi<T>(L);
-    T* rhs = lrhs<T>(L);
-    if (L.n <= COARSE_N && d.nlev - l >= 2) {
-        CoarseLevels C{};
-        C.nlev = d.nlev - l;
-        for (int q = 0; q < C.nlev; ++q) {
-            MGLevel& M = d.lev[l + q];
-            C.n[q] = M.n;
-            C.phi[q] = lphi<T>(M);
-            C.rhs[q] = lrhs<T>(M);
-        }
+    T* const phi = lphi<T>(L);
+    const T* rhs = lrhs<T>(L);
+    if (L.n <= COARSE_N) {
+        allow_smem(k_vcycle_coarse<T>, sizeof(CoarseSmem<T>));
         ++g_launches;
-        k_vcycle_coarse<T><<<R, 1024, 0, s>>>(C, nu1, nu2, 48);
-        return;
-    }
-    if (l == d.nlev - 1) {
-        const int cells = G.n * G.n * G.n;
-        const size_t sm = 2 * sizeof(T) * cells;
-        ++g_launches;
-        k_bottom<T><<<R, 256, sm, s>>>(phi, rhs, G.n, 48);
+        k_vcycle_coarse<T><<<R * COARSE_CL, COARSE_TPB, sizeof(CoarseSmem<T>), s>>>(CoarseTop<T>{ phi, rhs, G.n }, zero,
+                                                                                    nu1, nu2);
         return;
     }
     const int tpb = 256;
-    for (int it = 0; it < nu1; ++it) {
-        ++g_launches;
-        k_smooth<T><<<gridsz(G.cells / 2, tpb), tpb, 0, s>>>(phi, rhs, G, 0);
-        ++g_launches;
-        k_smooth<T><<<gridsz(G.cells / 2, tpb), tpb, 0, s>>>(phi, rhs, G, 1);
-    }
+    T* cur = phi;
+    auto sweeps = [&](int nu, int c0) {
+        for (; nu >= 2; nu -= 2) {
+            T* to = cur == phi ? reinterpret_cast<T*>(L.alt) : phi;
+            launch_sweep4<T>(zero ? nullptr : cur, rhs, to, G, c0, s);
+            cur = to;
+            zero = false;
+        }
+        if (zero) cudaMemsetAsync(cur, 0, G.cells * sizeof(T), s);
+        zero = false;
+        if (nu == 1)
+            for (int c = 0; c < 2; ++c) {
+                ++g_launches;
+                k_smooth<T><<<gridsz(G.cells / 2, tpb), tpb, 0, s>>>(cur, rhs, G, c0 ^ c);
+            }
+    };
+    sweeps(nu1, 0);
     MGLevel& C = d.lev[l + 1];
     const Geo Gc = geo(d, l + 1, R);
     ++g_launches;
-    k_resid_restrict<T, T><<<gridsz(Gc.cells, tpb), tpb, 0, s>>>(phi, rhs, lrhs<T>(C), Gc, G.n);
+    k_resid_restrict<T><<<gridsz(Gc.cells, tpb), tpb, 0, s>>>(cur, rhs, lrhs<T>(C), Gc, G.n);
+    vcycle<T>(d, l + 1, R, nu1, nu2, s, true);
     ++g_launches;
-    k_zero<T><<<gridsz(Gc.cells, tpb), tpb, 0, s>>>(lphi<T>(C), Gc.cells);
-    vcycle<T>(d, l + 1, R, nu1, nu2, s);
-    ++g_launches;
-    k_prolong<T><<<gridsz(G.cells, tpb), tpb, 0, s>>>(phi, lphi<T>(C), G);
-    for (int it = 0; it < nu2; ++it) {
-        ++g_launches;
-        k_smooth<T><<<gridsz(G.cells / 2, tpb), tpb, 0, s>>>(phi, rhs, G, 1);
-        ++g_launches;
-        k_smooth<T><<<gridsz(G.cells / 2, tpb), tpb, 0, s>>>(phi, rhs, G, 0);
-    }
+    k_prolong<T><<<gridsz(G.cells, tpb), tpb, 0, s>>>(cur, lphi<T>(C), G);
+    sweeps(nu2, 1);
+    if (cur != phi) cudaMemcpyAsync(phi, cur, G.cells * sizeof(T), cudaMemcpyDeviceToDevice, s);
 }
 
 
@@ -712,7 +1358,9 @@ __global__ void k_coef_restrict(const double* __restrict__ cf, double* __restric
 }
 
 // The coarse end of the variable-coefficient V-cycle (levels of at most 16^3
-// cells) in one launch, one block per realization (as k_vcycle_coarse).
+// cells) in one launch, one block per realization.
+constexpr int COARSE_VC_N = 16;
+
 struct CoarseVC {
     int nlev;
     int n[MAX_LEVELS];
@@ -856,8 +1504,8 @@ __global__ void k_coef_from_ne(const unsigned long long* __restrict__ ne_fix, do
 constexpr int MAX_REAL_NORM = 4096;
 
 // Replays (capturing first if needed) the graph of kind k on stream s:
-// k = 0: one FP64 V-cycle; k = 1: zero the FP32 correction, two FP32
-// V-cycles.  The launches of a cycle depend only on the level pointers and
+// k = 0: one FP64 V-cycle; k = 1: two FP32 V-cycles from a zero correction;
+// k = 3: one fixed-point V-cycle.  The launches of a cycle depend only on the level pointers and
 // the smoother counts, so one capture per (nu1, nu2) serves every solve.
 // Launches directly when d.direct_cycles is set (a solve on per-call
 // buffers, whose graphs could not be reused) or capture is not possible.
@@ -865,13 +1513,12 @@ void run_cycles(Dev& d, int k, int R, int nu1, int nu2, cudaStream_t s)
 {
     auto direct = [&]() {
         if (k == 0) {
-            vcycle<double>(d, 0, R, nu1, nu2, s);
+            vcycle<double>(d, 0, R, nu1, nu2, s, false);
+        } else if (k == 3) {
+            vcycle<long long>(d, 0, R, nu1, nu2, s, false);
         } else {
-            const Geo G0 = geo(d, 0, R);
-            ++g_launches;
-            k_zero<float><<<gridsz(G0.cells, 256), 256, 0, s>>>(d.lev[0].phi32, G0.cells);
-            vcycle<float>(d, 0, R, nu1, nu2, s);
-            vcycle<float>(d, 0, R, nu1, nu2, s);
+            vcycle<float>(d, 0, R, nu1, nu2, s, true);
+            vcycle<float>(d, 0, R, nu1, nu2, s, false);
         }
     };
     if (d.direct_cycles) {
@@ -932,6 +1579,24 @@ void lower_phi_scale(const Params& P, Dev& d, int F, cudaStream_t s)
     d.phi_F = F;
 }
 
+// FP64 form, before the cycles: start guess, scale, Phi and B.
+void fix_begin(const Params& P, Dev& d, bool extrapolate, cudaStream_t s)
+{
+    MGLevel& L0 = d.lev[0];
+    const Geo G0 = geo(d, 0, P.R);
+    double qscale, bc_top;
+    rhs_consts(P, qscale, bc_top);
+    const bool ex = extrapolate && d.phi_prev;
+    cudaMemsetAsync(d.fix, 0, sizeof(FixScale), s);
+    g_launches += 3;
+    k_fix_start<<<gridsz(G0.cells, 256), 256, 0, s>>>(L0.phi, reinterpret_cast<double*>(d.phi_prev), ex, d.have_prev,
+                                                     L0.rhs, G0, bc_top * (L0.h * L0.h), d.fix);
+    k_fix_scale<<<1, 1, 0, s>>>(d.fix, P.E0 * (P.hi[2] - P.lo[2]), G0.n, ex && d.have_prev, 0);
+    k_fix_load<<<gridsz(G0.cells, 256), 256, 0, s>>>(L0.phi, L0.rhs, L0.phi_fix, L0.rhs_fix, G0.cells, d.fix, 0);
+    if (ex) d.have_prev = true;
+    d.fix_result = true;
+}
+
 int field_solve(const Params& P, Dev& d, int precision, double rtol, int nu1, int nu2, unsigned long long rho_absmax,
                 int max_cycles, cudaStream_t s, int* cycles_out, double* rel_out, bool extrapolate)
 {
@@ -942,13 +1607,15 @@ int field_solve(const Params& P, Dev& d, int precision, double rtol, int nu1, in
     const int items = (int)(per_real / NORM_TPB < 8 ? per_real / NORM_TPB : 8);
     const int nblk = (int)(G0.cells / ((uint64_t)NORM_TPB * items));
     const int bpr = nblk / R;
-    double* h_norm = d.norm_host;       // 2 R doubles of host memory owned by the caller
+    double* h_norm = d.norm_host;       // 2 R + FIX_DOUBLES doubles of host memory owned by the caller
     double bnorm[MAX_REAL_NORM];
     if (R > MAX_REAL_NORM) return -1;
     double worst = 0.0;
     int cyc = 0;
     int status = -6;
     const bool fixed = precision == 2;
+    bool fix = precision == 0;          // FP64 form in fixed point (until it cannot go on)
+    d.fix_result = false;
     long long* Phi = reinterpret_cast<long long*>(L0.phi);
     long long* Bfix = reinterpret_cast<long long*>(L0.rhs);
     if (fixed) {
@@ -959,21 +1626,18 @@ int field_solve(const Params& P, Dev& d, int precision, double rtol, int nu1, in
         ++g_launches;
         k_rhs_fixed<<<gridsz(G0.cells, 256), 256, 0, s>>>(d.rho, Bfix, G0, qscale, bc_top,
                                                          L0.h * L0.h * std::ldexp(1.0, d.phi_F));
+        // initial guess 2 phi_k - phi_{k-1} (the previous potential is kept)
+        if (extrapolate && d.phi_prev) {
+            ++g_launches;
+            k_extrapolate<<<gridsz(G0.cells, 256), 256, 0, s>>>(Phi, reinterpret_cast<long long*>(d.phi_prev), G0.cells,
+                                                               d.have_prev);
+            d.have_prev = true;
+        }
     }
-    // initial guess 2 phi_k - phi_{k-1} (the previous potential is kept)
-    if (extrapolate && d.phi_prev) {
-        ++g_launches;
-        if (fixed)
-            k_extrapolate<long long><<<gridsz(G0.cells, 256), 256, 0, s>>>(
-                Phi, reinterpret_cast<long long*>(d.phi_prev), G0.cells, d.have_prev);
-        else
-            k_extrapolate<double><<<gridsz(G0.cells, 256), 256, 0, s>>>(
-                L0.phi, reinterpret_cast<double*>(d.phi_prev), G0.cells, d.have_prev);
-        d.have_prev = true;
-    }
+    if (fix) fix_begin(P, d, extrapolate, s);
     const float rsc = (float)std::ldexp(1.0, -d.phi_F);
     const float esc = (float)std::ldexp(1.0, d.phi_F);
-    // FP64 V-cycles: the residual norm only serves the convergence test, so
+    // FP64 form: the residual norm only serves the convergence test, so
     // it is evaluated at cycle 0 and then at the cycle the observed
     // convergence factor predicts (refinement forms need the residual every
     // outer iteration as the right-hand side of the correction).
@@ -982,27 +1646,59 @@ int field_solve(const Params& P, Dev& d, int precision, double rtol, int nu1, in
     int prev_cyc = 0;
     for (cyc = 0; cyc <= max_cycles; ++cyc) {
         if (precision == 0 && cyc < next_check && cyc < max_cycles) {
-            run_cycles(d, 0, R, nu1, nu2, s);
+            run_cycles(d, fix ? 3 : 0, R, nu1, nu2, s);
             continue;
         }
         ++g_launches;
         if (fixed)
             k_resid_fixed<<<nblk, NORM_TPB, 0, s>>>(Phi, Bfix, L0.rhs32, G0, rsc, d.norm_part, cyc == 0, items);
+        else if (fix)
+            k_resid_norm_fix<<<nblk, NORM_TPB, 0, s>>>(L0.phi_fix, L0.rhs_fix, G0, d.norm_part, cyc == 0, items, d.fix);
         else
             k_resid_norm<<<nblk, NORM_TPB, 0, s>>>(L0.phi, L0.rhs, precision == 1 ? L0.rhs32 : nullptr, G0,
-                                                   d.norm_part, cyc == 0, items);
+                                                   d.norm_part, prev_rel < 0.0, items);
         ++g_launches;
         k_norm_final<<<R, 256, 0, s>>>(d.norm_part, bpr, R, d.norm_out);
         cudaMemcpyAsync(h_norm, d.norm_out, 2 * R * sizeof(double), cudaMemcpyDeviceToHost, s);
+        if (fix) cudaMemcpyAsync(h_norm + 2 * R, d.fix, sizeof(FixScale), cudaMemcpyDeviceToHost, s);
         if (cudaStreamSynchronize(s) != cudaSuccess) return -3;
         worst = 0.0;
         bool done = true;
         for (int r = 0; r < R; ++r) {
-            if (cyc == 0) bnorm[r] = h_norm[2 * r + 1];
+            if (prev_rel < 0.0) bnorm[r] = h_norm[2 * r + 1];
             const double rn = std::sqrt(h_norm[2 * r]), bn = std::sqrt(bnorm[r]);
             const double rel = bn > 0.0 ? rn / bn : rn;
             if (rel > worst || !(rel == rel)) worst = rel;
             if (!(rn <= rtol * bn)) done = false;
+        }
+        if (fix) {
+            FixScale fs;
+            std::memcpy(&fs, h_norm + 2 * R, sizeof fs);
+            // out of the integer range, or no further progress in it: the
+            // potential reached so far goes on in FP64 cycles
+            const bool range = !fs.use64 && fs.max_fix < (unsigned long long)FIX_LIM && std::isfinite(worst);
+            if (!range || (!done && prev_rel >= 0.0 && worst > 0.9 * prev_rel)) {
+                if (range) {
+                    ++g_launches;
+                    k_fix_store<<<gridsz(G0.cells, 256), 256, 0, s>>>(L0.phi_fix, L0.phi, G0.cells, d.fix);
+                }
+                fix = false;
+                d.fix_result = false;
+                prev_rel = -1.0;
+                --cyc;                                  // the same check again, in FP64
+                continue;
+            }
+            // a loose bound left the leading bits unused: more of them
+            if (!done && cyc > 0 && fs.max_fix && fs.max_fix < (1ull << 52)) {
+                int lead = 0;
+                while ((fs.max_fix >> lead) > 1) ++lead;
+                const int sh = 55 - lead;
+                g_launches += 2;
+                k_fix_scale<<<1, 1, 0, s>>>(d.fix, P.E0 * (P.hi[2] - P.lo[2]), G0.n, 0, sh);
+                k_fix_load<<<gridsz(G0.cells, 256), 256, 0, s>>>(L0.phi, L0.rhs, L0.phi_fix, L0.rhs_fix, G0.cells, d.fix,
+                                                                sh);
+                for (int r = 0; r < R; ++r) bnorm[r] = std::ldexp(bnorm[r], 2 * sh);
+            }
         }
         if (done) { status = 0; break; }
         if (cyc == max_cycles || !std::isfinite(worst)) break;
@@ -1011,11 +1707,11 @@ int field_solve(const Params& P, Dev& d, int precision, double rtol, int nu1, in
                 rho_est = std::pow(worst / prev_rel, 1.0 / (cyc - prev_cyc));
                 rho_est = std::min(0.5, std::max(0.02, rho_est));
             }
-            prev_rel = worst;
-            prev_cyc = cyc;
             const double need = worst > 0.0 ? std::log(rtol / worst) / std::log(rho_est) : 1.0;
             next_check = cyc + std::max(1, (int)std::floor(need));
         }
+        prev_rel = worst;
+        prev_cyc = cyc;
         if (precision >= 1) {
             // inner solve of A e = r in FP32: two V-cycles per outer residual
             run_cycles(d, 1, R, nu1, nu2, s);
@@ -1025,7 +1721,7 @@ int field_solve(const Params& P, Dev& d, int precision, double rtol, int nu1, in
             else
                 k_add_correction<<<gridsz(G0.cells, 256), 256, 0, s>>>(L0.phi, L0.phi32, G0.cells);
         } else {
-            run_cycles(d, 0, R, nu1, nu2, s);
+            run_cycles(d, fix ? 3 : 0, R, nu1, nu2, s);
         }
     }
     if (cycles_out) *cycles_out = cyc;
@@ -1052,22 +1748,21 @@ void field_solve_fixed(const Params& P, Dev& d, int precision, int nu1, int nu2,
     const bool fixed = precision == 2;
     long long* Phi = reinterpret_cast<long long*>(L0.phi);
     long long* Bfix = reinterpret_cast<long long*>(L0.rhs);
+    d.fix_result = false;
     if (fixed) {
         double qscale, bc_top;
         rhs_consts(P, qscale, bc_top);
         ++g_launches;
         k_rhs_fixed<<<gridsz(G0.cells, 256), 256, 0, s>>>(d.rho, Bfix, G0, qscale, bc_top,
                                                          L0.h * L0.h * std::ldexp(1.0, d.phi_F));
-    }
-    if (d.phi_prev) {
-        ++g_launches;
-        if (fixed)
-            k_extrapolate<long long><<<gridsz(G0.cells, 256), 256, 0, s>>>(
-                Phi, reinterpret_cast<long long*>(d.phi_prev), G0.cells, d.have_prev);
-        else
-            k_extrapolate<double><<<gridsz(G0.cells, 256), 256, 0, s>>>(
-                L0.phi, reinterpret_cast<double*>(d.phi_prev), G0.cells, d.have_prev);
-        d.have_prev = true;
+        if (d.phi_prev) {
+            ++g_launches;
+            k_extrapolate<<<gridsz(G0.cells, 256), 256, 0, s>>>(Phi, reinterpret_cast<long long*>(d.phi_prev), G0.cells,
+                                                               d.have_prev);
+            d.have_prev = true;
+        }
+    } else if (precision == 0) {
+        fix_begin(P, d, true, s);
     }
     const float rsc = (float)std::ldexp(1.0, -d.phi_F);
     const float esc = (float)std::ldexp(1.0, d.phi_F);
@@ -1075,13 +1770,14 @@ void field_solve_fixed(const Params& P, Dev& d, int precision, int nu1, int nu2,
         ++g_launches;
         if (fixed)
             k_resid_fixed<<<nblk, NORM_TPB, 0, s>>>(Phi, Bfix, L0.rhs32, G0, rsc, d.norm_part, first, items);
+        else if (precision == 0)
+            k_resid_norm_fix<<<nblk, NORM_TPB, 0, s>>>(L0.phi_fix, L0.rhs_fix, G0, d.norm_part, first, items, d.fix);
         else
-            k_resid_norm<<<nblk, NORM_TPB, 0, s>>>(L0.phi, L0.rhs, precision == 1 ? L0.rhs32 : nullptr, G0,
-                                                   d.norm_part, first, items);
+            k_resid_norm<<<nblk, NORM_TPB, 0, s>>>(L0.phi, L0.rhs, L0.rhs32, G0, d.norm_part, first, items);
     };
     for (int c = 0; c < cycles; ++c) {
         if (precision == 0) {
-            run_cycles(d, 0, R, nu1, nu2, s);
+            run_cycles(d, 3, R, nu1, nu2, s);
             continue;
         }
         resid(false);
@@ -1147,7 +1843,12 @@ void launch_efield_to(const Params& P, Dev& d, cudaStream_t s, E64* E, float4* E
     const Geo G0 = geo(d, 0, P.R);
     const double phi_top = P.E0 * (P.hi[2] - P.lo[2]);
     ++g_launches;
-    if (d.phi_F > 0)
+    if (d.fix_result) {
+        // of a solve in fixed point: E and the FP64 potential in one pass
+        k_efield_fix<<<gridsz(G0.cells, 256), 256, 0, s>>>(d.lev[0].phi_fix, E, E32, d.lev[0].phi, G0,
+                                                          1.0 / (2.0 * d.lev[0].h), d.fix);
+        d.fix_result = false;
+    } else if (d.phi_F > 0)
         k_efield_fixed<<<gridsz(G0.cells, 256), 256, 0, s>>>(
             reinterpret_cast<const long long*>(d.lev[0].phi), E, E32, G0,
             std::ldexp(1.0, -d.phi_F) / (2.0 * d.lev[0].h), std::llrint(std::ldexp(phi_top, d.phi_F)));
@@ -1182,7 +1883,7 @@ static void vcycle_vc(const Dev& d, int l, int R, int nu1, int nu2, cudaStream_t
     double* phi = d.lev[l].phi;
     const double* rhs = d.lev[l].rhs;
     const int tpb = 256;
-    if (G.n <= COARSE_N && d.nlev - l >= 2) {
+    if (G.n <= COARSE_VC_N && d.nlev - l >= 2) {
         CoarseVC C{};
         C.nlev = d.nlev - l;
         for (int q = 0; q < C.nlev; ++q) {
@@ -1202,9 +1903,9 @@ static void vcycle_vc(const Dev& d, int l, int R, int nu1, int nu2, cudaStream_t
     };
     for (int it = 0; it < nu1; ++it) { sweep(0); sweep(1); }
     const Geo Gc = geo(d, l + 1, R);
-    g_launches += 3;
+    g_launches += 2;
     k_resid_restrict_vc<<<gridsz(Gc.cells, tpb), tpb, 0, s>>>(phi, rhs, A, d.lev[l + 1].rhs, Gc, G.n);
-    k_zero<double><<<gridsz(Gc.cells, tpb), tpb, 0, s>>>(d.lev[l + 1].phi, Gc.cells);
+    cudaMemsetAsync(d.lev[l + 1].phi, 0, Gc.cells * sizeof(double), s);
     vcycle_vc(d, l + 1, R, nu1, nu2, s);
     k_prolong<double><<<gridsz(G.cells, tpb), tpb, 0, s>>>(phi, d.lev[l + 1].phi, G);
     for (int it = 0; it < nu2; ++it) { sweep(1); sweep(0); }
@@ -1425,29 +2126,42 @@ extern "C" int itokmc_field_solve_noalloc(const itokmc_config* cfg, const int64_
     P.frac_bits = cfg->frac_bits;
     Dev d;
     d.direct_cycles = true;            // no graph objects: nothing is instantiated per call
+    // the field is formed after the cycles, so its array shares its place with
+    // the finest level's right-hand sides and second array
     size_t off = 0;
+    d.E = reinterpret_cast<E64*>(base + carve(off, (size_t)P.n3 * sizeof(E64)));
+    d.E32 = nullptr;
+    size_t top = 0;
     int l = 0;
     for (int m = n; m >= 4 && l < MAX_LEVELS; m >>= 1, ++l) {
         MGLevel& L = d.lev[l];
         const size_t cells = (size_t)m * m * m;
+        size_t& at = l == 0 ? top : off;
         L.n = m;
         L.h = P.h[0] * (double)(n / m);
-        L.phi = l == 0 ? phi : reinterpret_cast<double*>(base + carve(off, cells * sizeof(double)));
-        L.rhs = reinterpret_cast<double*>(base + carve(off, cells * sizeof(double)));
-        L.res = nullptr;
+        L.phi = l == 0 ? phi : reinterpret_cast<double*>(base + carve(at, cells * sizeof(double)));
+        L.rhs = reinterpret_cast<double*>(base + carve(at, cells * sizeof(double)));
+        L.alt = base + carve(at, cells * sizeof(double));
+        L.rhs_fix = reinterpret_cast<long long*>(l == 0 ? base + carve(at, cells * sizeof(long long))
+                                                        : reinterpret_cast<unsigned char*>(L.rhs));
+        L.phi_fix = reinterpret_cast<long long*>(l == 0 ? base + carve(off, cells * sizeof(long long))
+                                                        : reinterpret_cast<unsigned char*>(L.phi));
         L.phi32 = reinterpret_cast<float*>(base + carve(off, cells * sizeof(float)));
         L.rhs32 = reinterpret_cast<float*>(base + carve(off, cells * sizeof(float)));
     }
     d.nlev = l;
     d.norm_part = reinterpret_cast<double*>(base + carve(off, 2 * ((size_t)P.n3 / 256 + 16) * sizeof(double)));
     d.norm_out = reinterpret_cast<double*>(base + carve(off, 2 * sizeof(double)));
-    d.E = reinterpret_cast<E64*>(base + carve(off, (size_t)P.n3 * sizeof(E64)));
-    d.E32 = nullptr;
+    d.fix = reinterpret_cast<FixScale*>(base + carve(off, sizeof(FixScale)));
+    if (top > (size_t)P.n3 * sizeof(E64)) {
+        set_global_error("field_solve_noalloc: scratch layout exceeds the static array");
+        return ITOKMC_ERR_ARG;
+    }
     if (off > NOALLOC_BYTES) {
         set_global_error("field_solve_noalloc: scratch layout exceeds the static array");
         return ITOKMC_ERR_ARG;
     }
-    double norm_host[2];               // stack memory: no allocation
+    double norm_host[2 + FIX_DOUBLES]; // stack memory: no allocation
     d.norm_host = norm_host;
     const double dV = P.h[0] * P.h[1] * P.h[2];
     const double qscale = 1.602176634e-19 * ldexp(1.0, -3 * P.frac_bits) / dV;

@@ -83,9 +83,26 @@ struct VCLevel {
 struct MGLevel {
     int n;                 // cells per axis on this level
     double h;              // cell size
-    double* phi;  double* rhs;  double* res;   // FP64 (size R n^3)
+    double* phi;  double* rhs;                  // FP64 (size R n^3)
     float* phi32; float* rhs32;                 // FP32 inner V-cycles
+    // fixed-point V-cycles of the FP64 form (below the finest level in the
+    // FP64 arrays' place) and the second potential array of the out-of-place
+    // sweeps (levels above 32^3; elements as wide as the widest form in use)
+    long long* phi_fix; long long* rhs_fix;
+    void* alt;
 };
+
+// Scale of the FP64 form's fixed-point potential (device memory, one per
+// handle): Phi = phi 2^F, down = 2^-F, top the electrode potential; the
+// largest |phi|, |h^2 b| (bits of the doubles) and |Phi|; use64: the integers
+// cannot hold this solve.
+struct FixScale {
+    int F, use64;
+    double down;
+    long long top;
+    unsigned long long max_phi, max_b, max_fix;
+};
+constexpr int FIX_DOUBLES = (int)(sizeof(FixScale) / sizeof(double));
 
 constexpr int MAX_LEVELS = 12;
 
@@ -130,7 +147,9 @@ struct Dev {
     MGLevel lev[MAX_LEVELS];
     int nlev = 0;
     double* norm_part = nullptr;  double* norm_out = nullptr;  size_t norm_blocks = 0;
-    double* norm_host = nullptr;       // 2 R doubles (pinned or stack) for the norm readback
+    double* norm_host = nullptr;       // 2 R + FIX_DOUBLES doubles (pinned or stack) for the readback of a check
+    FixScale* fix = nullptr;           // FP64 form: the fixed-point scale
+    bool fix_result = false;           // the last solve's potential is in phi_fix (launch_efield_to stores it)
     // counters
     Counters* ctr = nullptr;
     Counters* ctr_host = nullptr;      // pinned mirror
@@ -138,11 +157,11 @@ struct Dev {
     uint32_t mover_cap = 0, photo_cap = 0;
     uint64_t work_cap = 0;             // merge work area, 32-byte units
     double* stage = nullptr;           // 3 G doubles: field upload/readback
-    // CUDA graphs of the correction sweep (FP32: zero + two V-cycles) and of
-    // one FP64 V-cycle, captured once per smoother pair and replayed
-    cudaGraphExec_t vgraph[3] = { nullptr, nullptr, nullptr };
-    int vgraph_nu[3][2] = { { 0, 0 }, { 0, 0 }, { 0, 0 } };
-    unsigned long long vgraph_kernels[3] = { 0, 0, 0 };
+    // CUDA graphs of the cycles (run_cycles), captured once per smoother pair
+    // and replayed
+    cudaGraphExec_t vgraph[4] = {};
+    int vgraph_nu[4][2] = {};
+    unsigned long long vgraph_kernels[4] = {};
     VCLevel vc[MAX_LEVELS];            // semi-implicit operator per level (allocated on first use)
     bool direct_cycles = false;        // launch the cycles directly (no capture)
     cudaStream_t side = nullptr;       // merge tiers 1 and 2 run beside tier 0
