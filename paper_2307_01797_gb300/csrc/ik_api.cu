@@ -216,6 +216,18 @@ void fill_params(const itokmc_config* cfg, ik::Params& P)
         P.lo[a] = cfg->lo[a]; P.hi[a] = cfg->hi[a]; P.h[a] = (cfg->hi[a] - cfg->lo[a]) / n;
         P.rh[a] = 1.0 / P.h[a];
     }
+    {
+        // h = mh 2^h_exp; floor(2^148 / mh) in two steps (2^96 - 1 for a power
+        // of two, whose quotient needs 97 bits)
+        uint64_t b;
+        std::memcpy(&b, &P.h[0], sizeof b);
+        const uint64_t mh = (b & 0xfffffffffffffull) | (1ull << 52);
+        const unsigned __int128 p127 = (unsigned __int128)1 << 127;
+        unsigned __int128 R = (p127 / mh << 21) + ((p127 % mh) << 21) / mh;
+        if (R >> 96) R = ((unsigned __int128)1 << 96) - 1;
+        for (int k = 0; k < 3; ++k) P.rh96[k] = (uint32_t)(R >> (32 * k));
+        P.h_exp = (int)(b >> 52) - 1075;
+    }
     P.mu = cfg->mu; P.D = cfg->D; P.alpha_A = cfg->alpha_A; P.alpha_B = cfg->alpha_B; P.eta = cfg->eta;
     P.photon_ratio = cfg->photon_ratio; P.kappa_lo = cfg->kappa_lo; P.kappa_hi = cfg->kappa_hi; P.eps = cfg->eps;
     set_step_consts(cfg, P, cfg->dt);

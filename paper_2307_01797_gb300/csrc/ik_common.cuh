@@ -24,6 +24,10 @@ struct Params {
     int ppc, n_new, n_crit, n_ssa, frac_bits;
     int dep_win;            // largest shared deposit window (cells) a push block uses, <= DEP_WIN_MAX
     double lo[3], hi[3], h[3], rh[3];   // rh = 1/h
+    // 1/h to 96 bits (cells are cubes): h = mh 2^h_exp with 53-bit mh, and
+    // floor(2^148 / mh) in three words, lowest first
+    uint32_t rh96[3];
+    int h_exp;
     double dt, mu, D, alpha_A, alpha_B, eta, photon_ratio, kappa_lo, kappa_hi, eps;
     double sdt;             // sqrt(2 D dt)
     double k_ep, k_np;      // recombination frequencies per pair, beta / dV (1/s)

@@ -20,7 +20,6 @@
 #include "ik_state.h"
 
 namespace ik {
-
 namespace {
 
 __device__ __forceinline__ P64 ld_p64(const P64* p)
@@ -76,6 +75,44 @@ __device__ __forceinline__ bool qsplit(double qd, QSplit& r)
     else { r.i0 = r.qc - 1; r.F = fb + half; }
     return true;
 }
+// The quotient q = (x - lo) / h of axis a (grid_quot) rounded to 53 bits and
+// split, by integer multiplication with the 96-bit reciprocal: the product's
+// upper 96 bits are within a few units of 2^-96 of the quotient, and grid_quot's
+// result is the quotient rounded to nearest up to an error of 2^-52 units of
+// the last place before its rounding; so both round the same way unless the
+// bits below the 53rd lie within 2^-29 of a half.  Those, and quotients
+// outside qsplit's range, return false (the caller takes grid_quot).  GB300 has
+// 2 FP64 lanes per SM and clock: the three FP64 instructions of a quotient
+// hold the pipe for the time in which an SM issues 192 others.  (Products
+// rounded by integer instructions, about 50 each, gained nothing.)
+__device__ __forceinline__ bool quot_split(const Params& P, double x, int a, QSplit& r)
+{
+    double d = x;
+    if (__double_as_longlong(P.lo[a]) != 0) d = x - P.lo[a];
+    const uint32_t dh = (uint32_t)__double2hiint(d), dl = (uint32_t)__double2loint(d);
+    const int e = (int)(dh >> 20);                  // biased exponent (>= 2048 when negative)
+    const uint32_t m1 = (dh << 11) | (dl >> 21) | 0x80000000u, m0 = dl << 11;
+    const uint64_t u = (uint64_t)m1 * P.rh96[1], v = (uint64_t)m0 * P.rh96[2];
+    const uint64_t w = (uint64_t)(uint32_t)u + (uint32_t)v + __umulhi(m1, P.rh96[0]) + __umulhi(m0, P.rh96[1]);
+    uint64_t top = (uint64_t)m1 * P.rh96[2] + (u >> 32) + (v >> 32) + (w >> 32);
+    uint32_t g = (uint32_t)w;
+    int E = e - 1075 - P.h_exp;                     // q = top 2^(E - 63)
+    if (!(top >> 63)) {
+        top = (top << 1) | (g >> 31);
+        g <<= 1;
+        --E;
+    }
+    const uint32_t low = ((uint32_t)top << 21) | (g >> 11);
+    const int sh = 52 - E;                          // fraction bits
+    if (e == 0 || e >= 2047 || sh < 22 || sh > 53 || low - 0x7ffffffcu <= 8u) return false;
+    const uint64_t m = (top >> 11) + (low >> 31);
+    const uint64_t fb = m & ((1ull << sh) - 1ull), half = 1ull << (sh - 1);
+    r.qc = (int)(m >> sh);
+    r.sh = sh;
+    if (fb >= half) { r.i0 = r.qc; r.F = fb - half; }
+    else { r.i0 = r.qc - 1; r.F = fb + half; }
+    return true;
+}
 // F 2^-sh as a double (F < 2^sh, sh <= 53: exact).
 __device__ __forceinline__ double qfrac(unsigned long long F, int sh)
 {
@@ -87,13 +124,17 @@ __device__ __forceinline__ double qfrac(unsigned long long F, int sh)
 // cic_axis with the split above (the FP64 steps for qd < 1/2); g = 1 - f,
 // exact: 2^sh - F is at most 2^sh, so (2^sh - F) 2^-sh is the same double
 // as the FP64 subtraction 1 - f.
-__device__ __forceinline__ void cic_axis_q(double x, double lo, double h, double rh, int n, int& ia, int& ib,
-                                           double& f, double& g)
+__device__ __forceinline__ void cic_axis_q(const Params& P, double x, int a, int& ia, int& ib, double& f, double& g)
 {
-    const double qd = grid_quot(x, lo, h, rh);
     QSplit t;
     int i0;
-    if (qsplit(qd, t)) {
+    double qd = 0.0;
+    bool split = quot_split(P, x, a, t);
+    if (!split) {
+        qd = grid_quot(x, P.lo[a], P.h[a], P.rh[a]);
+        split = qsplit(qd, t);
+    }
+    if (split) {
         i0 = t.i0;
         f = qfrac(t.F, t.sh);
         g = t.F == 0 ? 1.0 : qfrac((1ull << t.sh) - t.F, t.sh);
@@ -104,8 +145,8 @@ __device__ __forceinline__ void cic_axis_q(double x, double lo, double h, double
         f = u - fl;
         g = 1.0 - f;
     }
-    ia = clampi(i0, n);
-    ib = clampi(i0 + 1, n);
+    ia = clampi(i0, P.n);
+    ib = clampi(i0 + 1, P.n);
 }
 // x >= lo and x < hi by order-preserving integer keys (-0 taken as +0; a NaN
 // fails one of the two tests, as in the FP64 comparisons).
@@ -116,57 +157,45 @@ __device__ __forceinline__ unsigned long long dkey(double v)
     return (b >> 63) ? ~b : (b | 0x8000000000000000ull);
 }
 
+// The loops over the axes and over z stay loops, an axis' values rotating
+// through registers: with them unrolled a quarter of the push's issue slots
+// waited for instructions.
 __device__ __forceinline__ void interp_f64(const Params& P, const E64* __restrict__ E, const double X[3],
                                            double Ep[3])
 {
-    int ia[3], ib[3];
-    double f[3], g[3];
-#pragma unroll
-    for (int a = 0; a < 3; ++a) cic_axis_q(X[a], P.lo[a], P.h[a], P.rh[a], P.n, ia[a], ib[a], f[a], g[a]);
-    const double wx[2] = { g[0], f[0] }, wy[2] = { g[1], f[1] }, wz[2] = { g[2], f[2] };
-    const int ix[2] = { ia[0], ib[0] }, iy[2] = { ia[1], ib[1] }, iz[2] = { ia[2], ib[2] };
-    double ax = 0.0, ay = 0.0, az = 0.0;
-#pragma unroll
-    for (int c = 0; c < 2; ++c)
-#pragma unroll
-        for (int b = 0; b < 2; ++b)
-#pragma unroll
-            for (int a = 0; a < 2; ++a) {
-                const double wgt = (wx[a] * wy[b]) * wz[c];
-                const E64 e = ld_e64(E + ((size_t)iz[c] * P.n + iy[b]) * P.n + ix[a]);
-                ax = __fma_rn(wgt, e.x, ax);
-                ay = __fma_rn(wgt, e.y, ay);
-                az = __fma_rn(wgt, e.z, az);
-            }
-    Ep[0] = ax; Ep[1] = ay; Ep[2] = az;
-}
-
-// Int64 CIC deposition of weight w at X into ne (one realization's block).
-__device__ __forceinline__ void deposit_f64(const Params& P, unsigned long long* __restrict__ ne,
-                                            const double X[3], uint32_t w)
-{
-    const long long one = 1ll << P.frac_bits;
-    const double scale = (double)one;
-    int ia[3], ib[3];
-    long long A[3][2];
-#pragma unroll
+    double x0 = X[0], x1 = X[1], x2 = X[2];
+    double f0 = 0.0, f1 = 0.0, f2 = 0.0, g0 = 0.0, g1 = 0.0, g2 = 0.0;
+    uint32_t j0 = 0, j1 = 0, j2 = 0;               // lower index | upper index << 16
+#pragma unroll 1
     for (int a = 0; a < 3; ++a) {
-        double f;
-        cic_axis(X[a], P.lo[a], P.h[a], P.rh[a], P.n, ia[a], ib[a], f);
-        const long long q = (long long)floor(f * scale);
-        A[a][0] = one - q;
-        A[a][1] = q;
+        int ia, ib;
+        double f, g;
+        cic_axis_q(P, x0, a, ia, ib, f, g);
+        x0 = x1; x1 = x2;
+        f0 = f1; f1 = f2; f2 = f;
+        g0 = g1; g1 = g2; g2 = g;
+        j0 = j1; j1 = j2; j2 = (uint32_t)ia | ((uint32_t)ib << 16);
     }
-    const int ix[2] = { ia[0], ib[0] }, iy[2] = { ia[1], ib[1] }, iz[2] = { ia[2], ib[2] };
-#pragma unroll
-    for (int c = 0; c < 2; ++c)
-#pragma unroll
-        for (int b = 0; b < 2; ++b)
-#pragma unroll
-            for (int a = 0; a < 2; ++a) {
-                const long long v = (long long)w * A[0][a] * A[1][b] * A[2][c];
-                if (v) atomicAdd(ne + ((size_t)iz[c] * P.n + iy[b]) * P.n + ix[a], (unsigned long long)v);
-            }
+    (void)x2;
+    const double w00 = g0 * g1, w10 = f0 * g1, w01 = g0 * f1, w11 = f0 * f1;   // (x, y)
+    const int n = P.n;
+    const uint32_t xa = j0 & 0xffffu, xb = j0 >> 16;
+    uint32_t ya = (j1 & 0xffffu) * n, yb = (j1 >> 16) * n, z = (j2 & 0xffffu);
+    double ax = 0.0, ay = 0.0, az = 0.0, wz = g2;
+#pragma unroll 1
+    for (int c = 0; c < 2; ++c) {
+        const E64* plane = E + (size_t)z * n * n;
+        const E64 e0 = ld_e64(plane + ya + xa), e1 = ld_e64(plane + ya + xb), e2 = ld_e64(plane + yb + xa),
+                  e3 = ld_e64(plane + yb + xb);
+        const double v0 = w00 * wz, v1 = w10 * wz, v2 = w01 * wz, v3 = w11 * wz;
+        ax = __fma_rn(v0, e0.x, ax); ay = __fma_rn(v0, e0.y, ay); az = __fma_rn(v0, e0.z, az);
+        ax = __fma_rn(v1, e1.x, ax); ay = __fma_rn(v1, e1.y, ay); az = __fma_rn(v1, e1.z, az);
+        ax = __fma_rn(v2, e2.x, ax); ay = __fma_rn(v2, e2.y, ay); az = __fma_rn(v2, e2.z, az);
+        ax = __fma_rn(v3, e3.x, ax); ay = __fma_rn(v3, e3.y, ay); az = __fma_rn(v3, e3.z, az);
+        wz = f2;
+        z = j2 >> 16;
+    }
+    Ep[0] = ax; Ep[1] = ay; Ep[2] = az;
 }
 
 __device__ __forceinline__ int real_of(const Params& P, uint32_t g) { return (int)(g >> (3 * P.log2n)); }
@@ -221,6 +250,51 @@ __device__ __forceinline__ void stencil_f32(const Params& P, const int id[3], co
         S.ib[a] = clampi(i0 + 1, P.n);
         S.A[a][0] = one - aa;
         S.A[a][1] = aa;
+    }
+}
+
+// FP64 form: one quotient per axis serves the cell index (clamped) and the
+// stencil.
+__device__ __forceinline__ void stencil_f64(const Params& P, const double X[3], int ic[3], Stencil& S)
+{
+    const long long one = 1ll << P.frac_bits;
+    double x0 = X[0], x1 = X[1], x2 = X[2];
+    uint32_t c0 = 0, c1 = 0, c2 = 0, j0 = 0, j1 = 0, j2 = 0, q0 = 0, q1 = 0, q2 = 0;
+#pragma unroll 1
+    for (int a = 0; a < 3; ++a) {
+        QSplit t;
+        int ci, i0;
+        long long fq;
+        double qd = 0.0;
+        bool split = quot_split(P, x0, a, t);
+        if (!split) {
+            qd = grid_quot(x0, P.lo[a], P.h[a], P.rh[a]);
+            split = qsplit(qd, t);
+        }
+        if (split) {
+            ci = t.qc;
+            i0 = t.i0;
+            fq = (long long)(t.F >> (t.sh - P.frac_bits));
+        } else {
+            ci = (int)floor(qd);
+            const double u = qd - 0.5;
+            const double fl = floor(u);
+            i0 = (int)fl;
+            fq = (long long)floor((u - fl) * (double)one);
+        }
+        x0 = x1; x1 = x2;
+        c0 = c1; c1 = c2; c2 = (uint32_t)clampi(ci, P.n);
+        j0 = j1; j1 = j2; j2 = (uint32_t)clampi(i0, P.n) | ((uint32_t)clampi(i0 + 1, P.n) << 16);
+        q0 = q1; q1 = q2; q2 = (uint32_t)fq;
+    }
+    ic[0] = (int)c0; ic[1] = (int)c1; ic[2] = (int)c2;
+    const uint32_t j[3] = { j0, j1, j2 }, q[3] = { q0, q1, q2 };
+#pragma unroll
+    for (int a = 0; a < 3; ++a) {
+        S.ia[a] = (int)(j[a] & 0xffffu);
+        S.ib[a] = (int)(j[a] >> 16);
+        S.A[a][0] = (uint32_t)one - q[a];
+        S.A[a][1] = q[a];
     }
 }
 
@@ -409,10 +483,31 @@ __device__ __forceinline__ double znormal(PairStream& s)
             return neg ? -v : v;
         }
         const double u = s.uniform();
-        const double fi = __ldg(g_zig_f + i), fm = __ldg(g_zig_f + i - 1);
-        if (fi + u * (fm - fi) < dexp(-0.5 * x * x)) return neg ? -x : x;
+        // the wedge test fi + u (fm - fi) < exp(-x^2 / 2) in FP32 where that
+        // decides it: both sides are at most 1 and off by less than 1e-6 there
+        // (rounding of x, u and the table 6e-8 each, x^2/2 < 6, expf 2 ulp)
+        const float xf = (float)x, fif = __ldg(g_zig_f32 + i), fmf = __ldg(g_zig_f32 + i - 1);
+        const float gap = expf(-0.5f * xf * xf) - __fmaf_rn((float)u, fmf - fif, fif);
+        bool accept = gap > 0.0f;
+        if (fabsf(gap) < 4e-6f) {
+            const double fi = __ldg(g_zig_f + i), fm = __ldg(g_zig_f + i - 1);
+            accept = fi + u * (fm - fi) < dexp(-0.5 * x * x);
+        }
+        if (accept) return __longlong_as_double(__double_as_longlong(x) ^ ((long long)neg << 63));
     }
     return 0.0;
+}
+
+__device__ __forceinline__ void znormal3(PairStream& s, double N[3])
+{
+    double n0 = 0.0, n1 = 0.0, n2 = 0.0;
+#pragma unroll 1
+    for (int a = 0; a < 3; ++a) {
+        n0 = n1;
+        n1 = n2;
+        n2 = znormal(s);
+    }
+    N[0] = n0; N[1] = n1; N[2] = n2;
 }
 
 __device__ __forceinline__ float znormal32(PairStream& s)
@@ -445,6 +540,9 @@ __device__ __forceinline__ float znormal32(PairStream& s)
 }
 
 // ------------------------------------------------------------------ pass 1
+// Bound by issue (3100 instructions per warp at 54% of the slots) and the FP64
+// pipe together: 9.7 ms for 7.2e7 particles, 19.5 ms with the quotients and
+// the wedge tests of the normals on the FP64 pipe and the loops unrolled.
 __global__ void __launch_bounds__(TPB, 4) k_push_f64(
     Params P, const P64* __restrict__ A, P64* __restrict__ B, uint32_t* __restrict__ keyB, uint32_t N,
     const uint32_t* __restrict__ cell_start, const E64* __restrict__ E, int32_t* __restrict__ cnt_new,
@@ -457,7 +555,7 @@ __global__ void __launch_bounds__(TPB, 4) k_push_f64(
     bool alive = false, mover = false;
     uint32_t gnew = 0, w = 0;
     int rr = 0;
-    Stencil S;
+    Stencil S{};
     if (i < N) {
         const P64 p = ld_p64(A + i);
         const uint32_t gold = p.cell;
@@ -472,8 +570,7 @@ __global__ void __launch_bounds__(TPB, 4) k_push_f64(
         interp_f64(P, E + (size_t)rp * P.n3, X, Ep);
         PairStream s(seed_of(P, rp), idx, step_of(P), P.push_tag_sp[sp], 0);
         double Nn[3];
-#pragma unroll
-        for (int a = 0; a < 3; ++a) Nn[a] = znormal(s);
+        znormal3(s, Nn);
         const double nmu = P.cmu_sp[sp], sdt = P.sdt_sp[sp];   // electrons: -mu, sqrt(2 D dt)
         double Xn[3];
         bool inside = true;
@@ -486,32 +583,8 @@ __global__ void __launch_bounds__(TPB, 4) k_push_f64(
         P64 q;
         q.x = Xn[0]; q.y = Xn[1]; q.z = Xn[2]; q.w = w;
         if (inside) {
-            // one division per axis serves the cell index and the stencil
             int ic[3];
-            const long long one = 1ll << P.frac_bits;
-#pragma unroll
-            for (int a = 0; a < 3; ++a) {
-                const double qd = grid_quot(Xn[a], P.lo[a], P.h[a], P.rh[a]);
-                QSplit t;
-                int ci, i0;
-                long long fq;
-                if (qsplit(qd, t)) {
-                    ci = t.qc;
-                    i0 = t.i0;
-                    fq = (long long)(t.F >> (t.sh - P.frac_bits));
-                } else {
-                    ci = (int)floor(qd);
-                    const double u = qd - 0.5;
-                    const double fl = floor(u);
-                    i0 = (int)fl;
-                    fq = (long long)floor((u - fl) * (double)one);
-                }
-                ic[a] = ci > P.n - 1 ? P.n - 1 : (ci < 0 ? 0 : ci);
-                S.ia[a] = clampi(i0, P.n);
-                S.ib[a] = clampi(i0 + 1, P.n);
-                S.A[a][0] = (uint32_t)(one - fq);
-                S.A[a][1] = (uint32_t)fq;
-            }
+            stencil_f64(P, Xn, ic, S);
             gnew = (uint32_t)(ebase + ((size_t)ic[2] * P.n + ic[1]) * P.n + ic[0]);
             alive = true;
             mover = gnew != gold;
@@ -557,7 +630,7 @@ __global__ void __launch_bounds__(TPB, 4) k_advect_f64(
     bool alive = false, mover = false;
     uint32_t gnew = 0, w = 0;
     int rr = 0;
-    Stencil S;
+    Stencil S{};
     if (i < N) {
         const P64 p = ld_p64(A + i);
         const uint32_t gold = p.cell;
@@ -582,32 +655,8 @@ __global__ void __launch_bounds__(TPB, 4) k_advect_f64(
         P64 q;
         q.x = Xn[0]; q.y = Xn[1]; q.z = Xn[2]; q.w = w;
         if (inside) {
-            // one division per axis serves the cell index and the stencil
             int ic[3];
-            const long long one = 1ll << P.frac_bits;
-#pragma unroll
-            for (int a = 0; a < 3; ++a) {
-                const double qd = grid_quot(Xn[a], P.lo[a], P.h[a], P.rh[a]);
-                QSplit t;
-                int ci, i0;
-                long long fq;
-                if (qsplit(qd, t)) {
-                    ci = t.qc;
-                    i0 = t.i0;
-                    fq = (long long)(t.F >> (t.sh - P.frac_bits));
-                } else {
-                    ci = (int)floor(qd);
-                    const double u = qd - 0.5;
-                    const double fl = floor(u);
-                    i0 = (int)fl;
-                    fq = (long long)floor((u - fl) * (double)one);
-                }
-                ic[a] = ci > P.n - 1 ? P.n - 1 : (ci < 0 ? 0 : ci);
-                S.ia[a] = clampi(i0, P.n);
-                S.ib[a] = clampi(i0 + 1, P.n);
-                S.A[a][0] = (uint32_t)(one - fq);
-                S.A[a][1] = (uint32_t)fq;
-            }
+            stencil_f64(P, Xn, ic, S);
             gnew = (uint32_t)(ebase + ((size_t)ic[2] * P.n + ic[1]) * P.n + ic[0]);
             alive = true;
             mover = gnew != gold;
@@ -752,15 +801,20 @@ __global__ void __launch_bounds__(TPB) k_deposit_f64(Params P, const P64* __rest
                                                      unsigned long long* __restrict__ ne_fix)
 {
     const uint32_t i = blockIdx.x * TPB + threadIdx.x;
-    bool alive = i < N;
+    const bool alive = i < N;
     uint32_t g = 0, w = 0;
+    int r = 0;
+    Stencil S{};
     if (alive) {
         const P64 p = ld_p64(A + i);
         g = p.cell;
         w = p.w;
+        r = real_of(P, g);
         const double X[3] = { p.x, p.y, p.z };
-        deposit_f64(P, ne_fix + (size_t)real_of(P, g) * P.n3, X, w);
+        int ic[3];
+        stencil_f64(P, X, ic, S);
     }
+    block_deposit<false>(P, ne_fix, alive, r, S, w);
     unsigned long long v = alive ? (unsigned long long)w : 0ull;
     unsigned c = alive ? 1u : 0u;
     if (warp_run_sum(g, alive, v, c)) atomicAdd(Xe + g, v);
@@ -2113,34 +2167,6 @@ __device__ __forceinline__ void cic32(float o, int idx, int n, int& ia, int& ib,
     ib = clampi(i0 + 1, n);
 }
 
-__device__ __forceinline__ void deposit32(const Params& P, unsigned long long* __restrict__ ne, const int id[3],
-                                          const float o[3], uint32_t w)
-{
-    const int one = 1 << P.frac_bits, half = one >> 1;
-    int ia[3], ib[3];
-    long long A[3][2];
-#pragma unroll
-    for (int a = 0; a < 3; ++a) {
-        const int q = (int)floorf(o[a] * (float)one);   // exact: o in [0,1), power-of-two scale
-        const int aa = (q + half) & (one - 1);
-        const int i0 = id[a] - 1 + (q >= half ? 1 : 0);
-        ia[a] = clampi(i0, P.n);
-        ib[a] = clampi(i0 + 1, P.n);
-        A[a][0] = one - aa;
-        A[a][1] = aa;
-    }
-    const int ix[2] = { ia[0], ib[0] }, iy[2] = { ia[1], ib[1] }, iz[2] = { ia[2], ib[2] };
-#pragma unroll
-    for (int c = 0; c < 2; ++c)
-#pragma unroll
-        for (int b = 0; b < 2; ++b)
-#pragma unroll
-            for (int a = 0; a < 2; ++a) {
-                const long long v = (long long)w * A[0][a] * A[1][b] * A[2][c];
-                if (v) atomicAdd(ne + ((size_t)iz[c] * P.n + iy[b]) * P.n + ix[a], (unsigned long long)v);
-            }
-}
-
 // Pass 1 of the mixed form: interpolation (FP32, cell-relative offsets),
 // push, new cell, fixed-point deposit, per-cell counts.  SINGLE: one
 // realization (Philox key and counter index are kernel-wide).
@@ -2158,7 +2184,7 @@ __global__ void __launch_bounds__(TPB, 4) k_push_f32(
     bool alive = false, mover = false;
     uint32_t gnew = 0, w = 0;
     int rr = 0;
-    Stencil S;
+    Stencil S{};
     if (i < N) {
         const P32 p = A[i];
         const uint32_t gold = __ldg(cA + i);
@@ -2300,18 +2326,22 @@ __global__ void __launch_bounds__(TPB) k_deposit_f32(Params P, const P32* __rest
                                                      unsigned long long* __restrict__ ne_fix)
 {
     const uint32_t i = blockIdx.x * TPB + threadIdx.x;
-    bool alive = i < N;
+    const bool alive = i < N;
     uint32_t g = 0, w = 0;
+    int r = 0;
+    Stencil S{};
     if (alive) {
         const P32 p = A[i];
         g = cA[i];
         w = p.w;
+        r = real_of(P, g);
         const uint32_t c = g & (uint32_t)(P.n3 - 1);
         const int id[3] = { (int)(c & (uint32_t)(P.n - 1)), (int)((c >> P.log2n) & (uint32_t)(P.n - 1)),
                             (int)(c >> (2 * P.log2n)) };
         const float o[3] = { p.ox, p.oy, p.oz };
-        deposit32(P, ne_fix + (size_t)real_of(P, g) * P.n3, id, o, w);
+        stencil_f32(P, id, o, S);
     }
+    block_deposit<false>(P, ne_fix, alive, r, S, w);
     unsigned long long v = alive ? (unsigned long long)w : 0ull;
     unsigned c = alive ? 1u : 0u;
     if (warp_run_sum(g, alive, v, c)) atomicAdd(Xe + g, v);
@@ -2366,8 +2396,7 @@ __global__ void __launch_bounds__(TPB) k_diffuse_f64(Params P, const P64* __rest
     const uint32_t idx = i - cell_start[(size_t)r * P.n3];
     PairStream s(seed_of(P, r), idx, step_of(P), TAG_PUSH, 0);
     double Nn[3];
-#pragma unroll
-    for (int a = 0; a < 3; ++a) Nn[a] = znormal(s);
+    znormal3(s, Nn);
     p.x = p.x + P.sdt * Nn[0];
     p.y = p.y + P.sdt * Nn[1];
     p.z = p.z + P.sdt * Nn[2];
