@@ -1572,6 +1572,7 @@ struct MergeScanOp {
         list_n[0] = (uint32_t)t[3];
         list_n[1] = (uint32_t)t[4];
         list_n[2] = (uint32_t)t[5];
+        list_n[3] = 0;            // cells that the merge by presorted lists leaves to k_merge_lv
     }
 };
 
@@ -1689,6 +1690,179 @@ __device__ __forceinline__ V grp_max(int gs, V v, unsigned lane)
 
 constexpr uint8_t NO_SPLIT = 0xff;
 
+// The list of one cell for its merge: existing particles with w > 0 in
+// canonical order, then the new ones in (source cell, products before
+// photoelectrons, slot) order, each handed to put(place, element).  One warp;
+// scratch holds np 8-byte words.  Returns the length, or NO_CELL when the cell
+// does not fit (more than max_m elements, or the arrays' capacities).
+constexpr uint32_t NO_CELL = 0xffffffffu;
+
+template <class E, class F>
+__device__ __forceinline__ uint32_t gather_cell(
+    const Params& P, const P64* __restrict__ A, const P32* __restrict__ A32, const uint32_t* __restrict__ cs,
+    const int64_t* __restrict__ gain, const Photo* __restrict__ photos, const uint32_t* __restrict__ photo_sorted,
+    const uint32_t* __restrict__ photo_off, const uint32_t* __restrict__ out_start, uint64_t Gphys, uint32_t cap,
+    uint32_t photo_cap, uint64_t g, uint32_t max_m, unsigned long long* pkey, unsigned lane, Counters* __restrict__ ctr,
+    F put)
+{
+    constexpr bool MX = std::is_same<E, MP32>::value;
+    const int b = real_of(P, (uint32_t)g);
+    const int sp = species_of(P, b), r = phys_of(P, b);
+    const uint32_t c = (uint32_t)(g & (uint64_t)(P.n3 - 1));
+    const long long dN = gain[g];
+    const uint32_t e0 = cs[g], e1 = cs[g + 1];
+    const uint32_t mprod = dN > 0 ? (uint32_t)(dN < P.n_new ? dN : P.n_new) : 0u;
+    // the photons absorbed in this cell: photoelectrons of the electron
+    // block and, with mobile ions, photo-ions of the positive-ion block
+    const uint64_t ge = g - (uint64_t)sp * Gphys;
+    const uint32_t p0 = sp <= 1 ? photo_off[ge] : 0u, np = sp <= 1 ? photo_off[ge + 1] - p0 : 0u;
+    const uint32_t Mmax = (e1 - e0) + mprod + np;
+    if (Mmax > max_m) {
+        if (lane == 0) atomicOr(&ctr->err, DERR_INTERNAL);
+        return NO_CELL;
+    }
+    if ((uint64_t)p0 + np > photo_cap || out_start[g + 1] > cap) {
+        if (lane == 0) atomicOr(&ctr->err, DERR_CAPACITY);
+        return NO_CELL;
+    }
+    // ---- gather: existing particles with w > 0 (canonical order)
+    uint32_t M = 0;
+    for (uint32_t b = e0; b < e1; b += 32) {
+        const uint32_t q = b + lane;
+        E e;
+        bool ok = false;
+        if (q < e1) {
+            if constexpr (MX) {
+                const P32 p = A32[q];
+                e.x = p.ox; e.y = p.oy; e.z = p.oz; e.w = p.w;
+            } else {
+                const P64 p = ld_p64(A + q);
+                e.x = p.x; e.y = p.y; e.z = p.z; e.w = p.w; e.pad = 0;
+            }
+            ok = e.w > 0;
+        }
+        const unsigned bal = __ballot_sync(0xffffffffu, ok);
+        if (ok) put(M + __popc(bal & ((1u << lane) - 1u)), e);
+        M += __popc(bal);
+    }
+    // photoelectrons ranked by (source cell, slot): keys staged in pkey
+    uint32_t n_lt = 0;
+    for (uint32_t j = lane; j < np; j += 32) {
+        const Photo& pj = photos[photo_sorted[p0 + j]];
+        pkey[j] = ((unsigned long long)pj.src << 8) | pj.slot;
+        n_lt += pj.src < c;
+    }
+    n_lt = __reduce_add_sync(0xffffffffu, n_lt);
+    __syncwarp();
+    for (uint32_t j = lane; j < np; j += 32) {
+        const unsigned long long kj = pkey[j];
+        uint32_t rank = 0;
+        for (uint32_t k = 0; k < np; ++k) rank += pkey[k] < kj;
+        const Photo pj = photos[photo_sorted[p0 + j]];
+        E e;
+        e.x = pj.x; e.y = pj.y; e.z = pj.z; e.w = pj.w;
+        if constexpr (!MX) e.pad = 0;
+        put(M + (rank < n_lt ? rank : rank + mprod), e);
+    }
+    // products: uniform in the cell, the remainder on the first
+    if (mprod) {
+        // dN <= n_new products weigh 1 each; else the products number n_new
+        long long wq = 1, rem = 0;
+        if (dN > P.n_new) {
+            if (dN < (1ll << 32)) {
+                wq = (uint32_t)dN / mprod;
+                rem = (uint32_t)dN % mprod;
+            } else {
+                wq = dN / (long long)mprod;
+                rem = dN % (long long)mprod;
+            }
+        }
+        const int ijk[3] = { (int)(c & (uint32_t)(P.n - 1)), (int)((c >> P.log2n) & (uint32_t)(P.n - 1)),
+                             (int)(c >> (2 * P.log2n)) };
+        for (uint32_t j = lane; j < mprod; j += 32) {
+            Stream st(seed_of(P, r), c, step_of(P), P.prod_tag_sp[sp], j);
+            E e;
+            if constexpr (MX) {
+                // FP32 uniforms from the high words of the FP64 ones
+                float X[3];
+#pragma unroll
+                for (int a = 0; a < 3; ++a) {
+                    X[a] = uniform_f32(st.u32());
+                    (void)st.u32();
+                }
+                e.x = X[0]; e.y = X[1]; e.z = X[2];
+            } else {
+                double X[3];
+#pragma unroll
+                for (int a = 0; a < 3; ++a) X[a] = P.lo[a] + ((double)ijk[a] + st.uniform()) * P.h[a];
+                e.x = X[0]; e.y = X[1]; e.z = X[2];
+            }
+            const long long wj = wq + (j == 0 ? rem : 0);
+            if (wj > 0xffffffffll) atomicOr(&ctr->err, DERR_OVERFLOW);
+            e.w = (uint32_t)wj;
+            if constexpr (!MX) e.pad = 0;
+            put(M + n_lt + j, e);
+        }
+    }
+    __syncwarp();
+    return M + mprod + np;
+}
+
+// One leaf, positions q0..q1 - 1 of the list at(q), to output place o: weight
+// sum, weight-averaged position (list order).
+template <class E, class F>
+__device__ __forceinline__ void write_leaf(uint32_t q0, uint32_t q1, uint32_t o, uint32_t g, P64* __restrict__ out,
+                                           P32* __restrict__ out32, uint32_t* __restrict__ cout,
+                                           Counters* __restrict__ ctr, F at)
+{
+    constexpr bool MX = std::is_same<E, MP32>::value;
+    if constexpr (MX) {
+        // mixed form: a one-element leaf keeps its offsets; the
+        // weighted mean of a larger leaf is taken in FP32
+        P32 r;
+        if (q1 - q0 == 1) {
+            const E e = at(q0);
+            r.ox = e.x; r.oy = e.y; r.oz = e.z; r.w = e.w;
+        } else {
+            float sx = 0.f, sy = 0.f, sz = 0.f;
+            unsigned long long Wl = 0;
+            for (uint32_t q = q0; q < q1; ++q) {
+                const E e = at(q);
+                const float wf = (float)e.w;
+                sx = __fmaf_rn(wf, e.x, sx);
+                sy = __fmaf_rn(wf, e.y, sy);
+                sz = __fmaf_rn(wf, e.z, sz);
+                Wl += e.w;
+            }
+            if (Wl > 0xffffffffull) atomicOr(&ctr->err, DERR_OVERFLOW);
+            const float Wf = (float)Wl;
+            r.ox = clamp_offf(sx / Wf); r.oy = clamp_offf(sy / Wf); r.oz = clamp_offf(sz / Wf);
+            r.w = (uint32_t)Wl;
+        }
+        out32[o] = r;
+        cout[o] = g;
+    } else {
+        double sx = 0.0, sy = 0.0, sz = 0.0;
+        unsigned long long Wl = 0;
+        for (uint32_t q = q0; q < q1; ++q) {
+            const E e = at(q);
+            const double wd = (double)e.w;
+            sx = __fma_rn(wd, e.x, sx);
+            sy = __fma_rn(wd, e.y, sy);
+            sz = __fma_rn(wd, e.z, sz);
+            Wl += e.w;
+        }
+        if (Wl > 0xffffffffull) atomicOr(&ctr->err, DERR_OVERFLOW);
+        // quotients by the reciprocal of W with one fused correction
+        const double Wd = (double)Wl, rw = 1.0 / Wd;
+        P64 r;
+        r.x = quot_r(sx, Wd, rw); r.y = quot_r(sy, Wd, rw); r.z = quot_r(sz, Wd, rw);
+        r.cell = g;
+        r.w = (uint32_t)Wl;
+        st_p64(out + o, r);
+    }
+}
+
 // Merge/split of whole cells, one warp per cell, all nodes of a tree level
 // at once.  The cell's list (existing particles with w > 0 in canonical
 // order, then new ones in (source cell, products before photoelectrons,
@@ -1725,35 +1899,23 @@ __global__ void __launch_bounds__(128, GLOBAL ? 4 : (std::is_same<E, MP32>::valu
     unsigned long long t_cells = 0, t_el = 0, t_sq = 0, t_max = 0;
     for (uint32_t li = blockIdx.x * nw + wid; li < ncells; li += gridDim.x * nw) {
         const uint64_t g = list[li];                  // particle cell
-        const int b = real_of(P, (uint32_t)g);
-        const int sp = species_of(P, b), r = phys_of(P, b);
-        const uint32_t c = (uint32_t)(g & (uint64_t)(P.n3 - 1));
-        const long long dN = gain[g];
-        const uint32_t e0 = cs[g], e1 = cs[g + 1];
-        const uint32_t mprod = dN > 0 ? (uint32_t)(dN < P.n_new ? dN : P.n_new) : 0u;
-        // the photons absorbed in this cell: photoelectrons of the electron
-        // block and, with mobile ions, photo-ions of the positive-ion block
-        const uint64_t ge = g - (uint64_t)sp * Gphys;
-        const uint32_t p0 = sp <= 1 ? photo_off[ge] : 0u, np = sp <= 1 ? photo_off[ge + 1] - p0 : 0u;
-        const uint32_t Mmax = (e1 - e0) + mprod + np;
-        if ((uint64_t)p0 + np > photo_cap || out_start[g + 1] > cap) {
-            if (lane == 0) atomicOr(&ctr->err, DERR_CAPACITY);
-            continue;
-        }
         MLayout L;
         unsigned char* base;
+        uint32_t max_m;
         if constexpr (GLOBAL) {
-            L = merge_layout(Mmax + T, T, sizeof(E), sizeof(K));
+            const uint64_t gp = g - (uint64_t)species_of(P, real_of(P, (uint32_t)g)) * Gphys;
+            const bool ph = g < 2 * Gphys;              // electrons and positive ions take photo particles
+            const long long dN = gain[g];
+            max_m = (cs[g + 1] - cs[g]) + (dN > 0 ? (uint32_t)(dN < P.n_new ? dN : P.n_new) : 0u) +
+                    (ph ? photo_off[gp + 1] - photo_off[gp] : 0u);
+            L = merge_layout(max_m + T, T, sizeof(E), sizeof(K));
             if (work_off[g] * 32 + L.bytes > work_cap * 32) {
                 if (lane == 0) atomicOr(&ctr->err, DERR_CAPACITY);
                 continue;
             }
             base = work + work_off[g] * 32;
         } else {
-            if (Mmax + T > CAP) {
-                if (lane == 0) atomicOr(&ctr->err, DERR_INTERNAL);
-                continue;
-            }
+            max_m = CAP - T;
             L = merge_layout(CAP, T, sizeof(E), sizeof(K));
             base = msm + (size_t)wid * L.bytes;
         }
@@ -1775,77 +1937,10 @@ __global__ void __launch_bounds__(128, GLOBAL ? 4 : (std::is_same<E, MP32>::valu
         uint8_t* nax = reinterpret_cast<uint8_t*>(base + L.nax);
         uint8_t* nfl = reinterpret_cast<uint8_t*>(base + L.nfl);
 
-        // ---- gather: existing particles with w > 0 (canonical order)
-        uint32_t M = 0;
-        for (uint32_t b = e0; b < e1; b += 32) {
-            const uint32_t q = b + lane;
-            E e;
-            bool ok = false;
-            if (q < e1) {
-                if constexpr (MX) {
-                    const P32 p = A32[q];
-                    e.x = p.ox; e.y = p.oy; e.z = p.oz; e.w = p.w;
-                } else {
-                    const P64 p = ld_p64(A + q);
-                    e.x = p.x; e.y = p.y; e.z = p.z; e.w = p.w; e.pad = 0;
-                }
-                ok = e.w > 0;
-            }
-            const unsigned bal = __ballot_sync(0xffffffffu, ok);
-            if (ok) cur[M + __popc(bal & ((1u << lane) - 1u))] = e;
-            M += __popc(bal);
-        }
-        // photoelectrons ranked by (source cell, slot): keys staged in tmp
-        unsigned long long* pkey = reinterpret_cast<unsigned long long*>(tmp);
-        uint32_t n_lt = 0;
-        for (uint32_t j = lane; j < np; j += 32) {
-            const Photo& pj = photos[photo_sorted[p0 + j]];
-            pkey[j] = ((unsigned long long)pj.src << 8) | pj.slot;
-            n_lt += pj.src < c;
-        }
-        n_lt = __reduce_add_sync(0xffffffffu, n_lt);
-        __syncwarp();
-        for (uint32_t j = lane; j < np; j += 32) {
-            const unsigned long long kj = pkey[j];
-            uint32_t rank = 0;
-            for (uint32_t k = 0; k < np; ++k) rank += pkey[k] < kj;
-            const Photo pj = photos[photo_sorted[p0 + j]];
-            E e;
-            e.x = pj.x; e.y = pj.y; e.z = pj.z; e.w = pj.w;
-            if constexpr (!MX) e.pad = 0;
-            cur[M + (rank < n_lt ? rank : rank + mprod)] = e;
-        }
-        // products: uniform in the cell, the remainder on the first
-        if (mprod) {
-            const long long wq = dN / (long long)mprod, rem = dN % (long long)mprod;
-            const int ijk[3] = { (int)(c & (uint32_t)(P.n - 1)), (int)((c >> P.log2n) & (uint32_t)(P.n - 1)),
-                                 (int)(c >> (2 * P.log2n)) };
-            for (uint32_t j = lane; j < mprod; j += 32) {
-                Stream st(seed_of(P, r), c, step_of(P), P.prod_tag_sp[sp], j);
-                E e;
-                if constexpr (MX) {
-                    // FP32 uniforms from the high words of the FP64 ones
-                    float X[3];
-#pragma unroll
-                    for (int a = 0; a < 3; ++a) {
-                        X[a] = uniform_f32(st.u32());
-                        (void)st.u32();
-                    }
-                    e.x = X[0]; e.y = X[1]; e.z = X[2];
-                } else {
-                    double X[3];
-#pragma unroll
-                    for (int a = 0; a < 3; ++a) X[a] = P.lo[a] + ((double)ijk[a] + st.uniform()) * P.h[a];
-                    e.x = X[0]; e.y = X[1]; e.z = X[2];
-                }
-                const long long wj = wq + (j == 0 ? rem : 0);
-                if (wj > 0xffffffffll) atomicOr(&ctr->err, DERR_OVERFLOW);
-                e.w = (uint32_t)wj;
-                if constexpr (!MX) e.pad = 0;
-                cur[M + n_lt + j] = e;
-            }
-        }
-        M += mprod + np;
+        const uint32_t M = gather_cell<E>(
+            P, A, A32, cs, gain, photos, photo_sorted, photo_off, out_start, Gphys, cap, photo_cap, g, max_m,
+            reinterpret_cast<unsigned long long*>(tmp), lane, ctr, [&](uint32_t j, const E& e) { cur[j] = e; });
+        if (M == NO_CELL) continue;
         if (lane == 0) {
             t_cells += 1; t_el += M; t_sq += (unsigned long long)M * M; t_max = M > t_max ? M : t_max;
             nb[0] = 0;
@@ -2096,57 +2191,367 @@ __global__ void __launch_bounds__(128, GLOBAL ? 4 : (std::is_same<E, MP32>::valu
             if (lane == 0) atomicOr(&ctr->err, DERR_INTERNAL);
         } else {
             for (int d = lane; d < nnodes; d += 32) {
-                if constexpr (MX) {
-                    // mixed form: a one-element leaf keeps its offsets; the
-                    // weighted mean of a larger leaf is taken in FP32
-                    const uint32_t q0 = nb[d], q1 = nb[d + 1];
-                    P32 o;
-                    if (q1 - q0 == 1) {
-                        const E e = cur[q0];
-                        o.ox = e.x; o.oy = e.y; o.oz = e.z; o.w = e.w;
-                    } else {
-                        float sx = 0.f, sy = 0.f, sz = 0.f;
-                        unsigned long long Wl = 0;
-                        for (uint32_t q = q0; q < q1; ++q) {
-                            const E e = cur[q];
-                            const float wf = (float)e.w;
-                            sx = __fmaf_rn(wf, e.x, sx);
-                            sy = __fmaf_rn(wf, e.y, sy);
-                            sz = __fmaf_rn(wf, e.z, sz);
-                            Wl += e.w;
-                        }
-                        if (Wl > 0xffffffffull) atomicOr(&ctr->err, DERR_OVERFLOW);
-                        const float Wf = (float)Wl;
-                        o.ox = clamp_offf(sx / Wf); o.oy = clamp_offf(sy / Wf); o.oz = clamp_offf(sz / Wf);
-                        o.w = (uint32_t)Wl;
-                    }
-                    out32[o0 + d] = o;
-                    cout[o0 + d] = (uint32_t)g;
-                } else {
-                    double sx = 0.0, sy = 0.0, sz = 0.0;
-                    unsigned long long Wl = 0;
-                    for (uint32_t q = nb[d]; q < nb[d + 1]; ++q) {
-                        const E e = cur[q];
-                        const double wd = (double)e.w;
-                        sx = __fma_rn(wd, e.x, sx);
-                        sy = __fma_rn(wd, e.y, sy);
-                        sz = __fma_rn(wd, e.z, sz);
-                        Wl += e.w;
-                    }
-                    if (Wl > 0xffffffffull) atomicOr(&ctr->err, DERR_OVERFLOW);
-                    // quotients by the reciprocal of W with one fused correction
-                    const double Wd = (double)Wl, rw = 1.0 / Wd;
-                    P64 o;
-                    o.x = quot_r(sx, Wd, rw); o.y = quot_r(sy, Wd, rw); o.z = quot_r(sz, Wd, rw);
-                    o.cell = (uint32_t)g;
-                    o.w = (uint32_t)Wl;
-                    st_p64(out + o0 + d, o);
-                }
+                write_leaf<E>(nb[d], nb[d + 1], o0 + d, (uint32_t)g, out, out32, cout, ctr,
+                              [&](uint32_t q) { return cur[q]; });
             }
         }
         __syncwarp();
     }
     // workload counters, one atomic each per warp
+    if (lane == 0 && t_cells) {
+        atomicAdd(&ctr->merge_cells, t_cells);
+        atomicAdd(&ctr->merge_elems, t_el);
+        atomicAdd(&ctr->merge_elems2, t_sq);
+        atomicMax(&ctr->merge_maxm, t_max);
+    }
+}
+
+// ------------------------------------------------------------------ merge by presorted lists
+// The same tree as k_merge_lv, without a sort per level: the cell's elements
+// are ranked along each axis once, and every level keeps the three lists (the
+// nodes' elements in x, y and z order) by a stable partition.  A node's
+// bounds are then the ends of its three segments, and the weighted median is
+// one running sum along the list of its axis.  An entry is an element with a
+// weight; a median that is divided gets a second entry, a copy with the rest
+// of the weight.  A position's word holds the entries of the x, y and z list
+// there (one byte each) and its node.  The last level needs no lists: its
+// leaves are ranges of the lists it splits.
+// The order of equal coordinates depends on the splits before, which the
+// presorted lists do not know: cells with two equal coordinates along an axis
+// (as after a split of one particle without diffusion), and cells of 2^31
+// electrons or more (the sums here have 32 bits), are listed for k_merge_lv.
+// Bound by instruction issue (80% of the slots; about 4000 per warp and cell
+// of 28 elements, k_merge_lv twice that in the FP64 form); seven blocks per SM
+// measured best of six to nine.
+struct __align__(16) MNode {     // a node
+    uint32_t W, S;               // weight; weights of the nodes before it
+    uint16_t s0, n;              // first position, entries
+    uint8_t ax, pax;             // split axis; the axis of the split that made it
+    uint16_t pad;
+};
+struct __align__(8) MMed {       // its weighted median
+    uint32_t C;                  // weights up to and with it
+    uint16_t pm;                 // its place in the node
+    uint16_t e;                  // its entry
+};
+struct __align__(16) MRec {      // a node's split, for its entries
+    uint16_t s0, pm;
+    uint16_t pr, pl;             // right entries of the nodes before; left entries up to and with this node
+    uint8_t ax, med, child, fresh;   // axis; the median's side (0 left, 1 right, 2 both); first child; second entry
+    uint32_t pad;
+};
+struct __align__(16) MLeaf {     // a leaf of the last level: positions q0..q1 - 1 of the list of axis ax,
+    uint16_t q0, q1;             // the one at qs (0xffff: none) with weight w
+    uint16_t qs, ax;
+    uint32_t w, pad;
+};
+struct PreLayout {
+    uint32_t key[3], ew, list, side, node, rec, med, bytes;
+};
+__host__ __device__ inline PreLayout pre_layout(uint32_t cap, uint32_t T, uint32_t ksize)
+{
+    PreLayout L;
+    uint32_t o = 0;
+    for (int a = 0; a < 3; ++a) L.key[a] = ml_take(o, cap * ksize);
+    L.ew = ml_take(o, cap * 4);
+    L.list = ml_take(o, 8 * cap);     // the words of this and the next level (first 8-byte scratch of the gather)
+    L.side = ml_take(o, cap);
+    L.node = ml_take(o, 2 * T * (uint32_t)sizeof(MNode));      // the leaves take the second half at the last level
+    L.rec = ml_take(o, T * (uint32_t)sizeof(MRec));
+    L.med = ml_take(o, T * (uint32_t)sizeof(MMed));
+    L.bytes = o;
+    return L;
+}
+
+template <class E>
+__global__ void __launch_bounds__(128, 7) k_merge_pre(
+    Params P, const P64* __restrict__ A, const P32* __restrict__ A32, const uint32_t* __restrict__ cs,
+    const int64_t* __restrict__ gain, const Photo* __restrict__ photos, const uint32_t* __restrict__ photo_sorted,
+    const uint32_t* __restrict__ photo_off, const uint32_t* __restrict__ out_start, P64* __restrict__ out,
+    P32* __restrict__ out32, uint32_t* __restrict__ cout, uint64_t Gphys, uint32_t cap, uint32_t photo_cap,
+    const uint32_t* __restrict__ list, uint32_t* __restrict__ list_n, int tier, uint32_t CAP,
+    uint32_t* __restrict__ tie_list, Counters* __restrict__ ctr)
+{
+    constexpr bool MX = std::is_same<E, MP32>::value;
+    constexpr unsigned FULL = 0xffffffffu;
+    using K = typename EKey<E>::K;
+    extern __shared__ __align__(16) unsigned char msm[];
+    const unsigned lane = lane_id(), wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
+    const unsigned lt = (1u << lane) - 1u;
+    const int T = P.ppc;
+    const uint32_t ncells = list_n[tier];
+    const PreLayout L = pre_layout(CAP, T, sizeof(K));
+    unsigned char* const base = msm + (size_t)wid * L.bytes;
+    K* const key0 = reinterpret_cast<K*>(base + L.key[0]);
+    const uint32_t KS = (L.key[1] - L.key[0]) / (uint32_t)sizeof(K);   // keys from one axis to the next
+    uint32_t* const ew = reinterpret_cast<uint32_t*>(base + L.ew);
+    uint8_t* const side = base + L.side;
+    MRec* const rec = reinterpret_cast<MRec*>(base + L.rec);
+    MMed* const med = reinterpret_cast<MMed*>(base + L.med);
+    unsigned long long t_cells = 0, t_el = 0, t_sq = 0, t_max = 0;
+    for (uint32_t li = blockIdx.x * nw + wid; li < ncells; li += gridDim.x * nw) {
+        const uint64_t g = list[li];
+        uint32_t* ls = reinterpret_cast<uint32_t*>(base + L.list);    // words of this level
+        uint32_t* ls2 = ls + CAP;
+        MNode* nd = reinterpret_cast<MNode*>(base + L.node);
+        MNode* nd2 = nd + T;
+        const uint32_t M = gather_cell<E>(
+            P, A, A32, cs, gain, photos, photo_sorted, photo_off, out_start, Gphys, cap, photo_cap, g, CAP - T,
+            reinterpret_cast<unsigned long long*>(ls), lane, ctr, [&](uint32_t j, const E& e) {
+#pragma unroll
+                for (int a = 0; a < 3; ++a) key0[a * KS + j] = ET<E>::key(e, a);
+                ew[j] = e.w;
+            });
+        if (M == NO_CELL) continue;
+        constexpr uint32_t VEC = 16 / sizeof(K);
+        for (uint32_t j = M + lane; j < ((M + VEC - 1) & ~(VEC - 1)); j += 32)
+#pragma unroll
+            for (int a = 0; a < 3; ++a) key0[a * KS + j] = (K)~(K)0;     // never below a real key
+        __syncwarp();
+        // ---- ranks along the axes; equal keys share a rank, so that the ranks
+        // then do not add up to M (M - 1) / 2
+        unsigned long long wroot = 0;
+        bool other = false;
+#pragma unroll 1
+        for (int a = 0; a < 3; ++a) {
+            const K* ka = key0 + a * KS;
+            uint32_t total = 0;
+            for (uint32_t b0 = 0; b0 < M; b0 += 32) {
+                const uint32_t j = b0 + lane;
+                const bool ok = j < M;
+                const K kj = ka[ok ? j : 0];
+                uint32_t rk = 0;
+                if constexpr (MX) {
+#pragma unroll 2
+                    for (uint32_t k = 0; k < M; k += 4) {
+                        const uint4 q = *reinterpret_cast<const uint4*>(ka + k);
+                        rk += (q.x < kj) + (q.y < kj) + (q.z < kj) + (q.w < kj);
+                    }
+                } else {
+#pragma unroll 2
+                    for (uint32_t k = 0; k < M; k += 2) {
+                        const ulonglong2 q = *reinterpret_cast<const ulonglong2*>(ka + k);
+                        rk += (q.x < kj) + (q.y < kj);
+                    }
+                }
+                if (ok) {
+                    uint8_t* w = reinterpret_cast<uint8_t*>(ls + rk);
+                    w[a] = (uint8_t)j;
+                    total += rk;
+                    if (a == 0) {
+                        w[3] = 0;
+                        wroot += ew[j];
+                    }
+                }
+            }
+            other |= __reduce_add_sync(FULL, total) != M * (M - 1) / 2;
+        }
+#pragma unroll
+        for (int dd = 16; dd > 0; dd >>= 1) wroot += __shfl_xor_sync(FULL, wroot, dd);
+        if (other || wroot >= (1ull << 31)) {
+            if (lane == 0) tie_list[atomicAdd(list_n + 3, 1u)] = (uint32_t)g;
+            __syncwarp();
+            continue;
+        }
+        if (lane == 0) {
+            t_cells += 1; t_el += M; t_sq += (unsigned long long)M * M; t_max = M > t_max ? M : t_max;
+            nd[0] = MNode{ (uint32_t)wroot, 0u, 0, (uint16_t)M, 0, 0, 0 };
+        }
+        uint32_t n = M, nent = M;
+        int nnodes = 1;
+        bool leaves = false;                      // the leaves stand in nd2
+        __syncwarp();
+
+        for (int level = 1; level < T; level *= 2) {
+            const bool last = level * 2 >= T;
+            // ---- split axis of every node (NO_SPLIT below weight 2)
+            bool any_split = false;
+            for (int d = lane; d < nnodes; d += 32) {
+                const MNode q = nd[d];
+                uint8_t ax = NO_SPLIT;
+                if (q.W >= 2) {
+                    K lo[3], hi[3];
+                    const uint32_t w0 = ls[q.s0], w1 = ls[q.s0 + q.n - 1u];
+#pragma unroll
+                    for (int a = 0; a < 3; ++a) {
+                        lo[a] = key0[a * KS + ((w0 >> (8 * a)) & 255u)];
+                        hi[a] = key0[a * KS + ((w1 >> (8 * a)) & 255u)];
+                    }
+                    ax = (uint8_t)widest_axis<E>(lo, hi);
+                    any_split = true;
+                }
+                nd[d].ax = ax;
+            }
+            if (!__any_sync(FULL, any_split)) break;
+            __syncwarp();
+            // ---- weighted medians: the running weight along each node's list
+            uint32_t run = 0;
+            for (uint32_t b0 = 0; b0 < n; b0 += 32) {
+                const uint32_t p = b0 + lane, pc = p < n ? p : n - 1u;
+                const uint32_t word = ls[pc], d = word >> 24;
+                const MNode q = nd[d];
+                const uint32_t e = (word >> (q.ax == NO_SPLIT ? 0u : 8u * q.ax)) & 255u;
+                const uint32_t w = p < n ? ew[e] : 0u;
+                uint32_t x = w;
+#pragma unroll
+                for (int k = 1; k < 32; k <<= 1) {
+                    const uint32_t y = __shfl_up_sync(FULL, x, k);
+                    if ((int)lane >= k) x += y;
+                }
+                x += run;
+                run = __shfl_sync(FULL, x, 31);
+                const uint32_t v = x - q.S;
+                if (p < n && q.ax != NO_SPLIT && 2u * v > q.W && 2u * (v - w) <= q.W)
+                    med[d] = MMed{ v, (uint16_t)(p - q.s0), (uint16_t)e };
+            }
+            __syncwarp();
+            // ---- per node: median rule, the children's places
+            uint32_t cL = 0, cR = 0, cN = 0, cE = 0;     // left, right entries, children, new entries so far
+            for (int d0 = 0; d0 < nnodes; d0 += 32) {
+                const int d = d0 + (int)lane;
+                MNode q{};
+                MMed m{};
+                uint32_t lsz = 0, rsz = 0, cnt = 0, both = 0, a = 0, b = 0, wl = 0;
+                uint8_t medside = 0;
+                if (d < nnodes) {
+                    q = nd[d];
+                    cnt = 1;
+                    lsz = q.n;
+                    m.pm = q.n;
+                    wl = q.W;
+                    if (q.ax != NO_SPLIT) {
+                        m = med[d];
+                        const uint32_t wm = ew[m.e], WL = m.C - wm;
+                        // a unit weight joins the lighter side (left on ties), a
+                        // heavier one is divided (W + 1) / 2 - W_L : rest
+                        if (wm == 1) {
+                            a = WL <= q.W - m.C;
+                            b = 1u - a;
+                        } else {
+                            a = (q.W + 1u) / 2u - WL;
+                            b = wm - a;
+                        }
+                        const uint32_t lm = a > 0, rm = b > 0;
+                        cnt = 2;
+                        wl = WL + a;
+                        both = lm & rm;
+                        medside = both ? 2 : (lm ? 0 : 1);
+                        lsz = m.pm + lm;
+                        rsz = q.n - m.pm - 1u + rm;
+                    }
+                }
+                uint32_t k1 = lsz | (rsz << 16), k2 = cnt | (both << 16);
+                const int reach = nnodes - d0;
+                for (int k = 1; k < 32 && k < reach; k <<= 1) {
+                    const uint32_t y1 = __shfl_up_sync(FULL, k1, k), y2 = __shfl_up_sync(FULL, k2, k);
+                    if ((int)lane >= k) { k1 += y1; k2 += y2; }
+                }
+                const uint32_t pl = cL + (k1 & 0xffffu), pr = cR + (k1 >> 16) - rsz;
+                const uint32_t child = cN + (k2 & 0xffffu) - cnt, fresh = nent + cE + (k2 >> 16) - both;
+                if (d < nnodes && last) {
+                    MLeaf* lf = reinterpret_cast<MLeaf*>(nd2) + child;
+                    const uint32_t s0 = q.s0;
+                    if (q.ax == NO_SPLIT) {
+                        lf[0] = MLeaf{ q.s0, (uint16_t)(s0 + q.n), 0xffff, q.pax, 0u, 0u };
+                    } else {
+                        const uint32_t qm = s0 + m.pm;
+                        lf[0] = MLeaf{ q.s0, (uint16_t)(qm + (a > 0)), (uint16_t)(a > 0 ? qm : 0xffffu), q.ax, a, 0u };
+                        lf[1] = MLeaf{ (uint16_t)(qm + (b > 0 ? 0u : 1u)), (uint16_t)(s0 + q.n),
+                                       (uint16_t)(b > 0 ? qm : 0xffffu), q.ax, b, 0u };
+                    }
+                } else if (d < nnodes) {
+                    rec[d] = MRec{ q.s0, m.pm, (uint16_t)pr, (uint16_t)pl, (uint8_t)(q.ax == NO_SPLIT ? 0 : q.ax), medside,
+                                   (uint8_t)child, (uint8_t)fresh, 0u };
+                    if (both) {
+                        ew[m.e] = a;
+                        ew[fresh] = b;
+#pragma unroll
+                        for (int x = 0; x < 3; ++x) key0[x * KS + fresh] = key0[x * KS + m.e];
+                    }
+                    const uint32_t start = pl - lsz + pr;
+                    const uint8_t cax = q.ax == NO_SPLIT ? q.pax : q.ax;
+                    nd2[child] = MNode{ wl, q.S, (uint16_t)start, (uint16_t)lsz, 0, cax, 0 };
+                    if (q.ax != NO_SPLIT)
+                        nd2[child + 1] = MNode{ q.W - wl, q.S + wl, (uint16_t)(start + lsz), (uint16_t)rsz, 0, cax, 0 };
+                }
+                const int top = reach < 32 ? reach - 1 : 31;
+                const uint32_t e1 = __shfl_sync(FULL, k1, top), e2 = __shfl_sync(FULL, k2, top);
+                cL += e1 & 0xffffu;
+                cR += e1 >> 16;
+                cN += e2 & 0xffffu;
+                cE += e2 >> 16;
+            }
+            nnodes = (int)cN;
+            __syncwarp();
+            if (last) { leaves = true; break; }
+            // ---- each entry's side, from its place along the split axis
+            for (uint32_t p = lane; p < n; p += 32) {
+                const uint32_t word = ls[p];
+                const MRec r = rec[word >> 24];
+                const uint32_t at = p - r.s0;
+                side[(word >> (8 * r.ax)) & 255u] = at < r.pm ? 0 : (at > r.pm ? 1 : r.med);
+            }
+            __syncwarp();
+            // ---- stable partition of the three lists
+            uint32_t runL[3] = { 0, 0, 0 }, runR[3] = { 0, 0, 0 };
+            for (uint32_t b0 = 0; b0 < n; b0 += 32) {
+                const uint32_t p = b0 + lane, pc = p < n ? p : n - 1u;
+                const uint32_t word = ls[pc];
+                const MRec r = rec[word >> 24];
+                const bool more = b0 + 32 < n;
+                uint8_t* const to = reinterpret_cast<uint8_t*>(ls2);
+#pragma unroll
+                for (int a = 0; a < 3; ++a) {
+                    const uint32_t e = (word >> (8 * a)) & 255u;
+                    const uint32_t sd = p < n ? side[e] : 3u;
+                    const bool gl = !(sd & 1u), gr = sd - 1u < 2u;        // left: 0, 2; right: 1, 2
+                    const unsigned bl = __ballot_sync(FULL, gl), br = __ballot_sync(FULL, gr);
+                    const uint32_t ql = runL[a] + __popc(bl & lt) + r.pr, qr = runR[a] + __popc(br & lt) + r.pl;
+                    if (gl) {
+                        to[4 * ql + a] = (uint8_t)e;
+                        if (a == 0) to[4 * ql + 3] = r.child;
+                    }
+                    if (gr) {
+                        to[4 * qr + a] = sd == 2u ? r.fresh : (uint8_t)e;
+                        if (a == 0) to[4 * qr + 3] = (uint8_t)(r.child + 1u);
+                    }
+                    if (more) {
+                        runL[a] += __popc(bl);
+                        runR[a] += __popc(br);
+                    }
+                }
+            }
+            n = cL + cR;
+            nent += cE;
+            { uint32_t* t = ls; ls = ls2; ls2 = t; }
+            { MNode* t = nd; nd = nd2; nd2 = t; }
+            __syncwarp();
+        }
+        // ---- leaves, in the order along the axis of the split that made them
+        // (one particle per cell: the whole list in its own order)
+        const uint32_t o0 = out_start[g];
+        if ((uint32_t)nnodes != out_start[g + 1] - o0) {
+            if (lane == 0) atomicOr(&ctr->err, DERR_INTERNAL);
+        } else {
+            for (int d = lane; d < nnodes; d += 32) {
+                MLeaf f;
+                if (leaves) {
+                    f = reinterpret_cast<const MLeaf*>(nd2)[d];
+                } else {
+                    const MNode q = nd[d];
+                    f = MLeaf{ q.s0, (uint16_t)(q.s0 + q.n), 0xffff, q.pax, 0u, 0u };
+                }
+                write_leaf<E>(f.q0, f.q1, o0 + d, (uint32_t)g, out, out32, cout, ctr, [&](uint32_t q) {
+                    const uint32_t en = T > 1 ? (ls[q] >> (8 * f.ax)) & 255u : q;
+                    E e;
+                    e.x = okey_val(key0[en]); e.y = okey_val(key0[KS + en]); e.z = okey_val(key0[2 * KS + en]);
+                    e.w = q == f.qs ? f.w : ew[en];
+                    return e;
+                });
+            }
+        }
+        __syncwarp();
+    }
     if (lane == 0 && t_cells) {
         atomicAdd(&ctr->merge_cells, t_cells);
         atomicAdd(&ctr->merge_elems, t_el);
@@ -2647,15 +3052,17 @@ void launch_merge_tiers(const Params& P, Dev& d, uint64_t G, cudaStream_t s, con
     using E = typename std::conditional<MX, MP32, MP>::type;
     using K = typename EKey<E>::K;
     const uint32_t cap0 = merge_cap0((int)sizeof(E));
-    const MLayout L0 = merge_layout(cap0, P.ppc, sizeof(E), sizeof(K));
-    const MLayout L1 = merge_layout(MERGE_CAP1, P.ppc, sizeof(E), sizeof(K));
-    const size_t sm0 = (size_t)L0.bytes * MERGE_NW0, sm1 = (size_t)L1.bytes * MERGE_NW1;
+    const size_t sm0 = (size_t)pre_layout(cap0, P.ppc, sizeof(K)).bytes * MERGE_NW0;
+    const size_t sm1 = (size_t)pre_layout(MERGE_CAP1, P.ppc, sizeof(K)).bytes * MERGE_NW1;
+    const size_t smt = (size_t)merge_layout(MERGE_CAP1, P.ppc, sizeof(E), sizeof(K)).bytes * MERGE_NW1;
     static bool attr = false;
     if (!attr) {
         cudaFuncSetAttribute(k_merge_lv<E, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
+        cudaFuncSetAttribute(k_merge_pre<E>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
         attr = true;
     }
-    g_launches += 3;
+    g_launches += 4;
+    const uint64_t Gphys = (uint64_t)P.R * P.n3;
     // tiers 1 and 2 (few, long cells) on the side stream beside tier 0
     cudaStream_t s12 = s;
     if (d.side) {
@@ -2663,19 +3070,24 @@ void launch_merge_tiers(const Params& P, Dev& d, uint64_t G, cudaStream_t s, con
         cudaStreamWaitEvent(d.side, d.side_fork, 0);
         s12 = d.side;
     }
-    k_merge_lv<E, false><<<152 * 8, MERGE_NW1 * 32, sm1, s12>>>(
-        P, A, A32, d.cell_start, d.gain, d.photos, d.photo_sorted, d.photo_off, d.out_start, d.work_off, d.work,
-        d.work_cap, out, out32, cout, (uint64_t)P.R * P.n3, d.mover_cap, d.photo_cap, d.mid_list, d.list_n, 1, MERGE_CAP1, d.ctr);
+    auto pre = [&](cudaStream_t st, int blocks, size_t sm, const uint32_t* list, int tier, uint32_t CAP) {
+        k_merge_pre<E><<<blocks, 128, sm, st>>>(P, A, A32, d.cell_start, d.gain, d.photos, d.photo_sorted, d.photo_off,
+                                                d.out_start, out, out32, cout, Gphys, d.mover_cap, d.photo_cap, list,
+                                                d.list_n, tier, CAP, d.tie_list, d.ctr);
+    };
+    pre(s12, 152 * 8, sm1, d.mid_list, 1, MERGE_CAP1);
     k_merge_lv<E, true><<<152 * 4, 128, 0, s12>>>(
         P, A, A32, d.cell_start, d.gain, d.photos, d.photo_sorted, d.photo_off, d.out_start, d.work_off, d.work,
-        d.work_cap, out, out32, cout, (uint64_t)P.R * P.n3, d.mover_cap, d.photo_cap, d.big_list, d.list_n, 2, 0, d.ctr);
-    k_merge_lv<E, false><<<152 * 16, MERGE_NW0 * 32, sm0, s>>>(
-        P, A, A32, d.cell_start, d.gain, d.photos, d.photo_sorted, d.photo_off, d.out_start, d.work_off, d.work,
-        d.work_cap, out, out32, cout, (uint64_t)P.R * P.n3, d.mover_cap, d.photo_cap, d.small_list, d.list_n, 0, cap0, d.ctr);
+        d.work_cap, out, out32, cout, Gphys, d.mover_cap, d.photo_cap, d.big_list, d.list_n, 2, 0, d.ctr);
+    pre(s, 152 * 16, sm0, d.small_list, 0, cap0);
     if (d.side) {
         cudaEventRecord(d.side_join, d.side);
         cudaStreamWaitEvent(s, d.side_join, 0);
     }
+    // the cells of tiers 0 and 1 that it left
+    k_merge_lv<E, false><<<152 * 4, MERGE_NW1 * 32, smt, s>>>(
+        P, A, A32, d.cell_start, d.gain, d.photos, d.photo_sorted, d.photo_off, d.out_start, d.work_off, d.work,
+        d.work_cap, out, out32, cout, Gphys, d.mover_cap, d.photo_cap, d.tie_list, d.list_n, 3, MERGE_CAP1, d.ctr);
 }
 
 void launch_merges(const Params& P, Dev& d, uint64_t G, cudaStream_t s)
