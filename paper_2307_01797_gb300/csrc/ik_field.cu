@@ -18,6 +18,7 @@
 #include <algorithm>
 #include <cmath>
 #include <cstdio>
+#include <cstddef>
 #include <cstring>
 #include <mutex>
 #include <type_traits>
@@ -695,10 +696,11 @@ Geo geo(const Dev& d, int l, int R)
 // slab's two outer planes into the neighbour blocks' halo planes (distributed
 // shared memory) and ends with a cluster barrier.  The 8^3 level runs in the
 // cluster's first block, the 4^3 bottom (48 red-black sweep pairs) in one warp
-// with the cells in registers.  What bounds it is a chain of latencies (21
-// cluster barriers, 96 warp half-sweeps), not bandwidth: 39 us in fixed point,
-// 31 us in FP32 from 32^3 down; one block per realization from 16^3 down took
-// 159 us in FP64 and 96 us in FP32, after 10 launches for the 32^3 level.
+// with the cells in registers (64-bit forms: solved by its eigenvectors).
+// What bounds it is a chain of latencies (21 cluster barriers, 96 warp
+// half-sweeps), not bandwidth: 32 us in fixed point, 28 us in FP32 from 32^3
+// down; one block per realization from 16^3 down took 159 us in FP64 and 96 us
+// in FP32, after 10 launches for the 32^3 level.
 constexpr int COARSE_N = 32, COARSE_CL = 8, COARSE_TPB = 512, BOTTOM_SWEEPS = 48;
 
 template <class T>
@@ -748,6 +750,52 @@ __device__ void bottom_solve(T* phi, const T* rhs, unsigned lane)
     phi[c1] = b;
 }
 
+// The 4^3 level solved by its eigenvectors, for the 64-bit forms: cosines along
+// x and y (Neumann sides), sines along z (electrodes), six products with 4 x 4
+// matrices by 64 threads; all threads of the block call this.  The sweeps
+// above leave 4e-5 of the bottom's error; 1.6k clocks against 18k for them in
+// fixed point.
+__constant__ double BOTTOM_C[16] = {   // normalised cos(pi m (i + 1/2) / 4), row m
+    0.5, 0.5, 0.5, 0.5,
+    0.65328148243818826, 0.27059805007309850, -0.27059805007309850, -0.65328148243818826,
+    0.5, -0.5, -0.5, 0.5,
+    0.27059805007309850, -0.65328148243818826, 0.65328148243818826, -0.27059805007309850 };
+__constant__ double BOTTOM_S[16] = {   // normalised sin(pi (m + 1) (k + 1/2) / 4), row m
+    0.27059805007309850, 0.65328148243818826, 0.65328148243818826, 0.27059805007309850,
+    0.5, 0.5, -0.5, -0.5,
+    0.65328148243818826, -0.27059805007309850, -0.27059805007309850, 0.65328148243818826,
+    0.5, -0.5, 0.5, -0.5 };
+__constant__ double BOTTOM_L[5] = {    // 2 - 2 cos(pi m / 4)
+    0.0, 0.58578643762690485, 2.0, 3.4142135623730949, 4.0 };
+
+template <class T>
+__device__ void bottom_solve_exact(T* phi, const T* rhs, double* w)
+{
+    const int t = threadIdx.x, i = t & 3, j = (t >> 2) & 3, k = t >> 4;
+    double* a = w;
+    double* b = w + 64;
+    if (t < 64) a[t] = (double)rhs[t];
+    __syncthreads();
+    // forward along z, y, x, divide, back along x, y, z
+#pragma unroll 1
+    for (int st = 0; st < 6; ++st) {
+        if (t < 64) {
+            const int ax = st < 3 ? 2 - st : st - 3;
+            const int row = ax == 0 ? i : (ax == 1 ? j : k), step = 1 << (2 * ax), first = t - row * step;
+            const double* Q = ax == 2 ? BOTTOM_S : BOTTOM_C;
+            double s = 0.0;
+#pragma unroll
+            for (int m = 0; m < 4; ++m) s = __fma_rn(st < 3 ? Q[row * 4 + m] : Q[m * 4 + row], a[first + m * step], s);
+            if (st == 2) s = -s / ((BOTTOM_L[i] + BOTTOM_L[j]) + BOTTOM_L[k + 1]);
+            b[t] = s;
+        }
+        __syncthreads();
+        double* x = a; a = b; b = x;
+    }
+    if (t < 64) phi[t] = std::is_same<T, long long>::value ? (T)__double2ll_rn(a[t]) : (T)a[t];
+    __syncthreads();
+}
+
 // The planes of one level in one block: PL own planes and a halo plane below
 // and above, each as two colour arrays with a rim of zeros.
 template <int N, int PLANES>
@@ -762,6 +810,7 @@ struct CoarseSmem {
     T res[4 * 1024];               // residuals of a level's slab, then corrections of the level below, in cell order
     T r16[2 * 256], r8[512], e8[512];
     T p4[64], r4[64];
+    double w4[128];                // the bottom's transforms
 };
 
 // A thread's pair column of a level: PER planes of the PLANES in the block.
@@ -891,9 +940,11 @@ __global__ void __cluster_dims__(COARSE_CL, 1, 1) __launch_bounds__(COARSE_TPB)
     T* gp = top.phi + base;
     const T* gr = top.rhs + base;
     // zeros everywhere (rims, domain halos, the corrections' start)
-    for (int t = threadIdx.x; t < SlabShape<32, 4>::SIZE; t += COARSE_TPB) S.p32[t] = (T)0;
-    for (int t = threadIdx.x; t < SlabShape<16, 2>::SIZE; t += COARSE_TPB) S.p16[t] = (T)0;
-    for (int t = threadIdx.x; t < SlabShape<8, 8>::SIZE; t += COARSE_TPB) S.p8[t] = (T)0;
+    {
+        constexpr int WORDS = (SlabShape<32, 4>::SIZE + SlabShape<16, 2>::SIZE + SlabShape<8, 8>::SIZE) * (int)sizeof(T) / 16;
+        static_assert(WORDS * 16 == (int)offsetof(CoarseSmem<T>, res), "the three levels first, in whole 16-byte words");
+        for (int t = threadIdx.x; t < WORDS; t += COARSE_TPB) reinterpret_cast<uint4*>(&S)[t] = make_uint4(0, 0, 0, 0);
+    }
     Slab<T, 32, 4, 4> a;
     Slab<T, 16, 2, 2> b;
     Slab<T, 8, 8, 1> c;
@@ -949,8 +1000,12 @@ __global__ void __cluster_dims__(COARSE_CL, 1, 1) __launch_bounds__(COARSE_TPB)
         restrict_planes<T, 8>(S.res, S.r4, 4);
         if (threadIdx.x < 64) S.p4[threadIdx.x] = (T)0;
         __syncthreads();
-        if (threadIdx.x < 32) bottom_solve(S.p4, S.r4, threadIdx.x);
-        __syncthreads();
+        if constexpr (sizeof(T) == 8) {
+            bottom_solve_exact(S.p4, S.r4, S.w4);
+        } else {
+            if (threadIdx.x < 32) bottom_solve(S.p4, S.r4, threadIdx.x);
+            __syncthreads();
+        }
         c.correct(S.p4, 0);
         __syncthreads();
         for (int it = 0; it < nu2; ++it) {
@@ -1020,11 +1075,16 @@ __global__ void __cluster_dims__(COARSE_CL, 1, 1) __launch_bounds__(COARSE_TPB)
 // same to the last bit.  Two sweeps of 256^3 cells: 202 us in fixed point (66%
 // issue utilisation: bound by its integer instructions, 1.9 TB/s of DRAM)
 // against 508 us for four FP64 half-sweeps (FP64 pipe 82% busy).
-template <class T>
+//
+// The tile: 64 x 32 in FP32 (two pairs per thread), 32 x 32 in 64 bits.  A
+// 64^3 level has too few of these for the chip's SMs: 32 x 16 there, with one
+// pair per thread (17.9 -> 12.9 us in fixed point, 16.0 -> 10.6 us in FP32: a
+// step takes as long as its warps need to issue).
+template <class T, int TX_, int TY_, int PP_>
 struct SweepTile {
-    static constexpr int TX = sizeof(T) == 4 ? 64 : 32, TY = 32, H = 4;
+    static constexpr int TX = TX_, TY = TY_, H = 4;
     static constexpr int EX = TX + 2 * H, EY = TY + 2 * H, PX = EX / 2;
-    static constexpr int NT = sizeof(T) == 4 ? 720 : 800, PP = sizeof(T) == 4 ? 2 : 1, RING = 5;
+    static constexpr int PP = PP_, NT = PX * EY / PP, RING = 5;
     static constexpr int GUARD = PX + 1;           // elements before and after the ring that rim pairs read
     static constexpr size_t SMEM = sizeof(T) * (RING * EX * EY + 2 * GUARD);
     static_assert(PX * EY == PP * NT, "whole pairs per thread");
@@ -1033,11 +1093,10 @@ struct SweepTile {
 template <class T>
 struct __align__(2 * sizeof(T)) Pair { T v[2]; };
 
-template <class T>
-__global__ void __launch_bounds__(SweepTile<T>::NT, 1)
+template <class T, class Q>
+__global__ void __launch_bounds__(Q::NT, 1)
     k_sweep4(const T* __restrict__ src, const T* __restrict__ rhs, T* __restrict__ dst, int n, int c0, int zc)
 {
-    using Q = SweepTile<T>;
     constexpr int H = Q::H, PP = Q::PP, PX = Q::PX, EY = Q::EY, PLH = PX * EY;   // PLH: the cells of one colour
     extern __shared__ __align__(16) unsigned char ssm[];
     T* ring = reinterpret_cast<T*>(ssm) + Q::GUARD;
@@ -1170,27 +1229,34 @@ template <>
 long long* lrhs<long long>(MGLevel& L) { return L.rhs_fix; }
 
 // Shared memory beyond 48 KB needs an opt-in per kernel and device.
+constexpr int SMALL_R = 4;
+
 template <class F>
 void allow_smem(F* kernel, size_t bytes)
 {
     static std::mutex mtx;
-    static bool done[64] = {};
+    static F* seen[8] = {};                     // kernels of one signature
+    static unsigned long long done[8] = {};     // devices they are opted in on
     int dev = 0;
     cudaGetDevice(&dev);
     std::lock_guard<std::mutex> lk(mtx);
-    if (dev >= 0 && dev < 64 && done[dev]) return;
+    int k = 0;
+    while (k < 8 && seen[k] && seen[k] != kernel) ++k;
+    if (k < 8 && dev >= 0 && dev < 64 && seen[k] && ((done[k] >> dev) & 1u)) return;
     cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
-    if (dev >= 0 && dev < 64) done[dev] = true;
+    if (k < 8 && dev >= 0 && dev < 64) {
+        seen[k] = kernel;
+        done[k] |= 1ull << dev;
+    }
 }
 
 // Two sweeps of level l from src (nullptr: zeros) into dst.  The z chunk is
 // the one with the least modelled time: waves of resident blocks (one per SM)
 // times the planes each block marches over, the chunk and its halo of 2 x 4.
-template <class T>
-void launch_sweep4(const T* src, const T* rhs, T* dst, const Geo& G, int c0, cudaStream_t s)
+template <class T, class Q>
+void launch_sweep4_tile(const T* src, const T* rhs, T* dst, const Geo& G, int c0, cudaStream_t s)
 {
-    using Q = SweepTile<T>;
-    allow_smem(k_sweep4<T>, Q::SMEM);
+    allow_smem(k_sweep4<T, Q>, Q::SMEM);
     const uint64_t tiles = (uint64_t)(G.n / Q::TX) * (G.n / Q::TY);
     int zc = G.n;
     uint64_t best = ~0ull;
@@ -1199,7 +1265,15 @@ void launch_sweep4(const T* src, const T* rhs, T* dst, const Geo& G, int c0, cud
         if (cost < best) { best = cost; zc = c; }
     }
     ++g_launches;
-    k_sweep4<T><<<dim3((unsigned)tiles, G.n / zc, G.R), Q::NT, Q::SMEM, s>>>(src, rhs, dst, G.n, c0, zc);
+    k_sweep4<T, Q><<<dim3((unsigned)tiles, G.n / zc, G.R), Q::NT, Q::SMEM, s>>>(src, rhs, dst, G.n, c0, zc);
+}
+
+template <class T>
+void launch_sweep4(const T* src, const T* rhs, T* dst, const Geo& G, int c0, cudaStream_t s)
+{
+    constexpr int TX = sizeof(T) == 4 ? 64 : 32;
+    if (G.n == 64 && G.R < SMALL_R) launch_sweep4_tile<T, SweepTile<T, 32, 16, 1>>(src, rhs, dst, G, c0, s);
+    else launch_sweep4_tile<T, SweepTile<T, TX, 32, TX / 32>>(src, rhs, dst, G, c0, s);
 }
 
 // One V-cycle from level l; zero: the level's potential counts as zero (it is
