@@ -186,22 +186,57 @@ __global__ void k_smooth(T* __restrict__ phi, const T* __restrict__ rhs, Geo G, 
 // into the coarse right-hand side.  Every level stores h^2 b (the multigrid
 // systems are scaled by h^2), so the coarse value h_c^2 mean(r) is half the
 // sum of the children's h_f^2 r = h_f^2 b - (neighbour sum - diag phi).
+// A thread reads its 2 x 2 x 2 cells and their rim by rows of pairs: 12 pairs
+// and 8 single values for eight residuals.
 template <class T>
-__global__ void k_resid_restrict(const T* __restrict__ phi, const T* __restrict__ rhs, T* __restrict__ rhs_c,
-                                 Geo Gc, int nf)
+struct __align__(2 * sizeof(T)) Pair { T v[2]; };
+
+template <class T>
+__global__ void __launch_bounds__(256) k_resid_restrict(const T* __restrict__ phi, const T* __restrict__ rhs,
+                                                        T* __restrict__ rhs_c, Geo Gc, int nf)
 {
+    const int nc = Gc.n;
     for (uint64_t t = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; t < Gc.cells; t += (uint64_t)gridDim.x * blockDim.x) {
         int r, K, J, I;
         decode(t, Gc.log2n, r, K, J, I);
+        const uint64_t sy = (uint64_t)nf, sz = (uint64_t)nf * nf;
+        const T* p = phi + ((uint64_t)r * nf + 2 * K) * sz + (2 * J) * sy + 2 * I;
+        const T* b = rhs + (p - phi);
+        auto row = [&](int k, int j, bool in) {    // the x pair of plane k, row j from the thread's own
+            Pair<T> v;
+            v.v[0] = v.v[1] = (T)0;
+            if (in) v = *reinterpret_cast<const Pair<T>*>(p + (int64_t)k * (int64_t)sz + (int64_t)j * (int64_t)sy);
+            return v;
+        };
+        const bool xl = I > 0, xr = I < nc - 1, yl = J > 0, yr = J < nc - 1, zl = K > 0, zr = K < nc - 1;
+        // own pairs with a row before and after, per plane; the planes before and after
+        Pair<T> v[4][4];
+#pragma unroll
+        for (int k = -1; k <= 2; ++k)
+#pragma unroll
+            for (int j = -1; j <= 2; ++j) {
+                const bool edge_k = k < 0 || k > 1, edge_j = j < 0 || j > 1;
+                if (edge_k && edge_j) continue;
+                v[k + 1][j + 1] = row(k, j, (k >= 0 || zl) && (k <= 1 || zr) && (j >= 0 || yl) && (j <= 1 || yr));
+            }
         T acc = 0;
 #pragma unroll
-        for (int c = 0; c < 8; ++c) {
-            const int i = 2 * I + (c & 1), j = 2 * J + ((c >> 1) & 1), k = 2 * K + (c >> 2);
-            const uint64_t idx = (((uint64_t)r * nf + k) * nf + j) * nf + i;
-            int diag;
-            const T s = nbr_sum(phi, idx, nf, i, j, k, diag);
-            acc += MG<T>::resid(s, rhs[idx], phi[idx], diag);
-        }
+        for (int k = 0; k < 2; ++k)
+#pragma unroll
+            for (int j = 0; j < 2; ++j) {
+                const uint64_t o = (uint64_t)k * sz + (uint64_t)j * sy;
+                const Pair<T> c = v[k + 1][j + 1], f = *reinterpret_cast<const Pair<T>*>(b + o);
+                const T left = xl ? p[o - 1] : (T)0, right = xr ? p[o + 2] : (T)0;
+#pragma unroll
+                for (int x = 0; x < 2; ++x) {
+                    T s = (x ? c.v[0] : left) + (x ? right : c.v[1]);      // a side without a cell adds zero
+                    s += v[k + 1][j].v[x];
+                    s += v[k + 1][j + 2].v[x];
+                    s += v[k][j + 1].v[x];
+                    s += v[k + 2][j + 1].v[x];
+                    acc += MG<T>::resid(s, f.v[x], c.v[x], diag_count(2 * I + x, 2 * J + j, 2 * K + k, nf));
+                }
+            }
         rhs_c[t] = MG<T>::half(acc);
     }
 }
@@ -233,14 +268,47 @@ __device__ __forceinline__ T prolong_at(const T* __restrict__ ec, int nc, int i,
     return MG<T>::div64(MG<T>::axpy3(m[0], sz < (T)0 ? -m[1] : m[1]));
 }
 
+// A thread takes the x pair (2 I, 2 I + 1) of rows 2 J and 2 J + 1 of plane k:
+// three coarse values in each of 2 x 3 rows serve four cells (eight loads and
+// index computations per cell otherwise).  Each cell gets prolong_at's
+// operations.
 template <class T>
-__global__ void k_prolong(T* __restrict__ phi_f, const T* __restrict__ e_c, Geo Gf)
+__global__ void __launch_bounds__(256) k_prolong(T* __restrict__ phi_f, const T* __restrict__ e_c, Geo Gf)
 {
-    const int nc = Gf.n / 2;
-    for (uint64_t t = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; t < Gf.cells; t += (uint64_t)gridDim.x * blockDim.x) {
-        int r, k, j, i;
-        decode(t, Gf.log2n, r, k, j, i);
-        phi_f[t] += prolong_at(e_c + (uint64_t)r * nc * nc * nc, nc, i, j, k);
+    const int n = Gf.n, nc = n / 2, lc = Gf.log2n - 1;
+    const uint64_t groups = Gf.cells >> 2;
+    for (uint64_t t = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; t < groups; t += (uint64_t)gridDim.x * blockDim.x) {
+        const int I = (int)(t & (uint64_t)(nc - 1)), J = (int)((t >> lc) & (uint64_t)(nc - 1));
+        const int k = (int)((t >> (2 * lc)) & (uint64_t)(n - 1));
+        const uint64_t r = t >> (2 * lc + Gf.log2n);
+        const int K = k >> 1;
+        int K2 = K + ((k & 1) ? 1 : -1);
+        bool neg = false;
+        if (K2 < 0 || K2 >= nc) { K2 = K; neg = true; }
+        const int Il = I > 0 ? I - 1 : I, Ir = I < nc - 1 ? I + 1 : I;
+        const int Jl = J > 0 ? J - 1 : J, Jr = J < nc - 1 ? J + 1 : J;
+        T m[2][2][2];                              // [plane][fine row][cell]
+#pragma unroll
+        for (int c = 0; c < 2; ++c) {
+            const T* pl = e_c + (r * nc + (c ? K2 : K)) * (uint64_t)nc * nc;
+            const T *r0 = pl + J * nc, *rl = pl + Jl * nc, *rr = pl + Jr * nc;
+            const T a = r0[I], al = r0[Il], ar = r0[Ir];
+            const T b = rl[I], bl = rl[Il], br = rl[Ir];
+            const T d = rr[I], dl = rr[Il], dr = rr[Ir];
+            const T q0 = MG<T>::axpy3(a, al), q1 = MG<T>::axpy3(a, ar);
+            m[c][0][0] = MG<T>::axpy3(q0, MG<T>::axpy3(b, bl));
+            m[c][0][1] = MG<T>::axpy3(q1, MG<T>::axpy3(b, br));
+            m[c][1][0] = MG<T>::axpy3(q0, MG<T>::axpy3(d, dl));
+            m[c][1][1] = MG<T>::axpy3(q1, MG<T>::axpy3(d, dr));
+        }
+#pragma unroll
+        for (int y = 0; y < 2; ++y) {
+            Pair<T>* p = reinterpret_cast<Pair<T>*>(phi_f + ((r * n + k) * n + 2 * J + y) * (uint64_t)n + 2 * I);
+            Pair<T> v = *p;
+#pragma unroll
+            for (int x = 0; x < 2; ++x) v.v[x] += MG<T>::div64(MG<T>::axpy3(m[0][y][x], neg ? -m[1][y][x] : m[1][y][x]));
+            *p = v;
+        }
     }
 }
 
@@ -326,6 +394,22 @@ __global__ void k_add_correction(double* __restrict__ phi, const float* __restri
 // thread and FP64 across the block in a fixed order.
 constexpr long long PHI_LIM = 1ll << 59;
 
+// A block covers items rows of NORM_TPB cells of one realization (cells in
+// index order, as k_norm_final's fixed order wants them).
+struct RowCell {             // one thread's cell in the rows of a block
+    int i, j, k, n;
+    uint64_t t;
+};
+
+__device__ __forceinline__ long long fixed_sum(const long long* __restrict__ p, const RowCell& c)
+{
+    const int64_t sy = c.n, sz = (int64_t)c.n * c.n;
+    const long long xm = c.i > 0 ? p[-1] : 0, xp = c.i < c.n - 1 ? p[1] : 0;
+    const long long ym = c.j > 0 ? p[-sy] : 0, yp = c.j < c.n - 1 ? p[sy] : 0;
+    const long long zm = c.k > 0 ? p[-sz] : 0, zp = c.k < c.n - 1 ? p[sz] : 0;
+    return (xm + xp + ym) + (yp + zm + zp);
+}
+
 __global__ void __launch_bounds__(NORM_TPB) k_resid_fixed(const long long* __restrict__ Phi,
                                                           const long long* __restrict__ B, float* __restrict__ r32,
                                                           Geo G, float sc, double* __restrict__ part, int with_b,
@@ -335,17 +419,21 @@ __global__ void __launch_bounds__(NORM_TPB) k_resid_fixed(const long long* __res
     const uint64_t base = ((uint64_t)blockIdx.x * NORM_TPB) * items;
     float acc = 0.f, bacc = 0.f;
     bool bad = false;
+    RowCell c;
+    c.n = G.n;
+#pragma unroll 4
     for (int q = 0; q < items; ++q) {
         const uint64_t t = base + (uint64_t)q * NORM_TPB + threadIdx.x;
         if (t >= G.cells) break;
-        int r, k, j, i;
-        decode(t, G.log2n, r, k, j, i);
-        int diag;
-        const long long s = nbr_sum(Phi, t, G.n, i, j, k, diag);
+        const uint32_t u = (uint32_t)t;                        // a realization has at most 2^30 cells
+        c.i = (int)(u & (uint32_t)(G.n - 1));
+        c.j = (int)((u >> G.log2n) & (uint32_t)(G.n - 1));
+        c.k = (int)((u >> (2 * G.log2n)) & (uint32_t)(G.n - 1));
+        const long long s = fixed_sum(Phi + t, c);
         const long long pc = Phi[t];
         bad |= pc >= PHI_LIM || pc <= -PHI_LIM;
         const long long b = B[t];
-        const float res = __ll2float_rn(b - (s - (long long)diag * pc)) * sc;
+        const float res = __ll2float_rn(MG<long long>::resid(s, b, pc, diag_count(c.i, c.j, c.k, c.n))) * sc;
         r32[t] = res;
         acc = __fmaf_rn(res, res, acc);
         if (with_b) {
@@ -528,17 +616,21 @@ __global__ void __launch_bounds__(NORM_TPB) k_resid_norm_fix(const long long* __
     const uint64_t base = ((uint64_t)blockIdx.x * NORM_TPB) * items;
     float acc = 0.f, bacc = 0.f;
     unsigned long long mx = 0;
+    RowCell c;
+    c.n = G.n;
+#pragma unroll 4
     for (int q = 0; q < items; ++q) {
         const uint64_t t = base + (uint64_t)q * NORM_TPB + threadIdx.x;
         if (t >= G.cells) break;
-        int r, k, j, i;
-        decode(t, G.log2n, r, k, j, i);
-        int diag;
-        const long long s = nbr_sum(Phi, t, G.n, i, j, k, diag);
+        const uint32_t u = (uint32_t)t;                        // a realization has at most 2^30 cells
+        c.i = (int)(u & (uint32_t)(G.n - 1));
+        c.j = (int)((u >> G.log2n) & (uint32_t)(G.n - 1));
+        c.k = (int)((u >> (2 * G.log2n)) & (uint32_t)(G.n - 1));
+        const long long s = fixed_sum(Phi + t, c);
         const long long pc = Phi[t], b = B[t];
         const unsigned long long ap = (unsigned long long)(pc < 0 ? -pc : pc);
         mx = ap > mx ? ap : mx;
-        const float res = __ll2float_rn(MG<long long>::resid(s, b, pc, diag)) * 0x1p-30f;
+        const float res = __ll2float_rn(MG<long long>::resid(s, b, pc, diag_count(c.i, c.j, c.k, c.n))) * 0x1p-30f;
         acc = __fmaf_rn(res, res, acc);
         if (with_b) {
             const float bf = __ll2float_rn(b) * 0x1p-30f;
@@ -608,9 +700,14 @@ __global__ void k_rhs_fixed(const int64_t* __restrict__ rho, long long* __restri
 {
     for (uint64_t t = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; t < G.cells; t += (uint64_t)gridDim.x * blockDim.x) {
         const int k = (int)((t >> (2 * G.log2n)) & (uint64_t)(G.n - 1));
-        double b = -((double)rho[t] * qscale);
-        if (k == G.n - 1) b = b - bc_top;
-        B[t] = __double2ll_rn(b * bfix);
+        const int64_t q = rho[t];
+        long long v = 0;                          // a cell without charge below the electrode's
+        if (q != 0 || k == G.n - 1) {
+            double b = -((double)q * qscale);
+            if (k == G.n - 1) b = b - bc_top;
+            v = __double2ll_rn(b * bfix);
+        }
+        B[t] = v;
     }
 }
 
@@ -1090,9 +1187,6 @@ struct SweepTile {
     static_assert(PX * EY == PP * NT, "whole pairs per thread");
 };
 
-template <class T>
-struct __align__(2 * sizeof(T)) Pair { T v[2]; };
-
 template <class T, class Q>
 __global__ void __launch_bounds__(Q::NT, 1)
     k_sweep4(const T* __restrict__ src, const T* __restrict__ rhs, T* __restrict__ dst, int n, int c0, int zc)
@@ -1317,7 +1411,7 @@ void vcycle(Dev& d, int l, int R, int nu1, int nu2, cudaStream_t s, bool zero)
     k_resid_restrict<T><<<gridsz(Gc.cells, tpb), tpb, 0, s>>>(cur, rhs, lrhs<T>(C), Gc, G.n);
     vcycle<T>(d, l + 1, R, nu1, nu2, s, true);
     ++g_launches;
-    k_prolong<T><<<gridsz(G.cells, tpb), tpb, 0, s>>>(cur, lphi<T>(C), G);
+    k_prolong<T><<<gridsz(G.cells / 4, tpb), tpb, 0, s>>>(cur, lphi<T>(C), G);
     sweeps(nu2, 1);
     if (cur != phi) cudaMemcpyAsync(phi, cur, G.cells * sizeof(T), cudaMemcpyDeviceToDevice, s);
 }
@@ -1981,7 +2075,7 @@ static void vcycle_vc(const Dev& d, int l, int R, int nu1, int nu2, cudaStream_t
     k_resid_restrict_vc<<<gridsz(Gc.cells, tpb), tpb, 0, s>>>(phi, rhs, A, d.lev[l + 1].rhs, Gc, G.n);
     cudaMemsetAsync(d.lev[l + 1].phi, 0, Gc.cells * sizeof(double), s);
     vcycle_vc(d, l + 1, R, nu1, nu2, s);
-    k_prolong<double><<<gridsz(G.cells, tpb), tpb, 0, s>>>(phi, d.lev[l + 1].phi, G);
+    k_prolong<double><<<gridsz(G.cells / 4, tpb), tpb, 0, s>>>(phi, d.lev[l + 1].phi, G);
     for (int it = 0; it < nu2; ++it) { sweep(1); sweep(0); }
 }
 
