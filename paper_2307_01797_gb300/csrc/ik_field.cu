@@ -394,53 +394,75 @@ __global__ void k_add_correction(double* __restrict__ phi, const float* __restri
 // thread and FP64 across the block in a fixed order.
 constexpr long long PHI_LIM = 1ll << 59;
 
-// A block covers items rows of NORM_TPB cells of one realization (cells in
-// index order, as k_norm_final's fixed order wants them).
-struct RowCell {             // one thread's cell in the rows of a block
-    int i, j, k, n;
-    uint64_t t;
+// The cells of one block: a column of TX x TY cells over ZC planes of one
+// realization, one (x, y) per thread, marching up in z with the planes below
+// and at the cell in registers; the row's and the next rows' values were just
+// loaded by the block (a block of consecutive cells reads three planes from L2
+// for each one).
+struct MarchGeo {
+    int tx, log2tx, zc;          // x cells of a block (a power of two), planes of a block
+    int bx, bxy, bpr;            // blocks per row of blocks, per plane of blocks, per realization
 };
 
-__device__ __forceinline__ long long fixed_sum(const long long* __restrict__ p, const RowCell& c)
+__host__ __device__ inline MarchGeo march_geo(int n)
 {
-    const int64_t sy = c.n, sz = (int64_t)c.n * c.n;
-    const long long xm = c.i > 0 ? p[-1] : 0, xp = c.i < c.n - 1 ? p[1] : 0;
-    const long long ym = c.j > 0 ? p[-sy] : 0, yp = c.j < c.n - 1 ? p[sy] : 0;
-    const long long zm = c.k > 0 ? p[-sz] : 0, zp = c.k < c.n - 1 ? p[sz] : 0;
-    return (xm + xp + ym) + (yp + zm + zp);
+    MarchGeo m;
+    m.tx = n < 64 ? n : 64;
+    m.log2tx = 0;
+    while ((1 << m.log2tx) < m.tx) ++m.log2tx;
+    const int ty = NORM_TPB / m.tx < n ? NORM_TPB / m.tx : n;
+    m.zc = n <= 64 ? 4 : 16;     // small grids: more blocks rather than longer marches
+    m.bx = n / m.tx;
+    m.bxy = m.bx * (n / ty);
+    m.bpr = m.bxy * (n / m.zc);
+    return m;
+}
+
+// Calls f(cell index, value, neighbour sum, diagonal) for the thread's cells.
+template <class F>
+__device__ __forceinline__ void march_cells(const long long* __restrict__ Phi, int n, const MarchGeo& m, F f)
+{
+    const int ty = NORM_TPB / m.tx < n ? NORM_TPB / m.tx : n;
+    const int r = blockIdx.x / m.bpr, b = blockIdx.x - r * m.bpr, bz = b / m.bxy, bb = b - bz * m.bxy, by = bb / m.bx,
+              bx = bb - by * m.bx;
+    const int row = threadIdx.x >> m.log2tx;
+    if (row >= ty) return;
+    const int i = bx * m.tx + (threadIdx.x & (m.tx - 1)), j = by * ty + row, k0 = bz * m.zc;
+    const int64_t sy = n, sz = (int64_t)n * n;
+    uint64_t t = (uint64_t)r * n * sz + (uint64_t)k0 * sz + (uint64_t)j * sy + i;
+    const int dxy = 6 - (i == 0) - (i == n - 1) - (j == 0) - (j == n - 1);
+    long long below = k0 > 0 ? Phi[t - sz] : 0, own = Phi[t];
+#pragma unroll 2
+    for (int q = 0; q < m.zc; ++q, t += sz) {
+        const int k = k0 + q;
+        const long long above = k < n - 1 ? Phi[t + sz] : 0;
+        const long long xm = i > 0 ? Phi[t - 1] : 0, xp = i < n - 1 ? Phi[t + 1] : 0;
+        const long long ym = j > 0 ? Phi[t - sy] : 0, yp = j < n - 1 ? Phi[t + sy] : 0;
+        f(t, own, (xm + xp + ym) + (yp + below + above), dxy + (k == 0) + (k == n - 1));
+        below = own;
+        own = above;
+    }
 }
 
 __global__ void __launch_bounds__(NORM_TPB) k_resid_fixed(const long long* __restrict__ Phi,
                                                           const long long* __restrict__ B, float* __restrict__ r32,
                                                           Geo G, float sc, double* __restrict__ part, int with_b,
-                                                          int items)
+                                                          MarchGeo m)
 {
     __shared__ double red[NORM_TPB / 32][2];
-    const uint64_t base = ((uint64_t)blockIdx.x * NORM_TPB) * items;
     float acc = 0.f, bacc = 0.f;
     bool bad = false;
-    RowCell c;
-    c.n = G.n;
-#pragma unroll 4
-    for (int q = 0; q < items; ++q) {
-        const uint64_t t = base + (uint64_t)q * NORM_TPB + threadIdx.x;
-        if (t >= G.cells) break;
-        const uint32_t u = (uint32_t)t;                        // a realization has at most 2^30 cells
-        c.i = (int)(u & (uint32_t)(G.n - 1));
-        c.j = (int)((u >> G.log2n) & (uint32_t)(G.n - 1));
-        c.k = (int)((u >> (2 * G.log2n)) & (uint32_t)(G.n - 1));
-        const long long s = fixed_sum(Phi + t, c);
-        const long long pc = Phi[t];
+    march_cells(Phi, G.n, m, [&](uint64_t t, long long pc, long long s, int diag) {
         bad |= pc >= PHI_LIM || pc <= -PHI_LIM;
         const long long b = B[t];
-        const float res = __ll2float_rn(MG<long long>::resid(s, b, pc, diag_count(c.i, c.j, c.k, c.n))) * sc;
+        const float res = __ll2float_rn(MG<long long>::resid(s, b, pc, diag)) * sc;
         r32[t] = res;
         acc = __fmaf_rn(res, res, acc);
         if (with_b) {
             const float bf = __ll2float_rn(b) * sc;
             bacc = __fmaf_rn(bf, bf, bacc);
         }
-    }
+    });
     double a = bad ? (double)INFINITY : (double)acc, bb = (double)bacc;
 #pragma unroll
     for (int d = 16; d > 0; d >>= 1) {
@@ -608,35 +630,24 @@ __global__ void k_fix_store(const long long* __restrict__ Phi, double* __restric
 // |Phi|.  The norms serve the convergence test alone.
 __global__ void __launch_bounds__(NORM_TPB) k_resid_norm_fix(const long long* __restrict__ Phi,
                                                              const long long* __restrict__ B, Geo G,
-                                                             double* __restrict__ part, int with_b, int items,
+                                                             double* __restrict__ part, int with_b, MarchGeo m,
                                                              FixScale* __restrict__ fs)
 {
     __shared__ double red[NORM_TPB / 32][2];
     __shared__ unsigned long long redm[NORM_TPB / 32];
-    const uint64_t base = ((uint64_t)blockIdx.x * NORM_TPB) * items;
     float acc = 0.f, bacc = 0.f;
     unsigned long long mx = 0;
-    RowCell c;
-    c.n = G.n;
-#pragma unroll 4
-    for (int q = 0; q < items; ++q) {
-        const uint64_t t = base + (uint64_t)q * NORM_TPB + threadIdx.x;
-        if (t >= G.cells) break;
-        const uint32_t u = (uint32_t)t;                        // a realization has at most 2^30 cells
-        c.i = (int)(u & (uint32_t)(G.n - 1));
-        c.j = (int)((u >> G.log2n) & (uint32_t)(G.n - 1));
-        c.k = (int)((u >> (2 * G.log2n)) & (uint32_t)(G.n - 1));
-        const long long s = fixed_sum(Phi + t, c);
-        const long long pc = Phi[t], b = B[t];
+    march_cells(Phi, G.n, m, [&](uint64_t t, long long pc, long long s, int diag) {
+        const long long b = B[t];
         const unsigned long long ap = (unsigned long long)(pc < 0 ? -pc : pc);
         mx = ap > mx ? ap : mx;
-        const float res = __ll2float_rn(MG<long long>::resid(s, b, pc, diag_count(c.i, c.j, c.k, c.n))) * 0x1p-30f;
+        const float res = __ll2float_rn(MG<long long>::resid(s, b, pc, diag)) * 0x1p-30f;
         acc = __fmaf_rn(res, res, acc);
         if (with_b) {
             const float bf = __ll2float_rn(b) * 0x1p-30f;
             bacc = __fmaf_rn(bf, bf, bacc);
         }
-    }
+    });
     double a = fs->use64 || mx >= (unsigned long long)FIX_LIM ? (double)INFINITY : (double)acc, bb = (double)bacc;
 #pragma unroll
     for (int d = 16; d > 0; d >>= 1) {
@@ -1775,6 +1786,7 @@ int field_solve(const Params& P, Dev& d, int precision, double rtol, int nu1, in
     const int items = (int)(per_real / NORM_TPB < 8 ? per_real / NORM_TPB : 8);
     const int nblk = (int)(G0.cells / ((uint64_t)NORM_TPB * items));
     const int bpr = nblk / R;
+    const MarchGeo march = march_geo(G0.n);     // the integer residuals' blocks
     double* h_norm = d.norm_host;       // 2 R + FIX_DOUBLES doubles of host memory owned by the caller
     double bnorm[MAX_REAL_NORM];
     if (R > MAX_REAL_NORM) return -1;
@@ -1819,14 +1831,14 @@ int field_solve(const Params& P, Dev& d, int precision, double rtol, int nu1, in
         }
         ++g_launches;
         if (fixed)
-            k_resid_fixed<<<nblk, NORM_TPB, 0, s>>>(Phi, Bfix, L0.rhs32, G0, rsc, d.norm_part, cyc == 0, items);
+            k_resid_fixed<<<R * march.bpr, NORM_TPB, 0, s>>>(Phi, Bfix, L0.rhs32, G0, rsc, d.norm_part, cyc == 0, march);
         else if (fix)
-            k_resid_norm_fix<<<nblk, NORM_TPB, 0, s>>>(L0.phi_fix, L0.rhs_fix, G0, d.norm_part, cyc == 0, items, d.fix);
+            k_resid_norm_fix<<<R * march.bpr, NORM_TPB, 0, s>>>(L0.phi_fix, L0.rhs_fix, G0, d.norm_part, cyc == 0, march, d.fix);
         else
             k_resid_norm<<<nblk, NORM_TPB, 0, s>>>(L0.phi, L0.rhs, precision == 1 ? L0.rhs32 : nullptr, G0,
                                                    d.norm_part, prev_rel < 0.0, items);
         ++g_launches;
-        k_norm_final<<<R, 256, 0, s>>>(d.norm_part, bpr, R, d.norm_out);
+        k_norm_final<<<R, 256, 0, s>>>(d.norm_part, fixed || fix ? march.bpr : bpr, R, d.norm_out);
         cudaMemcpyAsync(h_norm, d.norm_out, 2 * R * sizeof(double), cudaMemcpyDeviceToHost, s);
         if (fix) cudaMemcpyAsync(h_norm + 2 * R, d.fix, sizeof(FixScale), cudaMemcpyDeviceToHost, s);
         if (cudaStreamSynchronize(s) != cudaSuccess) return -3;
@@ -1913,6 +1925,7 @@ void field_solve_fixed(const Params& P, Dev& d, int precision, int nu1, int nu2,
     const int items = (int)(per_real / NORM_TPB < 8 ? per_real / NORM_TPB : 8);
     const int nblk = (int)(G0.cells / ((uint64_t)NORM_TPB * items));
     const int bpr = nblk / R;
+    const MarchGeo march = march_geo(G0.n);     // the integer residuals' blocks
     const bool fixed = precision == 2;
     long long* Phi = reinterpret_cast<long long*>(L0.phi);
     long long* Bfix = reinterpret_cast<long long*>(L0.rhs);
@@ -1937,9 +1950,9 @@ void field_solve_fixed(const Params& P, Dev& d, int precision, int nu1, int nu2,
     auto resid = [&](bool first) {
         ++g_launches;
         if (fixed)
-            k_resid_fixed<<<nblk, NORM_TPB, 0, s>>>(Phi, Bfix, L0.rhs32, G0, rsc, d.norm_part, first, items);
+            k_resid_fixed<<<R * march.bpr, NORM_TPB, 0, s>>>(Phi, Bfix, L0.rhs32, G0, rsc, d.norm_part, first, march);
         else if (precision == 0)
-            k_resid_norm_fix<<<nblk, NORM_TPB, 0, s>>>(L0.phi_fix, L0.rhs_fix, G0, d.norm_part, first, items, d.fix);
+            k_resid_norm_fix<<<R * march.bpr, NORM_TPB, 0, s>>>(L0.phi_fix, L0.rhs_fix, G0, d.norm_part, first, march, d.fix);
         else
             k_resid_norm<<<nblk, NORM_TPB, 0, s>>>(L0.phi, L0.rhs, L0.rhs32, G0, d.norm_part, first, items);
     };
@@ -1958,7 +1971,7 @@ void field_solve_fixed(const Params& P, Dev& d, int precision, int nu1, int nu2,
     }
     resid(true);
     ++g_launches;
-    k_norm_final<<<R, 256, 0, s>>>(d.norm_part, bpr, R, d.norm_out);
+    k_norm_final<<<R, 256, 0, s>>>(d.norm_part, precision == 1 ? bpr : march.bpr, R, d.norm_out);
 }
 
 __global__ void k_pack_field(const double* __restrict__ E3, E64* __restrict__ E, float4* __restrict__ E32, uint64_t G)
