@@ -588,6 +588,7 @@ bool graph_eligible(itokmc_handle* h)
 {
     const itokmc_config& c = h->cfg;
     if (!c.graph_step || c.dt_adapt || c.coupling != ITOKMC_EXPLICIT || h->stage != 0) return false;
+    if (h->d.kmc_stale) return false;            // the next KMC clears every cell's firings first
     if (h->steps_done < 1 || h->graph_cycles < 1 || h->graph_cycles > c.mg_max_cycles) return false;
     if ((uint64_t)h->N * 3 > (uint64_t)h->cap * 2 || h->N == 0) return false;
     // the transport grids cover the next power of two of the count (at most
@@ -954,6 +955,8 @@ int itokmc_init(const itokmc_config* cfg, itokmc_handle** out)
     d.tie_list = dalloc_n<uint32_t>(h, Gp, &rc);
     d.list_n = dalloc_n<uint32_t>(h, 4, &rc);
     d.pc_list = dalloc_n<uint32_t>(h, G, &rc);
+    d.kmc_list = dalloc_n<uint32_t>(h, G, &rc);
+    d.kmc_n = dalloc_n<uint32_t>(h, 1, &rc);
     set_work(h, reinterpret_cast<unsigned char*>(dalloc(h, d.work_cap * 32, &rc)), d.work_cap);
     const size_t se = 2 * std::max(std::max(ik::scan_scratch_elems(Gp, 6), ik::scan_scratch_elems(nblk, 3)),
                                    ik::radix_scratch_elems(h->cap));

@@ -170,6 +170,7 @@ extern "C" int itokmc_load(itokmc_handle* h, const char* path)
     }
     std::vector<unsigned char> buf;
     bool ok = true;
+    v.d->kmc_stale = true;               // the file's firings are of cells that this handle's list does not hold
     for (const Blob& b : blobs_of(v, F.N)) {
         for (size_t o = 0; ok && o < b.bytes; o += CHUNK) {
             const size_t mm = b.bytes - o < CHUNK ? b.bytes - o : CHUNK;

@@ -696,7 +696,8 @@ struct BlockScanOp {
     __device__ void total(const long long*) const {}
 };
 
-// Cell scan: new offsets, stayer offsets, mover offsets.
+// Cell scan: new offsets, stayer offsets, mover offsets (channels: particles,
+// stayers, movers of a cell).
 struct TransportScanOp {
     const int32_t* cnt_new;
     const int32_t* in_cnt;
@@ -705,16 +706,36 @@ struct TransportScanOp {
     int64_t* delta;
     uint32_t* in_off;
     uint64_t G;
-    __device__ void load(uint64_t g, long long v[3]) const
+    __device__ void sum8(uint64_t g, uint32_t s[3]) const
     {
-        const int cn = cnt_new[g], ic = in_cnt[g];
-        v[0] = cn; v[1] = cn - ic; v[2] = ic;
+        uint32_t v[8][3];
+        get8(g, v);
+#pragma unroll
+        for (int k = 0; k < 8; ++k) { s[0] += v[k][0]; s[1] += v[k][1]; s[2] += v[k][2]; }
     }
-    __device__ void store(uint64_t g, const long long ex[3], const long long*) const
+    __device__ void get8(uint64_t g, uint32_t v[8][3]) const
     {
-        new_start[g] = (uint32_t)ex[0];
-        delta[g] = ex[0] + in_before[g] - ex[1];
-        in_off[g] = (uint32_t)ex[2];
+        uint32_t cn[8], ic[8];
+        load8(reinterpret_cast<const uint32_t*>(cnt_new) + g, cn);
+        load8(reinterpret_cast<const uint32_t*>(in_cnt) + g, ic);
+#pragma unroll
+        for (int k = 0; k < 8; ++k) { v[k][0] = cn[k]; v[k][1] = cn[k] - ic[k]; v[k][2] = ic[k]; }
+    }
+    __device__ void put8(uint64_t g, const uint32_t ex[3], const uint32_t v[8][3]) const
+    {
+        uint32_t ib[8], ns[8], io[8], e0 = ex[0], e1 = ex[1], e2 = ex[2];
+        long long dl[8];
+        load8(reinterpret_cast<const uint32_t*>(in_before) + g, ib);
+#pragma unroll
+        for (int k = 0; k < 8; ++k) {
+            ns[k] = e0;
+            io[k] = e2;
+            dl[k] = (long long)e0 + ib[k] - (long long)e1;
+            e0 += v[k][0]; e1 += v[k][1]; e2 += v[k][2];
+        }
+        store8(new_start + g, ns);
+        store8(in_off + g, io);
+        store8(reinterpret_cast<long long*>(delta) + g, dl);
     }
     __device__ void total(const long long t[3]) const
     {
@@ -1116,8 +1137,9 @@ __device__ int kmc_cell(const Params& P, Stream& s, const long long X0[3], const
 // Cells with electrons -- or, with ion-ion recombination on, ions of both
 // signs -- listed for the KMC (one thread per listed cell keeps the warps'
 // lanes busy: the active cells are a small part of the grid); the other
-// cells fire nothing.  The recombination blocks of the firings are touched
-// only when their reaction is on.
+// cells fire nothing, and their firings stay zero (k_kmc_clear).  The
+// recombination blocks of the firings are touched only when their reaction is
+// on.
 // The ion counts of cell g: the NGP counts of the ion blocks' last deposit
 // (mobile ions), else the per-cell counts.
 __device__ __forceinline__ void ion_counts(const Params& P, const unsigned long long* __restrict__ Xe,
@@ -1129,11 +1151,9 @@ __device__ __forceinline__ void ion_counts(const Params& P, const unsigned long 
 }
 
 __global__ void k_kmc_list(Params P, const unsigned long long* __restrict__ Xe, const int64_t* __restrict__ Npos,
-                           const int64_t* __restrict__ Nneg, int64_t* __restrict__ fired,
-                           int64_t* __restrict__ gain, uint64_t G, uint32_t* __restrict__ list,
+                           const int64_t* __restrict__ Nneg, uint64_t G, uint32_t* __restrict__ list,
                            Counters* __restrict__ ctr)
 {
-    const bool rec = P.k_ep > 0.0 || P.k_np > 0.0;
     const bool ion_only = P.k_np > 0.0;
     for (uint64_t g = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; g < G; g += (uint64_t)gridDim.x * blockDim.x) {
         bool run = Xe[g] > 0;
@@ -1142,18 +1162,27 @@ __global__ void k_kmc_list(Params P, const unsigned long long* __restrict__ Xe, 
             ion_counts(P, Xe, Npos, Nneg, G, g, xp, xm);
             run = xp > 0 && xm > 0;
         }
-        if (run) {
-            list[warp_slot32(&ctr->n_kmc_cells)] = (uint32_t)g;
-        } else {
-            fired[g] = 0;
-            fired[G + g] = 0;
-            fired[2 * G + g] = 0;
-            if (rec) {
-                fired[3 * G + g] = 0;
-                fired[4 * G + g] = 0;
-            }
-            for (int s = 0; s < P.S; ++s) gain[(uint64_t)s * G + g] = 0;
+        if (run) list[warp_slot32(&ctr->n_kmc_cells)] = (uint32_t)g;
+    }
+}
+
+// The cells of the last KMC's list back to no firings: all others hold zeros
+// already (32 bytes per active cell instead of per cell of the grid).
+__global__ void k_kmc_clear(Params P, int64_t* __restrict__ fired, int64_t* __restrict__ gain, uint64_t G,
+                            const uint32_t* __restrict__ list, const uint32_t* __restrict__ n_last)
+{
+    const bool rec = P.k_ep > 0.0 || P.k_np > 0.0;
+    const uint32_t n = *n_last;
+    for (uint32_t t = blockIdx.x * blockDim.x + threadIdx.x; t < n; t += gridDim.x * blockDim.x) {
+        const uint64_t g = list[t];
+        fired[g] = 0;
+        fired[G + g] = 0;
+        fired[2 * G + g] = 0;
+        if (rec) {
+            fired[3 * G + g] = 0;
+            fired[4 * G + g] = 0;
         }
+        for (int s = 0; s < P.S; ++s) gain[(uint64_t)s * G + g] = 0;
     }
 }
 
@@ -1289,12 +1318,18 @@ __global__ void k_kmc0d(Params P, double Em, long long X0, uint32_t nreal, int n
 // Systematic integer removal of L = -dN electrons from the cell's particles
 // in canonical order: particle p loses floor((C_p L + R)/W) -
 // floor((C_{p-1} L + R)/W), R = (64-bit draw) mod W.
-// Gp particle cells: each block's species loses from its own particles,
-// against its own NGP count, with its own stream tag.
+// Each block's species loses from its own particles, against its own NGP
+// count, with its own stream tag.  Runs over the cells of the KMC's list
+// (only those have firings), for each species.
 __global__ void k_loss(Params P, uint32_t* __restrict__ wbase, int wstride, const uint32_t* __restrict__ cs,
-                       const unsigned long long* __restrict__ Xe, const int64_t* __restrict__ gain, uint64_t G)
+                       const unsigned long long* __restrict__ Xe, const int64_t* __restrict__ gain, uint64_t G,
+                       const uint32_t* __restrict__ list, const Counters* __restrict__ ctr)
 {
-    for (uint64_t g = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; g < G; g += (uint64_t)gridDim.x * blockDim.x) {
+    const uint32_t n = ctr->n_kmc_cells;
+    for (uint64_t t = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; t < (uint64_t)n * P.S;
+         t += (uint64_t)gridDim.x * blockDim.x) {
+        const uint64_t sp = (uint64_t)(t >= n) + (uint64_t)(t >= 2ull * n);
+        const uint64_t g = sp * G + list[t - sp * n];
         const long long dN = gain[g];
         if (dN >= 0) continue;
         const unsigned long long L = (unsigned long long)(-dN);
@@ -1517,64 +1552,123 @@ constexpr int MERGE_NW0 = 4, MERGE_NW1 = 4;
 __host__ __device__ inline uint32_t merge_cap0(int esize) { return esize == 16 ? MERGE_CAP0_MP32 : MERGE_CAP0_MP; }
 
 // Per particle cell: W = X + dN + photo weight -> min(W, ppc) leaves; photo
-// offsets; work-area units (32 B) for tier-2 cells; the tier lists.  The
-// photons of physical cell c are the electron block's photoelectrons and the
-// positive-ion block's photo-ions (mobile ions); the photo offsets count
-// them once, over the electron blocks.
+// offsets; the tier lists.  The photons of physical cell c are the electron
+// block's photoelectrons and the positive-ion block's photo-ions (mobile
+// ions); the photo offsets count them once, over the electron blocks.
+// Channels: leaves, photons, cells of tier 0, 1, 2.  The first pass leaves
+// each cell's leaves and tier in code, which the second reads in the place of
+// five arrays.
 struct MergeScanOp {
     const unsigned long long* Xe;
     const int64_t* gain;
     const unsigned long long* photo_w;
     const int32_t* photo_cnt;
     const uint32_t* cs;
+    uint32_t* code;           // leaves | (tier + 1) << 16 (0: no particles)
     uint32_t* out_start;
     uint32_t* photo_off;
-    uint64_t* work_off;
     uint32_t* small_list;     // non-empty cells of tier 0
     uint32_t* mid_list;       // ... tier 1
     uint32_t* big_list;       // ... tier 2
     uint32_t* list_n;         // [3]: lengths
     uint64_t G;               // particle cells
     uint64_t Gphys;           // physical cells (one block per realization)
-    int ppc, n_new, esize, ksize;
-    __device__ void load(uint64_t g, long long v[6]) const
+    int ppc, n_new, esize;
+    // species of cell g (a group of eight lies in one block)
+    __device__ uint64_t species(uint64_t g) const { return (uint64_t)(g >= Gphys) + (uint64_t)(g >= 2 * Gphys); }
+    __device__ void sum8(uint64_t g, uint32_t s[5]) const
     {
-        const long long dN = gain[g];
-        const uint64_t sp = (uint64_t)(g >= Gphys) + (uint64_t)(g >= 2 * Gphys), gph = g - sp * Gphys;
-        const long long pw = sp <= 1 ? (long long)photo_w[gph] : 0, pc = sp <= 1 ? photo_cnt[gph] : 0;
-        const long long W = (long long)Xe[g] + dN + pw;
-        v[0] = W < ppc ? W : ppc;
-        v[1] = sp == 0 ? pc : 0;
-        const long long M = (long long)(cs[g + 1] - cs[g]) + (dN > 0 ? (dN < n_new ? dN : n_new) : 0) + pc;
-        const long long S = M + ppc;
-        const int tier = S <= (long long)merge_cap0(esize) ? 0 : (S <= MERGE_CAP1 ? 1 : 2);
-        v[2] = (v[0] > 0 && tier == 2)
-                   ? ((long long)merge_layout((uint32_t)S, (uint32_t)ppc, (uint32_t)esize, (uint32_t)ksize).bytes + 31) / 32
-                   : 0;
-        v[3] = (v[0] > 0 && tier == 0) ? 1 : 0;
-        v[4] = (v[0] > 0 && tier == 1) ? 1 : 0;
-        v[5] = (v[0] > 0 && tier == 2) ? 1 : 0;
+        const uint64_t sp = species(g), gph = g - sp * Gphys;
+        long long X[8], dN[8], pw[8];
+        uint32_t pc[8], c[8], o[8];
+        load8(reinterpret_cast<const long long*>(Xe) + g, X);
+        load8(reinterpret_cast<const long long*>(gain) + g, dN);
+#pragma unroll
+        for (int k = 0; k < 8; ++k) { pw[k] = 0; pc[k] = 0; }
+        if (sp <= 1) {
+            load8(reinterpret_cast<const long long*>(photo_w) + gph, pw);
+            load8(reinterpret_cast<const uint32_t*>(photo_cnt) + gph, pc);
+        }
+        load8(cs + g, c);
+        const uint32_t end = cs[g + 8];
+#pragma unroll
+        for (int k = 0; k < 8; ++k) {
+            const long long W = X[k] + dN[k] + pw[k];
+            const uint32_t leaves = (uint32_t)(W < ppc ? W : ppc);
+            const long long M = (long long)((k < 7 ? c[k < 7 ? k + 1 : 7] : end) - c[k]) +
+                                (dN[k] > 0 ? (dN[k] < n_new ? dN[k] : n_new) : 0) + pc[k];
+            const long long S = M + ppc;
+            const uint32_t tier = S <= (long long)merge_cap0(esize) ? 0u : (S <= MERGE_CAP1 ? 1u : 2u);
+            o[k] = leaves ? leaves | ((tier + 1u) << 16) : 0u;
+            s[0] += leaves;
+            s[1] += sp == 0 ? pc[k] : 0u;
+            s[2] += leaves && tier == 0u;
+            s[3] += leaves && tier == 1u;
+            s[4] += leaves && tier == 2u;
+        }
+        store8(code + g, o);
     }
-    __device__ void store(uint64_t g, const long long ex[6], const long long* v) const
+    __device__ void get8(uint64_t g, uint32_t v[8][5]) const
     {
-        out_start[g] = (uint32_t)ex[0];
-        photo_off[g] = (uint32_t)ex[1];
-        work_off[g] = (uint64_t)ex[2];
-        if (v[3]) small_list[ex[3]] = (uint32_t)g;
-        if (v[4]) mid_list[ex[4]] = (uint32_t)g;
-        if (v[5]) big_list[ex[5]] = (uint32_t)g;
+        uint32_t o[8], pc[8];
+        load8(code + g, o);
+#pragma unroll
+        for (int k = 0; k < 8; ++k) pc[k] = 0;
+        if (g < Gphys) load8(reinterpret_cast<const uint32_t*>(photo_cnt) + g, pc);
+#pragma unroll
+        for (int k = 0; k < 8; ++k) {
+            v[k][0] = o[k] & 0xffffu;
+            v[k][1] = pc[k];
+            v[k][2] = (o[k] >> 16) == 1u;
+            v[k][3] = (o[k] >> 16) == 2u;
+            v[k][4] = (o[k] >> 16) == 3u;
+        }
     }
-    __device__ void total(const long long t[6]) const
+    __device__ void put8(uint64_t g, const uint32_t ex[5], const uint32_t v[8][5]) const
+    {
+        uint32_t os[8], po[8], e[5] = { ex[0], ex[1], ex[2], ex[3], ex[4] };
+#pragma unroll
+        for (int k = 0; k < 8; ++k) {
+            os[k] = e[0];
+            po[k] = e[1];
+            if (v[k][2]) small_list[e[2]] = (uint32_t)(g + k);
+            if (v[k][3]) mid_list[e[3]] = (uint32_t)(g + k);
+            if (v[k][4]) big_list[e[4]] = (uint32_t)(g + k);
+#pragma unroll
+            for (int c = 0; c < 5; ++c) e[c] += v[k][c];
+        }
+        store8(out_start + g, os);
+        store8(photo_off + g, po);
+    }
+    __device__ void total(const long long t[5]) const
     {
         out_start[G] = (uint32_t)t[0];
         photo_off[G] = (uint32_t)t[1];
-        work_off[G] = (uint64_t)t[2];
-        list_n[0] = (uint32_t)t[3];
-        list_n[1] = (uint32_t)t[4];
-        list_n[2] = (uint32_t)t[5];
+        list_n[0] = (uint32_t)t[2];
+        list_n[1] = (uint32_t)t[3];
+        list_n[2] = (uint32_t)t[4];
         list_n[3] = 0;            // cells that the merge by presorted lists leaves to k_merge_lv
     }
 };
+
+// Work-area places (32-byte units) of the tier-2 cells in list order of
+// arrival: the scratch needs no order.  total: zeroed before.
+__global__ void k_big_work(Params P, const uint32_t* __restrict__ big_list, const uint32_t* __restrict__ list_n,
+                           const uint32_t* __restrict__ cs, const int64_t* __restrict__ gain,
+                           const int32_t* __restrict__ photo_cnt, uint64_t Gphys, uint32_t esize, uint32_t ksize,
+                           uint64_t* __restrict__ work_off, unsigned long long* __restrict__ total)
+{
+    const uint32_t n = list_n[2];
+    for (uint32_t li = blockIdx.x * blockDim.x + threadIdx.x; li < n; li += gridDim.x * blockDim.x) {
+        const uint64_t g = big_list[li];
+        const uint64_t sp = (uint64_t)(g >= Gphys) + (uint64_t)(g >= 2 * Gphys);
+        const long long dN = gain[g];
+        const long long M = (long long)(cs[g + 1] - cs[g]) + (dN > 0 ? (dN < P.n_new ? dN : P.n_new) : 0) +
+                            (sp <= 1 ? photo_cnt[g - sp * Gphys] : 0);
+        const unsigned long long units = (merge_layout((uint32_t)(M + P.ppc), (uint32_t)P.ppc, esize, ksize).bytes + 31ull) / 32;
+        work_off[li] = atomicAdd(total, units);
+    }
+}
 
 // ------------------------------------------------------------------ merge
 struct MP32 {         // merge work element (mixed form: cell offsets)
@@ -1909,11 +2003,11 @@ __global__ void __launch_bounds__(128, GLOBAL ? 4 : (std::is_same<E, MP32>::valu
             max_m = (cs[g + 1] - cs[g]) + (dN > 0 ? (uint32_t)(dN < P.n_new ? dN : P.n_new) : 0u) +
                     (ph ? photo_off[gp + 1] - photo_off[gp] : 0u);
             L = merge_layout(max_m + T, T, sizeof(E), sizeof(K));
-            if (work_off[g] * 32 + L.bytes > work_cap * 32) {
+            if (work_off[li] * 32 + L.bytes > work_cap * 32) {
                 if (lane == 0) atomicOr(&ctr->err, DERR_CAPACITY);
                 continue;
             }
-            base = work + work_off[g] * 32;
+            base = work + work_off[li] * 32;
         } else {
             max_m = CAP - T;
             L = merge_layout(CAP, T, sizeof(E), sizeof(K));
@@ -2845,7 +2939,7 @@ void launch_advect(const Params& P, Dev& d, uint32_t N, cudaStream_t s)
 void launch_transport_finish(const Params& P, Dev& d, uint32_t N, uint64_t G, cudaStream_t s, const uint32_t* Ndev)
 {
     TransportScanOp op{ d.cnt_new, d.in_cnt, d.in_before, d.cell_start_B, d.delta, d.in_off, G };
-    run_scan<3>(op, G, d.scan_blk, s);
+    run_gscan<3>(op, G, d.scan_blk, s);
     const uint32_t nblk = (N + TPB - 1) / TPB;
     if (N > 0) {
         BlockScanOp bop{ d.blk_stay, d.blk_prefix };
@@ -3001,21 +3095,30 @@ void launch_kmc(const Params& P, Dev& d, uint64_t G, cudaStream_t s)
     static_assert(offsetof(Counters, n_kmc_cells) > offsetof(Counters, ion), "counter layout");
     cudaMemsetAsync(reinterpret_cast<char*>(d.ctr) + offsetof(Counters, ion), 0,
                     offsetof(Counters, n_kmc_cells) + sizeof(unsigned int) - offsetof(Counters, ion), s);
-    // the merge's tier-0 list is free until the merge scan of this step
+    if (d.kmc_stale) {
+        // firings that no list covers (a loaded state): every cell once
+        cudaMemsetAsync(d.fired, 0, 5 * G * sizeof(int64_t), s);
+        cudaMemsetAsync(d.gain, 0, (uint64_t)P.S * G * sizeof(int64_t), s);
+        d.kmc_stale = false;
+    } else {
+        ++g_launches;
+        k_kmc_clear<<<grid_for(G, 256, 152 * 8), 256, 0, s>>>(P, d.fired, d.gain, G, d.kmc_list, d.kmc_n);
+    }
     g_launches += 2;
-    k_kmc_list<<<grid_for(G, 256, 152 * 32), 256, 0, s>>>(P, d.Xe, d.Npos, d.Nneg, d.fired, d.gain, G, d.small_list,
-                                                          d.ctr);
+    k_kmc_list<<<grid_for(G, 256, 152 * 32), 256, 0, s>>>(P, d.Xe, d.Npos, d.Nneg, G, d.kmc_list, d.ctr);
+    cudaMemcpyAsync(d.kmc_n, reinterpret_cast<const char*>(d.ctr) + offsetof(Counters, n_kmc_cells), sizeof(uint32_t),
+                    cudaMemcpyDeviceToDevice, s);
     const int nb = grid_for(G, 128, 152 * 64);
     const bool rec = P.k_ep > 0.0 || P.k_np > 0.0;
     if (d.mixed) {
-        if (rec) k_kmc<float, true><<<nb, 128, 0, s>>>(P, d.Xe, d.E, d.E32, d.fired, d.gain, d.Npos, d.Nneg, G, d.small_list,
+        if (rec) k_kmc<float, true><<<nb, 128, 0, s>>>(P, d.Xe, d.E, d.E32, d.fired, d.gain, d.Npos, d.Nneg, G, d.kmc_list,
                                                        d.pc_list, d.ctr);
-        else k_kmc<float, false><<<nb, 128, 0, s>>>(P, d.Xe, d.E, d.E32, d.fired, d.gain, d.Npos, d.Nneg, G, d.small_list,
+        else k_kmc<float, false><<<nb, 128, 0, s>>>(P, d.Xe, d.E, d.E32, d.fired, d.gain, d.Npos, d.Nneg, G, d.kmc_list,
                                                     d.pc_list, d.ctr);
     } else {
-        if (rec) k_kmc<double, true><<<nb, 128, 0, s>>>(P, d.Xe, d.E, d.E32, d.fired, d.gain, d.Npos, d.Nneg, G, d.small_list,
+        if (rec) k_kmc<double, true><<<nb, 128, 0, s>>>(P, d.Xe, d.E, d.E32, d.fired, d.gain, d.Npos, d.Nneg, G, d.kmc_list,
                                                         d.pc_list, d.ctr);
-        else k_kmc<double, false><<<nb, 128, 0, s>>>(P, d.Xe, d.E, d.E32, d.fired, d.gain, d.Npos, d.Nneg, G, d.small_list,
+        else k_kmc<double, false><<<nb, 128, 0, s>>>(P, d.Xe, d.E, d.E32, d.fired, d.gain, d.Npos, d.Nneg, G, d.kmc_list,
                                                      d.pc_list, d.ctr);
     }
 }
@@ -3032,16 +3135,21 @@ void launch_particles_a(const Params& P, Dev& d, uint64_t G, cudaStream_t s)
     uint32_t* wbase = d.mixed ? reinterpret_cast<uint32_t*>(d.rA32) + 3 : reinterpret_cast<uint32_t*>(d.recA) + 7;
     const int wstride = d.mixed ? 4 : 8;
     ++g_launches;
-    k_loss<<<grid_for(Gp, 128, 152 * 64), 128, 0, s>>>(P, wbase, wstride, d.cell_start, d.Xe, d.gain, Gp);
+    k_loss<<<grid_for(Gp, 128, 152 * 64), 128, 0, s>>>(P, wbase, wstride, d.cell_start, d.Xe, d.gain, G, d.kmc_list, d.ctr);
     if (P.photon_ratio > 0.0) {
         ++g_launches;
         k_photons<<<152 * 16, 256, 0, s>>>(P, d.mixed ? 1 : 0, d.fired, G, d.pc_list, d.photos, d.photo_cap,
                                             d.photo_cnt, d.photo_w, d.Npos, d.ctr);
     }
-    MergeScanOp op{ d.Xe, d.gain, d.photo_w, d.photo_cnt, d.cell_start, d.out_start, d.photo_off, d.work_off,
-                    d.small_list, d.mid_list, d.big_list, d.list_n, Gp, G, P.ppc, P.n_new,
-                    d.mixed ? (int)sizeof(MP32) : (int)sizeof(MP), d.mixed ? 4 : 8 };
-    run_scan<6>(op, Gp, d.scan_blk, s);
+    const int esize = d.mixed ? (int)sizeof(MP32) : (int)sizeof(MP);
+    MergeScanOp op{ d.Xe, d.gain, d.photo_w, d.photo_cnt, d.cell_start, reinterpret_cast<uint32_t*>(d.cnt_new), d.out_start,
+                    d.photo_off, d.small_list, d.mid_list, d.big_list, d.list_n, Gp, G, P.ppc, P.n_new, esize };
+    run_gscan<5>(op, Gp, d.scan_blk, s);
+    unsigned long long* total = reinterpret_cast<unsigned long long*>(d.work_off) + Gp;
+    cudaMemsetAsync(total, 0, sizeof *total, s);
+    ++g_launches;
+    k_big_work<<<152, 256, 0, s>>>(P, d.big_list, d.list_n, d.cell_start, d.gain, d.photo_cnt, G, (uint32_t)esize,
+                                   d.mixed ? 4u : 8u, d.work_off, total);
 }
 
 

@@ -182,6 +182,7 @@ int seed_blobs(itokmc_handle* h, const itokmc_seed_blob* blobs, int nb, int flag
         return handle_fail(h, ITOKMC_ERR_ARG, "seed_blobs: too many blobs");
     SeedBlob* dB = reinterpret_cast<SeedBlob*>(d.photos);
     int64_t* cnt = d.fired;                      // counts in the first G of the firing array
+    d.kmc_stale = true;
     cudaStream_t s = v.s;
     if (nb > 0 && cudaMemcpyAsync(dB, hb.data(), nb * sizeof(SeedBlob), cudaMemcpyHostToDevice, s) != cudaSuccess)
         return handle_fail(h, ITOKMC_ERR_CUDA, "seed_blobs: copy");

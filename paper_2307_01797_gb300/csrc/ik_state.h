@@ -141,6 +141,9 @@ struct Dev {
     uint32_t* tie_list = nullptr;      // Gp: cells of tiers 0 and 1 left to the merge with a sort per level
     uint32_t* list_n = nullptr;        // 4 counts: tiers 0, 1, 2 and the ties
     uint32_t* pc_list = nullptr;       // G: photon-emitting cells
+    uint32_t* kmc_list = nullptr;      // G: cells of the last KMC (outside them fired and gain are zero)
+    uint32_t* kmc_n = nullptr;         // its length
+    bool kmc_stale = false;            // fired was set from outside: kmc_list does not cover it
     unsigned char* work = nullptr;  size_t work_bytes = 0;   // merge scratch of tier-2 cells
     // scans
     long long* scan_blk = nullptr;  size_t scan_blk_elems = 0;
