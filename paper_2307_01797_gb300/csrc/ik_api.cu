@@ -128,6 +128,19 @@ void dfree(itokmc_handle* h, void* p)
     else cudaFreeAsync(p, h->s);
 }
 
+// Whether kernels can read the array p where it is: memory of the handle's
+// device, aligned to its elements.  NULL (an array that is not given) passes.
+bool readable_here(itokmc_handle* h, const void* p, size_t align)
+{
+    if (!p) return true;
+    cudaPointerAttributes a;
+    if (cudaPointerGetAttributes(&a, p) != cudaSuccess) {
+        cudaGetLastError();
+        return false;
+    }
+    return a.type == cudaMemoryTypeDevice && a.device == h->device && reinterpret_cast<uintptr_t>(p) % align == 0;
+}
+
 // Grows the photon list to hold at least `need` superphotons (geometric).
 int ensure_photo_cap(itokmc_handle* h, uint64_t need)
 {
@@ -1085,17 +1098,28 @@ int itokmc_set_particles_species(itokmc_handle* h, const double* x, const double
     uint32_t* dw = reinterpret_cast<uint32_t*>(dz + n);
     int32_t* dr = realization ? reinterpret_cast<int32_t*>(dw + n) : nullptr;
     const cudaMemcpyKind k = mem == ITOKMC_HOST ? cudaMemcpyHostToDevice : cudaMemcpyDeviceToDevice;
-    if (n > 0) {
+    // arrays in this device's memory are read where they are
+    const bool in_place = mem == ITOKMC_DEVICE && n > 0 && readable_here(h, x, 8) && readable_here(h, y, 8) &&
+                          readable_here(h, z, 8) && readable_here(h, w, 4) && readable_here(h, realization, 4) &&
+                          readable_here(h, species, 4);
+    const double *sx = dx, *sy = dy, *sz = dz;
+    const uint32_t* sw = dw;
+    const int32_t *sr = dr, *ssp = nullptr;
+    if (in_place) {
+        sx = x; sy = y; sz = z; sw = w; sr = realization; ssp = species;
+    } else if (n > 0) {
         IK_CHECK(h, cudaMemcpyAsync(dx, x, n * sizeof(double), k, h->s));
         IK_CHECK(h, cudaMemcpyAsync(dy, y, n * sizeof(double), k, h->s));
         IK_CHECK(h, cudaMemcpyAsync(dz, z, n * sizeof(double), k, h->s));
         IK_CHECK(h, cudaMemcpyAsync(dw, w, n * sizeof(uint32_t), k, h->s));
         if (dr) IK_CHECK(h, cudaMemcpyAsync(dr, realization, n * sizeof(int32_t), k, h->s));
+        // the species (mobile ions) in the push keys' buffer, free until the next push
+        if (species) {
+            IK_CHECK(h, cudaMemcpyAsync(h->d.keyB, species, n * sizeof(int32_t), k, h->s));
+            ssp = reinterpret_cast<const int32_t*>(h->d.keyB);
+        }
     }
-    // the species (mobile ions) in the push keys' buffer, free until the next push
-    int32_t* dsp = (species && n > 0) ? reinterpret_cast<int32_t*>(h->d.keyB) : nullptr;
-    if (dsp) IK_CHECK(h, cudaMemcpyAsync(dsp, species, n * sizeof(int32_t), k, h->s));
-    ik::launch_set_particles(h->P, h->d, dx, dy, dz, dw, dr, dsp, (uint32_t)n, h->Gp, h->s);
+    ik::launch_set_particles(h->P, h->d, sx, sy, sz, sw, sr, ssp, (uint32_t)n, h->Gp, h->s);
     int rc = readback(h);
     if (rc) return rc;
     if (h->rb->ctr.err) {
@@ -1175,8 +1199,12 @@ int itokmc_set_field(itokmc_handle* h, const double* E, int32_t mem)
     IK_GUARD(h);
     if (!E) return fail(h, ITOKMC_ERR_ARG, "NULL field");
     const cudaMemcpyKind k = mem == ITOKMC_HOST ? cudaMemcpyHostToDevice : cudaMemcpyDeviceToDevice;
-    IK_CHECK(h, cudaMemcpyAsync(h->d.stage, E, 3 * h->G * sizeof(double), k, h->s));
-    ik::launch_pack_field(h->P, h->d, h->d.stage, h->s);
+    const double* src = E;
+    if (!(mem == ITOKMC_DEVICE && readable_here(h, E, 8))) {
+        IK_CHECK(h, cudaMemcpyAsync(h->d.stage, E, 3 * h->G * sizeof(double), k, h->s));
+        src = h->d.stage;
+    }
+    ik::launch_pack_field(h->P, h->d, src, h->s);
     IK_CHECK(h, cudaStreamSynchronize(h->s));
     return cuda_check(h, cudaGetLastError(), "set_field");
 }

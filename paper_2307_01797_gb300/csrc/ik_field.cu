@@ -1974,10 +1974,50 @@ void field_solve_fixed(const Params& P, Dev& d, int precision, int nu1, int nu2,
     k_norm_final<<<R, 256, 0, s>>>(d.norm_part, precision == 1 ? bpr : march.bpr, R, d.norm_out);
 }
 
+// The FP32 value of a double that is one (false: it is not, or is not a normal
+// number).
+__device__ __forceinline__ bool as_float(double v, float& f)
+{
+    const unsigned long long b = (unsigned long long)__double_as_longlong(v);
+    const int e = (int)((b >> 52) & 0x7ff);
+    if (b << 1 == 0) { f = 0.f; return true; }
+    if ((b & 0x1fffffffull) != 0 || e < 1023 - 126 || e > 1023 + 126) return false;
+    f = __uint_as_float((uint32_t)((b >> 32) & 0x80000000u) | ((uint32_t)(e - 896) << 23) | (uint32_t)((b >> 29) & 0x7fffffu));
+    return true;
+}
+
+// |E| of three FP32 components rounded to FP32 as (float)sqrt((ex ex + ey ey) +
+// ez ez) in FP64 is, from sums of two floats (relative error below 2^-40):
+// false where that is too near a rounding boundary to tell, or out of range.
+__device__ __forceinline__ bool norm3(float x, float y, float z, float& m)
+{
+    const float a = x * x, b = y * y, c = z * z;
+    const float ea = __fmaf_rn(x, x, -a), eb = __fmaf_rn(y, y, -b), ec = __fmaf_rn(z, z, -c);
+    const float s1 = a + b, t1 = s1 - a, e1 = (a - (s1 - t1)) + (b - t1);       // two-sums
+    const float s = s1 + c, t2 = s - s1, e2 = (s1 - (s - t2)) + (c - t2);
+    const float lo = ((ea + eb) + ec) + (e1 + e2);
+    if (!(s > 1e-20f && s < 1e30f)) return false;
+    const float r = sqrtf(s);
+    const float d = __fdiv_rn(__fmaf_rn(-r, r, s) + lo, r + r);                  // sqrt(s + lo) = r + d
+    m = r + d;
+    const float off = fabsf((r - m) + d);                                        // what the rounding left
+    const float half = 0.5f * (__uint_as_float(__float_as_uint(m) + 1u) - m);
+    // (a power of two has its lower boundary at half the distance)
+    return fabsf(off - half) > half * 1e-3f && fabsf(off - 0.5f * half) > half * 1e-3f;
+}
+
+// The handle's field from three blocks of components: E64 (FP64 form) or
+// float4 (mixed form).  An FP32 field (one read from the mixed form) takes
+// |E| without the FP64 pipe, whose square root bounds the pass otherwise.
 __global__ void k_pack_field(const double* __restrict__ E3, E64* __restrict__ E, float4* __restrict__ E32, uint64_t G)
 {
     for (uint64_t t = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; t < G; t += (uint64_t)gridDim.x * blockDim.x) {
         const double ex = E3[t], ey = E3[G + t], ez = E3[2 * G + t];
+        float fx, fy, fz, fm;
+        if (!E && as_float(ex, fx) && as_float(ey, fy) && as_float(ez, fz) && norm3(fx, fy, fz, fm)) {
+            E32[t] = make_float4(fx, fy, fz, fm);
+            continue;
+        }
         const double m = sqrt((ex * ex + ey * ey) + ez * ez);
         if (E) {
             reinterpret_cast<double2*>(E + t)[0] = make_double2(ex, ey);

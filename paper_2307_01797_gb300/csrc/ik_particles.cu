@@ -50,69 +50,6 @@ __device__ __forceinline__ E64 ld_e64(const E64* p)
 
 // Trilinear interpolation of the cell-centred field at (x,y,z); sum order z
 // outer, y, x inner; weight (wx*wy)*wz.
-// Cell quotients qd in [1/2, 2^31) split from their bits.  For such qd the
-// stencil coordinate u = qd - 1/2 is exact (1/2 is a multiple of ulp(qd)),
-// and so are floor(u), the fraction f = u - floor(u) = F 2^-sh and
-// floor(f 2^s) = F >> (sh - s): the FP64 subtract / floor / convert
-// sequence yields the same values, and these integer steps keep the FP64
-// pipe (a small fraction of the FP32 rate on GB300) for the arithmetic
-// that rounds.  qc = floor(qd) is the cell index.
-struct QSplit {
-    int qc, i0, sh;
-    unsigned long long F;
-};
-__device__ __forceinline__ bool qsplit(double qd, QSplit& r)
-{
-    const unsigned long long b = (unsigned long long)__double_as_longlong(qd);
-    const int e = (int)(b >> 52);                  // biased exponent (>= 2048 when negative)
-    if (e < 1022 || e > 1053) return false;        // qd < 1/2, qd >= 2^31, negative, NaN
-    const unsigned long long m = (b & 0xfffffffffffffull) | (1ull << 52);
-    const int sh = 1075 - e;                       // fraction bits of qd, 22..53
-    const unsigned long long fb = m & ((1ull << sh) - 1ull), half = 1ull << (sh - 1);
-    r.qc = (int)(m >> sh);
-    r.sh = sh;
-    if (fb >= half) { r.i0 = r.qc; r.F = fb - half; }
-    else { r.i0 = r.qc - 1; r.F = fb + half; }
-    return true;
-}
-// The quotient q = (x - lo) / h of axis a (grid_quot) rounded to 53 bits and
-// split, by integer multiplication with the 96-bit reciprocal: the product's
-// upper 96 bits are within a few units of 2^-96 of the quotient, and grid_quot's
-// result is the quotient rounded to nearest up to an error of 2^-52 units of
-// the last place before its rounding; so both round the same way unless the
-// bits below the 53rd lie within 2^-29 of a half.  Those, and quotients
-// outside qsplit's range, return false (the caller takes grid_quot).  GB300 has
-// 2 FP64 lanes per SM and clock: the three FP64 instructions of a quotient
-// hold the pipe for the time in which an SM issues 192 others.  (Products
-// rounded by integer instructions, about 50 each, gained nothing.)
-__device__ __forceinline__ bool quot_split(const Params& P, double x, int a, QSplit& r)
-{
-    double d = x;
-    if (__double_as_longlong(P.lo[a]) != 0) d = x - P.lo[a];
-    const uint32_t dh = (uint32_t)__double2hiint(d), dl = (uint32_t)__double2loint(d);
-    const int e = (int)(dh >> 20);                  // biased exponent (>= 2048 when negative)
-    const uint32_t m1 = (dh << 11) | (dl >> 21) | 0x80000000u, m0 = dl << 11;
-    const uint64_t u = (uint64_t)m1 * P.rh96[1], v = (uint64_t)m0 * P.rh96[2];
-    const uint64_t w = (uint64_t)(uint32_t)u + (uint32_t)v + __umulhi(m1, P.rh96[0]) + __umulhi(m0, P.rh96[1]);
-    uint64_t top = (uint64_t)m1 * P.rh96[2] + (u >> 32) + (v >> 32) + (w >> 32);
-    uint32_t g = (uint32_t)w;
-    int E = e - 1075 - P.h_exp;                     // q = top 2^(E - 63)
-    if (!(top >> 63)) {
-        top = (top << 1) | (g >> 31);
-        g <<= 1;
-        --E;
-    }
-    const uint32_t low = ((uint32_t)top << 21) | (g >> 11);
-    const int sh = 52 - E;                          // fraction bits
-    if (e == 0 || e >= 2047 || sh < 22 || sh > 53 || low - 0x7ffffffcu <= 8u) return false;
-    const uint64_t m = (top >> 11) + (low >> 31);
-    const uint64_t fb = m & ((1ull << sh) - 1ull), half = 1ull << (sh - 1);
-    r.qc = (int)(m >> sh);
-    r.sh = sh;
-    if (fb >= half) { r.i0 = r.qc; r.F = fb - half; }
-    else { r.i0 = r.qc - 1; r.F = fb + half; }
-    return true;
-}
 // F 2^-sh as a double (F < 2^sh, sh <= 53: exact).
 __device__ __forceinline__ double qfrac(unsigned long long F, int sh)
 {
@@ -148,15 +85,6 @@ __device__ __forceinline__ void cic_axis_q(const Params& P, double x, int a, int
     ia = clampi(i0, P.n);
     ib = clampi(i0 + 1, P.n);
 }
-// x >= lo and x < hi by order-preserving integer keys (-0 taken as +0; a NaN
-// fails one of the two tests, as in the FP64 comparisons).
-__device__ __forceinline__ unsigned long long dkey(double v)
-{
-    unsigned long long b = (unsigned long long)__double_as_longlong(v);
-    b = b == 0x8000000000000000ull ? 0ull : b;
-    return (b >> 63) ? ~b : (b | 0x8000000000000000ull);
-}
-
 // The loops over the axes and over z stay loops, an axis' values rotating
 // through registers: with them unrolled a quarter of the push's issue slots
 // waited for instructions.

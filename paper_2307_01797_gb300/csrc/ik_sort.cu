@@ -17,8 +17,10 @@ constexpr int RS_TILE = RS_TPB * RS_ROUNDS;
 constexpr int RS_BINS = 256;
 
 __global__ void __launch_bounds__(RS_TPB) k_rs_hist(const uint32_t* __restrict__ keys, uint32_t n, int shift,
-                                                    uint32_t nblk, uint32_t* __restrict__ hist)
+                                                    uint32_t nblk, uint32_t* __restrict__ hist,
+                                                    const unsigned* __restrict__ unsorted)
 {
+    if (*unsorted == 0) return;
     __shared__ uint32_t h[RS_BINS];
     h[threadIdx.x] = 0;
     __syncthreads();
@@ -42,8 +44,9 @@ struct HistScanOp {
 __global__ void __launch_bounds__(RS_TPB) k_rs_scatter(const uint32_t* __restrict__ keys, const uint32_t* __restrict__ vals,
                                                        uint32_t n, int shift, uint32_t nblk,
                                                        const uint32_t* __restrict__ off, uint32_t* __restrict__ kout,
-                                                       uint32_t* __restrict__ vout)
+                                                       uint32_t* __restrict__ vout, const unsigned* __restrict__ unsorted)
 {
+    if (*unsorted == 0) return;
     __shared__ uint32_t running[RS_BINS];
     __shared__ uint32_t wc[RS_TPB / 32][RS_BINS];
     const unsigned lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
@@ -87,13 +90,19 @@ __global__ void k_pack(Params P, const double* __restrict__ x, const double* __r
         const int r0 = real ? real[i] : 0, sp = species ? species[i] : 0;
         bool ok = r0 >= 0 && r0 < P.R && sp >= 0 && sp < P.S && w[i] > 0;
         const int r = sp * P.R + r0;             // particle block
-        for (int a = 0; a < 3; ++a) ok = ok && X[a] >= P.lo[a] && X[a] < P.hi[a];
+        int ic[3];
+#pragma unroll
+        for (int a = 0; a < 3; ++a) {
+            const unsigned long long kx = dkey(X[a]);
+            ok = ok && kx >= dkey(P.lo[a]) && kx < dkey(P.hi[a]);
+            // the cell from the quotient's integer split (the FP64 quotient
+            // where that does not serve)
+            QSplit t;
+            ic[a] = ok ? (quot_split(P, X[a], a, t) ? clampi(t.qc, P.n) : cell_axis(X[a], P.lo[a], P.h[a], P.rh[a], P.n)) : 0;
+        }
         uint32_t g = 0;
         if (ok) {
-            const int ix = cell_axis(X[0], P.lo[0], P.h[0], P.rh[0], P.n);
-            const int iy = cell_axis(X[1], P.lo[1], P.h[1], P.rh[1], P.n);
-            const int iz = cell_axis(X[2], P.lo[2], P.h[2], P.rh[2], P.n);
-            g = (uint32_t)((size_t)r * P.n3 + ((size_t)iz * P.n + iy) * P.n + ix);
+            g = (uint32_t)((size_t)r * P.n3 + ((size_t)ic[2] * P.n + ic[1]) * P.n + ic[0]);
         } else {
             atomicOr(&ctr->err, DERR_INTERNAL);
         }
@@ -105,24 +114,58 @@ __global__ void k_pack(Params P, const double* __restrict__ x, const double* __r
     }
 }
 
-__global__ void k_gather(const P64* __restrict__ in, const uint32_t* __restrict__ perm, uint32_t n, P64* __restrict__ out)
+// *unsorted is set where a key is followed by a smaller one.  Particles
+// often come in the library's own order (a restart, a coupled code): the sort
+// is then the identity and its passes return at once.
+__global__ void k_find_unsorted(const uint32_t* __restrict__ keys, uint32_t n, unsigned* __restrict__ unsorted)
 {
-    for (uint32_t j = blockIdx.x * blockDim.x + threadIdx.x; j < n; j += gridDim.x * blockDim.x) out[j] = in[perm[j]];
+    bool bad = false;
+    for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i + 1 < n; i += gridDim.x * blockDim.x) bad |= keys[i] > keys[i + 1];
+    if (__any_sync(__activemask(), bad) && bad) atomicOr(unsorted, 1u);
+}
+
+__global__ void k_gather(const P64* __restrict__ in, const uint32_t* __restrict__ perm, uint32_t n, P64* __restrict__ out,
+                         const unsigned* __restrict__ unsorted)
+{
+    const bool sorted = *unsorted == 0;
+    for (uint32_t j = blockIdx.x * blockDim.x + threadIdx.x; j < n; j += gridDim.x * blockDim.x) {
+        const double2* p = reinterpret_cast<const double2*>(in + (sorted ? j : perm[j]));
+        const double2 a = p[0], b = p[1];
+        reinterpret_cast<double2*>(out + j)[0] = a;
+        reinterpret_cast<double2*>(out + j)[1] = b;
+    }
+}
+
+// The result of an odd number of passes, back from the tmp buffers.
+__global__ void k_rs_copy(const uint32_t* __restrict__ ka, const uint32_t* __restrict__ va, uint32_t* __restrict__ kb,
+                          uint32_t* __restrict__ vb, uint32_t n, const unsigned* __restrict__ unsorted)
+{
+    if (*unsorted == 0) return;
+    for (uint32_t j = blockIdx.x * blockDim.x + threadIdx.x; j < n; j += gridDim.x * blockDim.x) {
+        kb[j] = ka[j];
+        vb[j] = va[j];
+    }
 }
 
 // Mixed form: (cell, FP32 offset in cell units) from the sorted FP64 records.
 __global__ void k_gather32(Params P, const P64* __restrict__ in, const uint32_t* __restrict__ perm, uint32_t n,
-                           P32* __restrict__ out, uint32_t* __restrict__ cout)
+                           P32* __restrict__ out, uint32_t* __restrict__ cout, const unsigned* __restrict__ unsorted)
 {
+    const bool sorted = *unsorted == 0;
     for (uint32_t j = blockIdx.x * blockDim.x + threadIdx.x; j < n; j += gridDim.x * blockDim.x) {
-        const P64 p = in[perm[j]];
+        const P64 p = in[sorted ? j : perm[j]];
         const uint32_t c = p.cell & (uint32_t)(P.n3 - 1);
         const int id[3] = { (int)(c & (uint32_t)(P.n - 1)), (int)((c >> P.log2n) & (uint32_t)(P.n - 1)),
                             (int)(c >> (2 * P.log2n)) };
         const double X[3] = { p.x, p.y, p.z };
         float o[3];
         for (int a = 0; a < 3; ++a) {
-            float f = (float)(grid_quot(X[a], P.lo[a], P.h[a], P.rh[a]) - (double)id[a]);
+            // q - id in FP64 is exact for id = floor(q): the quotient's fraction
+            // bits, rounded once to FP32
+            QSplit t;
+            float f;
+            if (quot_split(P, X[a], a, t) && t.qc == id[a]) f = __ull2float_rn(t.fb) * __int_as_float((127 - t.sh) << 23);
+            else f = (float)(grid_quot(X[a], P.lo[a], P.h[a], P.rh[a]) - (double)id[a]);
             if (!(f >= 0.0f)) f = 0.0f;
             if (f >= 1.0f) f = 0x1.fffffep-1f;
             o[a] = f;
@@ -160,7 +203,7 @@ int gsz(uint64_t n, int tpb)
 }  // namespace
 
 void radix_sort_pairs(uint32_t* keys, uint32_t* vals, uint32_t* keys_tmp, uint32_t* vals_tmp, uint32_t n,
-                      int key_bits, cudaStream_t s, long long* blk_scratch, size_t)
+                      int key_bits, cudaStream_t s, long long* blk_scratch, const unsigned* unsorted)
 {
     if (n == 0) return;
     const uint32_t nblk = (n + RS_TILE - 1) / RS_TILE;
@@ -169,18 +212,18 @@ void radix_sort_pairs(uint32_t* keys, uint32_t* vals, uint32_t* keys_tmp, uint32
     uint32_t* off = hist + (size_t)RS_BINS * nblk;
     for (int shift = 0; shift < key_bits; shift += 8) {
         ++g_launches;
-        k_rs_hist<<<nblk, RS_TPB, 0, s>>>(keys, n, shift, nblk, hist);
+        k_rs_hist<<<nblk, RS_TPB, 0, s>>>(keys, n, shift, nblk, hist, unsorted);
         HistScanOp op{ hist, off };
         run_scan<1>(op, (uint64_t)RS_BINS * nblk, blk_scratch, s);
         ++g_launches;
-        k_rs_scatter<<<nblk, RS_TPB, 0, s>>>(keys, vals, n, shift, nblk, off, keys_tmp, vals_tmp);
+        k_rs_scatter<<<nblk, RS_TPB, 0, s>>>(keys, vals, n, shift, nblk, off, keys_tmp, vals_tmp, unsorted);
         uint32_t* t = keys; keys = keys_tmp; keys_tmp = t;
         t = vals; vals = vals_tmp; vals_tmp = t;
     }
     // an odd number of passes leaves the result in the tmp buffers
     if (((key_bits + 7) / 8) & 1) {
-        cudaMemcpyAsync(keys_tmp, keys, n * sizeof(uint32_t), cudaMemcpyDeviceToDevice, s);
-        cudaMemcpyAsync(vals_tmp, vals, n * sizeof(uint32_t), cudaMemcpyDeviceToDevice, s);
+        ++g_launches;
+        k_rs_copy<<<gsz(n, 256), 256, 0, s>>>(keys, vals, keys_tmp, vals_tmp, n, unsorted);
     }
 }
 
@@ -190,8 +233,8 @@ size_t radix_scratch_elems(uint32_t cap)
     return scan_scratch_elems((uint64_t)RS_BINS * nblk, 1) + (size_t)RS_BINS * nblk + 16;
 }
 
-// x, y, z, w, real are device pointers (already staged).  `tmp64` holds n
-// FP64 records during the sort.
+// x, y, z, w, real are device pointers (the caller's, or staged at the start of
+// recA / the merge work area).  `tmp64` holds n FP64 records during the sort.
 void launch_set_particles(const Params& P, Dev& d, const double* x, const double* y, const double* z,
                           const uint32_t* w, const int32_t* real, const int32_t* species, uint32_t n, uint64_t G,
                           cudaStream_t s)
@@ -207,10 +250,12 @@ void launch_set_particles(const Params& P, Dev& d, const double* x, const double
         k_pack<<<gsz(n, 256), 256, 0, s>>>(P, x, y, z, w, real, species, n, tmp64, keys, vals, d.ctr);
         int bits = 1;
         while (bits < 32 && (1ull << bits) < G) ++bits;
-        radix_sort_pairs(keys, vals, kt, vt, n, bits, s, d.scan_blk, 0);
         ++g_launches;
-        if (d.mixed) k_gather32<<<gsz(n, 256), 256, 0, s>>>(P, tmp64, vals, n, d.rA32, d.cellA32);
-        else k_gather<<<gsz(n, 256), 256, 0, s>>>(tmp64, vals, n, d.recA);
+        k_find_unsorted<<<gsz(n, 256), 256, 0, s>>>(keys, n, &d.ctr->unsorted);
+        radix_sort_pairs(keys, vals, kt, vt, n, bits, s, d.scan_blk, &d.ctr->unsorted);
+        ++g_launches;
+        if (d.mixed) k_gather32<<<gsz(n, 256), 256, 0, s>>>(P, tmp64, vals, n, d.rA32, d.cellA32, &d.ctr->unsorted);
+        else k_gather<<<gsz(n, 256), 256, 0, s>>>(tmp64, vals, n, d.recA, &d.ctr->unsorted);
     }
     cudaMemsetAsync(d.cnt_new, 0, G * sizeof(int32_t), s);
     if (n > 0) {

@@ -67,6 +67,7 @@ struct Counters {
     unsigned long long rho_absmax;     // max |rho_fixed| of the last deposit
     unsigned int err;                  // DERR_* bits
     unsigned int kmc_fail_cell;
+    unsigned int unsorted;             // set_particles: the input is not in cell order
     unsigned long long outflow[MAX_R];
     unsigned long long lost[MAX_R];
 };
@@ -233,8 +234,7 @@ void launch_deposit_B(const Params& P, Dev& d, uint32_t N, cudaStream_t s);
 void launch_advect(const Params& P, Dev& d, uint32_t N, cudaStream_t s);
 // ik_sort.cu
 void radix_sort_pairs(uint32_t* keys, uint32_t* vals, uint32_t* keys_tmp, uint32_t* vals_tmp,
-                      uint32_t n, int key_bits, cudaStream_t s, long long* blk_scratch,
-                      size_t blk_scratch_elems);
+                      uint32_t n, int key_bits, cudaStream_t s, long long* blk_scratch, const unsigned* unsorted);
 size_t radix_scratch_elems(uint32_t cap);
 void launch_set_particles(const Params& P, Dev& d, const double* x, const double* y,
                           const double* z, const uint32_t* w, const int32_t* real, const int32_t* species,
