@@ -87,6 +87,14 @@ __device__ __forceinline__ double u53(uint64_t k)
     return __longlong_as_double((long long)bits);
 }
 
+// m 2^-53 for m < 2^53, exact.
+__device__ __forceinline__ double u53_mul(uint64_t m)
+{
+    if (m == 0) return 0.0;
+    const int p = 63 - __clzll((long long)m);
+    return __longlong_as_double((long long)(((uint64_t)(p - 53 + 1023) << 52) | ((m << (52 - p)) & 0x000fffffffffffffull)));
+}
+
 struct Stream {
     uint32_t k0, k1, c0, c1, c2, blk;
     u32x4 buf;
@@ -107,12 +115,12 @@ struct Stream {
         return v;
     }
     // uniform on (0,1): k = 52 random bits, (2k+1) 2^-53 (exact)
-    __device__ __forceinline__ double uniform()
+    __device__ __forceinline__ double uniform() { return u53(bits52()); }
+    __device__ __forceinline__ uint64_t bits52()
     {
         const uint32_t a = u32();
         const uint32_t b = u32();
-        const uint64_t k = ((uint64_t)a << 20) | (uint64_t)(b >> 12);
-        return u53(k);
+        return ((uint64_t)a << 20) | (uint64_t)(b >> 12);
     }
 };
 
@@ -291,50 +299,196 @@ __device__ __forceinline__ double dlogfact(int64_t k)
     return (((x + 0.5) * dlog(x) - x) + 0.91893853320467274178) + ser;
 }
 
+// ---- pairs of floats: a value hi + lo to about 2^-44
+// The Poisson draws are whole numbers: FP64 arithmetic only decides floors and
+// comparisons.  These pairs decide the same ones outside a margin that covers
+// their error many times over, with FP32 instructions (GB300 issues 64 of them
+// in the time of one FP64 instruction); inside the margin FP64 decides (5e-5 of
+// the trials, 2e-3 of the logarithmic tests).  k_kmc over a channel with
+// recombination on 128^3 is bound by that pipe: 857 us with FP64 draws, 224 us
+// with these (6.26 million FP64 warp instructions to 2.74 million).
+struct FF { float h, l; };
+__device__ __forceinline__ FF ff_norm(float h, float l)            // |h| >= |l|
+{
+    const float s = h + l;
+    return FF{ s, l - (s - h) };
+}
+__device__ __forceinline__ FF ff_add(FF a, FF b)
+{
+    const float s = a.h + b.h, t = s - a.h, e = (a.h - (s - t)) + (b.h - t);
+    return ff_norm(s, e + (a.l + b.l));
+}
+__device__ __forceinline__ FF ff_mul(FF a, FF b)
+{
+    const float p = a.h * b.h, e = __fmaf_rn(a.h, b.h, -p);
+    return ff_norm(p, __fmaf_rn(a.h, b.l, __fmaf_rn(a.l, b.h, e)));
+}
+__device__ __forceinline__ FF ff_div(FF a, FF b)
+{
+    const float q = __fdividef(a.h, b.h);
+    const float r = __fmaf_rn(-q, b.h, a.h) + __fmaf_rn(-q, b.l, a.l);      // a - q b
+    return ff_norm(q, __fdividef(r, b.h));
+}
+// The constant c to 48 bits.
+#define IK_FF(c) (FF{ (float)(c), (float)((c) - (double)(float)(c)) })
+// m 2^-53 for m < 2^53.
+__device__ __forceinline__ FF ff_frac53(uint64_t m)
+{
+    const float h = (float)(uint32_t)(m >> 29), l = (float)(uint32_t)(m & 0x1fffffffu);   // 24 and 29 bits
+    return ff_norm(h * 0x1p-24f, l * 0x1p-53f);
+}
+// The same for small m: its own leading bits.
+__device__ __forceinline__ FF ff_small53(uint64_t m)
+{
+    const int z = __clzll((long long)m) - 11;                      // m > 0
+    const FF f = ff_frac53(m << z);
+    const float sc = __int_as_float((127 - z) << 23);
+    return FF{ f.h * sc, f.l * sc };
+}
+// A positive double in float's range.
+__device__ __forceinline__ FF ff_from(double v)
+{
+    const uint64_t b = (uint64_t)__double_as_longlong(v);
+    const int e = (int)(b >> 52) - 1023;
+    const uint64_t m = (b & 0xfffffffffffffull) | (1ull << 52);
+    const FF f = ff_frac53(m);                                     // v 2^-(e + 1)
+    const float sc = __int_as_float((e + 128) << 23);
+    return FF{ f.h * sc, f.l * sc };
+}
+
+// One PTRS acceptance test by logarithms, in FP64 (the specification).
+static __device__ __noinline__ bool ptrs_log_test(double mu, double kd, double us, double V)
+{
+    const double b = 0.931 + 2.53 * sqrt(mu);
+    const double a = -0.059 + 0.02483 * b;
+    const double invalpha = 1.1239 + 1.1328 / (b - 3.4);
+    // the acceptance test as one logarithm (Hoermann's form)
+    const double lhs = dlog((V * invalpha) / ((a / (us * us)) + b));
+    const double rhs = ((-mu) + kd * dlog(mu)) - dlogfact((int64_t)kd);
+    return lhs <= rhs;
+}
+// The trial's count and its test against vr, in FP64.
+static __device__ __noinline__ double ptrs_trial(double mu, double U, double us, double V, bool& below_vr)
+{
+    const double b = 0.931 + 2.53 * sqrt(mu);
+    const double a = -0.059 + 0.02483 * b;
+    below_vr = V <= 0.9277 - 3.6224 / (b - 2.0);
+    return floor(((((2.0 * a) / us) + b) * U + mu) + 0.43);
+}
+// Inversion by sequential search, in FP64.
+static __device__ __noinline__ int64_t poisson_search(double mu, double u)
+{
+    double p = dexp(-mu);
+    double F = p;
+    int64_t k = 0;
+    while (u > F && k < 200) {
+        k += 1;
+        p = (p * mu) / (double)k;
+        F = F + p;
+    }
+    return k;
+}
+
 // P(mu): 0 without a draw for mu <= 0; inversion by sequential search (one
 // uniform) for mu < 10; PTRS transformed rejection (Hoermann 1993, two
 // uniforms per trial) above.  Returns -1 if PTRS exhausts its trial limit.
-static __device__ __noinline__ int64_t dpoisson(Stream& s, double mu)
+__device__ __forceinline__ int64_t dpoisson_inl(Stream& s, double mu)
 {
     if (!(mu > 0.0)) return 0;
-    if (mu < 10.0) {
-        const double u = s.uniform();
-        double p = dexp(-mu);
-        double F = p;
-        int64_t k = 0;
-        while (u > F && k < 200) {
-            k += 1;
-            p = (p * mu) / (double)k;
-            F = F + p;
+    const bool small = mu < 10.0;
+    // the pairs serve means up to 2^24; a search whose first term would leave
+    // float's range does not occur (exp(-10) = 4.5e-5), a mean near 0 does
+    const bool pairs = mu < 0x1p24 && mu > 0x1p-60;
+    const FF m = ff_from(pairs ? mu : 1.0);
+    if (small) {
+        const uint32_t a = s.u32(), c = s.u32();
+        const uint64_t ku = ((uint64_t)a << 20) | (uint64_t)(c >> 12);
+        if (pairs) {
+            // errors below 1e-5: expf and p to 1e-6 relative over the few steps
+            const float u = ff_frac53(2 * ku + 1).h, mf = m.h;
+            float p = expf(-mf), F = p;
+            int k = 0;
+            bool clear = fabsf(u - F) > 1e-5f;
+            while (clear && u > F && k < 100) {
+                k += 1;
+                p = __fdividef(p * mf, (float)k);
+                F += p;
+                clear = fabsf(u - F) > 1e-5f;
+            }
+            if (clear && k < 100) return k;
         }
-        return k;
+        return poisson_search(mu, u53(ku));
     }
-    const double slam = sqrt(mu);
-    const double b = 0.931 + 2.53 * slam;
-    const double a = -0.059 + 0.02483 * b;
-    const double vr = 0.9277 - 3.6224 / (b - 2.0);
-    // ln(mu) and 1/alpha serve only the slow test: formed on first use (the
-    // same values, so the draws are unchanged)
-    double loglam = 0.0, invalpha = 0.0;
-    bool slow_ready = false;
+    // b, a and vr of the transformed rejection
+    const float r0 = sqrtf(m.h), rl = __fdividef(__fmaf_rn(-r0, r0, m.h) + m.l, r0 + r0);
+    const FF b = ff_add(IK_FF(0.931), ff_mul(IK_FF(2.53), ff_norm(r0, rl)));
+    const FF a = ff_add(IK_FF(-0.059), ff_mul(IK_FF(0.02483), b));
+    const float vr = 0.9277f - __fdividef(3.6224f, b.h - 2.0f);
+    const float invalpha = 1.1239f + __fdividef(1.1328f, b.h - 3.4f);
     for (int it = 0; it < 1000000; ++it) {
-        const double U = s.uniform() - 0.5;
-        const double V = s.uniform();
-        const double us = 0.5 - fabs(U);
-        const double kd = floor(((((2.0 * a) / us) + b) * U + mu) + 0.43);
-        if (us >= 0.07 && V <= vr) return (int64_t)kd;
-        if (kd < 0.0 || (us < 0.013 && V > us)) continue;
-        if (!slow_ready) {
-            loglam = dlog(mu);
-            invalpha = 1.1239 + 1.1328 / (b - 3.4);
-            slow_ready = true;
+        const uint32_t w0 = s.u32(), w1 = s.u32(), w2 = s.u32(), w3 = s.u32();
+        const uint64_t ku = 2ull * (((uint64_t)w0 << 20) | (uint64_t)(w1 >> 12)) + 1ull;
+        const uint64_t kv = 2ull * (((uint64_t)w2 << 20) | (uint64_t)(w3 >> 12)) + 1ull;
+        // U = ku 2^-53 - 1/2, us = 1/2 - |U| and V = kv 2^-53 are exact: so are
+        // the comparisons among them
+        const bool neg = ku < (1ull << 52);
+        const uint64_t au = neg ? (1ull << 52) - ku : ku - (1ull << 52), kus = (1ull << 52) - au;
+        const FF us = ff_small53(kus), Uabs = ff_frac53(au);
+        const FF U = neg ? FF{ -Uabs.h, -Uabs.l } : Uabs;
+        double kd = 0.0;
+        int64_t kk = 0;
+        bool below_vr = false, known = false;
+        if (pairs) {
+            const FF q = ff_div(FF{ 2.0f * a.h, 2.0f * a.l }, us);
+            const FF v = ff_add(ff_add(ff_mul(ff_add(q, b), U), m), IK_FF(0.43));
+            const float fh = floorf(v.h), fr = (v.h - fh) + v.l, fl = floorf(fr), at = fr - fl;
+            const float slack = 1e-5f + (m.h + fabsf(v.h)) * 0x1p-38f, dv = ff_frac53(kv).h - vr;
+            known = at > slack && at < 1.0f - slack && fabsf(dv) > 1e-5f && fabsf(v.h) < 0x1p30f;
+            kk = (int64_t)(int)fh + (int)fl;
+            below_vr = dv < 0.0f;
         }
-        // the acceptance test as one logarithm (Hoermann's form)
-        const double lhs = dlog((V * invalpha) / ((a / (us * us)) + b));
-        const double rhs = ((-mu) + kd * loglam) - dlogfact((int64_t)kd);
-        if (lhs <= rhs) return (int64_t)kd;
+        if (!known) {
+            kd = ptrs_trial(mu, neg ? -u53_mul(au) : u53_mul(au), u53_mul(kus), u53_mul(kv), below_vr);
+            kk = (int64_t)kd;
+        }
+        if (kus >= 630503947831870ull && below_vr) return kk;             // us >= 0.07
+        const bool negk = known ? kk < 0 : kd < 0.0;
+        if (negk || (kus < 117093590311633ull && kv > kus)) continue;     // us < 0.013
+        if (known && kk >= 4 && us.h > 1e-9f) {
+            // k ln mu - mu - ln k! = -(k h(x) + ln(2 pi k) / 2 + 1 / 12 k - 1 / 360 k^3 + ...)
+            // with x = (mu - k) / k, h(x) = x - ln(1 + x): errors below 1e-4
+            const float kf = (float)kk, d = (m.h - kf) + (m.l - (float)(kk - (int64_t)kf));
+            const float x = __fdividef(d, kf);
+            const float h = fabsf(x) < 0.05f
+                                ? x * x * (0.5f + x * (-1.0f / 3.0f + x * (0.25f + x * (-0.2f + x * (1.0f / 6.0f + x * (-1.0f / 7.0f))))))
+                                : x - log1pf(x);
+            const float rk = __fdividef(1.0f, kf);
+            const float rhs = -(kf * h) - 0.5f * logf(6.2831853f * kf) - rk * (1.0f / 12.0f - rk * rk * (1.0f / 360.0f));
+            const float lhs = logf(__fdividef(ff_frac53(kv).h * invalpha, __fdividef(a.h, us.h * us.h) + b.h));
+            const float gap = rhs - lhs;
+            // kf h carries the relative errors of d and of the logarithm
+            if (fabsf(gap) > 1e-3f + kf * h * 1e-4f) {
+                if (gap > 0.0f) return kk;
+                continue;
+            }
+        }
+        if (ptrs_log_test(mu, known ? (double)kk : kd, u53_mul(kus), u53_mul(kv))) return kk;
     }
     return -1;
+}
+static __device__ __noinline__ int64_t dpoisson(Stream& s, double mu) { return dpoisson_inl(s, mu); }
+
+// An exponential time -ln(u) / A, u the uniform of the bits k; infinity where
+// it lies above the limit for certain (the caller does nothing else with such
+// a time), which FP32 decides for most draws.  logf and the rounding of u
+// to 24 bits are off by less than 2e-7 (1 + l).
+static __device__ __noinline__ double exp_time_exact(uint64_t k, double A) { return (-dlog(u53(k))) / A; }
+__device__ __forceinline__ double exp_time(Stream& s, double A, double limit)
+{
+    const uint64_t k = s.bits52();
+    const float l = -logf(ff_frac53(2 * k + 1).h);
+    if (l - 1e-5f * (1.0f + l) > (float)(A * limit) * 1.00001f) return __longlong_as_double(0x7ff0000000000000ll);
+    return exp_time_exact(k, A);
 }
 
 // ---------------------------------------------------------------- grid

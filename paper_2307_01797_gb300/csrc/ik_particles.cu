@@ -823,9 +823,9 @@ __global__ void k_rho(Params P, const int64_t* __restrict__ Npos, const int64_t*
 template <class T> struct KT;
 template <> struct KT<double> {
     static __device__ __forceinline__ double uni(Stream& s) { return s.uniform(); }
-    static __device__ __forceinline__ double lg(double x) { return dlog(x); }
+    static __device__ __forceinline__ double after(Stream& s, double A, double limit) { return exp_time(s, A, limit); }
     static __device__ __forceinline__ double inf() { return __longlong_as_double(0x7ff0000000000000ll); }
-    static __device__ __forceinline__ long long poisson(Stream& s, double mu) { return dpoisson(s, mu); }
+    static __device__ __forceinline__ long long poisson(Stream& s, double mu) { return dpoisson_inl(s, mu); }
 };
 template <> struct KT<float> {
     static __device__ __forceinline__ float uni(Stream& s)
@@ -834,7 +834,7 @@ template <> struct KT<float> {
         (void)s.u32();
         return uniform_f32(a);
     }
-    static __device__ __forceinline__ float lg(float x) { return logf(x); }
+    static __device__ __forceinline__ float after(Stream& s, float A, float) { return (-logf(uni(s))) / A; }
     static __device__ __forceinline__ float inf() { return __int_as_float(0x7f800000); }
     static __device__ long long poisson(Stream& s, float mu);
 };
@@ -990,7 +990,8 @@ __device__ int kmc_cell(const Params& P, Stream& s, const long long X0[3], const
                     kmc_props<T, REC>(kr, Xs, as);
                     const T As = kmc_total<T, REC>(as);
                     if (!(As > (T)0)) { t = dtau; break; }
-                    const T dte = (-K::lg(K::uni(s))) / As;
+                    // 1e-9 dtau covers the rounding of t + dte
+                    const T dte = K::after(s, As, (dtau - t) + (T)1e-9 * dtau);
                     if (t + dte > dtau) { t = dtau; break; }
                     t = t + dte;
                     const T target = K::uni(s) * As;
@@ -1011,7 +1012,7 @@ __device__ int kmc_cell(const Params& P, Stream& s, const long long X0[3], const
                 }
                 adv = t;
             } else {
-                if (dtc < (T)0) dtc = (Ac > (T)0) ? (-K::lg(K::uni(s))) / Ac : K::inf();
+                if (dtc < (T)0) dtc = (Ac > (T)0) ? K::after(s, Ac, rem) : K::inf();
                 if (dtc < dtnc && dtc < rem) {
                     dtau = dtc;
                     const T target = K::uni(s) * Ac;
@@ -1028,13 +1029,23 @@ __device__ int kmc_cell(const Params& P, Stream& s, const long long X0[3], const
 #pragma unroll
                     for (int r = 0; r < NR; ++r) k[r] += (rc == r);
                 }
-#pragma unroll
+                // one copy of the sampler (its code is long): the reactions' values
+                // are selected in a loop that stays one
+                bool failed = false;
+#pragma unroll 1
                 for (int r = 0; r < NR; ++r) {
-                    if (crit[r]) continue;
-                    const long long kk = K::poisson(s, a[r] * dtau);
-                    if (kk < 0) return -1;
-                    k[r] += kk;
+                    T ar = a[0];
+                    bool cr = crit[0];
+#pragma unroll
+                    for (int q = 1; q < NR; ++q)
+                        if (r == q) { ar = a[q]; cr = crit[q]; }
+                    if (cr) continue;
+                    const long long kk = K::poisson(s, ar * dtau);
+                    failed |= kk < 0;
+#pragma unroll
+                    for (int q = 0; q < NR; ++q) k[q] += r == q ? kk : 0;
                 }
+                if (failed) return -1;
                 adv = dtau;
             }
             const long long Xn0 = X[0] + k[0] - k[1] - k[3];
