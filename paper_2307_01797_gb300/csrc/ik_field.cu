@@ -143,6 +143,7 @@ struct Inv {
     T v;
     __device__ __forceinline__ Inv() {}
     __device__ __forceinline__ explicit Inv(int d) : v(inv_diag<T>(d)) {}
+    static __device__ __forceinline__ Inv zero() { Inv i; i.v = (T)0; return i; }
     __device__ __forceinline__ T relax(T sum, T rhs) const { return (sum - rhs) * v; }
 };
 template <>
@@ -150,6 +151,7 @@ struct Inv<long long> {
     int mh, ml;
     __device__ __forceinline__ Inv() {}
     __device__ __forceinline__ explicit Inv(int d) { MG<long long>::magic(d, mh, ml); }
+    static __device__ __forceinline__ Inv zero() { Inv i; i.mh = i.ml = 0; return i; }
     __device__ __forceinline__ long long relax(long long sum, long long rhs) const
     {
         return MG<long long>::mul(sum - rhs + 3, mh, ml);
@@ -308,6 +310,60 @@ __global__ void __launch_bounds__(256) k_prolong(T* __restrict__ phi_f, const T*
 #pragma unroll
             for (int x = 0; x < 2; ++x) v.v[x] += MG<T>::div64(MG<T>::axpy3(m[0][y][x], neg ? -m[1][y][x] : m[1][y][x]));
             *p = v;
+        }
+    }
+}
+
+// The same with kp fine planes per thread, from the bottom up: a coarse plane's
+// interpolation is formed once for the two fine planes on either side.
+template <class T>
+__global__ void __launch_bounds__(256) k_prolong_march(T* __restrict__ phi_f, const T* __restrict__ e_c, Geo Gf, int kp)
+{
+    const int n = Gf.n, nc = n / 2, lc = Gf.log2n - 1;
+    const uint64_t t = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x;
+    const int I = (int)(t & (uint64_t)(nc - 1)), J = (int)((t >> lc) & (uint64_t)(nc - 1));
+    const uint64_t z = (t >> (2 * lc)) * (uint64_t)kp, r = z >> Gf.log2n;      // first plane over all realizations
+    if (z >= Gf.cells >> (2 * Gf.log2n)) return;
+    const int k0 = (int)(z & (uint64_t)(n - 1));
+    const int il = I > 0 ? -1 : 0, ir = I < nc - 1 ? 1 : 0;
+    const int64_t jl = J > 0 ? -nc : 0, jr = J < nc - 1 ? nc : 0;
+    struct M { T v[2][2]; };                       // in-plane interpolation: [fine row][cell]
+    auto plane = [&](int K, M& m) {                // ghosts beyond the electrodes: the outermost plane, negated
+        const bool neg = K < 0 || K >= nc;
+        const int Kc = K < 0 ? 0 : (K >= nc ? nc - 1 : K);
+        const T *r0 = e_c + ((r * nc + Kc) * (uint64_t)nc + J) * (uint64_t)nc + I, *rl = r0 + jl, *rr = r0 + jr;
+        const T a = r0[0], al = r0[il], ar = r0[ir];
+        const T b = rl[0], bl = rl[il], br = rl[ir];
+        const T d = rr[0], dl = rr[il], dr = rr[ir];
+        const T q0 = MG<T>::axpy3(a, al), q1 = MG<T>::axpy3(a, ar);
+        m.v[0][0] = MG<T>::axpy3(q0, MG<T>::axpy3(b, bl));
+        m.v[0][1] = MG<T>::axpy3(q1, MG<T>::axpy3(b, br));
+        m.v[1][0] = MG<T>::axpy3(q0, MG<T>::axpy3(d, dl));
+        m.v[1][1] = MG<T>::axpy3(q1, MG<T>::axpy3(d, dr));
+        if (neg)
+#pragma unroll
+            for (int q = 0; q < 4; ++q) m.v[q >> 1][q & 1] = -m.v[q >> 1][q & 1];
+    };
+    T* f = phi_f + (z * (uint64_t)n + 2 * J) * (uint64_t)n + 2 * I;
+    M own, oth;                                    // plane k's coarse plane and the one beside it
+    plane(k0 >> 1, own);
+    plane((k0 >> 1) + ((k0 & 1) ? 1 : -1), oth);
+    for (int k = k0;; ++k, f += (int64_t)n * n) {
+#pragma unroll
+        for (int y = 0; y < 2; ++y) {
+            Pair<T>* p = reinterpret_cast<Pair<T>*>(f + y * n);
+            Pair<T> v = *p;
+#pragma unroll
+            for (int x = 0; x < 2; ++x) v.v[x] += MG<T>::div64(MG<T>::axpy3(own.v[y][x], oth.v[y][x]));
+            *p = v;
+        }
+        if (k + 1 == k0 + kp) break;
+        if (k & 1) {
+            const M m = own;
+            own = oth;
+            oth = m;
+        } else {
+            plane((k >> 1) + 1, oth);
         }
     }
 }
@@ -1180,13 +1236,15 @@ __global__ void __cluster_dims__(COARSE_CL, 1, 1) __launch_bounds__(COARSE_TPB)
 // of place (dst must not be src): neighbouring blocks read the halo's old
 // values.  src == nullptr: a zero initial guess.  Every cell gets the
 // operations of four plain half-sweeps in their order, so the result is the
-// same to the last bit.  Two sweeps of 256^3 cells: 202 us in fixed point (66%
-// issue utilisation: bound by its integer instructions, 1.9 TB/s of DRAM)
-// against 508 us for four FP64 half-sweeps (FP64 pipe 82% busy).
+// same to the last bit.  Cells outside the domain relax like the others, with
+// a divisor of zero: no branch per cell (FP32 at 512^3 564 -> 521 us, fixed
+// point at 256^3 202 -> 180 us).  Two sweeps of 256^3 cells: 180 us in fixed
+// point (bound by its integer instructions) against 508 us for four FP64
+// half-sweeps (FP64 pipe 82% busy).
 //
 // The tile: 64 x 32 in FP32 (two pairs per thread), 32 x 32 in 64 bits.  A
 // 64^3 level has too few of these for the chip's SMs: 32 x 16 there, with one
-// pair per thread (17.9 -> 12.9 us in fixed point, 16.0 -> 10.6 us in FP32: a
+// pair per thread (17.9 -> 12.2 us in fixed point, 16.0 -> 10.4 us in FP32: a
 // step takes as long as its warps need to issue).
 template <class T, int TX_, int TY_, int PP_>
 struct SweepTile {
@@ -1195,47 +1253,45 @@ struct SweepTile {
     static constexpr int PP = PP_, NT = PX * EY / PP, RING = 5;
     static constexpr int GUARD = PX + 1;           // elements before and after the ring that rim pairs read
     static constexpr size_t SMEM = sizeof(T) * (RING * EX * EY + 2 * GUARD);
-    static_assert(PX * EY == PP * NT, "whole pairs per thread");
+    static_assert(PX * EY == PP * NT && NT % PX == 0 && (PP == 1 || EY / PP % 2 == 0), "whole pairs per thread, rows of one parity");
 };
 
 template <class T, class Q>
 __global__ void __launch_bounds__(Q::NT, 1)
     k_sweep4(const T* __restrict__ src, const T* __restrict__ rhs, T* __restrict__ dst, int n, int c0, int zc)
 {
-    constexpr int H = Q::H, PP = Q::PP, PX = Q::PX, EY = Q::EY, PLH = PX * EY;   // PLH: the cells of one colour
+    constexpr int H = Q::H, PP = Q::PP, PX = Q::PX, EY = Q::EY, DY = EY / PP, PLH = PX * EY;   // PLH: the cells of one colour
     extern __shared__ __align__(16) unsigned char ssm[];
     T* ring = reinterpret_cast<T*>(ssm) + Q::GUARD;
     const int tiles_x = n / Q::TX;
     const int x0 = (int)(blockIdx.x % tiles_x) * Q::TX - H, y0 = (int)(blockIdx.x / tiles_x) * Q::TY - H;
     const int z0 = (int)blockIdx.y * zc, z1 = z0 + zc;
     const int64_t nn = (int64_t)n * n;
+    // a thread's pairs lie DY rows apart (an even number): one x, one parity
+    const int px = (int)threadIdx.x % PX, ey0 = (int)threadIdx.x / PX, gi = x0 + 2 * px, gj0 = y0 + ey0;
+    const unsigned odd = (unsigned)(gj0 + c0);
+    const int off0 = gj0 * n + gi;
     bool in[PP], tile[PP];                         // inside the domain; inside the block's own column
-    int d0[PP], d1[PP];                            // in-plane diagonal counts of the even and the odd cell
-    unsigned odd[PP];                              // y + c0
-    Inv<T> i0[PP], i1[PP];
-    int64_t off[PP];
+    Inv<T> i0[PP], i1[PP];                         // of the even and the odd cell; outside the domain zero: cells stay zero
+    auto diag = [&](int m, int x) { return 6 - (gj0 + m * DY == 0) - (gj0 + m * DY == n - 1) - (x ? gi + 2 == n : gi == 0); };
 #pragma unroll
     for (int m = 0; m < PP; ++m) {
-        const int q = threadIdx.x + m * Q::NT;
-        const int ey = q / PX, px = q - ey * PX, gi = x0 + 2 * px, gj = y0 + ey;
+        const int ey = ey0 + m * DY, gj = gj0 + m * DY;
         in[m] = gi >= 0 && gi < n && gj >= 0 && gj < n;       // pairs lie wholly inside or outside
         tile[m] = px >= H / 2 && px < PX - H / 2 && ey >= H && ey < EY - H;
-        const int dy = 6 - (gj == 0) - (gj == n - 1);
-        d0[m] = dy - (gi == 0);
-        d1[m] = dy - (gi + 2 == n);
-        i0[m] = Inv<T>(d0[m]);
-        i1[m] = Inv<T>(d1[m]);
-        odd[m] = (unsigned)(gj + c0);
-        off[m] = (int64_t)blockIdx.z * nn * n + (int64_t)gj * n + gi;
+        i0[m] = in[m] ? Inv<T>(diag(m, 0)) : Inv<T>::zero();
+        i1[m] = in[m] ? Inv<T>(diag(m, 1)) : Inv<T>::zero();
     }
     // in step t: v[K] and r[K - 1] are plane t - K's values and right-hand
     // side, colour A in .v[0], colour B in .v[1]
     Pair<T> v[H + 2][PP], r[H][PP], nv[PP], nr[PP];
+    auto plane_of = [&](int p) { return ((int64_t)blockIdx.z * n + p) * nn; };
     auto fetch = [&](const T* __restrict__ a, int p, Pair<T>* to) {
+        const T* pl = a + plane_of(p);
 #pragma unroll
         for (int m = 0; m < PP; ++m) {
             to[m].v[0] = to[m].v[1] = (T)0;
-            if (in[m] && p >= 0 && p < n) to[m] = *reinterpret_cast<const Pair<T>*>(a + off[m] + (int64_t)p * nn);
+            if (in[m] && p >= 0 && p < n) to[m] = *reinterpret_cast<const Pair<T>*>(pl + (off0 + m * DY * n));
         }
     };
 #pragma unroll
@@ -1252,16 +1308,16 @@ __global__ void __launch_bounds__(Q::NT, 1)
     // domain face (else no plane needs a look)
     auto step = [&](auto edge, int t) {
         constexpr bool EDGE = decltype(edge)::value;
-        bool par[PP];
+        const bool par = (odd + (unsigned)t + 1u) & 1u;
+        const int xo = par ? 1 : -1;
         Inv<T> ic[PP];
 #pragma unroll
         for (int m = 0; m < PP; ++m) {
-            par[m] = (odd[m] + (unsigned)t + 1u) & 1u;
-            ic[m] = par[m] ? i1[m] : i0[m];
+            ic[m] = par ? i1[m] : i0[m];
             T* c = ring + s * (2 * PLH) + threadIdx.x + m * Q::NT;
             if (src) {
-                v[0][m].v[0] = par[m] ? nv[m].v[0] : nv[m].v[1];
-                v[0][m].v[1] = par[m] ? nv[m].v[1] : nv[m].v[0];
+                v[0][m].v[0] = par ? nv[m].v[0] : nv[m].v[1];
+                v[0][m].v[1] = par ? nv[m].v[1] : nv[m].v[0];
             }
             c[0] = v[0][m].v[0];
             c[PLH] = v[0][m].v[1];
@@ -1277,23 +1333,21 @@ __global__ void __launch_bounds__(Q::NT, 1)
             T* plane = ring + (s >= K ? s - K : s + Q::RING - K) * (2 * PLH) + threadIdx.x;
 #pragma unroll
             for (int m = 0; m < PP; ++m) {
-                if (!in[m]) continue;                         // cells outside the domain stay zero
                 const T* oth = plane + o * PLH + m * Q::NT;
-                T sum = v[K][m].v[o] + oth[par[m] ? 1 : -1];
+                T sum = v[K][m].v[o] + oth[xo];
                 sum += oth[-PX];
                 sum += oth[PX];
                 sum += v[K + 1][m].v[o];
                 sum += v[K - 1][m].v[o];
-                T w;
-                if (EDGE && dz) w = Inv<T>((par[m] ? d1[m] : d0[m]) + dz).relax(sum, r[K - 1][m].v[c]);
-                else w = ic[m].relax(sum, r[K - 1][m].v[c]);
+                T w = ic[m].relax(sum, r[K - 1][m].v[c]);
+                if (EDGE && dz && in[m]) w = Inv<T>(diag(m, par) + dz).relax(sum, r[K - 1][m].v[c]);
                 v[K][m].v[c] = w;
                 if (K < H) plane[c * PLH + m * Q::NT] = w;
                 if (K == H && tile[m]) {
                     Pair<T> q;
-                    q.v[0] = par[m] ? v[H][m].v[0] : w;
-                    q.v[1] = par[m] ? w : v[H][m].v[0];
-                    *reinterpret_cast<Pair<T>*>(dst + off[m] + (int64_t)p * nn) = q;
+                    q.v[0] = par ? v[H][m].v[0] : w;
+                    q.v[1] = par ? w : v[H][m].v[0];
+                    *reinterpret_cast<Pair<T>*>(dst + plane_of(p) + (off0 + m * DY * n)) = q;
                 }
             }
         }
@@ -1304,8 +1358,8 @@ __global__ void __launch_bounds__(Q::NT, 1)
             for (int K = H + 1; K > 0; --K) v[K][m] = v[K - 1][m];
 #pragma unroll
             for (int K = H - 1; K > 0; --K) r[K][m] = r[K - 1][m];
-            r[0][m].v[0] = par[m] ? nr[m].v[0] : nr[m].v[1];
-            r[0][m].v[1] = par[m] ? nr[m].v[1] : nr[m].v[0];
+            r[0][m].v[0] = par ? nr[m].v[0] : nr[m].v[1];
+            r[0][m].v[1] = par ? nr[m].v[1] : nr[m].v[0];
         }
         s = s + 1 == Q::RING ? 0 : s + 1;
     };
@@ -1381,6 +1435,24 @@ void launch_sweep4(const T* src, const T* rhs, T* dst, const Geo& G, int c0, cud
     else launch_sweep4_tile<T, SweepTile<T, TX, 32, TX / 32>>(src, rhs, dst, G, c0, s);
 }
 
+// FP32 grids of 2^25 cells and more march over eight planes (512^3: 235 us
+// against 300 us, 16 x 128^3: 61 against 76); at 2^24 cells both take 33 us,
+// smaller ones want the threads (64^3: 4.5 us against 5.6), and 64-bit values
+// the registers (256^3 in fixed point: 50 us against 59).
+template <class T>
+void launch_prolong(T* phi, const T* ec, const Geo& G, cudaStream_t s)
+{
+    ++g_launches;
+    if constexpr (sizeof(T) == 4) {
+        if (G.cells >= (1u << 25)) {
+            constexpr int kp = 8;
+            k_prolong_march<T><<<(unsigned)((G.cells / (4 * kp) + 255) / 256), 256, 0, s>>>(phi, ec, G, kp);
+            return;
+        }
+    }
+    k_prolong<T><<<gridsz(G.cells / 4, 256), 256, 0, s>>>(phi, ec, G);
+}
+
 // One V-cycle from level l; zero: the level's potential counts as zero (it is
 // not read).  Levels of 64^3 and more take two sweeps per pass, between the
 // level's two arrays; an odd sweep runs as two plain half-sweeps in place.
@@ -1421,8 +1493,7 @@ void vcycle(Dev& d, int l, int R, int nu1, int nu2, cudaStream_t s, bool zero)
     ++g_launches;
     k_resid_restrict<T><<<gridsz(Gc.cells, tpb), tpb, 0, s>>>(cur, rhs, lrhs<T>(C), Gc, G.n);
     vcycle<T>(d, l + 1, R, nu1, nu2, s, true);
-    ++g_launches;
-    k_prolong<T><<<gridsz(G.cells / 4, tpb), tpb, 0, s>>>(cur, lphi<T>(C), G);
+    launch_prolong<T>(cur, lphi<T>(C), G, s);
     sweeps(nu2, 1);
     if (cur != phi) cudaMemcpyAsync(phi, cur, G.cells * sizeof(T), cudaMemcpyDeviceToDevice, s);
 }
@@ -2124,11 +2195,11 @@ static void vcycle_vc(const Dev& d, int l, int R, int nu1, int nu2, cudaStream_t
     };
     for (int it = 0; it < nu1; ++it) { sweep(0); sweep(1); }
     const Geo Gc = geo(d, l + 1, R);
-    g_launches += 2;
+    ++g_launches;
     k_resid_restrict_vc<<<gridsz(Gc.cells, tpb), tpb, 0, s>>>(phi, rhs, A, d.lev[l + 1].rhs, Gc, G.n);
     cudaMemsetAsync(d.lev[l + 1].phi, 0, Gc.cells * sizeof(double), s);
     vcycle_vc(d, l + 1, R, nu1, nu2, s);
-    k_prolong<double><<<gridsz(G.cells / 4, tpb), tpb, 0, s>>>(phi, d.lev[l + 1].phi, G);
+    launch_prolong<double>(phi, d.lev[l + 1].phi, G, s);
     for (int it = 0; it < nu2; ++it) { sweep(1); sweep(0); }
 }
 
