@@ -247,7 +247,7 @@ __global__ void __launch_bounds__(256) k_resid_restrict(const T* __restrict__ ph
 // weights 3/4, 1/4 per axis written as (3 a + b) / 4 with fused multiply-
 // adds (ghosts: Neumann e, Dirichlet -e, i.e. (3 a - a) / 4 in z).
 template <class T>
-__device__ __forceinline__ T prolong_at(const T* __restrict__ ec, int nc, int i, int j, int k, int z0 = 0)
+__device__ __forceinline__ T prolong_at(const T* __restrict__ ec, int nc, int i, int j, int k)
 {
     const int I = i >> 1, J = j >> 1, K = k >> 1;
     int I2 = I + ((i & 1) ? 1 : -1), J2 = J + ((j & 1) ? 1 : -1), K2 = K + ((k & 1) ? 1 : -1);
@@ -255,7 +255,7 @@ __device__ __forceinline__ T prolong_at(const T* __restrict__ ec, int nc, int i,
     if (I2 < 0 || I2 >= nc) I2 = I;
     if (J2 < 0 || J2 >= nc) J2 = J;
     if (K2 < 0 || K2 >= nc) { K2 = K; sz = (T)-1; }
-    const int iz[2] = { K - z0, K2 - z0 }, iy[2] = { J, J2 };
+    const int iz[2] = { K, K2 }, iy[2] = { J, J2 };
     T m[2];
 #pragma unroll
     for (int c = 0; c < 2; ++c) {
@@ -862,8 +862,10 @@ Geo geo(const Dev& d, int l, int R)
 // cluster's first block, the 4^3 bottom (48 red-black sweep pairs) in one warp
 // with the cells in registers (64-bit forms: solved by its eigenvectors).
 // What bounds it is a chain of latencies (21 cluster barriers, 96 warp
-// half-sweeps), not bandwidth: 32 us in fixed point, 28 us in FP32 from 32^3
-// down; one block per realization from 16^3 down took 159 us in FP64 and 96 us
+// half-sweeps), not bandwidth: 31 us in fixed point, 27 us in FP32 from 32^3
+// down (33 and 28 with the interpolation cell by cell and every thread's fence
+// at the barriers; clusters of 16 blocks take 29.5 and 26 when they find 16 free
+// SMs in one GPC, which other streams' kernels may hold); one block per realization from 16^3 down took 159 us in FP64 and 96 us
 // in FP32, after 10 launches for the 32^3 level.
 constexpr int COARSE_N = 32, COARSE_CL = 8, COARSE_TPB = 512, BOTTOM_SWEEPS = 48;
 
@@ -1064,15 +1066,41 @@ struct Slab {
             for (int c = 0; c < 2; ++c)
                 out[cell(q + 1, par(q, c))] = own[c * S::COLOR + (q + 1) * S::PLANE + at];
     }
-    // plus the correction of the level below (cell order, planes from z0 on)
+    // plus the correction of the level below (cell order, planes from z0 on):
+    // prolong_at's operations, with each coarse plane's share formed once
     __device__ __forceinline__ void correct(const T* ec, int z0)
     {
+        static_assert(PL == 1 || PL % 2 == 0, "a column of several planes starts at an even one");
         if (!act) return;
+        constexpr int NC = N / 2;
+        const int J = j >> 1, il = ih > 0 ? -1 : 0, ir = ih < NC - 1 ? 1 : 0;
+        const int dj = (j & 1) ? (J < NC - 1 ? NC : 0) : (J > 0 ? -NC : 0);
+        auto plane = [&](int K, Pair<T>& m) {
+            const bool neg = K < 0 || K >= NC;
+            const T* a = ec + ((neg ? (K < 0 ? 0 : NC - 1) : K) - z0) * (NC * NC) + J * NC + ih;
+            const T* b = a + dj;
+            m.v[0] = MG<T>::axpy3(MG<T>::axpy3(a[0], a[il]), MG<T>::axpy3(b[0], b[il]));
+            m.v[1] = MG<T>::axpy3(MG<T>::axpy3(a[0], a[ir]), MG<T>::axpy3(b[0], b[ir]));
+            if (neg) { m.v[0] = -m.v[0]; m.v[1] = -m.v[1]; }
+        };
+        Pair<T> own, oth;
+        plane(k0 >> 1, own);
+        plane((k0 >> 1) + ((k0 & 1) ? 1 : -1), oth);
 #pragma unroll
-        for (int q = 0; q < PL; ++q)
-#pragma unroll
-            for (int c = 0; c < 2; ++c)
-                put(q, c, v[q][c] + prolong_at(ec, N / 2, 2 * ih + par(q, c), j, k0 + q, z0));
+        for (int q = 0; q < PL; ++q) {
+            if (q & 1) {
+                plane(((k0 + q) >> 1) + 1, oth);
+            } else if (q > 0) {
+                const Pair<T> m = own;
+                own = oth;
+                oth = m;
+            }
+            const T c0 = MG<T>::div64(MG<T>::axpy3(own.v[0], oth.v[0]));
+            const T c1 = MG<T>::div64(MG<T>::axpy3(own.v[1], oth.v[1]));
+            const bool p = par(q, 0);
+            put(q, 0, v[q][0] + (p ? c1 : c0));
+            put(q, 1, v[q][1] + (p ? c0 : c1));
+        }
     }
 };
 
@@ -1089,6 +1117,16 @@ __device__ __forceinline__ void restrict_planes(const T* res, T* rc, int planes)
         for (int c = 0; c < 8; ++c) acc += res[((2 * K + (c >> 2)) * N + 2 * J + ((c >> 1) & 1)) * N + 2 * I + (c & 1)];
         rc[t] = MG<T>::half(acc);
     }
+}
+
+// cluster.sync() with one warp's fence for the block: the block's stores come
+// before its barrier, and the fence after it is cumulative.
+__device__ __forceinline__ void cluster_step()
+{
+    __syncthreads();
+    if (threadIdx.x < 32) asm volatile("fence.acq_rel.cluster;" ::: "memory");
+    asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory");
+    asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
 }
 
 // zero: the starting level's potential is taken as zero (not read).
@@ -1127,15 +1165,15 @@ __global__ void __cluster_dims__(COARSE_CL, 1, 1) __launch_bounds__(COARSE_TPB)
 #pragma unroll
             for (int x = 0; x < 2; ++x) L.put(q, x, gp[o + L.cell(q, L.par(q, x))]);
     };
-    cl.sync();                                        // zeros in place before a neighbour's store
+    cluster_step();                                        // zeros in place before a neighbour's store
     if (n == 32) load(a, 32);
     if (n == 16) load(b, 16);
     if (n == 8 && rank == 0) load(c, 8);
-    cl.sync();
+    cluster_step();
     if (n >= 32) {
         for (int it = 0; it < nu1; ++it) {
-            a.relax(0); cl.sync();
-            a.relax(1); cl.sync();
+            a.relax(0); cluster_step();
+            a.relax(1); cluster_step();
         }
         a.residuals(S.res);
         __syncthreads();
@@ -1145,13 +1183,13 @@ __global__ void __cluster_dims__(COARSE_CL, 1, 1) __launch_bounds__(COARSE_TPB)
     }
     if (n >= 16) {
         for (int it = 0; it < nu1; ++it) {
-            b.relax(0); cl.sync();
-            b.relax(1); cl.sync();
+            b.relax(0); cluster_step();
+            b.relax(1); cluster_step();
         }
         b.residuals(S.res);
         __syncthreads();
         restrict_planes<T, 16>(S.res, cl.map_shared_rank(S.r8, 0) + rank * 64, 1);
-        cl.sync();
+        cluster_step();
     }
     if (rank == 0) {
         if (n >= 16) c.set_rhs(S.r8 + c.k0 * 64);
@@ -1181,15 +1219,15 @@ __global__ void __cluster_dims__(COARSE_CL, 1, 1) __launch_bounds__(COARSE_TPB)
             for (int x = 0; x < 2; ++x) (n == 8 ? gp : S.e8)[c.k0 * 64 + c.cell(0, c.par(0, x))] = c.v[0][x];
     }
     if (n >= 16) {
-        cl.sync();
+        cluster_step();
         const T* e0 = cl.map_shared_rank(S.e8, 0);
         for (int t = threadIdx.x; t < 512; t += COARSE_TPB) S.res[t] = e0[t];
         __syncthreads();
         b.correct(S.res, 0);
-        cl.sync();
+        cluster_step();
         for (int it = 0; it < nu2; ++it) {
-            b.relax(1); cl.sync();
-            b.relax(0); cl.sync();
+            b.relax(1); cluster_step();
+            b.relax(0); cluster_step();
         }
     }
     auto store = [&](auto& L, int N) {
@@ -1203,16 +1241,16 @@ __global__ void __cluster_dims__(COARSE_CL, 1, 1) __launch_bounds__(COARSE_TPB)
         b.values(S.res);
         __syncthreads();
         a.correct(S.res, rank * 2 - 1);
-        cl.sync();
+        cluster_step();
         for (int it = 0; it < nu2; ++it) {
-            a.relax(1); cl.sync();
-            a.relax(0); cl.sync();
+            a.relax(1); cluster_step();
+            a.relax(0); cluster_step();
         }
         store(a, 32);
     } else if (n == 16) {
         store(b, 16);
     }
-    cl.sync();                     // no block's shared memory goes while another may still write to it
+    cluster_step();                     // no block's shared memory goes while another may still write to it
 }
 
 // ---------------------------------------------------------------------------
