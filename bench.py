@@ -40,15 +40,15 @@ sys.path.insert(0, ROOT)
 # particle count (both grids hold about the same particles per cell, so the
 # per-cell arrays weigh alike per particle; the 256^3 field array no longer
 # fits in L2, which makes the full-size figure somewhat higher).  Captured:
-# FP64 1.401 GB, mixed 0.855 GB.  The cudaMemsetAsync zeroing of the
+# FP64 1.388 GB, mixed 0.835 GB.  The cudaMemsetAsync zeroing of the
 # per-cell count arrays is not a kernel and is not in the figure.
-TRANSPORT_DRAM_PER_PARTICLE = {True: 140.5, False: 85.8}
+TRANSPORT_DRAM_PER_PARTICLE = {True: 139.2, False: 83.7}
 # FP64 arithmetic of the FP64 push per particle (ncu thread-instruction counts
 # of DADD, DMUL and DFMA over a launch, divided by its particles; an FMA
-# counts as two operations: 12.4 + 30.6 + 2 x 37.1).  The peak it is set
+# counts as two operations: 6.0 + 24.1 + 2 x 24.1).  The peak it is set
 # against is measured in the run (itokmc_probe_fp64_peak: register-resident
 # FMA chains on every SM).
-FP64_FLOP_PER_PARTICLE = 117.3
+FP64_FLOP_PER_PARTICLE = 78.2
 
 METRIC = "particle-steps/s (push+sort+deposit+KMC), HBM roofline %; FP32 vs FP64 at stated err"
 

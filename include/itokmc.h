@@ -489,7 +489,8 @@ int itokmc_probe_fp64_peak(void* stream, double* tflops_out, double* ms_out);
  *           mg_nu1/nu2, mg_max_cycles, precision/field_precision and
  *           stream; particle and allocator fields are ignored.  The field
  *           form is field_precision, or precision when that is -1:
- *           ITOKMC_FP64 runs FP64 V-cycles; ITOKMC_MIXED runs FP32 V-cycles
+ *           ITOKMC_FP64 runs V-cycles in 64-bit fixed point (FP64 ones where
+ *           its range does not serve); ITOKMC_MIXED runs FP32 V-cycles
  *           inside FP64 residual refinement (an FP64 potential, not the
  *           fixed-point potential a handle of the mixed form keeps).  Any
  *           other value is ITOKMC_ERR_ARG before anything is launched.

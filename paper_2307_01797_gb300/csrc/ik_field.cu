@@ -6,8 +6,9 @@
 // conditions of Sec. 5.1: plane electrodes (Dirichlet, phi = 0 at z = lo,
 // E0 L at z = hi; ghost 2 phi_b - phi_1) and homogeneous Neumann side faces
 // (ghost = phi_1).  Cell-centred hierarchy down to 4^3: averaging
-// restriction, trilinear cell-centred prolongation, and a one-block
-// red-black solve at the bottom (the paper uses BiCGSTAB there).
+// restriction, trilinear cell-centred prolongation, and at the bottom red-black
+// sweeps in FP32 or the level's eigenvectors in the 64-bit forms (the paper
+// uses BiCGSTAB there).
 //
 // Two forms: V-cycles on the system in 64-bit fixed point (the FP64 form; with
 // FP64 V-cycles where the integers' range does not serve), or FP32 V-cycles
