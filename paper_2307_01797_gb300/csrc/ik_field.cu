@@ -863,10 +863,11 @@ Geo geo(const Dev& d, int l, int R)
 // cluster's first block, the 4^3 bottom (48 red-black sweep pairs) in one warp
 // with the cells in registers (64-bit forms: solved by its eigenvectors).
 // What bounds it is a chain of latencies (21 cluster barriers, 96 warp
-// half-sweeps), not bandwidth: 31 us in fixed point, 27 us in FP32 from 32^3
-// down (33 and 28 with the interpolation cell by cell and every thread's fence
-// at the barriers; clusters of 16 blocks take 29.5 and 26 when they find 16 free
-// SMs in one GPC, which other streams' kernels may hold); one block per realization from 16^3 down took 159 us in FP64 and 96 us
+// half-sweeps), not bandwidth: 29 us in fixed point, 25 us in FP32 from 32^3
+// down (33 and 28 with the interpolation cell by cell, every thread's fence at
+// the barriers, a divisor formed per cell and the loads after the zeros; clusters
+// of 16 blocks took 1 us off when they found 16 free SMs in one GPC, which other
+// streams' kernels may hold); one block per realization from 16^3 down took 159 us in FP64 and 96 us
 // in FP32, after 10 launches for the 32^3 level.
 constexpr int COARSE_N = 32, COARSE_CL = 8, COARSE_TPB = 512, BOTTOM_SWEEPS = 48;
 
@@ -999,11 +1000,16 @@ struct Slab {
         ih = threadIdx.x % (N / 2);
         j = threadIdx.x / (N / 2) % N;
         at = z * S::PLANE + (j + 1) * S::W + ih + 1;
+        // between the electrodes a column has two divisors
+        const int dy = 6 - (j == 0) - (j == N - 1);
+        const Inv<T> even(dy - (ih == 0)), odd(dy - (ih == N / 2 - 1));
 #pragma unroll
         for (int q = 0; q < PL; ++q)
 #pragma unroll
             for (int c = 0; c < 2; ++c) {
-                inv[q][c] = Inv<T>(diag_count(2 * ih + ((j + k0 + q + c) & 1), j, k0 + q, N));
+                inv[q][c] = par(q, c) ? odd : even;
+                if ((q == 0 && k0 == 0) || (q == PL - 1 && k0 + q == N - 1))
+                    inv[q][c] = Inv<T>(diag_count(2 * ih + par(q, c), j, k0 + q, N));
                 v[q][c] = r[q][c] = (T)0;
             }
     }
@@ -1132,7 +1138,7 @@ __device__ __forceinline__ void cluster_step()
 
 // zero: the starting level's potential is taken as zero (not read).
 template <class T>
-__global__ void __cluster_dims__(COARSE_CL, 1, 1) __launch_bounds__(COARSE_TPB)
+__global__ void __cluster_dims__(COARSE_CL, 1, 1) __launch_bounds__(COARSE_TPB, 1)
     k_vcycle_coarse(CoarseTop<T> top, int zero, int nu1, int nu2)
 {
     extern __shared__ __align__(16) unsigned char csm[];
@@ -1142,12 +1148,6 @@ __global__ void __cluster_dims__(COARSE_CL, 1, 1) __launch_bounds__(COARSE_TPB)
     const uint64_t base = (uint64_t)(blockIdx.x / COARSE_CL) * n * n * n;
     T* gp = top.phi + base;
     const T* gr = top.rhs + base;
-    // zeros everywhere (rims, domain halos, the corrections' start)
-    {
-        constexpr int WORDS = (SlabShape<32, 4>::SIZE + SlabShape<16, 2>::SIZE + SlabShape<8, 8>::SIZE) * (int)sizeof(T) / 16;
-        static_assert(WORDS * 16 == (int)offsetof(CoarseSmem<T>, res), "the three levels first, in whole 16-byte words");
-        for (int t = threadIdx.x; t < WORDS; t += COARSE_TPB) reinterpret_cast<uint4*>(&S)[t] = make_uint4(0, 0, 0, 0);
-    }
     Slab<T, 32, 4, 4> a;
     Slab<T, 16, 2, 2> b;
     Slab<T, 8, 8, 1> c;
@@ -1156,21 +1156,32 @@ __global__ void __cluster_dims__(COARSE_CL, 1, 1) __launch_bounds__(COARSE_TPB)
     a.init(S.p32, lower(S.p32), upper(S.p32), rank * 4);
     b.init(S.p16, lower(S.p16), upper(S.p16), rank * 2);
     c.init(S.p8, nullptr, nullptr, 0);
-    // the starting level's right-hand side and potential
+    // the starting level's right-hand side, on its way while the zeros are
+    // written, and potential
+    if (n == 32) a.set_rhs(gr + (int64_t)a.k0 * 1024);
+    if (n == 16) b.set_rhs(gr + (int64_t)b.k0 * 256);
+    if (n == 8 && rank == 0) c.set_rhs(gr + (int64_t)c.k0 * 64);
+    // zeros everywhere (rims, domain halos, the corrections' start)
+    {
+        constexpr int WORDS = (SlabShape<32, 4>::SIZE + SlabShape<16, 2>::SIZE + SlabShape<8, 8>::SIZE) * (int)sizeof(T) / 16;
+        static_assert(WORDS * 16 == (int)offsetof(CoarseSmem<T>, res), "the three levels first, in whole 16-byte words");
+        for (int t = threadIdx.x; t < WORDS; t += COARSE_TPB) reinterpret_cast<uint4*>(&S)[t] = make_uint4(0, 0, 0, 0);
+    }
     auto load = [&](auto& L, int N) {
         const int64_t o = (int64_t)L.k0 * N * N;
-        L.set_rhs(gr + o);
-        if (zero || !L.act) return;
+        if (!L.act) return;
 #pragma unroll
         for (int q = 0; q < L.PL; ++q)
 #pragma unroll
             for (int x = 0; x < 2; ++x) L.put(q, x, gp[o + L.cell(q, L.par(q, x))]);
     };
-    cluster_step();                                        // zeros in place before a neighbour's store
-    if (n == 32) load(a, 32);
-    if (n == 16) load(b, 16);
-    if (n == 8 && rank == 0) load(c, 8);
-    cluster_step();
+    cluster_step();                                    // zeros in place before a neighbour's store
+    if (!zero) {
+        if (n == 32) load(a, 32);
+        if (n == 16) load(b, 16);
+        if (n == 8 && rank == 0) load(c, 8);
+        cluster_step();
+    }
     if (n >= 32) {
         for (int it = 0; it < nu1; ++it) {
             a.relax(0); cluster_step();
