@@ -58,7 +58,7 @@ struct itokmc_handle {
     std::vector<void*> allocs;
     itokmc_stats st{};
     cudaEvent_t ev[8]{};
-    struct Readback { uint32_t N; uint32_t step; uint64_t work_need; ik::Counters ctr; }* rb = nullptr;  // pinned
+    struct Readback { uint32_t N; uint32_t step; uint64_t work_need; ik::Counters ctr, keep; }* rb = nullptr;  // pinned
 };
 
 namespace {
@@ -271,6 +271,25 @@ int readback(itokmc_handle* h)
     IK_CHECK(h, cudaStreamSynchronize(h->s));
     IK_CHECK(h, cudaGetLastError());
     h->N = h->rb->N;
+    return ITOKMC_OK;
+}
+
+// A call between two stages that uses the counters keeps the stages' own
+// aside: the particles stage still needs the KMC's list lengths.
+int keep_counters(itokmc_handle* h)
+{
+    if (h->stage == 0) return ITOKMC_OK;         // the next stage clears them
+    IK_CHECK(h, cudaMemcpyAsync(&h->rb->keep, h->d.ctr, sizeof(ik::Counters), cudaMemcpyDeviceToHost, h->s));
+    return ITOKMC_OK;
+}
+
+// new_rho: the call has left its charge in rho, whose largest value stays.
+int restore_counters(itokmc_handle* h, bool new_rho)
+{
+    if (h->stage == 0) return ITOKMC_OK;
+    IK_CHECK(h, cudaStreamSynchronize(h->s));
+    if (new_rho) h->rb->keep.rho_absmax = h->rb->ctr.rho_absmax;
+    IK_CHECK(h, cudaMemcpyAsync(h->d.ctr, &h->rb->keep, sizeof(ik::Counters), cudaMemcpyHostToDevice, h->s));
     return ITOKMC_OK;
 }
 
@@ -1212,10 +1231,13 @@ int itokmc_set_field(itokmc_handle* h, const double* E, int32_t mem)
 int itokmc_solve_field(itokmc_handle* h)
 {
     IK_GUARD(h);
-    cudaMemsetAsync(h->d.ctr, 0, sizeof(ik::Counters), h->s);
+    int rc = keep_counters(h);
+    if (rc) return rc;
+    IK_CHECK(h, cudaMemsetAsync(h->d.ctr, 0, sizeof(ik::Counters), h->s));
     ik::launch_deposit_only(h->P, h->d, h->N, h->s);
     ik::launch_rho(h->P, h->d, h->G, h->s);
-    int rc = readback(h);
+    rc = readback(h);
+    if (!rc) rc = restore_counters(h, true);
     if (rc) return rc;
     rc = status_of_err(h, h->rb->ctr.err);
     if (rc) return rc;
@@ -1310,6 +1332,8 @@ int itokmc_autotune(itokmc_handle* h, itokmc_tuning* out)
     if (h->N > 0 && d.work_bytes >= 3 * dep_bytes + 16) {
         IK_CHECK(h, cudaMemcpyAsync(d.work, d.ne_fix, dep_bytes, cudaMemcpyDeviceToDevice, h->s));
         IK_CHECK(h, cudaMemcpyAsync(d.work + dep_bytes, d.Xe, dep_bytes, cudaMemcpyDeviceToDevice, h->s));
+        const int kept = keep_counters(h);
+        if (kept) return kept;
         // every trial's deposit must equal the first one's (integer sums)
         unsigned long long* first = reinterpret_cast<unsigned long long*>(d.work + 2 * dep_bytes);
         unsigned int* differs = reinterpret_cast<unsigned int*>(d.work + 3 * dep_bytes);
@@ -1333,6 +1357,8 @@ int itokmc_autotune(itokmc_handle* h, itokmc_tuning* out)
         IK_CHECK(h, cudaMemcpyAsync(&diff, differs, sizeof diff, cudaMemcpyDeviceToHost, h->s));
         IK_CHECK(h, cudaMemcpyAsync(d.ne_fix, d.work, dep_bytes, cudaMemcpyDeviceToDevice, h->s));
         IK_CHECK(h, cudaMemcpyAsync(d.Xe, d.work + dep_bytes, dep_bytes, cudaMemcpyDeviceToDevice, h->s));
+        const int back = restore_counters(h, false);
+        if (back) return back;
         IK_CHECK(h, cudaStreamSynchronize(h->s));
         drop_graphs(h);                      // the kernels' parameters changed
         if (diff) return fail(h, ITOKMC_ERR_INTERNAL, "autotune: deposit windows gave different densities");

@@ -1266,9 +1266,9 @@ __global__ void k_kmc0d(Params P, double Em, long long X0, uint32_t nreal, int n
 // (only those have firings), for each species.
 __global__ void k_loss(Params P, uint32_t* __restrict__ wbase, int wstride, const uint32_t* __restrict__ cs,
                        const unsigned long long* __restrict__ Xe, const int64_t* __restrict__ gain, uint64_t G,
-                       const uint32_t* __restrict__ list, const Counters* __restrict__ ctr)
+                       const uint32_t* __restrict__ list, const uint32_t* __restrict__ list_n)
 {
-    const uint32_t n = ctr->n_kmc_cells;
+    const uint32_t n = *list_n;
     for (uint64_t t = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; t < (uint64_t)n * P.S;
          t += (uint64_t)gridDim.x * blockDim.x) {
         const uint64_t sp = (uint64_t)(t >= n) + (uint64_t)(t >= 2ull * n);
@@ -3125,7 +3125,7 @@ void launch_particles_a(const Params& P, Dev& d, uint64_t G, cudaStream_t s)
     uint32_t* wbase = d.mixed ? reinterpret_cast<uint32_t*>(d.rA32) + 3 : reinterpret_cast<uint32_t*>(d.recA) + 7;
     const int wstride = d.mixed ? 4 : 8;
     ++g_launches;
-    k_loss<<<grid_for(Gp, 128, 152 * 64), 128, 0, s>>>(P, wbase, wstride, d.cell_start, d.Xe, d.gain, G, d.kmc_list, d.ctr);
+    k_loss<<<grid_for(Gp, 128, 152 * 64), 128, 0, s>>>(P, wbase, wstride, d.cell_start, d.Xe, d.gain, G, d.kmc_list, d.kmc_n);
     if (P.photon_ratio > 0.0) {
         ++g_launches;
         k_photons<<<152 * 2, 256, 0, s>>>(P, d.mixed ? 1 : 0, d.fired, G, d.pc_list, d.photos, d.photo_cap,
