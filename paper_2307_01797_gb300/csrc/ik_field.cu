@@ -2470,6 +2470,10 @@ extern "C" int itokmc_field_solve_noalloc(const itokmc_config* cfg, const int64_
     d.direct_cycles = true;            // no graph objects: nothing is instantiated per call
     // the field is formed after the cycles, so its array shares its place with
     // the finest level's right-hand sides and second array
+    // the cycles load and store the potential by pairs: a caller's array that
+    // is not aligned to them (the ABI asks for a double's alignment) is solved
+    // in a copy, which shares that place too
+    const bool copy = reinterpret_cast<uintptr_t>(phi) % (2 * sizeof(double)) != 0;
     size_t off = 0;
     d.E = reinterpret_cast<E64*>(base + carve(off, (size_t)P.n3 * sizeof(E64)));
     d.E32 = nullptr;
@@ -2481,7 +2485,7 @@ extern "C" int itokmc_field_solve_noalloc(const itokmc_config* cfg, const int64_
         size_t& at = l == 0 ? top : off;
         L.n = m;
         L.h = P.h[0] * (double)(n / m);
-        L.phi = l == 0 ? phi : reinterpret_cast<double*>(base + carve(at, cells * sizeof(double)));
+        L.phi = l == 0 && !copy ? phi : reinterpret_cast<double*>(base + carve(at, cells * sizeof(double)));
         L.rhs = reinterpret_cast<double*>(base + carve(at, cells * sizeof(double)));
         L.alt = base + carve(at, cells * sizeof(double));
         L.rhs_fix = reinterpret_cast<long long*>(l == 0 ? base + carve(at, cells * sizeof(long long))
@@ -2510,6 +2514,8 @@ extern "C" int itokmc_field_solve_noalloc(const itokmc_config* cfg, const int64_
     const double phi_top = P.E0 * (P.hi[2] - P.lo[2]);
     ++g_launches;
     k_rhs_from_rho<<<gridsz((uint64_t)P.n3, 256), 256, 0, s>>>(rho, d.lev[0].rhs, n, P.log2n, qscale, phi_top, P.h[0]);
+    const size_t phi_bytes = (size_t)P.n3 * sizeof(double);
+    if (copy) cudaMemcpyAsync(d.lev[0].phi, phi, phi_bytes, cudaMemcpyDeviceToDevice, s);
     int cycles = 0;
     double rel = 0.0;
     const int st = field_solve(P, d, prec, cfg->mg_rtol, cfg->mg_nu1, cfg->mg_nu2, 0ull, cfg->mg_max_cycles, s, &cycles,
@@ -2519,6 +2525,10 @@ extern "C" int itokmc_field_solve_noalloc(const itokmc_config* cfg, const int64_
     if (st == -3) {
         set_global_error("field_solve_noalloc: CUDA error in the multigrid");
         return ITOKMC_ERR_CUDA;
+    }
+    if (copy) {
+        cudaMemcpyAsync(phi, d.lev[0].phi, phi_bytes, cudaMemcpyDeviceToDevice, s);
+        d.lev[0].phi = phi;
     }
     launch_efield(P, d, s);
     const uint64_t G = (uint64_t)P.n3;
