@@ -227,7 +227,8 @@ int itokmc_destroy(itokmc_handle* h);
  * These are the computational particles of Sec. 3.1 (position X_p, integer
  * weight w_p: the number of physical electrons a superparticle stands for,
  * Sec. 4.4).  Particles are stably sorted by (realization, cell), the
- * binning of Sec. 5.6; particles outside [lo, hi) are rejected with ERR_ARG.
+ * binning of Sec. 5.6; particles outside [lo, hi) are rejected with ERR_ARG,
+ * and so is device memory of cudaMalloc that ends before the n-th element.
  * ERR_CAPACITY if n > capacity. */
 int itokmc_set_particles(itokmc_handle* h, const double* x, const double* y, const double* z,
                          const uint32_t* w, const int32_t* realization, int64_t n, int32_t mem);
@@ -274,7 +275,8 @@ int itokmc_seed_blobs(itokmc_handle* h, const itokmc_seed_blob* blobs, int32_t n
 int itokmc_set_ions(itokmc_handle* h, const int64_t* npos, const int64_t* nneg, int32_t mem);
 
 /* Sets E directly (double, three blocks Ex, Ey, Ez of R n^3 each), bypassing
- * the field solve: used to feed a given field to the next step or stage. */
+ * the field solve: used to feed a given field to the next step or stage.
+ * ERR_ARG for device memory of cudaMalloc that ends before the last value. */
 int itokmc_set_field(itokmc_handle* h, const double* E, int32_t mem);
 
 /* Re-deposits the current particles (a4) and solves the field (a5) from

@@ -9,6 +9,8 @@
 #include <string>
 #include <vector>
 
+#include <cuda.h>
+
 #include "../../include/itokmc.h"
 #include "ik_common.cuh"
 #include "ik_state.h"
@@ -128,17 +130,46 @@ void dfree(itokmc_handle* h, void* p)
     else cudaFreeAsync(p, h->s);
 }
 
-// Whether kernels can read the array p where it is: memory of the handle's
-// device, aligned to its elements.  NULL (an array that is not given) passes.
-bool readable_here(itokmc_handle* h, const void* p, size_t align)
+// An entry point of the driver (the library links the runtime alone).
+template <class F>
+F* driver_fn(const char* name)
 {
-    if (!p) return true;
+    void* p = nullptr;
+    cudaDriverEntryPointQueryResult q;
+    if (cudaGetDriverEntryPointByVersion(name, &p, 12000, cudaEnableDefault, &q) != cudaSuccess ||
+        q != cudaDriverEntryPointSuccess) {
+        cudaGetLastError();
+        return nullptr;
+    }
+    return reinterpret_cast<F*>(p);
+}
+
+// How an array of `bytes` that the caller gave as device memory is taken: read
+// by the kernels where it is (memory of the handle's device, aligned to its
+// elements, all of it inside one allocation), copied first, or refused because
+// its allocation ends before the array does.  A copy checks the range itself;
+// kernels would read on.  Memory whose allocation the driver does not give in
+// one piece (mapped ranges, pools) and that seems short is copied.
+enum class Take { IN_PLACE, COPY, SHORT };
+Take take_array(itokmc_handle* h, const void* p, size_t bytes, size_t align)
+{
+    if (!p) return Take::IN_PLACE;               // not given
     cudaPointerAttributes a;
     if (cudaPointerGetAttributes(&a, p) != cudaSuccess) {
         cudaGetLastError();
-        return false;
+        return Take::COPY;
     }
-    return a.type == cudaMemoryTypeDevice && a.device == h->device && reinterpret_cast<uintptr_t>(p) % align == 0;
+    if (a.type != cudaMemoryTypeDevice || a.device != h->device || reinterpret_cast<uintptr_t>(p) % align) return Take::COPY;
+    static auto* const range = driver_fn<CUresult(CUdeviceptr*, size_t*, CUdeviceptr)>("cuMemGetAddressRange");
+    static auto* const attr = driver_fn<CUresult(void*, CUpointer_attribute, CUdeviceptr)>("cuPointerGetAttribute");
+    const CUdeviceptr at = reinterpret_cast<CUdeviceptr>(p);
+    CUdeviceptr base = 0;
+    size_t size = 0;
+    if (!range || !attr || range(&base, &size, at) != CUDA_SUCCESS) return Take::COPY;
+    if (at - base <= size && bytes <= size - (at - base)) return Take::IN_PLACE;
+    int whole = 0;                               // memory of cudaMalloc: the range is all of it
+    if (attr(&whole, CU_POINTER_ATTRIBUTE_IS_LEGACY_CUDA_IPC_CAPABLE, at) != CUDA_SUCCESS) whole = 0;
+    return whole ? Take::SHORT : Take::COPY;
 }
 
 // Grows the photon list to hold at least `need` superphotons (geometric).
@@ -1118,9 +1149,16 @@ int itokmc_set_particles_species(itokmc_handle* h, const double* x, const double
     int32_t* dr = realization ? reinterpret_cast<int32_t*>(dw + n) : nullptr;
     const cudaMemcpyKind k = mem == ITOKMC_HOST ? cudaMemcpyHostToDevice : cudaMemcpyDeviceToDevice;
     // arrays in this device's memory are read where they are
-    const bool in_place = mem == ITOKMC_DEVICE && n > 0 && readable_here(h, x, 8) && readable_here(h, y, 8) &&
-                          readable_here(h, z, 8) && readable_here(h, w, 4) && readable_here(h, realization, 4) &&
-                          readable_here(h, species, 4);
+    bool in_place = mem == ITOKMC_DEVICE && n > 0;
+    if (in_place) {
+        const Take t[6] = { take_array(h, x, n * 8, 8),           take_array(h, y, n * 8, 8),
+                            take_array(h, z, n * 8, 8),           take_array(h, w, n * 4, 4),
+                            take_array(h, realization, n * 4, 4), take_array(h, species, n * 4, 4) };
+        for (const Take k : t) {
+            if (k == Take::SHORT) return fail(h, ITOKMC_ERR_ARG, "bad particle arrays: device memory of fewer than n elements");
+            in_place = in_place && k == Take::IN_PLACE;
+        }
+    }
     const double *sx = dx, *sy = dy, *sz = dz;
     const uint32_t* sw = dw;
     const int32_t *sr = dr, *ssp = nullptr;
@@ -1219,7 +1257,9 @@ int itokmc_set_field(itokmc_handle* h, const double* E, int32_t mem)
     if (!E) return fail(h, ITOKMC_ERR_ARG, "NULL field");
     const cudaMemcpyKind k = mem == ITOKMC_HOST ? cudaMemcpyHostToDevice : cudaMemcpyDeviceToDevice;
     const double* src = E;
-    if (!(mem == ITOKMC_DEVICE && readable_here(h, E, 8))) {
+    const Take t = mem == ITOKMC_DEVICE ? take_array(h, E, 3 * h->G * sizeof(double), 8) : Take::COPY;
+    if (t == Take::SHORT) return fail(h, ITOKMC_ERR_ARG, "set_field: device memory of fewer than 3 R n^3 values");
+    if (t == Take::COPY) {
         IK_CHECK(h, cudaMemcpyAsync(h->d.stage, E, 3 * h->G * sizeof(double), k, h->s));
         src = h->d.stage;
     }
