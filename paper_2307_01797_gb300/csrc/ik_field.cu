@@ -682,9 +682,9 @@ __global__ void k_fix_store(const long long* __restrict__ Phi, double* __restric
         phi[t] = (double)Phi[t] * sc;
 }
 
-// Squared norms of the exact integer residual and of B (units of 2^30 steps:
-// FP32 holds their squares), summed as in k_resid_fixed, and the largest
-// |Phi|.  The norms serve the convergence test alone.
+// Squared norms of the exact integer residual and of B in FP64, summed in the
+// order of k_resid_fixed, and the largest |Phi|.  The norms decide where the
+// cycles end.
 __global__ void __launch_bounds__(NORM_TPB) k_resid_norm_fix(const long long* __restrict__ Phi,
                                                              const long long* __restrict__ B, Geo G,
                                                              double* __restrict__ part, int with_b, MarchGeo m,
@@ -692,20 +692,20 @@ __global__ void __launch_bounds__(NORM_TPB) k_resid_norm_fix(const long long* __
 {
     __shared__ double red[NORM_TPB / 32][2];
     __shared__ unsigned long long redm[NORM_TPB / 32];
-    float acc = 0.f, bacc = 0.f;
+    double acc = 0.0, bb = 0.0;
     unsigned long long mx = 0;
     march_cells(Phi, G.n, m, [&](uint64_t t, long long pc, long long s, int diag) {
         const long long b = B[t];
         const unsigned long long ap = (unsigned long long)(pc < 0 ? -pc : pc);
         mx = ap > mx ? ap : mx;
-        const float res = __ll2float_rn(MG<long long>::resid(s, b, pc, diag)) * 0x1p-30f;
-        acc = __fmaf_rn(res, res, acc);
+        const double res = __ll2double_rn(MG<long long>::resid(s, b, pc, diag));
+        acc = __fma_rn(res, res, acc);
         if (with_b) {
-            const float bf = __ll2float_rn(b) * 0x1p-30f;
-            bacc = __fmaf_rn(bf, bf, bacc);
+            const double bf = __ll2double_rn(b);
+            bb = __fma_rn(bf, bf, bb);
         }
     });
-    double a = fs->use64 || mx >= (unsigned long long)FIX_LIM ? (double)INFINITY : (double)acc, bb = (double)bacc;
+    double a = fs->use64 || mx >= (unsigned long long)FIX_LIM ? (double)INFINITY : acc;
 #pragma unroll
     for (int d = 16; d > 0; d >>= 1) {
         a += __shfl_xor_sync(0xffffffffu, a, d);
