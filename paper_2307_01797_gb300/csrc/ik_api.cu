@@ -1045,7 +1045,7 @@ int itokmc_init(const itokmc_config* cfg, itokmc_handle** out)
         if (l == 0 && f64) {
             L.phi_fix = dalloc_n<long long>(h, cells, &rc);
             L.rhs_fix = dalloc_n<long long>(h, cells, &rc);
-            d.fix = dalloc_n<ik::FixScale>(h, 1, &rc);
+            d.fix = dalloc_n<ik::FixScale>(h, R, &rc);
         }
     }
     d.nlev = l;
@@ -1054,7 +1054,7 @@ int itokmc_init(const itokmc_config* cfg, itokmc_handle** out)
     d.norm_out = dalloc_n<double>(h, 2 * R, &rc);
     if (!rc && cudaMallocHost(reinterpret_cast<void**>(&h->rb), sizeof(*h->rb)) != cudaSuccess)
         rc = fail(h, ITOKMC_ERR_OOM, "pinned host buffer");
-    if (!rc && cudaMallocHost(reinterpret_cast<void**>(&d.norm_host), (2 * R + ik::FIX_DOUBLES) * sizeof(double)) != cudaSuccess)
+    if (!rc && cudaMallocHost(reinterpret_cast<void**>(&d.norm_host), R * (2 + ik::FIX_DOUBLES) * sizeof(double)) != cudaSuccess)
         rc = fail(h, ITOKMC_ERR_OOM, "pinned host buffer");
     for (int e = 0; e < 8 && !rc; ++e)
         if (cudaEventCreate(&h->ev[e]) != cudaSuccess) rc = fail(h, ITOKMC_ERR_CUDA, "event create");

@@ -577,9 +577,21 @@ __global__ void k_efield_fixed(const long long* __restrict__ Phi, E64* __restric
 // h^2 b 2^F, |Phi| below 2^57 (2^-57 of the bound on |phi|, FP64 keeps 2^-53
 // of the value), with the relaxations, residuals and transfers of MG<long
 // long>.  The potential is FP64 before and after (the start guess, the
-// checkpoint, itokmc_read_densities).  FIX_LIM marks an iterate that left its
-// range: the solve then goes on with FP64 cycles.
+// checkpoint, itokmc_read_densities).  Each realization has its own scale: a
+// member of a batch keeps its bits beside one of a far higher potential.
+// FIX_LIM marks an iterate that left its range: the solve then goes on with
+// FP64 cycles.
 constexpr long long FIX_LIM = 1ll << 59;
+
+// The bits by which a scale can go up that a loose bound (k_fix_scale) left
+// too low: the largest |Phi| to [2^55, 2^56).
+__host__ __device__ inline int fix_shift(const FixScale& f)
+{
+    if (f.max_fix == 0 || f.max_fix >= (1ull << 52)) return 0;
+    int lead = 0;
+    while ((f.max_fix >> lead) > 1) ++lead;
+    return 55 - lead;
+}
 
 // x 2^F rounded to the nearest integer, |x| 2^F < 2^62, by integer steps.
 __device__ __forceinline__ long long to_fixed(double x, int F)
@@ -595,13 +607,18 @@ __device__ __forceinline__ long long to_fixed(double x, int F)
 
 // The start guess (extrapolated in time when asked) and the largest |guess|
 // and |h^2 b| (the electrode's share of the top layer's b taken out), as the
-// bits of the non-negative doubles.
+// bits of the non-negative doubles.  Block row r: realization r.
 __global__ void __launch_bounds__(256) k_fix_start(double* __restrict__ phi, double* __restrict__ prev, int extrapolate,
                                                    int have, const double* __restrict__ rhs, Geo G, double bc,
                                                    FixScale* __restrict__ fs)
 {
     unsigned long long mp = 0, mb = 0;
-    for (uint64_t t = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; t < G.cells; t += (uint64_t)gridDim.x * blockDim.x) {
+    const uint64_t n3 = 1ull << (3 * G.log2n), o = blockIdx.y * n3;
+    fs += blockIdx.y;
+    phi += o;
+    rhs += o;
+    if (prev) prev += o;
+    for (uint64_t t = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; t < n3; t += (uint64_t)gridDim.x * blockDim.x) {
         double v = phi[t];
         if (extrapolate) {
             const double old = v;
@@ -612,7 +629,7 @@ __global__ void __launch_bounds__(256) k_fix_start(double* __restrict__ phi, dou
             prev[t] = old;
         }
         double b = rhs[t];
-        if (((t >> (2 * G.log2n)) & (uint64_t)(G.n - 1)) == (uint64_t)(G.n - 1)) b += bc;
+        if ((t >> (2 * G.log2n)) == (uint64_t)(G.n - 1)) b += bc;
         const unsigned long long vb = (unsigned long long)__double_as_longlong(v) & 0x7fffffffffffffffull,
                                  bb = (unsigned long long)__double_as_longlong(b) & 0x7fffffffffffffffull;
         mp = vb > mp ? vb : mp;
@@ -637,15 +654,19 @@ __global__ void __launch_bounds__(256) k_fix_start(double* __restrict__ phi, dou
     }
 }
 
-// The scale.  Mc bounds |phi| of the solution: electrode potential plus the
+// The scale of each realization.  Mc bounds |phi| of the solution: electrode potential plus the
 // 1D Dirichlet bound max|h^2 b| n^2 / 8, doubled.  A guess extrapolated from
 // the last steps is near the solution: four times its modulus bounds it (Mc
 // is loose by orders of magnitude for a localised charge).  use64: the guess
 // is not finite or far above the solution.
-__global__ void k_fix_scale(FixScale* fs, double phi_top, int n, int near, int sh)
+__global__ void k_fix_scale(FixScale* fs, int R, double phi_top, int n, int near, int rescale)
 {
-    if (sh) {                                                   // a rescaling of a running solve
-        fs->F += sh;
+    const int r = blockIdx.x * blockDim.x + threadIdx.x;
+    if (r >= R) return;
+    fs += r;
+    fs->sh = rescale ? fix_shift(*fs) : 0;
+    if (rescale) {                                              // of a running solve
+        fs->F += fs->sh;
     } else {
         const double mp = __longlong_as_double((long long)fs->max_phi), mb = __longlong_as_double((long long)fs->max_b);
         const double Mc = 2.0 * (fabs(phi_top) + mb * (double)n * (double)n / 8.0);
@@ -660,25 +681,28 @@ __global__ void k_fix_scale(FixScale* fs, double phi_top, int n, int near, int s
     fs->top = to_fixed(phi_top, fs->F);
 }
 
-// Phi and B from phi and the right-hand side (sh = 0), or Phi shifted up by
-// sh bits and B formed again at the new scale.
+// Phi and B from phi and the right-hand side; rescale: Phi shifted up by sh
+// bits and B formed again at the new scale.  Block row r: realization r.
 __global__ void k_fix_load(const double* __restrict__ phi, const double* __restrict__ rhs, long long* __restrict__ Phi,
-                           long long* __restrict__ B, uint64_t cells, const FixScale* __restrict__ fs, int sh)
+                           long long* __restrict__ B, uint64_t n3, const FixScale* __restrict__ fs, int rescale)
 {
-    const int F = fs->F;
-    if (fs->use64) return;
-    for (uint64_t t = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; t < cells; t += (uint64_t)gridDim.x * blockDim.x) {
-        Phi[t] = sh ? Phi[t] << sh : to_fixed(phi[t], F);
+    fs += blockIdx.y;
+    const int F = fs->F, sh = fs->sh;
+    if (fs->use64 || (rescale && sh == 0)) return;
+    const uint64_t o = blockIdx.y * n3;
+    for (uint64_t t = o + blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; t < o + n3; t += (uint64_t)gridDim.x * blockDim.x) {
+        Phi[t] = rescale ? Phi[t] << sh : to_fixed(phi[t], F);
         B[t] = to_fixed(rhs[t], F);
     }
 }
 
-// The potential back in FP64.
-__global__ void k_fix_store(const long long* __restrict__ Phi, double* __restrict__ phi, uint64_t cells,
+// The potential back in FP64.  Block row r: realization r.
+__global__ void k_fix_store(const long long* __restrict__ Phi, double* __restrict__ phi, uint64_t n3,
                             const FixScale* __restrict__ fs)
 {
-    const double sc = fs->down;
-    for (uint64_t t = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; t < cells; t += (uint64_t)gridDim.x * blockDim.x)
+    const double sc = fs[blockIdx.y].down;
+    const uint64_t o = blockIdx.y * n3;
+    for (uint64_t t = o + blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; t < o + n3; t += (uint64_t)gridDim.x * blockDim.x)
         phi[t] = (double)Phi[t] * sc;
 }
 
@@ -694,6 +718,7 @@ __global__ void __launch_bounds__(NORM_TPB) k_resid_norm_fix(const long long* __
     __shared__ unsigned long long redm[NORM_TPB / 32];
     double acc = 0.0, bb = 0.0;
     unsigned long long mx = 0;
+    fs += blockIdx.x / m.bpr;
     march_cells(Phi, G.n, m, [&](uint64_t t, long long pc, long long s, int diag) {
         const long long b = B[t];
         const unsigned long long ap = (unsigned long long)(pc < 0 ? -pc : pc);
@@ -733,13 +758,13 @@ __global__ void __launch_bounds__(NORM_TPB) k_resid_norm_fix(const long long* __
 __global__ void k_efield_fix(const long long* __restrict__ Phi, E64* __restrict__ E, float4* __restrict__ E32,
                              double* __restrict__ phi, Geo G, double inv2h, const FixScale* __restrict__ fs)
 {
-    if (fs->use64) return;                        // nothing was solved here (replayed steps: the host solves again)
-    const double down = fs->down, sc = down * inv2h;
     const float inv2hf = (float)inv2h;
-    const long long top2 = 2 * fs->top;
     for (uint64_t t = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; t < G.cells; t += (uint64_t)gridDim.x * blockDim.x) {
         int r, k, j, i;
         decode(t, G.log2n, r, k, j, i);
+        if (fs[r].use64) continue;                // nothing was solved here (replayed steps: the host solves again)
+        const double down = fs[r].down, sc = down * inv2h;
+        const long long top2 = 2 * fs[r].top;
         const int n = G.n;
         const uint64_t sy = (uint64_t)n, sz = (uint64_t)n * n;
         const long long c = Phi[t];
@@ -849,6 +874,13 @@ Geo geo(const Dev& d, int l, int R)
     g.R = R;
     g.cells = (uint64_t)R * g.n * g.n * g.n;
     return g;
+}
+
+// Blocks for a pass whose block row r takes realization r.
+dim3 grid_per_real(const Geo& G)
+{
+    const int cap = 152 * 32 / G.R, b = gridsz(G.cells / G.R, 256);
+    return dim3(b < cap ? b : (cap > 1 ? cap : 1), G.R);
 }
 
 // ---------------------------------------------------------------------------
@@ -1887,12 +1919,12 @@ void fix_begin(const Params& P, Dev& d, bool extrapolate, cudaStream_t s)
     double qscale, bc_top;
     rhs_consts(P, qscale, bc_top);
     const bool ex = extrapolate && d.phi_prev;
-    cudaMemsetAsync(d.fix, 0, sizeof(FixScale), s);
+    cudaMemsetAsync(d.fix, 0, P.R * sizeof(FixScale), s);
     g_launches += 3;
-    k_fix_start<<<gridsz(G0.cells, 256), 256, 0, s>>>(L0.phi, reinterpret_cast<double*>(d.phi_prev), ex, d.have_prev,
-                                                     L0.rhs, G0, bc_top * (L0.h * L0.h), d.fix);
-    k_fix_scale<<<1, 1, 0, s>>>(d.fix, P.E0 * (P.hi[2] - P.lo[2]), G0.n, ex && d.have_prev, 0);
-    k_fix_load<<<gridsz(G0.cells, 256), 256, 0, s>>>(L0.phi, L0.rhs, L0.phi_fix, L0.rhs_fix, G0.cells, d.fix, 0);
+    k_fix_start<<<grid_per_real(G0), 256, 0, s>>>(L0.phi, reinterpret_cast<double*>(d.phi_prev), ex, d.have_prev, L0.rhs,
+                                                  G0, bc_top * (L0.h * L0.h), d.fix);
+    k_fix_scale<<<(P.R + 255) / 256, 256, 0, s>>>(d.fix, P.R, P.E0 * (P.hi[2] - P.lo[2]), G0.n, ex && d.have_prev, 0);
+    k_fix_load<<<grid_per_real(G0), 256, 0, s>>>(L0.phi, L0.rhs, L0.phi_fix, L0.rhs_fix, G0.cells / P.R, d.fix, 0);
     if (ex) d.have_prev = true;
     d.fix_result = true;
 }
@@ -1908,7 +1940,7 @@ int field_solve(const Params& P, Dev& d, int precision, double rtol, int nu1, in
     const int nblk = (int)(G0.cells / ((uint64_t)NORM_TPB * items));
     const int bpr = nblk / R;
     const MarchGeo march = march_geo(G0.n);     // the integer residuals' blocks
-    double* h_norm = d.norm_host;       // 2 R + FIX_DOUBLES doubles of host memory owned by the caller
+    double* h_norm = d.norm_host;       // R (2 + FIX_DOUBLES) doubles of host memory owned by the caller
     double bnorm[MAX_REAL_NORM];
     if (R > MAX_REAL_NORM) return -1;
     double worst = 0.0;
@@ -1961,7 +1993,7 @@ int field_solve(const Params& P, Dev& d, int precision, double rtol, int nu1, in
         ++g_launches;
         k_norm_final<<<R, 256, 0, s>>>(d.norm_part, fixed || fix ? march.bpr : bpr, R, d.norm_out);
         cudaMemcpyAsync(h_norm, d.norm_out, 2 * R * sizeof(double), cudaMemcpyDeviceToHost, s);
-        if (fix) cudaMemcpyAsync(h_norm + 2 * R, d.fix, sizeof(FixScale), cudaMemcpyDeviceToHost, s);
+        if (fix) cudaMemcpyAsync(h_norm + 2 * R, d.fix, R * sizeof(FixScale), cudaMemcpyDeviceToHost, s);
         if (cudaStreamSynchronize(s) != cudaSuccess) return -3;
         worst = 0.0;
         bool done = true;
@@ -1973,15 +2005,18 @@ int field_solve(const Params& P, Dev& d, int precision, double rtol, int nu1, in
             if (!(rn <= rtol * bn)) done = false;
         }
         if (fix) {
-            FixScale fs;
-            std::memcpy(&fs, h_norm + 2 * R, sizeof fs);
+            const FixScale* fs = reinterpret_cast<const FixScale*>(h_norm + 2 * R);
+            bool range = std::isfinite(worst), finer = false;
+            for (int r = 0; r < R; ++r) {
+                range = range && !fs[r].use64 && fs[r].max_fix < (unsigned long long)FIX_LIM;
+                finer = finer || fix_shift(fs[r]) > 0;
+            }
             // out of the integer range, or no further progress in it: the
             // potential reached so far goes on in FP64 cycles
-            const bool range = !fs.use64 && fs.max_fix < (unsigned long long)FIX_LIM && std::isfinite(worst);
             if (!range || (!done && prev_rel >= 0.0 && worst > 0.9 * prev_rel)) {
                 if (range) {
                     ++g_launches;
-                    k_fix_store<<<gridsz(G0.cells, 256), 256, 0, s>>>(L0.phi_fix, L0.phi, G0.cells, d.fix);
+                    k_fix_store<<<grid_per_real(G0), 256, 0, s>>>(L0.phi_fix, L0.phi, per_real, d.fix);
                 }
                 fix = false;
                 d.fix_result = false;
@@ -1990,15 +2025,11 @@ int field_solve(const Params& P, Dev& d, int precision, double rtol, int nu1, in
                 continue;
             }
             // a loose bound left the leading bits unused: more of them
-            if (!done && cyc > 0 && fs.max_fix && fs.max_fix < (1ull << 52)) {
-                int lead = 0;
-                while ((fs.max_fix >> lead) > 1) ++lead;
-                const int sh = 55 - lead;
+            if (!done && cyc > 0 && finer) {
                 g_launches += 2;
-                k_fix_scale<<<1, 1, 0, s>>>(d.fix, P.E0 * (P.hi[2] - P.lo[2]), G0.n, 0, sh);
-                k_fix_load<<<gridsz(G0.cells, 256), 256, 0, s>>>(L0.phi, L0.rhs, L0.phi_fix, L0.rhs_fix, G0.cells, d.fix,
-                                                                sh);
-                for (int r = 0; r < R; ++r) bnorm[r] = std::ldexp(bnorm[r], 2 * sh);
+                k_fix_scale<<<(R + 255) / 256, 256, 0, s>>>(d.fix, R, P.E0 * (P.hi[2] - P.lo[2]), G0.n, 0, 1);
+                k_fix_load<<<grid_per_real(G0), 256, 0, s>>>(L0.phi, L0.rhs, L0.phi_fix, L0.rhs_fix, per_real, d.fix, 1);
+                for (int r = 0; r < R; ++r) bnorm[r] = std::ldexp(bnorm[r], 2 * fix_shift(fs[r]));
             }
         }
         if (done) { status = 0; break; }
@@ -2507,7 +2538,7 @@ extern "C" int itokmc_field_solve_noalloc(const itokmc_config* cfg, const int64_
         set_global_error("field_solve_noalloc: scratch layout exceeds the static array");
         return ITOKMC_ERR_ARG;
     }
-    double norm_host[2 + FIX_DOUBLES]; // stack memory: no allocation
+    alignas(FixScale) double norm_host[2 + FIX_DOUBLES];   // stack memory: no allocation
     d.norm_host = norm_host;
     const double dV = P.h[0] * P.h[1] * P.h[2];
     const double qscale = 1.602176634e-19 * ldexp(1.0, -3 * P.frac_bits) / dV;

@@ -94,11 +94,11 @@ struct MGLevel {
 };
 
 // Scale of the FP64 form's fixed-point potential (device memory, one per
-// handle): Phi = phi 2^F, down = 2^-F, top the electrode potential; the
-// largest |phi|, |h^2 b| (bits of the doubles) and |Phi|; use64: the integers
-// cannot hold this solve.
+// realization): Phi = phi 2^F, down = 2^-F, top the electrode potential; the
+// largest |phi|, |h^2 b| (bits of the doubles) and |Phi|; sh: bits of the last
+// change of F; use64: the integers cannot hold this solve.
 struct FixScale {
-    int F, use64;
+    int F, sh, use64, pad;
     double down;
     long long top;
     unsigned long long max_phi, max_b, max_fix;
@@ -152,8 +152,8 @@ struct Dev {
     MGLevel lev[MAX_LEVELS];
     int nlev = 0;
     double* norm_part = nullptr;  double* norm_out = nullptr;  size_t norm_blocks = 0;
-    double* norm_host = nullptr;       // 2 R + FIX_DOUBLES doubles (pinned or stack) for the readback of a check
-    FixScale* fix = nullptr;           // FP64 form: the fixed-point scale
+    double* norm_host = nullptr;       // R (2 + FIX_DOUBLES) doubles (pinned or stack) for the readback of a check
+    FixScale* fix = nullptr;           // FP64 form: the fixed-point scales
     bool fix_result = false;           // the last solve's potential is in phi_fix (launch_efield_to stores it)
     // counters
     Counters* ctr = nullptr;

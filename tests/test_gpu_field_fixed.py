@@ -1,10 +1,11 @@
 """The FP64 form's solve in 64-bit fixed point keeps what FP64 cycles give: the
-residual norms in FP64."""
+residual norms in FP64, and a scale per realization."""
+import numpy as np
 import pytest
 
 from gpu_util import small_phys
 from paper_2307_01797_gb300 import itokmc
-from test_gpu_field_forms import rel_residual
+from test_gpu_field_forms import TOL, charges, rel_residual
 
 pytestmark = pytest.mark.gpu
 
@@ -13,10 +14,9 @@ pytestmark = pytest.mark.gpu
 def test_norms_are_fp64(n, ions):
     # a uniform charge: the sum of equal squares rounds the same way all along,
     # up to 2^-24 per term of a partial sum in FP32.  In FP64: 2^-53 per term
-    # and level of the sum (below 1e-14), and the rounding of the potential
-    # to FP64, 12 * 2^-53 |phi| per cell against a residual of 1e-3 b or more
-    # with |phi| < b n^2 / 8 (below 1e-9 at n = 64 if all signs agreed; they do
-    # not: 2^18 cells of either sign leave 2^-9 of it)
+    # and level of the sum (below 1e-14), and the rounding of the potential to
+    # FP64: 12 * 2^-53 |phi| per cell, |phi| < b n^2 / 8, of either sign over
+    # n^3 cells whose residual is 1e-2 b or more (below 2e-12 at n = 64)
     import torch
     ph = small_phys(n, E0=0.0, mg_rtol=0.2)
     rho = torch.full((n ** 3,), ions << 30, dtype=torch.int64, device="cuda")
@@ -26,3 +26,31 @@ def test_norms_are_fp64(n, ions):
     assert 1e-3 < rel <= 0.2
     want = rel_residual(phi.cpu().numpy(), rho.cpu().numpy(), ph)
     assert abs(rel - want) <= 1e-11 * want
+
+
+def bits_held(phi):
+    """Bits between the leading one of the largest |phi| and the last one set
+    in any value of at least a quarter of it."""
+    a = np.abs(phi)
+    m, e = np.frexp(a[a >= a.max() / 4])
+    mant = (m * 2.0 ** 53).astype(np.int64)
+    last = min(int(ee) - 53 + (int(v) & -int(v)).bit_length() - 1 for v, ee in zip(mant, e))
+    return int(np.frexp(a.max())[1]) - last
+
+
+@pytest.mark.parametrize("n", [16, 64])
+def test_a_weak_member_beside_a_strong_one(n):
+    # the strong member's potential is 2e4 times and more the weak ones'; FP64
+    # cycles hold 53 bits of each (54 and 55 where values of the next lower
+    # binades show), one scale for all leaves 39 to 42
+    ph = small_phys(n, E0=0.0)
+    H = itokmc.Handle(itokmc.make_config(ph, 100, realizations=3))
+    pos = np.concatenate([charges("cloud", n, 0), np.full(n ** 3, 10 ** 6), charges("cloud", n, 1)])
+    H.itokmc_set_ions(pos, np.zeros_like(pos))
+    H.itokmc_solve_field()
+    phi = H.itokmc_read_densities(itokmc.PHI, -1).reshape(3, -1)
+    rho = H.itokmc_read_densities(itokmc.RHO, -1).reshape(3, -1)
+    for r in range(3):
+        assert rel_residual(phi[r], rho[r], ph) <= TOL
+        assert bits_held(phi[r]) >= 53
+    H.close()
