@@ -409,9 +409,10 @@ __global__ void __launch_bounds__(NORM_TPB) k_resid_norm(const double* __restric
 }
 
 // Per realization (one block each): fixed-order strided sums, then a fixed
-// tree in shared memory -- the same result on every run.
+// tree in shared memory -- the same result on every run.  fs (FP64 form): the
+// largest |Phi| of the check is closed.
 __global__ void __launch_bounds__(256) k_norm_final(const double* __restrict__ part, int blocks_per_real, int R,
-                                                    double* __restrict__ out)
+                                                    double* __restrict__ out, FixScale* __restrict__ fs = nullptr)
 {
     __shared__ double sa[256], sb[256];
     const int r = blockIdx.x;
@@ -433,6 +434,10 @@ __global__ void __launch_bounds__(256) k_norm_final(const double* __restrict__ p
     if (threadIdx.x == 0) {
         out[2 * r] = sa[0];
         out[2 * r + 1] = sb[0];
+        if (fs) {
+            fs[r].seen = fs[r].max_fix;
+            fs[r].max_fix = 0;
+        }
     }
 }
 
@@ -583,14 +588,26 @@ __global__ void k_efield_fixed(const long long* __restrict__ Phi, E64* __restric
 // FP64 cycles.
 constexpr long long FIX_LIM = 1ll << 59;
 
-// The bits by which a scale can go up that a loose bound (k_fix_scale) left
-// too low: the largest |Phi| to [2^55, 2^56).
+// The bits by which a scale can go up that a loose bound (k_fix_scale) left too
+// low: the largest |Phi| (seen) holds fewer bits than a double.  It goes to [2^55,
+// 2^56); B (from max_b) and the electrode stay below 2^60 and 2^58.
+constexpr int FIX_BITS = 53;
+__host__ __device__ inline int lead_bit(unsigned long long v)
+{
+    int l = 0;
+    while ((v >> l) > 1) ++l;
+    return l;
+}
 __host__ __device__ inline int fix_shift(const FixScale& f)
 {
-    if (f.max_fix == 0 || f.max_fix >= (1ull << 52)) return 0;
-    int lead = 0;
-    while ((f.max_fix >> lead) > 1) ++lead;
-    return 55 - lead;
+    if (f.seen == 0 || f.seen >= (1ull << FIX_BITS)) return 0;
+    if (f.max_b == 0 && f.top == 0) return 0;      // no charge and no applied field: the guess decays to zero
+    int sh = 55 - lead_bit(f.seen);
+    const int eb = (int)(f.max_b >> 52) - 1023 + f.F;          // |B| < 2^(eb + 1)
+    if (f.max_b && sh > 58 - eb) sh = 58 - eb;
+    const int et = lead_bit((unsigned long long)(f.top < 0 ? -f.top : f.top));
+    if (f.top && sh > 56 - et) sh = 56 - et;
+    return sh > 0 ? sh : 0;
 }
 
 // x 2^F rounded to the nearest integer, |x| 2^F < 2^62, by integer steps.
@@ -657,20 +674,22 @@ __global__ void __launch_bounds__(256) k_fix_start(double* __restrict__ phi, dou
 // The scale of each realization.  Mc bounds |phi| of the solution: electrode potential plus the
 // 1D Dirichlet bound max|h^2 b| n^2 / 8, doubled.  A guess extrapolated from
 // the last steps is near the solution: four times its modulus bounds it (Mc
-// is loose by orders of magnitude for a localised charge).  use64: the guess
-// is not finite or far above the solution.
+// is loose by orders of magnitude for a localised charge; a single cell's
+// potential is about a quarter of its |h^2 b|, so that at least FIX_BITS bits
+// hold it).  use64: the guess is not finite or far above the solution.
 __global__ void k_fix_scale(FixScale* fs, int R, double phi_top, int n, int near, int rescale)
 {
     const int r = blockIdx.x * blockDim.x + threadIdx.x;
     if (r >= R) return;
     fs += r;
+    if (rescale == 2) fs->seen = fs->max_fix;                   // of k_fix_max
     fs->sh = rescale ? fix_shift(*fs) : 0;
     if (rescale) {                                              // of a running solve
         fs->F += fs->sh;
     } else {
         const double mp = __longlong_as_double((long long)fs->max_phi), mb = __longlong_as_double((long long)fs->max_b);
         const double Mc = 2.0 * (fabs(phi_top) + mb * (double)n * (double)n / 8.0);
-        double M = near && mp * 16384.0 >= Mc ? fmin(Mc, fmax(4.0 * mp, 2.0 * (mb + fabs(phi_top)))) : fmax(Mc, 2.0 * mp);
+        double M = near && mp > 0.0 ? fmin(Mc, fmax(4.0 * mp, 2.0 * (mb + fabs(phi_top)))) : fmax(Mc, 2.0 * mp);
         M = fmax(M, 0x1p-400);
         fs->use64 = !(mp <= 16.0 * Mc) || !(Mc < 0x1p400);
         if (!(M < 0x1p400)) M = 1.0;
@@ -679,6 +698,24 @@ __global__ void k_fix_scale(FixScale* fs, int R, double phi_top, int n, int near
     fs->max_fix = 0;
     fs->down = scalbn(1.0, -fs->F);
     fs->top = to_fixed(phi_top, fs->F);
+}
+
+// The largest |Phi|.  Block row r: realization r.
+__global__ void __launch_bounds__(256) k_fix_max(const long long* __restrict__ Phi, uint64_t n3, FixScale* __restrict__ fs)
+{
+    const uint64_t o = blockIdx.y * n3;
+    unsigned long long mx = 0;
+    for (uint64_t t = o + blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; t < o + n3; t += (uint64_t)gridDim.x * blockDim.x) {
+        const long long v = Phi[t];
+        const unsigned long long a = (unsigned long long)(v < 0 ? -v : v);
+        mx = a > mx ? a : mx;
+    }
+#pragma unroll
+    for (int d = 16; d > 0; d >>= 1) {
+        const unsigned long long a = __shfl_xor_sync(0xffffffffu, mx, d);
+        mx = a > mx ? a : mx;
+    }
+    if ((threadIdx.x & 31) == 0) atomicMax(&fs[blockIdx.y].max_fix, mx);
 }
 
 // Phi and B from phi and the right-hand side; rescale: Phi shifted up by sh
@@ -1912,7 +1949,8 @@ void lower_phi_scale(const Params& P, Dev& d, int F, cudaStream_t s)
 }
 
 // FP64 form, before the cycles: start guess, scale, Phi and B.
-void fix_begin(const Params& P, Dev& d, bool extrapolate, cudaStream_t s)
+// Returns whether the scale was taken from the guess (else from the bound).
+bool fix_begin(const Params& P, Dev& d, bool extrapolate, cudaStream_t s)
 {
     MGLevel& L0 = d.lev[0];
     const Geo G0 = geo(d, 0, P.R);
@@ -1925,8 +1963,10 @@ void fix_begin(const Params& P, Dev& d, bool extrapolate, cudaStream_t s)
                                                   G0, bc_top * (L0.h * L0.h), d.fix);
     k_fix_scale<<<(P.R + 255) / 256, 256, 0, s>>>(d.fix, P.R, P.E0 * (P.hi[2] - P.lo[2]), G0.n, ex && d.have_prev, 0);
     k_fix_load<<<grid_per_real(G0), 256, 0, s>>>(L0.phi, L0.rhs, L0.phi_fix, L0.rhs_fix, G0.cells / P.R, d.fix, 0);
+    const bool near = ex && d.have_prev;
     if (ex) d.have_prev = true;
     d.fix_result = true;
+    return near;
 }
 
 int field_solve(const Params& P, Dev& d, int precision, double rtol, int nu1, int nu2, unsigned long long rho_absmax,
@@ -1967,7 +2007,8 @@ int field_solve(const Params& P, Dev& d, int precision, double rtol, int nu1, in
             d.have_prev = true;
         }
     }
-    if (fix) fix_begin(P, d, extrapolate, s);
+    bool near = false;                  // fixed point: the scale is from a guess that ought to be near
+    if (fix) near = fix_begin(P, d, extrapolate, s);
     const float rsc = (float)std::ldexp(1.0, -d.phi_F);
     const float esc = (float)std::ldexp(1.0, d.phi_F);
     // FP64 form: the residual norm only serves the convergence test, so
@@ -1975,6 +2016,7 @@ int field_solve(const Params& P, Dev& d, int precision, double rtol, int nu1, in
     // convergence factor predicts (refinement forms need the residual every
     // outer iteration as the right-hand side of the correction).
     int next_check = 0;
+    bool first = true;                  // the check takes the right-hand sides' norms too
     double rho_est = 0.1, prev_rel = -1.0;
     int prev_cyc = 0;
     for (cyc = 0; cyc <= max_cycles; ++cyc) {
@@ -1984,54 +2026,74 @@ int field_solve(const Params& P, Dev& d, int precision, double rtol, int nu1, in
         }
         ++g_launches;
         if (fixed)
-            k_resid_fixed<<<R * march.bpr, NORM_TPB, 0, s>>>(Phi, Bfix, L0.rhs32, G0, rsc, d.norm_part, cyc == 0, march);
+            k_resid_fixed<<<R * march.bpr, NORM_TPB, 0, s>>>(Phi, Bfix, L0.rhs32, G0, rsc, d.norm_part, first, march);
         else if (fix)
-            k_resid_norm_fix<<<R * march.bpr, NORM_TPB, 0, s>>>(L0.phi_fix, L0.rhs_fix, G0, d.norm_part, cyc == 0, march, d.fix);
+            k_resid_norm_fix<<<R * march.bpr, NORM_TPB, 0, s>>>(L0.phi_fix, L0.rhs_fix, G0, d.norm_part, first, march, d.fix);
         else
             k_resid_norm<<<nblk, NORM_TPB, 0, s>>>(L0.phi, L0.rhs, precision == 1 ? L0.rhs32 : nullptr, G0,
-                                                   d.norm_part, prev_rel < 0.0, items);
+                                                   d.norm_part, first, items);
         ++g_launches;
-        k_norm_final<<<R, 256, 0, s>>>(d.norm_part, fixed || fix ? march.bpr : bpr, R, d.norm_out);
+        k_norm_final<<<R, 256, 0, s>>>(d.norm_part, fixed || fix ? march.bpr : bpr, R, d.norm_out, fix ? d.fix : nullptr);
         cudaMemcpyAsync(h_norm, d.norm_out, 2 * R * sizeof(double), cudaMemcpyDeviceToHost, s);
         if (fix) cudaMemcpyAsync(h_norm + 2 * R, d.fix, R * sizeof(FixScale), cudaMemcpyDeviceToHost, s);
         if (cudaStreamSynchronize(s) != cudaSuccess) return -3;
         worst = 0.0;
         bool done = true;
         for (int r = 0; r < R; ++r) {
-            if (prev_rel < 0.0) bnorm[r] = h_norm[2 * r + 1];
+            if (first) bnorm[r] = h_norm[2 * r + 1];
             const double rn = std::sqrt(h_norm[2 * r]), bn = std::sqrt(bnorm[r]);
             const double rel = bn > 0.0 ? rn / bn : rn;
             if (rel > worst || !(rel == rel)) worst = rel;
             if (!(rn <= rtol * bn)) done = false;
         }
+        first = false;
+        bool few = false;               // a scale that may be too low
         if (fix) {
             const FixScale* fs = reinterpret_cast<const FixScale*>(h_norm + 2 * R);
             bool range = std::isfinite(worst), finer = false;
             for (int r = 0; r < R; ++r) {
-                range = range && !fs[r].use64 && fs[r].max_fix < (unsigned long long)FIX_LIM;
+                range = range && !fs[r].use64 && fs[r].seen < (unsigned long long)FIX_LIM;
                 finer = finer || fix_shift(fs[r]) > 0;
+                const unsigned long long top = (unsigned long long)(fs[r].top < 0 ? -fs[r].top : fs[r].top);
+                few = few || (bnorm[r] > 0.0 && std::max(fs[r].seen, top) < (1ull << (FIX_BITS + 1)));
             }
-            // out of the integer range, or no further progress in it: the
-            // potential reached so far goes on in FP64 cycles
-            if (!range || (!done && prev_rel >= 0.0 && worst > 0.9 * prev_rel)) {
+            if (range && finer && cyc > 0 && cyc < max_cycles) {
+                // a loose bound left the leading bits unused: more of them, and
+                // a cycle that fills them
+                g_launches += 2;
+                k_fix_scale<<<(R + 255) / 256, 256, 0, s>>>(d.fix, R, P.E0 * (P.hi[2] - P.lo[2]), G0.n, 0, 1);
+                k_fix_load<<<grid_per_real(G0), 256, 0, s>>>(L0.phi, L0.rhs, L0.phi_fix, L0.rhs_fix, per_real, d.fix, 1);
+                first = true;
+                done = false;
+            } else if (!range && near) {
+                // the solution is far above the guess: once more, at the bound's scale
+                near = false;
+                g_launches += 2;
+                k_fix_scale<<<(R + 255) / 256, 256, 0, s>>>(d.fix, R, P.E0 * (P.hi[2] - P.lo[2]), G0.n, 0, 0);
+                k_fix_load<<<grid_per_real(G0), 256, 0, s>>>(L0.phi, L0.rhs, L0.phi_fix, L0.rhs_fix, per_real, d.fix, 0);
+                first = true;
+                prev_rel = -1.0;
+                next_check = 0;
+                cyc = -1;
+                continue;
+            } else if (!range || (!done && prev_rel >= 0.0 && worst > 0.9 * prev_rel)) {
+                // out of the integer range (the cycles start again from the
+                // guess), or no further progress in it (they go on): FP64 cycles
                 if (range) {
                     ++g_launches;
                     k_fix_store<<<grid_per_real(G0), 256, 0, s>>>(L0.phi_fix, L0.phi, per_real, d.fix);
                 }
                 fix = false;
                 d.fix_result = false;
+                first = true;
                 prev_rel = -1.0;
-                --cyc;                                  // the same check again, in FP64
+                cyc = range ? cyc - 1 : -1;                 // the check again, in FP64
+                next_check = cyc + 1;
                 continue;
             }
-            // a loose bound left the leading bits unused: more of them
-            if (!done && cyc > 0 && finer) {
-                g_launches += 2;
-                k_fix_scale<<<(R + 255) / 256, 256, 0, s>>>(d.fix, R, P.E0 * (P.hi[2] - P.lo[2]), G0.n, 0, 1);
-                k_fix_load<<<grid_per_real(G0), 256, 0, s>>>(L0.phi, L0.rhs, L0.phi_fix, L0.rhs_fix, per_real, d.fix, 1);
-                for (int r = 0; r < R; ++r) bnorm[r] = std::ldexp(bnorm[r], 2 * fix_shift(fs[r]));
-            }
         }
+        // a guess that needs no cycle stays as it is
+        if (fix && done && cyc == 0 && !near) d.fix_result = false;
         if (done) { status = 0; break; }
         if (cyc == max_cycles || !std::isfinite(worst)) break;
         if (precision == 0) {
@@ -2054,6 +2116,15 @@ int field_solve(const Params& P, Dev& d, int precision, double rtol, int nu1, in
                 k_add_correction<<<gridsz(G0.cells, 256), 256, 0, s>>>(L0.phi, L0.phi32, G0.cells);
         } else {
             run_cycles(d, fix ? 3 : 0, R, nu1, nu2, s);
+            if (fix && few && cyc == 0 && !near) {
+                // after one cycle the potential is known well enough for a
+                // scale that the bound left too low (no wait for it)
+                g_launches += 3;
+                k_fix_max<<<grid_per_real(G0), 256, 0, s>>>(L0.phi_fix, per_real, d.fix);
+                k_fix_scale<<<(R + 255) / 256, 256, 0, s>>>(d.fix, R, P.E0 * (P.hi[2] - P.lo[2]), G0.n, 0, 2);
+                k_fix_load<<<grid_per_real(G0), 256, 0, s>>>(L0.phi, L0.rhs, L0.phi_fix, L0.rhs_fix, per_real, d.fix, 1);
+                first = true;
+            }
         }
     }
     if (cycles_out) *cycles_out = cyc;

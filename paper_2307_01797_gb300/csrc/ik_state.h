@@ -95,13 +95,14 @@ struct MGLevel {
 
 // Scale of the FP64 form's fixed-point potential (device memory, one per
 // realization): Phi = phi 2^F, down = 2^-F, top the electrode potential; the
-// largest |phi|, |h^2 b| (bits of the doubles) and |Phi|; sh: bits of the last
-// change of F; use64: the integers cannot hold this solve.
+// largest |phi|, |h^2 b| (bits of the doubles) and |Phi| (max_fix while it is
+// taken, seen: of the last check); sh: bits of the last change of F; use64: the
+// integers cannot hold this solve.
 struct FixScale {
     int F, sh, use64, pad;
     double down;
     long long top;
-    unsigned long long max_phi, max_b, max_fix;
+    unsigned long long max_phi, max_b, max_fix, seen;
 };
 constexpr int FIX_DOUBLES = (int)(sizeof(FixScale) / sizeof(double));
 

@@ -1,5 +1,6 @@
 """The FP64 form's solve in 64-bit fixed point keeps what FP64 cycles give: the
-residual norms in FP64, and a scale per realization."""
+residual norms in FP64, a scale per realization, at least the 53 bits of a
+double for the largest potential, whatever the start guess."""
 import numpy as np
 import pytest
 
@@ -53,4 +54,58 @@ def test_a_weak_member_beside_a_strong_one(n):
     for r in range(3):
         assert rel_residual(phi[r], rho[r], ph) <= TOL
         assert bits_held(phi[r]) >= 53
+    H.close()
+
+
+def bits_of_largest(phi):
+    """Bits between the leading one of the largest |phi| and the last one set
+    in any value: the step in which the potential is held (n^3 values do not
+    all have a last bit of zero; a single value does every other time)."""
+    m, e = np.frexp(np.abs(phi[phi != 0.0]))
+    mant = (m * 2.0 ** 53).astype(np.int64)
+    low = np.log2((mant & -mant).astype(np.float64)).astype(np.int64)
+    return int(e.max() - (e.astype(np.int64) - 53 + low).min())
+
+
+@pytest.mark.parametrize("rtol", [1e-3, 1e-10])
+@pytest.mark.parametrize("kind", ["point", "corner", "cloud"])
+@pytest.mark.parametrize("n", [16, 64])
+def test_the_largest_potential_has_53_bits(n, kind, rtol):
+    # the bound from which a scale is taken is 2^12 above a single cell's potential
+    ph = small_phys(n, E0=0.0, mg_rtol=rtol)
+    H = itokmc.Handle(itokmc.make_config(ph, 100))
+    pos, none = charges(kind, n, 1), np.zeros(n ** 3, np.int64)
+    H.itokmc_set_ions(pos, none)
+    H.itokmc_solve_field()
+    phi = H.itokmc_read_densities(itokmc.PHI)
+    assert rel_residual(phi, H.itokmc_read_densities(itokmc.RHO), ph) <= 1.02 * rtol
+    assert bits_of_largest(phi) >= 53
+    # the same charge again: the guess needs no cycle and stays as it is
+    H.itokmc_solve_field()
+    if H.itokmc_get_stats()["mg_cycles"] == 0:
+        assert np.array_equal(H.itokmc_read_densities(itokmc.PHI), phi)
+    # a weaker charge: the guess' leading bits are not the solution's
+    H.itokmc_set_ions(charges("corner", n, 1), none)
+    H.itokmc_solve_field()
+    phi = H.itokmc_read_densities(itokmc.PHI)
+    assert rel_residual(phi, H.itokmc_read_densities(itokmc.RHO), ph) <= 1.02 * rtol
+    assert bits_of_largest(phi) >= 53
+    H.close()
+
+
+@pytest.mark.parametrize("factor", [30, 10 ** 6])
+@pytest.mark.parametrize("n,graph", [(16, 0), (64, 0), (16, 1)])
+def test_a_charge_that_jumps_between_steps(n, graph, factor):
+    # steps take their scale from the extrapolated potential
+    ph = small_phys(n, E0=0.0)
+    H = itokmc.Handle(itokmc.make_config(ph, 10000, graph_step=graph))
+    c = (np.arange(8) + 0.5) * (ph["hi"][0] - ph["lo"][0]) / 8 + ph["lo"][0]
+    H.itokmc_set_particles(c, c, c, np.ones(8, np.uint32))
+    none = np.zeros(n ** 3, np.int64)
+    for scale in (1, factor, 1):
+        H.itokmc_set_ions(scale * charges("cloud", n, 2), none)
+        for _ in range(3):
+            H.itokmc_step(1)
+            rho = H.itokmc_read_densities(itokmc.RHO)
+            assert rel_residual(H.itokmc_read_densities(itokmc.PHI), rho, ph) <= TOL
     H.close()
