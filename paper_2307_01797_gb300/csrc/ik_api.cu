@@ -1015,8 +1015,7 @@ int itokmc_init(const itokmc_config* cfg, itokmc_handle** out)
     d.small_list = dalloc_n<uint32_t>(h, Gp, &rc);
     d.mid_list = dalloc_n<uint32_t>(h, Gp, &rc);
     d.big_list = dalloc_n<uint32_t>(h, Gp, &rc);
-    d.tie_list = dalloc_n<uint32_t>(h, Gp, &rc);
-    d.list_n = dalloc_n<uint32_t>(h, 4, &rc);
+    d.list_n = dalloc_n<uint32_t>(h, 5, &rc);
     d.pc_list = dalloc_n<uint32_t>(h, G, &rc);
     d.kmc_list = dalloc_n<uint32_t>(h, G, &rc);
     d.kmc_n = dalloc_n<uint32_t>(h, 1, &rc);

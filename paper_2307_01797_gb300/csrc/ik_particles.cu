@@ -1637,7 +1637,7 @@ struct MergeScanOp {
         list_n[0] = (uint32_t)t[2];
         list_n[1] = (uint32_t)t[3];
         list_n[2] = (uint32_t)t[4];
-        list_n[3] = 0;            // cells that the merge by presorted lists leaves to k_merge_lv
+        list_n[3] = list_n[4] = 0;   // cells of tiers 0 and 1 that the merge by presorted lists leaves to k_merge_lv
     }
 };
 
@@ -2300,10 +2300,15 @@ __global__ void __launch_bounds__(128, GLOBAL ? 4 : (std::is_same<E, MP32>::valu
 // of the weight.  A position's word holds the entries of the x, y and z list
 // there (one byte each) and its node.  The last level needs no lists: its
 // leaves are ranges of the lists it splits.
-// The order of equal coordinates depends on the splits before, which the
-// presorted lists do not know: cells with two equal coordinates along an axis
-// (as after a split of one particle without diffusion), and cells of 2^31
-// electrons or more (the sums here have 32 bits), are listed for k_merge_lv.
+// The order of two elements with equal coordinates along an axis depends on the
+// splits before.  Copies (equal along all axes, as after a split of one particle
+// without diffusion) keep the cell's order through every stable sort, so they
+// take it in all three lists.  Cells with two elements that are equal along one
+// axis and not along another, and cells of 2^31 electrons or more (the sums here
+// have 32 bits), are listed for k_merge_lv, which sorts per level.  46000 cells
+// on 64^3 without diffusion, two thirds of them with copies: 250 us in the FP64
+// form and 175 us in the mixed one (365 and 220 us with all of those sorted per
+// level; k_merge_lv alone for every cell 250 and 148 us).
 // Bound by instruction issue (80% of the slots; about 4000 per warp and cell
 // of 28 elements, k_merge_lv twice that in the FP64 form); seven blocks per SM
 // measured best of six to nine.
@@ -2345,6 +2350,69 @@ __host__ __device__ inline PreLayout pre_layout(uint32_t cap, uint32_t T, uint32
     L.med = ml_take(o, T * (uint32_t)sizeof(MMed));
     L.bytes = o;
     return L;
+}
+
+// Keys below k among the first M of ka, read by 16 bytes (the keys from M on to
+// the next multiple of them are not below any).
+__device__ __forceinline__ uint32_t count_below(const uint32_t* ka, uint32_t M, uint32_t k)
+{
+    uint32_t n = 0;
+#pragma unroll 2
+    for (uint32_t i = 0; i < M; i += 4) {
+        const uint4 q = *reinterpret_cast<const uint4*>(ka + i);
+        n += (q.x < k) + (q.y < k) + (q.z < k) + (q.w < k);
+    }
+    return n;
+}
+__device__ __forceinline__ uint32_t count_below(const unsigned long long* ka, uint32_t M, unsigned long long k)
+{
+    uint32_t n = 0;
+#pragma unroll 2
+    for (uint32_t i = 0; i < M; i += 2) {
+        const ulonglong2 q = *reinterpret_cast<const ulonglong2*>(ka + i);
+        n += (q.x < k) + (q.y < k);
+    }
+    return n;
+}
+
+// The three lists of a cell with equal keys, these in the cell's order; returns
+// whether it holds for the levels too: no two elements are equal along one axis
+// and not along another.  (Not inlined: it would cost the kernel registers.)
+template <class K>
+__device__ __noinline__ bool rank_copies(const K* key0, uint32_t KS, uint32_t* ls, uint32_t M, unsigned lane)
+{
+    const unsigned full = 0xffffffffu;
+    __syncwarp();
+#pragma unroll 1
+    for (int a = 0; a < 3; ++a) {
+        const K* ka = key0 + a * KS;
+        for (uint32_t b0 = 0; b0 < M; b0 += 32) {
+            const uint32_t j = b0 + lane;
+            const bool ok = j < M;
+            const K kj = ka[ok ? j : 0];
+            uint32_t rk = count_below(ka, M, kj);
+            // equal ones before it: in the warp's chunk, and in the chunks before
+            rk += __popc(__match_any_sync(full, ok ? rk : 0x10000u + lane) & ((1u << lane) - 1u));
+            for (uint32_t k = 0; k < b0; ++k) rk += ka[k] == kj;
+            if (ok) {
+                uint8_t* w = reinterpret_cast<uint8_t*>(ls + rk);
+                w[a] = (uint8_t)j;
+                if (a == 0) w[3] = 0;
+            }
+        }
+    }
+    __syncwarp();
+    bool differ = false;
+    for (uint32_t j = lane; j + 1 < M; j += 32) {
+        const uint32_t w0 = ls[j], w1 = ls[j + 1];
+#pragma unroll
+        for (int a = 0; a < 3; ++a) {
+            const K *k0 = key0 + ((w0 >> (8 * a)) & 255u), *k1 = key0 + ((w1 >> (8 * a)) & 255u);
+            const int same = (k0[0] == k1[0]) + (k0[KS] == k1[KS]) + (k0[2 * KS] == k1[2 * KS]);
+            differ |= k0[a * KS] == k1[a * KS] && same < 3;
+        }
+    }
+    return !__any_sync(full, differ);
 }
 
 template <class E>
@@ -2404,20 +2472,7 @@ __global__ void __launch_bounds__(128, 7) k_merge_pre(
                 const uint32_t j = b0 + lane;
                 const bool ok = j < M;
                 const K kj = ka[ok ? j : 0];
-                uint32_t rk = 0;
-                if constexpr (MX) {
-#pragma unroll 2
-                    for (uint32_t k = 0; k < M; k += 4) {
-                        const uint4 q = *reinterpret_cast<const uint4*>(ka + k);
-                        rk += (q.x < kj) + (q.y < kj) + (q.z < kj) + (q.w < kj);
-                    }
-                } else {
-#pragma unroll 2
-                    for (uint32_t k = 0; k < M; k += 2) {
-                        const ulonglong2 q = *reinterpret_cast<const ulonglong2*>(ka + k);
-                        rk += (q.x < kj) + (q.y < kj);
-                    }
-                }
+                const uint32_t rk = count_below(ka, M, kj);
                 if (ok) {
                     uint8_t* w = reinterpret_cast<uint8_t*>(ls + rk);
                     w[a] = (uint8_t)j;
@@ -2430,10 +2485,11 @@ __global__ void __launch_bounds__(128, 7) k_merge_pre(
             }
             other |= __reduce_add_sync(FULL, total) != M * (M - 1) / 2;
         }
+        if (other) other = !rank_copies<K>(key0, KS, ls, M, lane);
 #pragma unroll
         for (int dd = 16; dd > 0; dd >>= 1) wroot += __shfl_xor_sync(FULL, wroot, dd);
         if (other || wroot >= (1ull << 31)) {
-            if (lane == 0) tie_list[atomicAdd(list_n + 3, 1u)] = (uint32_t)g;
+            if (lane == 0) tie_list[atomicAdd(list_n + 3 + tier, 1u)] = (uint32_t)g;
             __syncwarp();
             continue;
         }
@@ -3152,14 +3208,15 @@ void launch_merge_tiers(const Params& P, Dev& d, uint64_t G, cudaStream_t s, con
     const uint32_t cap0 = merge_cap0((int)sizeof(E));
     const size_t sm0 = (size_t)pre_layout(cap0, P.ppc, sizeof(K)).bytes * MERGE_NW0;
     const size_t sm1 = (size_t)pre_layout(MERGE_CAP1, P.ppc, sizeof(K)).bytes * MERGE_NW1;
-    const size_t smt = (size_t)merge_layout(MERGE_CAP1, P.ppc, sizeof(E), sizeof(K)).bytes * MERGE_NW1;
+    const size_t smt0 = (size_t)merge_layout(cap0, P.ppc, sizeof(E), sizeof(K)).bytes * MERGE_NW0;
+    const size_t smt1 = (size_t)merge_layout(MERGE_CAP1, P.ppc, sizeof(E), sizeof(K)).bytes * MERGE_NW1;
     static bool attr = false;
     if (!attr) {
         cudaFuncSetAttribute(k_merge_lv<E, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
         cudaFuncSetAttribute(k_merge_pre<E>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
         attr = true;
     }
-    g_launches += 4;
+    g_launches += 5;
     const uint64_t Gphys = (uint64_t)P.R * P.n3;
     // tiers 1 and 2 (few, long cells) on the side stream beside tier 0
     cudaStream_t s12 = s;
@@ -3168,24 +3225,26 @@ void launch_merge_tiers(const Params& P, Dev& d, uint64_t G, cudaStream_t s, con
         cudaStreamWaitEvent(d.side, d.side_fork, 0);
         s12 = d.side;
     }
-    auto pre = [&](cudaStream_t st, int blocks, size_t sm, const uint32_t* list, int tier, uint32_t CAP) {
+    // the cells that a tier's pass leaves follow it, with the tier's scratch;
+    // their lists lie in two arrays that only the transport fills
+    uint32_t* const left[2] = { reinterpret_cast<uint32_t*>(d.cnt_new), reinterpret_cast<uint32_t*>(d.in_cnt) };
+    auto tier = [&](cudaStream_t st, int t, int blocks, const uint32_t* list, uint32_t CAP, size_t sm, size_t smt) {
         k_merge_pre<E><<<blocks, 128, sm, st>>>(P, A, A32, d.cell_start, d.gain, d.photos, d.photo_sorted, d.photo_off,
                                                 d.out_start, out, out32, cout, Gphys, d.mover_cap, d.photo_cap, list,
-                                                d.list_n, tier, CAP, d.tie_list, d.ctr);
+                                                d.list_n, t, CAP, left[t], d.ctr);
+        k_merge_lv<E, false><<<blocks, 128, smt, st>>>(
+            P, A, A32, d.cell_start, d.gain, d.photos, d.photo_sorted, d.photo_off, d.out_start, d.work_off, d.work,
+            d.work_cap, out, out32, cout, Gphys, d.mover_cap, d.photo_cap, left[t], d.list_n, 3 + t, CAP, d.ctr);
     };
-    pre(s12, 152 * 8, sm1, d.mid_list, 1, MERGE_CAP1);
+    tier(s12, 1, 152 * 8, d.mid_list, MERGE_CAP1, sm1, smt1);
     k_merge_lv<E, true><<<152 * 4, 128, 0, s12>>>(
         P, A, A32, d.cell_start, d.gain, d.photos, d.photo_sorted, d.photo_off, d.out_start, d.work_off, d.work,
         d.work_cap, out, out32, cout, Gphys, d.mover_cap, d.photo_cap, d.big_list, d.list_n, 2, 0, d.ctr);
-    pre(s, 152 * 16, sm0, d.small_list, 0, cap0);
+    tier(s, 0, 152 * 16, d.small_list, cap0, sm0, smt0);
     if (d.side) {
         cudaEventRecord(d.side_join, d.side);
         cudaStreamWaitEvent(s, d.side_join, 0);
     }
-    // the cells of tiers 0 and 1 that it left
-    k_merge_lv<E, false><<<152 * 4, MERGE_NW1 * 32, smt, s>>>(
-        P, A, A32, d.cell_start, d.gain, d.photos, d.photo_sorted, d.photo_off, d.out_start, d.work_off, d.work,
-        d.work_cap, out, out32, cout, Gphys, d.mover_cap, d.photo_cap, d.tie_list, d.list_n, 3, MERGE_CAP1, d.ctr);
 }
 
 void launch_merges(const Params& P, Dev& d, uint64_t G, cudaStream_t s)

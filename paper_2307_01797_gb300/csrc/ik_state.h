@@ -140,8 +140,7 @@ struct Dev {
     uint32_t* small_list = nullptr;    // G: non-empty cells of merge tier 0 (small shared scratch)
     uint32_t* mid_list = nullptr;      // G: ... tier 1 (large shared scratch)
     uint32_t* big_list = nullptr;      // G: ... tier 2 (scratch in the work area)
-    uint32_t* tie_list = nullptr;      // Gp: cells of tiers 0 and 1 left to the merge with a sort per level
-    uint32_t* list_n = nullptr;        // 4 counts: tiers 0, 1, 2 and the ties
+    uint32_t* list_n = nullptr;        // 5 counts: tiers 0, 1, 2, and of tiers 0 and 1 those left to the merge with a sort per level
     uint32_t* pc_list = nullptr;       // G: photon-emitting cells
     uint32_t* kmc_list = nullptr;      // G: cells of the last KMC (outside them fired and gain are zero)
     uint32_t* kmc_n = nullptr;         // its length
