@@ -1014,13 +1014,13 @@ int itokmc_init(const itokmc_config* cfg, itokmc_handle** out)
     d.work_off = dalloc_n<uint64_t>(h, Gp + 1, &rc);
     d.small_list = dalloc_n<uint32_t>(h, Gp, &rc);
     d.mid_list = dalloc_n<uint32_t>(h, Gp, &rc);
-    d.big_list = dalloc_n<uint32_t>(h, Gp, &rc);
-    d.list_n = dalloc_n<uint32_t>(h, 5, &rc);
+    d.big_list = d.mid_list + (Gp - 1);
+    d.list_n = dalloc_n<uint32_t>(h, 6, &rc);
     d.pc_list = dalloc_n<uint32_t>(h, G, &rc);
     d.kmc_list = dalloc_n<uint32_t>(h, G, &rc);
-    d.kmc_n = dalloc_n<uint32_t>(h, 1, &rc);
+    d.kmc_n = d.list_n + 5;
     set_work(h, reinterpret_cast<unsigned char*>(dalloc(h, d.work_cap * 32, &rc)), d.work_cap);
-    const size_t se = 2 * std::max(std::max(ik::scan_scratch_elems(Gp, 6), ik::scan_scratch_elems(nblk, 3)),
+    const size_t se = 2 * std::max(std::max(ik::scan_scratch_elems(Gp, 5), ik::scan_scratch_elems(nblk, 3)),
                                    ik::radix_scratch_elems(h->cap));
     d.scan_blk = dalloc_n<long long>(h, se, &rc);
     d.scan_blk_elems = se;
@@ -1035,19 +1035,22 @@ int itokmc_init(const itokmc_config* cfg, itokmc_handle** out)
         L.h = P.h[0] * (double)(n / m);
         L.phi = dalloc_n<double>(h, cells, &rc);
         L.rhs = dalloc_n<double>(h, cells, &rc);
-        L.phi32 = dalloc_n<float>(h, cells, &rc);
-        L.rhs32 = dalloc_n<float>(h, cells, &rc);
+        L.phi32 = dalloc_n<float>(h, 2 * cells, &rc);
+        L.rhs32 = L.phi32 + cells;
+        // the sweeps' second array and the fixed-point arrays lie where this
+        // form of the solve keeps nothing: the FP64 form's second array (and
+        // the scales) over its FP32 ones, the mixed form's over the FP64
+        // potential of a coarse level and, on the finest, like the FP64 form's
+        // integers, in the last two thirds of the upload buffer (no call uses
+        // it during a solve but the autotuner, which keeps the first third)
         const bool f64 = h->field_prec == ITOKMC_FP64;
-        L.alt = m > 32 ? dalloc(h, cells * (f64 ? sizeof(double) : sizeof(float)), &rc) : nullptr;
-        L.phi_fix = reinterpret_cast<long long*>(L.phi);
-        L.rhs_fix = reinterpret_cast<long long*>(L.rhs);
-        if (l == 0 && f64) {
-            L.phi_fix = dalloc_n<long long>(h, cells, &rc);
-            L.rhs_fix = dalloc_n<long long>(h, cells, &rc);
-            d.fix = dalloc_n<ik::FixScale>(h, R, &rc);
-        }
+        L.alt = f64 ? static_cast<void*>(L.phi32) : l > 0 ? static_cast<void*>(L.phi) : d.stage + 2 * cells;
+        L.phi_fix = reinterpret_cast<long long*>(l == 0 ? d.stage + cells : L.phi);
+        L.rhs_fix = reinterpret_cast<long long*>(l == 0 ? d.stage + 2 * cells : L.rhs);
     }
     d.nlev = l;
+    // (64 R cells of two floats, for R scales)
+    if (h->field_prec == ITOKMC_FP64) d.fix = reinterpret_cast<ik::FixScale*>(d.lev[l - 1].phi32);
     const size_t nb = (size_t)R * n * n * n / 256 + 16;
     d.norm_part = dalloc_n<double>(h, 2 * nb, &rc);
     d.norm_out = dalloc_n<double>(h, 2 * R, &rc);
@@ -1313,7 +1316,8 @@ int itokmc_autotune(itokmc_handle* h, itokmc_tuning* out)
     ik::Dev& d = h->d;
     const size_t cells = h->G;
     double* phi0 = d.lev[0].phi;
-    // the stage buffer (3 G doubles) holds the initial potential
+    // the first third of the stage buffer holds the initial potential (the
+    // solves use the rest)
     IK_CHECK(h, cudaMemcpyAsync(d.stage, phi0, cells * sizeof(double), cudaMemcpyDeviceToDevice, h->s));
     const int F0 = d.phi_F;
     itokmc_tuning t{};

@@ -1559,7 +1559,7 @@ struct MergeScanOp {
     uint32_t* photo_off;
     uint32_t* small_list;     // non-empty cells of tier 0
     uint32_t* mid_list;       // ... tier 1
-    uint32_t* big_list;       // ... tier 2
+    uint32_t* big_list;       // ... tier 2 (downwards)
     uint32_t* list_n;         // [3]: lengths
     uint64_t G;               // particle cells
     uint64_t Gphys;           // physical cells (one block per realization)
@@ -1623,7 +1623,7 @@ struct MergeScanOp {
             po[k] = e[1];
             if (v[k][2]) small_list[e[2]] = (uint32_t)(g + k);
             if (v[k][3]) mid_list[e[3]] = (uint32_t)(g + k);
-            if (v[k][4]) big_list[e[4]] = (uint32_t)(g + k);
+            if (v[k][4]) *(big_list - e[4]) = (uint32_t)(g + k);
 #pragma unroll
             for (int c = 0; c < 5; ++c) e[c] += v[k][c];
         }
@@ -1650,7 +1650,7 @@ __global__ void k_big_work(Params P, const uint32_t* __restrict__ big_list, cons
 {
     const uint32_t n = list_n[2];
     for (uint32_t li = blockIdx.x * blockDim.x + threadIdx.x; li < n; li += gridDim.x * blockDim.x) {
-        const uint64_t g = big_list[li];
+        const uint64_t g = *(big_list - li);
         const uint64_t sp = (uint64_t)(g >= Gphys) + (uint64_t)(g >= 2 * Gphys);
         const long long dN = gain[g];
         const long long M = (long long)(cs[g + 1] - cs[g]) + (dN > 0 ? (dN < P.n_new ? dN : P.n_new) : 0) +
@@ -1982,7 +1982,7 @@ __global__ void __launch_bounds__(128, GLOBAL ? 4 : (std::is_same<E, MP32>::valu
     const uint32_t ncells = list_n[tier];
     unsigned long long t_cells = 0, t_el = 0, t_sq = 0, t_max = 0;
     for (uint32_t li = blockIdx.x * nw + wid; li < ncells; li += gridDim.x * nw) {
-        const uint64_t g = list[li];                  // particle cell
+        const uint64_t g = GLOBAL ? *(list - li) : list[li];      // particle cell
         MLayout L;
         unsigned char* base;
         uint32_t max_m;

@@ -139,7 +139,7 @@ struct Dev {
     uint64_t* work_off = nullptr;      // G + 1
     uint32_t* small_list = nullptr;    // G: non-empty cells of merge tier 0 (small shared scratch)
     uint32_t* mid_list = nullptr;      // G: ... tier 1 (large shared scratch)
-    uint32_t* big_list = nullptr;      // G: ... tier 2 (scratch in the work area)
+    uint32_t* big_list = nullptr;      // ... tier 2 (scratch in the work area), down from mid_list's end
     uint32_t* list_n = nullptr;        // 5 counts: tiers 0, 1, 2, and of tiers 0 and 1 those left to the merge with a sort per level
     uint32_t* pc_list = nullptr;       // G: photon-emitting cells
     uint32_t* kmc_list = nullptr;      // G: cells of the last KMC (outside them fired and gain are zero)
@@ -161,7 +161,7 @@ struct Dev {
     uint32_t* sort_tmp = nullptr;      // radix-sort scratch (4 x capacity u32)
     uint32_t mover_cap = 0, photo_cap = 0;
     uint64_t work_cap = 0;             // merge work area, 32-byte units
-    double* stage = nullptr;           // 3 G doubles: field upload/readback
+    double* stage = nullptr;           // 3 G doubles: field upload/readback; arrays of the field solve
     // CUDA graphs of the cycles (run_cycles), captured once per smoother pair
     // and replayed
     cudaGraphExec_t vgraph[4] = {};
