@@ -1506,27 +1506,7 @@ float* lrhs<float>(MGLevel& L) { return L.rhs32; }
 template <>
 long long* lrhs<long long>(MGLevel& L) { return L.rhs_fix; }
 
-// Shared memory beyond 48 KB needs an opt-in per kernel and device.
 constexpr int SMALL_R = 4;
-
-template <class F>
-void allow_smem(F* kernel, size_t bytes)
-{
-    static std::mutex mtx;
-    static F* seen[8] = {};                     // kernels of one signature
-    static unsigned long long done[8] = {};     // devices they are opted in on
-    int dev = 0;
-    cudaGetDevice(&dev);
-    std::lock_guard<std::mutex> lk(mtx);
-    int k = 0;
-    while (k < 8 && seen[k] && seen[k] != kernel) ++k;
-    if (k < 8 && dev >= 0 && dev < 64 && seen[k] && ((done[k] >> dev) & 1u)) return;
-    cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
-    if (k < 8 && dev >= 0 && dev < 64) {
-        seen[k] = kernel;
-        done[k] |= 1ull << dev;
-    }
-}
 
 // Two sweeps of level l from src (nullptr: zeros) into dst.  The z chunk is
 // the one with the least modelled time: waves of resident blocks (one per SM)

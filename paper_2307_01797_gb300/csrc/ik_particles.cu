@@ -3210,12 +3210,8 @@ void launch_merge_tiers(const Params& P, Dev& d, uint64_t G, cudaStream_t s, con
     const size_t sm1 = (size_t)pre_layout(MERGE_CAP1, P.ppc, sizeof(K)).bytes * MERGE_NW1;
     const size_t smt0 = (size_t)merge_layout(cap0, P.ppc, sizeof(E), sizeof(K)).bytes * MERGE_NW0;
     const size_t smt1 = (size_t)merge_layout(MERGE_CAP1, P.ppc, sizeof(E), sizeof(K)).bytes * MERGE_NW1;
-    static bool attr = false;
-    if (!attr) {
-        cudaFuncSetAttribute(k_merge_lv<E, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
-        cudaFuncSetAttribute(k_merge_pre<E>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
-        attr = true;
-    }
+    allow_smem(k_merge_lv<E, false>, 200 * 1024);
+    allow_smem(k_merge_pre<E>, 200 * 1024);
     g_launches += 5;
     const uint64_t Gphys = (uint64_t)P.R * P.n3;
     // tiers 1 and 2 (few, long cells) on the side stream beside tier 0

@@ -4,6 +4,7 @@
 #include <cstddef>
 #include <atomic>
 #include <cstdint>
+#include <mutex>
 #include <cmath>
 #include <cuda_runtime.h>
 
@@ -51,6 +52,27 @@ constexpr uint32_t KEY_MASK = 0x3fffffffu;
 
 constexpr int TPB = 256;        // threads per block of the particle passes
 constexpr int MAX_R = 1024;     // realizations per handle
+
+// Shared memory beyond 48 KB needs an opt-in per kernel and device (handles may
+// live on several, and launch from several threads).
+template <class F>
+void allow_smem(F* kernel, size_t bytes)
+{
+    static std::mutex mtx;
+    static F* seen[8] = {};                     // kernels of one signature
+    static unsigned long long done[8] = {};     // devices they are opted in on
+    int dev = 0;
+    cudaGetDevice(&dev);
+    std::lock_guard<std::mutex> lk(mtx);
+    int k = 0;
+    while (k < 8 && seen[k] && seen[k] != kernel) ++k;
+    if (k < 8 && dev >= 0 && dev < 64 && seen[k] && ((done[k] >> dev) & 1u)) return;
+    cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+    if (k < 8 && dev >= 0 && dev < 64) {
+        seen[k] = kernel;
+        done[k] |= 1ull << dev;
+    }
+}
 
 // Device counters of one step (zeroed at the start of each stage).
 struct Counters {
