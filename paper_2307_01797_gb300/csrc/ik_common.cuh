@@ -515,17 +515,6 @@ __device__ __forceinline__ double quot_r(double a, double b, double r)
     return __fma_rn(__fma_rn(-q0, b, a), r, q0);
 }
 
-__device__ __forceinline__ void cic_axis(double x, double lo, double h, double rh, int n, int& ia, int& ib,
-                                         double& f)
-{
-    const double u = grid_quot(x, lo, h, rh) - 0.5;
-    const double fl = floor(u);
-    const int i0 = (int)fl;
-    f = u - fl;
-    ia = clampi(i0, n);
-    ib = clampi(i0 + 1, n);
-}
-
 // Cell of a coordinate known to lie in [lo, hi): floor((x-lo)/h), clamped.
 __device__ __forceinline__ int cell_axis(double x, double lo, double h, double rh, int n)
 {

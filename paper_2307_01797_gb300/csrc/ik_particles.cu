@@ -48,8 +48,6 @@ __device__ __forceinline__ E64 ld_e64(const E64* p)
     return E64{ a.x, a.y, b.x, b.y };
 }
 
-// Trilinear interpolation of the cell-centred field at (x,y,z); sum order z
-// outer, y, x inner; weight (wx*wy)*wz.
 // F 2^-sh as a double (F < 2^sh, sh <= 53: exact).
 __device__ __forceinline__ double qfrac(unsigned long long F, int sh)
 {
@@ -58,9 +56,11 @@ __device__ __forceinline__ double qfrac(unsigned long long F, int sh)
     const unsigned long long mant = (F << (52 - pb)) & 0xfffffffffffffull;
     return __longlong_as_double((long long)(((unsigned long long)(pb - sh + 1023) << 52) | mant));
 }
-// cic_axis with the split above (the FP64 steps for qd < 1/2); g = 1 - f,
-// exact: 2^sh - F is at most 2^sh, so (2^sh - F) 2^-sh is the same double
-// as the FP64 subtraction 1 - f.
+// The two cells ia, ib (clamped) that the coordinate x of axis a lies between by
+// their centres, with the fraction f of the way to the second: u = (x - lo) / h
+// - 1/2, ia = floor(u), f = u - ia, from the quotient's split (in FP64 steps for
+// quotients below 1/2).  g = 1 - f, exact: 2^sh - F is at most 2^sh, so (2^sh -
+// F) 2^-sh is the same double as the FP64 subtraction 1 - f.
 __device__ __forceinline__ void cic_axis_q(const Params& P, double x, int a, int& ia, int& ib, double& f, double& g)
 {
     QSplit t;
@@ -85,7 +85,8 @@ __device__ __forceinline__ void cic_axis_q(const Params& P, double x, int a, int
     ia = clampi(i0, P.n);
     ib = clampi(i0 + 1, P.n);
 }
-// The loops over the axes and over z stay loops, an axis' values rotating
+// Trilinear interpolation of the cell-centred field at X; sum order z outer, y, x
+// inner; weight (wx*wy)*wz.  The loops over the axes and over z stay loops, an axis' values rotating
 // through registers: with them unrolled a quarter of the push's issue slots
 // waited for instructions.
 __device__ __forceinline__ void interp_f64(const Params& P, const E64* __restrict__ E, const double X[3],
