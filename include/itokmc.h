@@ -63,7 +63,8 @@ extern "C" {
 #define ITOKMC_ERR_INTERNAL (-10)  /* a self-check of the library failed     */
 
 /* ---- precision forms --------------------------------------------------- */
-#define ITOKMC_FP64 0   /* FP64 positions/push/KMC, FP64 multigrid (parity) */
+#define ITOKMC_FP64 0   /* FP64 positions/push/KMC and potential, multigrid */
+                        /* in 64-bit fixed point (parity)                   */
 #define ITOKMC_MIXED 1  /* FP32 cell-relative positions, push and KMC,      */
                         /* int64 fixed-point deposit; the potential held in */
                         /* int64 fixed point, its residual formed exactly   */

@@ -585,7 +585,12 @@ __global__ void k_efield_fixed(const long long* __restrict__ Phi, E64* __restric
 // checkpoint, itokmc_read_densities).  Each realization has its own scale: a
 // member of a batch keeps its bits beside one of a far higher potential.
 // FIX_LIM marks an iterate that left its range: the solve then goes on with
-// FP64 cycles.
+// FP64 cycles.  Sums, residuals and relaxations hold for |Phi| below it; the
+// interpolation forms 64 times a correction and holds for corrections below
+// 2^57, which the scales leave room for: guess and solution are at most half of
+// a bound below 2^57 each.  A correction beyond that (a cycle that overshoots, a
+// step whose potential grows more than fivefold) wraps, and the next check finds
+// a residual that has not fallen.
 constexpr long long FIX_LIM = 1ll << 59;
 
 // The bits by which a scale can go up that a loose bound (k_fix_scale) left too
@@ -671,12 +676,12 @@ __global__ void __launch_bounds__(256) k_fix_start(double* __restrict__ phi, dou
     }
 }
 
-// The scale of each realization.  Mc bounds |phi| of the solution: electrode potential plus the
-// 1D Dirichlet bound max|h^2 b| n^2 / 8, doubled.  A guess extrapolated from
-// the last steps is near the solution: four times its modulus bounds it (Mc
-// is loose by orders of magnitude for a localised charge; a single cell's
-// potential is about a quarter of its |h^2 b|, so that at least FIX_BITS bits
-// hold it).  use64: the guess is not finite or far above the solution.
+// The scale of each realization.  Mc bounds |phi| of the solution: electrode
+// potential plus the 1D Dirichlet bound max|h^2 b| n^2 / 8, doubled.  A guess
+// extrapolated from the last steps is near the solution: four times its modulus
+// bounds it (Mc is loose by orders of magnitude for a localised charge; a single
+// cell's potential is about a quarter of its |h^2 b|, so that at least FIX_BITS
+// bits hold it).  use64: the guess is not finite or far above the solution.
 __global__ void k_fix_scale(FixScale* fs, int R, double phi_top, int n, int near, int rescale)
 {
     const int r = blockIdx.x * blockDim.x + threadIdx.x;
@@ -931,13 +936,14 @@ dim3 grid_per_real(const Geo& G)
 // shared memory) and ends with a cluster barrier.  The 8^3 level runs in the
 // cluster's first block, the 4^3 bottom (48 red-black sweep pairs) in one warp
 // with the cells in registers (64-bit forms: solved by its eigenvectors).
-// What bounds it is a chain of latencies (21 cluster barriers, 96 warp
-// half-sweeps), not bandwidth: 29 us in fixed point, 25 us in FP32 from 32^3
-// down (33 and 28 with the interpolation cell by cell, every thread's fence at
-// the barriers, a divisor formed per cell and the loads after the zeros; clusters
-// of 16 blocks took 1 us off when they found 16 free SMs in one GPC, which other
-// streams' kernels may hold); one block per realization from 16^3 down took 159 us in FP64 and 96 us
-// in FP32, after 10 launches for the 32^3 level.
+// What bounds it is a chain of latencies (22 cluster barriers from 32^3 down with
+// two sweeps before and after; in FP32 96 warp half-sweeps at the bottom), not
+// bandwidth: 29 us in fixed point, 25 us in FP32 from 32^3 down (33 and 28 with
+// the interpolation cell by cell, every thread's fence at the barriers, a divisor
+// formed per cell and the loads after the zeros; clusters of 16 blocks took 1 us
+// off when they found 16 free SMs in one GPC, which other streams' kernels may
+// hold); one block per realization from 16^3 down took 159 us in FP64 and 96 us in
+// FP32, after 10 launches for the 32^3 level.
 constexpr int COARSE_N = 32, COARSE_CL = 8, COARSE_TPB = 512, BOTTOM_SWEEPS = 48;
 
 template <class T>
@@ -1358,8 +1364,9 @@ __global__ void __cluster_dims__(COARSE_CL, 1, 1) __launch_bounds__(COARSE_TPB, 
 // same to the last bit.  Cells outside the domain relax like the others, with
 // a divisor of zero: no branch per cell (FP32 at 512^3 564 -> 521 us, fixed
 // point at 256^3 202 -> 180 us).  Two sweeps of 256^3 cells: 180 us in fixed
-// point (bound by its integer instructions) against 508 us for four FP64
-// half-sweeps (FP64 pipe 82% busy).
+// point (128 blocks on 152 SMs, which issue 65% of the time; the next plane's
+// loads are the largest stall) against 508 us for four FP64 half-sweeps (FP64
+// pipe 82% busy).
 //
 // The tile: 64 x 32 in FP32 (two pairs per thread), 32 x 32 in 64 bits.  A
 // 64^3 level has too few of these for the chip's SMs: 32 x 16 there, with one
@@ -1854,8 +1861,8 @@ constexpr int MAX_REAL_NORM = 4096;
 
 // Replays (capturing first if needed) the graph of kind k on stream s:
 // k = 0: one FP64 V-cycle; k = 1: two FP32 V-cycles from a zero correction;
-// k = 3: one fixed-point V-cycle.  The launches of a cycle depend only on the level pointers and
-// the smoother counts, so one capture per (nu1, nu2) serves every solve.
+// k = 3: one fixed-point V-cycle.  The launches of a cycle depend only on the
+// level pointers and the smoother counts, so one capture per (nu1, nu2) serves every solve.
 // Launches directly when d.direct_cycles is set (a solve on per-call
 // buffers, whose graphs could not be reused) or capture is not possible.
 void run_cycles(Dev& d, int k, int R, int nu1, int nu2, cudaStream_t s)
@@ -1906,11 +1913,6 @@ void run_cycles(Dev& d, int k, int R, int nu1, int nu2, cudaStream_t s)
     cudaGraphLaunch(d.vgraph[k], s);
 }
 
-// precision: 0 FP64 V-cycles; 1 FP32 V-cycles in FP64 residual refinement;
-// 2 FP32 V-cycles in fixed-point residual refinement (potential in units of
-// 2^-phi_F V, right-hand side prepared by the charge kernel).  Returns 0 on
-// convergence, ITOKMC_ERR_NOCONV (-6) if max_cycles is reached or the
-// potential leaves the fixed-point range.
 // Lowers the fixed-point potential's scale to F bits (F < d.phi_F): the
 // potential and the kept previous one shifted right by the difference.
 void lower_phi_scale(const Params& P, Dev& d, int F, cudaStream_t s)
@@ -1949,6 +1951,13 @@ bool fix_begin(const Params& P, Dev& d, bool extrapolate, cudaStream_t s)
     return near;
 }
 
+// precision: 0 V-cycles in 64-bit fixed point, followed by FP64 ones where the
+// integers do not serve (a start guess or an iterate beyond their range, a
+// tolerance below what they reach); 1 FP32 V-cycles in FP64 residual refinement;
+// 2 FP32 V-cycles in fixed-point residual refinement (potential in units of
+// 2^-phi_F V, right-hand side prepared by the charge kernel).  Returns 0 on
+// convergence, ITOKMC_ERR_NOCONV (-6) if max_cycles is reached or the potential
+// of form 2 leaves its range.
 int field_solve(const Params& P, Dev& d, int precision, double rtol, int nu1, int nu2, unsigned long long rho_absmax,
                 int max_cycles, cudaStream_t s, int* cycles_out, double* rel_out, bool extrapolate)
 {

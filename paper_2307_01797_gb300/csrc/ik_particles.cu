@@ -469,9 +469,9 @@ __device__ __forceinline__ float znormal32(PairStream& s)
 }
 
 // ------------------------------------------------------------------ pass 1
-// Bound by issue (3100 instructions per warp at 54% of the slots) and the FP64
-// pipe together: 9.7 ms for 7.2e7 particles, 19.5 ms with the quotients and
-// the wedge tests of the normals on the FP64 pipe and the loops unrolled.
+// Bound by the FP64 pipe (81% busy; 2340 instructions per warp at 43% of the
+// issue slots): 9.7 ms for 7.2e7 particles, 19.5 ms with the quotients and the
+// wedge tests of the normals on the FP64 pipe and the loops unrolled.
 __global__ void __launch_bounds__(TPB, 4) k_push_f64(
     Params P, const P64* __restrict__ A, P64* __restrict__ B, uint32_t* __restrict__ keyB, uint32_t N,
     const uint32_t* __restrict__ cell_start, const E64* __restrict__ E, int32_t* __restrict__ cnt_new,
@@ -2310,9 +2310,9 @@ __global__ void __launch_bounds__(128, GLOBAL ? 4 : (std::is_same<E, MP32>::valu
 // on 64^3 without diffusion, two thirds of them with copies: 250 us in the FP64
 // form and 175 us in the mixed one (365 and 220 us with all of those sorted per
 // level; k_merge_lv alone for every cell 250 and 148 us).
-// Bound by instruction issue (80% of the slots; about 4000 per warp and cell
-// of 28 elements, k_merge_lv twice that in the FP64 form); seven blocks per SM
-// measured best of six to nine.
+// Bound by instruction issue (69% of the slots in the FP64 form, 75% in the mixed
+// one; about 4000 per warp and cell of 28 elements, k_merge_lv twice that in the
+// FP64 form); seven blocks per SM measured best of six to nine.
 struct __align__(16) MNode {     // a node
     uint32_t W, S;               // weight; weights of the nodes before it
     uint16_t s0, n;              // first position, entries
