@@ -681,7 +681,10 @@ __global__ void __launch_bounds__(256) k_fix_start(double* __restrict__ phi, dou
 // extrapolated from the last steps is near the solution: four times its modulus
 // bounds it (Mc is loose by orders of magnitude for a localised charge; a single
 // cell's potential is about a quarter of its |h^2 b|, so that at least FIX_BITS
-// bits hold it).  use64: the guess is not finite or far above the solution.
+// bits hold it).  near: 1 unless the guess is so far below the bound that the
+// charge may be another one (a looser scale is raised after the first cycle), 2 in
+// any case (replayed steps, whose scale stays).  use64: the guess is not finite or
+// far above the solution.
 __global__ void k_fix_scale(FixScale* fs, int R, double phi_top, int n, int near, int rescale)
 {
     const int r = blockIdx.x * blockDim.x + threadIdx.x;
@@ -694,7 +697,7 @@ __global__ void k_fix_scale(FixScale* fs, int R, double phi_top, int n, int near
     } else {
         const double mp = __longlong_as_double((long long)fs->max_phi), mb = __longlong_as_double((long long)fs->max_b);
         const double Mc = 2.0 * (fabs(phi_top) + mb * (double)n * (double)n / 8.0);
-        double M = near && mp > 0.0 ? fmin(Mc, fmax(4.0 * mp, 2.0 * (mb + fabs(phi_top)))) : fmax(Mc, 2.0 * mp);
+        double M = near && mp > 0.0 && (near == 2 || mp * 16384.0 >= Mc) ? fmin(Mc, fmax(4.0 * mp, 2.0 * (mb + fabs(phi_top)))) : fmax(Mc, 2.0 * mp);
         M = fmax(M, 0x1p-400);
         fs->use64 = !(mp <= 16.0 * Mc) || !(Mc < 0x1p400);
         if (!(M < 0x1p400)) M = 1.0;
@@ -1931,8 +1934,9 @@ void lower_phi_scale(const Params& P, Dev& d, int F, cudaStream_t s)
 }
 
 // FP64 form, before the cycles: start guess, scale, Phi and B.
-// Returns whether the scale was taken from the guess (else from the bound).
-bool fix_begin(const Params& P, Dev& d, bool extrapolate, cudaStream_t s)
+// Returns whether the scale may have been taken from the guess (else it is from
+// the bound).
+bool fix_begin(const Params& P, Dev& d, bool extrapolate, bool replayed, cudaStream_t s)
 {
     MGLevel& L0 = d.lev[0];
     const Geo G0 = geo(d, 0, P.R);
@@ -1943,7 +1947,8 @@ bool fix_begin(const Params& P, Dev& d, bool extrapolate, cudaStream_t s)
     g_launches += 3;
     k_fix_start<<<grid_per_real(G0), 256, 0, s>>>(L0.phi, reinterpret_cast<double*>(d.phi_prev), ex, d.have_prev, L0.rhs,
                                                   G0, bc_top * (L0.h * L0.h), d.fix);
-    k_fix_scale<<<(P.R + 255) / 256, 256, 0, s>>>(d.fix, P.R, P.E0 * (P.hi[2] - P.lo[2]), G0.n, ex && d.have_prev, 0);
+    k_fix_scale<<<(P.R + 255) / 256, 256, 0, s>>>(d.fix, P.R, P.E0 * (P.hi[2] - P.lo[2]), G0.n,
+                                                 ex && d.have_prev ? (replayed ? 2 : 1) : 0, 0);
     k_fix_load<<<grid_per_real(G0), 256, 0, s>>>(L0.phi, L0.rhs, L0.phi_fix, L0.rhs_fix, G0.cells / P.R, d.fix, 0);
     const bool near = ex && d.have_prev;
     if (ex) d.have_prev = true;
@@ -1997,7 +2002,7 @@ int field_solve(const Params& P, Dev& d, int precision, double rtol, int nu1, in
         }
     }
     bool near = false;                  // fixed point: the scale is from a guess that ought to be near
-    if (fix) near = fix_begin(P, d, extrapolate, s);
+    if (fix) near = fix_begin(P, d, extrapolate, false, s);
     const float rsc = (float)std::ldexp(1.0, -d.phi_F);
     const float esc = (float)std::ldexp(1.0, d.phi_F);
     // FP64 form: the residual norm only serves the convergence test, so
@@ -2105,7 +2110,7 @@ int field_solve(const Params& P, Dev& d, int precision, double rtol, int nu1, in
                 k_add_correction<<<gridsz(G0.cells, 256), 256, 0, s>>>(L0.phi, L0.phi32, G0.cells);
         } else {
             run_cycles(d, fix ? 3 : 0, R, nu1, nu2, s);
-            if (fix && few && cyc == 0 && !near) {
+            if (fix && few && cyc == 0) {
                 // after one cycle the potential is known well enough for a
                 // scale that the bound left too low (no wait for it)
                 g_launches += 3;
@@ -2155,7 +2160,7 @@ void field_solve_fixed(const Params& P, Dev& d, int precision, int nu1, int nu2,
             d.have_prev = true;
         }
     } else if (precision == 0) {
-        fix_begin(P, d, true, s);
+        fix_begin(P, d, true, true, s);
     }
     const float rsc = (float)std::ldexp(1.0, -d.phi_F);
     const float esc = (float)std::ldexp(1.0, d.phi_F);
