@@ -1015,10 +1015,10 @@ int itokmc_init(const itokmc_config* cfg, itokmc_handle** out)
     d.small_list = dalloc_n<uint32_t>(h, Gp, &rc);
     d.mid_list = dalloc_n<uint32_t>(h, Gp, &rc);
     d.big_list = d.mid_list + (Gp - 1);
-    d.list_n = dalloc_n<uint32_t>(h, 6, &rc);
+    d.list_n = dalloc_n<uint32_t>(h, ik::LIST_COUNTS, &rc);
     d.pc_list = dalloc_n<uint32_t>(h, G, &rc);
     d.kmc_list = dalloc_n<uint32_t>(h, G, &rc);
-    d.kmc_n = d.list_n + 5;
+    d.kmc_n = d.list_n + ik::LIST_KMC;
     set_work(h, reinterpret_cast<unsigned char*>(dalloc(h, d.work_cap * 32, &rc)), d.work_cap);
     const size_t se = 2 * std::max(std::max(ik::scan_scratch_elems(Gp, 5), ik::scan_scratch_elems(nblk, 3)),
                                    ik::radix_scratch_elems(h->cap));

@@ -1638,7 +1638,7 @@ struct MergeScanOp {
         list_n[0] = (uint32_t)t[2];
         list_n[1] = (uint32_t)t[3];
         list_n[2] = (uint32_t)t[4];
-        list_n[3] = list_n[4] = 0;   // cells of tiers 0 and 1 that the merge by presorted lists leaves to k_merge_lv
+        for (int t = 0; t < 2; ++t) list_n[LIST_TIED + t] = list_n[LIST_REST + t] = 0;
     }
 };
 
@@ -2304,12 +2304,14 @@ __global__ void __launch_bounds__(128, GLOBAL ? 4 : (std::is_same<E, MP32>::valu
 // The order of two elements with equal coordinates along an axis depends on the
 // splits before.  Copies (equal along all axes, as after a split of one particle
 // without diffusion) keep the cell's order through every stable sort, so they
-// take it in all three lists.  Cells with two elements that are equal along one
-// axis and not along another, and cells of 2^31 electrons or more (the sums here
-// have 32 bits), are listed for k_merge_lv, which sorts per level.  46000 cells
-// on 64^3 without diffusion, two thirds of them with copies: 250 us in the FP64
-// form and 175 us in the mixed one (365 and 220 us with all of those sorted per
-// level; k_merge_lv alone for every cell 250 and 148 us).
+// take it in all three lists: a cell with equal coordinates is listed for a second
+// pass (TIED), which ranks it so.  Cells with two elements that are equal along
+// one axis and not along another, and cells of 2^31 electrons or more (the sums
+// here have 32 bits), are left to k_merge_lv, which sorts per level.  A particles
+// stage on 64^3 without diffusion, two thirds of 46000 cells with copies: 0.50 ms
+// in the FP64 form and 0.35 ms in the mixed one (0.61 and 0.40 ms with all of
+// those sorted per level, 0.53 and 0.37 ms when that form merged every cell).
+// Ranking them in the first pass (0.47 and 0.32 ms) slows the others by 2% to 3%.
 // Bound by instruction issue (69% of the slots in the FP64 form, 75% in the mixed
 // one; about 4000 per warp and cell of 28 elements, k_merge_lv twice that in the
 // FP64 form); seven blocks per SM measured best of six to nine.
@@ -2378,9 +2380,9 @@ __device__ __forceinline__ uint32_t count_below(const unsigned long long* ka, ui
 
 // The three lists of a cell with equal keys, these in the cell's order; returns
 // whether it holds for the levels too: no two elements are equal along one axis
-// and not along another.  (Not inlined: it would cost the kernel registers.)
+// and not along another.
 template <class K>
-__device__ __noinline__ bool rank_copies(const K* key0, uint32_t KS, uint32_t* ls, uint32_t M, unsigned lane)
+__device__ __forceinline__ bool rank_copies(const K* key0, uint32_t KS, uint32_t* ls, uint32_t M, unsigned lane)
 {
     const unsigned full = 0xffffffffu;
     __syncwarp();
@@ -2416,14 +2418,15 @@ __device__ __noinline__ bool rank_copies(const K* key0, uint32_t KS, uint32_t* l
     return !__any_sync(full, differ);
 }
 
-template <class E>
+// TIED: the cells that the pass without it left.
+template <class E, bool TIED>
 __global__ void __launch_bounds__(128, 7) k_merge_pre(
     Params P, const P64* __restrict__ A, const P32* __restrict__ A32, const uint32_t* __restrict__ cs,
     const int64_t* __restrict__ gain, const Photo* __restrict__ photos, const uint32_t* __restrict__ photo_sorted,
     const uint32_t* __restrict__ photo_off, const uint32_t* __restrict__ out_start, P64* __restrict__ out,
     P32* __restrict__ out32, uint32_t* __restrict__ cout, uint64_t Gphys, uint32_t cap, uint32_t photo_cap,
-    const uint32_t* __restrict__ list, uint32_t* __restrict__ list_n, int tier, uint32_t CAP,
-    uint32_t* __restrict__ tie_list, Counters* __restrict__ ctr)
+    const uint32_t* __restrict__ list, const uint32_t* __restrict__ list_n, uint32_t CAP,
+    uint32_t* __restrict__ left, uint32_t* __restrict__ left_n, Counters* __restrict__ ctr)
 {
     constexpr bool MX = std::is_same<E, MP32>::value;
     constexpr unsigned FULL = 0xffffffffu;
@@ -2432,7 +2435,7 @@ __global__ void __launch_bounds__(128, 7) k_merge_pre(
     const unsigned lane = lane_id(), wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
     const unsigned lt = (1u << lane) - 1u;
     const int T = P.ppc;
-    const uint32_t ncells = list_n[tier];
+    const uint32_t ncells = *list_n;
     const PreLayout L = pre_layout(CAP, T, sizeof(K));
     unsigned char* const base = msm + (size_t)wid * L.bytes;
     K* const key0 = reinterpret_cast<K*>(base + L.key[0]);
@@ -2465,32 +2468,36 @@ __global__ void __launch_bounds__(128, 7) k_merge_pre(
         // then do not add up to M (M - 1) / 2
         unsigned long long wroot = 0;
         bool other = false;
+        if constexpr (TIED) {
+            for (uint32_t j = lane; j < M; j += 32) wroot += ew[j];
+            other = !rank_copies<K>(key0, KS, ls, M, lane);
+        } else {
 #pragma unroll 1
-        for (int a = 0; a < 3; ++a) {
-            const K* ka = key0 + a * KS;
-            uint32_t total = 0;
-            for (uint32_t b0 = 0; b0 < M; b0 += 32) {
-                const uint32_t j = b0 + lane;
-                const bool ok = j < M;
-                const K kj = ka[ok ? j : 0];
-                const uint32_t rk = count_below(ka, M, kj);
-                if (ok) {
-                    uint8_t* w = reinterpret_cast<uint8_t*>(ls + rk);
-                    w[a] = (uint8_t)j;
-                    total += rk;
-                    if (a == 0) {
-                        w[3] = 0;
-                        wroot += ew[j];
+            for (int a = 0; a < 3; ++a) {
+                const K* ka = key0 + a * KS;
+                uint32_t total = 0;
+                for (uint32_t b0 = 0; b0 < M; b0 += 32) {
+                    const uint32_t j = b0 + lane;
+                    const bool ok = j < M;
+                    const K kj = ka[ok ? j : 0];
+                    const uint32_t rk = count_below(ka, M, kj);
+                    if (ok) {
+                        uint8_t* w = reinterpret_cast<uint8_t*>(ls + rk);
+                        w[a] = (uint8_t)j;
+                        total += rk;
+                        if (a == 0) {
+                            w[3] = 0;
+                            wroot += ew[j];
+                        }
                     }
                 }
+                other |= __reduce_add_sync(FULL, total) != M * (M - 1) / 2;
             }
-            other |= __reduce_add_sync(FULL, total) != M * (M - 1) / 2;
         }
-        if (other) other = !rank_copies<K>(key0, KS, ls, M, lane);
 #pragma unroll
         for (int dd = 16; dd > 0; dd >>= 1) wroot += __shfl_xor_sync(FULL, wroot, dd);
         if (other || wroot >= (1ull << 31)) {
-            if (lane == 0) tie_list[atomicAdd(list_n + 3 + tier, 1u)] = (uint32_t)g;
+            if (lane == 0) left[atomicAdd(left_n, 1u)] = (uint32_t)g;
             __syncwarp();
             continue;
         }
@@ -3212,8 +3219,9 @@ void launch_merge_tiers(const Params& P, Dev& d, uint64_t G, cudaStream_t s, con
     const size_t smt0 = (size_t)merge_layout(cap0, P.ppc, sizeof(E), sizeof(K)).bytes * MERGE_NW0;
     const size_t smt1 = (size_t)merge_layout(MERGE_CAP1, P.ppc, sizeof(E), sizeof(K)).bytes * MERGE_NW1;
     allow_smem(k_merge_lv<E, false>, 200 * 1024);
-    allow_smem(k_merge_pre<E>, 200 * 1024);
-    g_launches += 5;
+    allow_smem(k_merge_pre<E, false>, 200 * 1024);
+    allow_smem(k_merge_pre<E, true>, 200 * 1024);
+    g_launches += 7;
     const uint64_t Gphys = (uint64_t)P.R * P.n3;
     // tiers 1 and 2 (few, long cells) on the side stream beside tier 0
     cudaStream_t s12 = s;
@@ -3223,15 +3231,20 @@ void launch_merge_tiers(const Params& P, Dev& d, uint64_t G, cudaStream_t s, con
         s12 = d.side;
     }
     // the cells that a tier's pass leaves follow it, with the tier's scratch;
-    // their lists lie in two arrays that only the transport fills
-    uint32_t* const left[2] = { reinterpret_cast<uint32_t*>(d.cnt_new), reinterpret_cast<uint32_t*>(d.in_cnt) };
+    // their lists lie in arrays that only the transport fills
+    uint32_t* const tied[2] = { reinterpret_cast<uint32_t*>(d.cnt_new), reinterpret_cast<uint32_t*>(d.in_cnt) };
+    uint32_t* const rest[2] = { reinterpret_cast<uint32_t*>(d.delta), reinterpret_cast<uint32_t*>(d.delta) + Gphys * P.S };
     auto tier = [&](cudaStream_t st, int t, int blocks, const uint32_t* list, uint32_t CAP, size_t sm, size_t smt) {
-        k_merge_pre<E><<<blocks, 128, sm, st>>>(P, A, A32, d.cell_start, d.gain, d.photos, d.photo_sorted, d.photo_off,
-                                                d.out_start, out, out32, cout, Gphys, d.mover_cap, d.photo_cap, list,
-                                                d.list_n, t, CAP, left[t], d.ctr);
+        auto pre = [&](auto kernel, const uint32_t* from, int n, uint32_t* left, int left_n) {
+            kernel<<<blocks, 128, sm, st>>>(P, A, A32, d.cell_start, d.gain, d.photos, d.photo_sorted, d.photo_off,
+                                            d.out_start, out, out32, cout, Gphys, d.mover_cap, d.photo_cap, from,
+                                            d.list_n + n, CAP, left, d.list_n + left_n, d.ctr);
+        };
+        pre(k_merge_pre<E, false>, list, t, tied[t], LIST_TIED + t);
+        pre(k_merge_pre<E, true>, tied[t], LIST_TIED + t, rest[t], LIST_REST + t);
         k_merge_lv<E, false><<<blocks, 128, smt, st>>>(
             P, A, A32, d.cell_start, d.gain, d.photos, d.photo_sorted, d.photo_off, d.out_start, d.work_off, d.work,
-            d.work_cap, out, out32, cout, Gphys, d.mover_cap, d.photo_cap, left[t], d.list_n, 3 + t, CAP, d.ctr);
+            d.work_cap, out, out32, cout, Gphys, d.mover_cap, d.photo_cap, rest[t], d.list_n, LIST_REST + t, CAP, d.ctr);
     };
     tier(s12, 1, 152 * 8, d.mid_list, MERGE_CAP1, sm1, smt1);
     k_merge_lv<E, true><<<152 * 4, 128, 0, s12>>>(

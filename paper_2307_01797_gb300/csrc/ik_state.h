@@ -130,6 +130,10 @@ constexpr int FIX_DOUBLES = (int)(sizeof(FixScale) / sizeof(double));
 
 constexpr int MAX_LEVELS = 12;
 
+// Counts in Dev::list_n: the tiers' cells, the KMC's, and of tiers 0 and 1 the cells
+// with equal coordinates (or 2^31 electrons) and those sorted per level.
+constexpr int LIST_TIED = 3, LIST_REST = 5, LIST_KMC = 7, LIST_COUNTS = 8;
+
 struct Dev {
     // particles (ping-pong)
     P64* recA = nullptr;  P64* recB = nullptr;
@@ -162,7 +166,7 @@ struct Dev {
     uint32_t* small_list = nullptr;    // G: non-empty cells of merge tier 0 (small shared scratch)
     uint32_t* mid_list = nullptr;      // G: ... tier 1 (large shared scratch)
     uint32_t* big_list = nullptr;      // ... tier 2 (scratch in the work area), down from mid_list's end
-    uint32_t* list_n = nullptr;        // 5 counts: tiers 0, 1, 2, and of tiers 0 and 1 those left to the merge with a sort per level
+    uint32_t* list_n = nullptr;        // LIST_COUNTS counts: tiers 0, 1, 2, and the cells that tiers 0 and 1 leave
     uint32_t* pc_list = nullptr;       // G: photon-emitting cells
     uint32_t* kmc_list = nullptr;      // G: cells of the last KMC (outside them fired and gain are zero)
     uint32_t* kmc_n = nullptr;         // its length
