@@ -723,7 +723,13 @@ __global__ void __launch_bounds__(256) k_fix_max(const long long* __restrict__ P
         const unsigned long long a = __shfl_xor_sync(0xffffffffu, mx, d);
         mx = a > mx ? a : mx;
     }
-    if ((threadIdx.x & 31) == 0) atomicMax(&fs[blockIdx.y].max_fix, mx);
+    __shared__ unsigned long long sm[8];
+    if ((threadIdx.x & 31) == 0) sm[threadIdx.x >> 5] = mx;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        for (int w = 1; w < 8; ++w) mx = sm[w] > mx ? sm[w] : mx;
+        atomicMax(&fs[blockIdx.y].max_fix, mx);
+    }
 }
 
 // Phi and B from phi and the right-hand side; rescale: Phi shifted up by sh
@@ -2114,7 +2120,8 @@ int field_solve(const Params& P, Dev& d, int precision, double rtol, int nu1, in
                 // after one cycle the potential is known well enough for a
                 // scale that the bound left too low (no wait for it)
                 g_launches += 3;
-                k_fix_max<<<grid_per_real(G0), 256, 0, s>>>(L0.phi_fix, per_real, d.fix);
+                const dim3 few_blocks(std::min<unsigned>(grid_per_real(G0).x, std::max(1, 152 * 8 / R)), R);
+                k_fix_max<<<few_blocks, 256, 0, s>>>(L0.phi_fix, per_real, d.fix);
                 k_fix_scale<<<(R + 255) / 256, 256, 0, s>>>(d.fix, R, P.E0 * (P.hi[2] - P.lo[2]), G0.n, 0, 2);
                 k_fix_load<<<grid_per_real(G0), 256, 0, s>>>(L0.phi, L0.rhs, L0.phi_fix, L0.rhs_fix, per_real, d.fix, 1);
                 first = true;

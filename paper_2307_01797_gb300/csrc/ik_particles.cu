@@ -3235,14 +3235,15 @@ void launch_merge_tiers(const Params& P, Dev& d, uint64_t G, cudaStream_t s, con
     uint32_t* const tied[2] = { reinterpret_cast<uint32_t*>(d.cnt_new), reinterpret_cast<uint32_t*>(d.in_cnt) };
     uint32_t* const rest[2] = { reinterpret_cast<uint32_t*>(d.delta), reinterpret_cast<uint32_t*>(d.delta) + Gphys * P.S };
     auto tier = [&](cudaStream_t st, int t, int blocks, const uint32_t* list, uint32_t CAP, size_t sm, size_t smt) {
-        auto pre = [&](auto kernel, const uint32_t* from, int n, uint32_t* left, int left_n) {
+        auto pre = [&](auto kernel, int blocks, const uint32_t* from, int n, uint32_t* left, int left_n) {
             kernel<<<blocks, 128, sm, st>>>(P, A, A32, d.cell_start, d.gain, d.photos, d.photo_sorted, d.photo_off,
                                             d.out_start, out, out32, cout, Gphys, d.mover_cap, d.photo_cap, from,
                                             d.list_n + n, CAP, left, d.list_n + left_n, d.ctr);
         };
-        pre(k_merge_pre<E, false>, list, t, tied[t], LIST_TIED + t);
-        pre(k_merge_pre<E, true>, tied[t], LIST_TIED + t, rest[t], LIST_REST + t);
-        k_merge_lv<E, false><<<blocks, 128, smt, st>>>(
+        // (the two that mostly find no cell: as many blocks as are resident)
+        pre(k_merge_pre<E, false>, blocks, list, t, tied[t], LIST_TIED + t);
+        pre(k_merge_pre<E, true>, 152 * 7, tied[t], LIST_TIED + t, rest[t], LIST_REST + t);
+        k_merge_lv<E, false><<<152 * 4, 128, smt, st>>>(
             P, A, A32, d.cell_start, d.gain, d.photos, d.photo_sorted, d.photo_off, d.out_start, d.work_off, d.work,
             d.work_cap, out, out32, cout, Gphys, d.mover_cap, d.photo_cap, rest[t], d.list_n, LIST_REST + t, CAP, d.ctr);
     };
